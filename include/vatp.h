@@ -35,7 +35,7 @@
  *     contiguous (stride fields 0); vatp_prefill_scores_from_lse and win_rows (hence vatp_compact
  *     with a history window) are not available with it (VATP_ERR_UNSUPPORTED), and the workspace
  *     holds a normaliser row per query head and G partial indicators.  The decode step takes
- *     the tensor-core kernel for bf16, head_dim 128 and G <= 8 (VATP_FLAG_DECODE_OVERLAP applies as in the multi-head case) and a
+ *     the tensor-core kernel for bf16 and G <= 8 (VATP_FLAG_DECODE_OVERLAP applies as in the multi-head case) and a
  *     general kernel otherwise; the history rebuild runs a general kernel.
  *   - Inputs are assumed finite.
  *   - A second build of the library (compiled with -DVATP_DEBUG_BOUNDS) range-checks every row, slot,
@@ -136,7 +136,7 @@ size_t vatp_workspace_bytes(const vatp_params* params);
  *           history window is then built by vatp_compact_window, which recomputes the kept columns.
  * workspace: >= vatp_workspace_bytes(params) bytes of device scratch, 256-byte aligned; holds the
  *           row normalisers between the two passes and two work-item counters.
- * bf16 with head_dim 128 runs on the tensor cores; other combinations use an fp32 FMA kernel.
+ * bf16 runs on the tensor cores, fp32 on an FMA kernel.
  */
 vatp_status vatp_prefill_scores(const vatp_params* params, const void* q, const void* k, const void* v,
                                 float* lse_out, float* attn_acc, float* vnorm, float* score,

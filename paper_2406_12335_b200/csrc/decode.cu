@@ -449,7 +449,7 @@ cudaError_t launch_decode(const Shape& s, int dtype, int B, int F, int R, const 
                           const void* k, const void* v, void* out, int32_t* evicted, int32_t* dev_status,
                           cudaStream_t st, bool may_overlap) {
   const bool win = s.window > 0;
-  if (dtype == VATP_BF16 && s.d == 128) {
+  if (dtype == VATP_BF16) {
     const cudaError_t e = launch_decode_mma(s, B, F, R, c, q, k, v, out, evicted, dev_status, st, may_overlap);
     if (e != cudaErrorNotSupported) return e;
   }

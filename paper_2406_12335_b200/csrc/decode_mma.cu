@@ -1,4 +1,4 @@
-// Decode step for bf16, head_dim 128 (the LLaMA2-7B shape): append, attend (Eq. 1), indicator
+// Decode step for bf16, head_dim 64 or 128: append, attend (Eq. 1), indicator
 // update (Eq. 2 / Eq. 3), importance (Eq. 4), release of the lowest-importance unprotected slot.
 //
 // The step is HBM-bound (every cached K and V row is read once) but so short - tens of megabytes -
@@ -53,11 +53,10 @@ namespace {
 // bit-identical whichever kernel a launch gets.
 constexpr int MW_BESIDE = 4, MW_ALONE = 8;
 constexpr int NSTREAM = 8;
-constexpr int HD = 128;
+// (the kernels' template parameter HD: head_dim, 64 or 128)
 constexpr int GROUP = 16;             // rows per MMA group = rows of K (and of V) per stage
-constexpr int ROW_BYTES = HD * 2;
 constexpr int TILE_BYTES = GROUP * 128;    // 16 rows x 64 bf16, 128-byte swizzled
-constexpr int STAGE_BYTES = 4 * TILE_BYTES; // K columns 0-63, K 64-127, V 0-63, V 64-127
+template <int HD> constexpr int stage_bytes = 2 * (HD / 64) * TILE_BYTES; // K columns 0-63 (, K 64-127), V 0-63 (, V 64-127)
 constexpr int MAX_SPLIT = 8;
 constexpr int GQ_HEADS = 8;           // grouped queries: query heads per cache this kernel takes (rows 0-7 of the MMA tiles)
 constexpr int GQ_MAX_SPLIT = MAX_SPLIT;   // ... and the CTAs a unit is split over at most
@@ -140,6 +139,7 @@ __device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier
 __device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // what the CTAs of a unit push into one another
+template <int HD>
 struct Exch {
   float m[MAX_SPLIT], l[MAX_SPLIT];       // in every rank: per rank the max of its logits (log2 domain) and the sum of exp2(s - m)
   float o[MAX_SPLIT][HD];                 // in rank 0: partial outputs of every rank
@@ -165,7 +165,7 @@ __device__ __forceinline__ unsigned long long warp_min_key(unsigned long long ke
 // streaming loop is the same instructions, and every K and V row is read once for the whole group; the maxima,
 // sums and partial outputs exist per head, and the indicator advances by the MEAN of the heads' probabilities.
 // Only the eight-warp kernel is built for it (the per-head partials take the room a second CTA would need).
-template <bool WINDOWED, int MW, int GT>
+template <int HD, bool WINDOWED, int MW, int GT>
 __global__ void __launch_bounds__(MW * 32 + 32, MW == MW_BESIDE ? 2 : 1)
 decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, int independent, int G,
                   int state_in_smem, int split, int chunk, int nstage, int B, int cap, int F, int R, int w, int norm, float scale_log2,
@@ -173,6 +173,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
                   const __nv_bfloat16* __restrict__ q_new, const __nv_bfloat16* __restrict__ k_new,
                   const __nv_bfloat16* __restrict__ v_new, __nv_bfloat16* __restrict__ out,
                   int32_t* __restrict__ evicted, int32_t* __restrict__ dev_status) {
+  constexpr int STAGE_BYTES = stage_bytes<HD>, NTILE = HD / 64, ROW_CHUNKS = HD / 8;   // tiles and 16-byte chunks of a row
   constexpr int WT = MW * 32;           // streaming threads (at least HD: one per output channel where outputs are formed)
   static_assert(WT >= HD, "one streaming thread per output channel");
   static_assert(GT == 1 || (GT == GQ_HEADS && MW == MW_ALONE), "grouped queries: the eight-warp kernel only");
@@ -194,7 +195,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   float* gq_xo = gq_part + NSTREAM * (GT > 1 ? G : 0) * HD;
 
   __shared__ __align__(8) uint64_t bars[MW * 4 + 1];
-  __shared__ __align__(16) Exch ex;
+  __shared__ __align__(16) Exch<HD> ex;
   constexpr int SPW = NSTREAM / MW;     // streams per warp
   static_assert(SPW == 1 || SPW == 2, "a warp folds one or two streams");
   __shared__ __align__(16) float part_o[NSTREAM][HD];
@@ -254,13 +255,13 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncwarp();
-  // lanes 0-3 fetch the four tiles of group g (rows beyond the caches arrive as zeros)
+  // lanes 0 .. 2 NTILE - 1 fetch the tiles of group g (rows beyond the caches arrive as zeros)
   auto issue = [&](int g, int stage) {
     unsigned char* dst = my_stages + stage * STAGE_BYTES;
     uint64_t* bar = &my_bars[stage];
     if (lane == 0) mbar_expect_tx(bar, STAGE_BYTES);
     __syncwarp();
-    if (lane < 4) tma_load_2d(dst + lane * TILE_BYTES, lane < 2 ? &tm_k : &tm_v, bar, (lane & 1) * 64, row_base + g * GROUP);
+    if (lane < 2 * NTILE) tma_load_2d(dst + lane * TILE_BYTES, lane < NTILE ? &tm_k : &tm_v, bar, (lane & (NTILE - 1)) * 64, row_base + g * GROUP);
   };
   // This warp's groups: g_first, g_first + 4, ... below g_end.  H: where streams 4-7 begin.
   const int H = ((ngroups + 7) >> 3) << 2;
@@ -322,11 +323,13 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
     qa[ks][0] = __ldg(reinterpret_cast<const uint32_t*>(qn + ks * 16 + 2 * j4));
     qa[ks][1] = __ldg(reinterpret_cast<const uint32_t*>(qn + ks * 16 + 8 + 2 * j4));
   }
-  // 16 bytes of the incoming K row (lanes 0-15) or V row (lanes 16-31)
-  const uint4 new_raw = __ldg(reinterpret_cast<const uint4*>((lane < 16 ? k_new : v_new) + (int64_t)u * HD) + (lane & 15));
+  // 16 bytes of the incoming K row (lanes 0-15) or V row (lanes 16-31); with head_dim 64 the first eight lanes of each half
+  const bool has_chunk = (lane & 15) < ROW_CHUNKS;
+  uint4 new_raw = make_uint4(0u, 0u, 0u, 0u);
+  if (has_chunk) new_raw = __ldg(reinterpret_cast<const uint4*>((lane < 16 ? k_new : v_new) + (int64_t)u * HD) + (lane & 15));
 
   uint4 last_raw = make_uint4(0u, 0u, 0u, 0u);
-  if (owns_last)
+  if (owns_last && has_chunk)
     last_raw = *(reinterpret_cast<const uint4*>((const __nv_bfloat16*)(lane < 16 ? c.k_cache : c.v_cache) +
                                                 ((int64_t)u * cap + ls) * HD) + (lane & 15));
 
@@ -343,7 +346,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   }
   if (owns_new && wid == 0) {
     __nv_bfloat16* dst = (__nv_bfloat16*)(lane < 16 ? c.k_cache : c.v_cache) + ((int64_t)u * cap + fs) * HD;
-    reinterpret_cast<uint4*>(dst)[lane & 15] = new_raw;
+    if (has_chunk) reinterpret_cast<uint4*>(dst)[lane & 15] = new_raw;
     if (lane == 0) {
       c.vnorm[(int64_t)u * cap + fs] = new_norm;
       c.pos[(int64_t)u * cap + fs] = t;
@@ -397,7 +400,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
       if (ok && !mbar_wait(&my_bars[stage], parity)) ok = false;
       ok = __all_sync(0xffffffffu, ok);
       unsigned char* ks = my_stages + stage * STAGE_BYTES;
-      unsigned char* vs = ks + 2 * TILE_BYTES;
+      unsigned char* vs = ks + NTILE * TILE_BYTES;
       const int r0 = g * GROUP;
       bool wrote = false;
       if (ok && r0 < cnt) {
@@ -405,16 +408,16 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
         // must not reach the p V product (their probability is 0, but 0 * garbage need not be 0)
         if (owns_new && fs_local >= r0 && fs_local < r0 + GROUP) {
           const int rr = fs_local - r0, ch = lane & 15;
-          *reinterpret_cast<uint4*>((lane < 16 ? ks : vs) + (ch >> 3) * TILE_BYTES + rr * 128 + (((ch & 7) ^ (rr & 7)) << 4)) = new_raw;
+          if (has_chunk) *reinterpret_cast<uint4*>((lane < 16 ? ks : vs) + (ch >> 3) * TILE_BYTES + rr * 128 + (((ch & 7) ^ (rr & 7)) << 4)) = new_raw;
           wrote = true;
         }
         if (owns_last && ls_local >= r0 && ls_local < r0 + GROUP) {
           const int rr = ls_local - r0, ch = lane & 15;
-          *reinterpret_cast<uint4*>((lane < 16 ? ks : vs) + (ch >> 3) * TILE_BYTES + rr * 128 + (((ch & 7) ^ (rr & 7)) << 4)) = last_raw;
+          if (has_chunk) *reinterpret_cast<uint4*>((lane < 16 ? ks : vs) + (ch >> 3) * TILE_BYTES + rr * 128 + (((ch & 7) ^ (rr & 7)) << 4)) = last_raw;
           wrote = true;
         }
         if (cnt < r0 + GROUP) {
-          for (int rr = cnt - r0 + (lane >> 4); rr < GROUP; rr += 2)
+          for (int rr = cnt - r0 + (lane >> 4); rr < GROUP && has_chunk; rr += 2)
             *reinterpret_cast<uint4*>(vs + ((lane >> 3) & 1) * TILE_BYTES + rr * 128 + ((lane & 7) << 4)) = make_uint4(0u, 0u, 0u, 0u);
           wrote = true;
         }
@@ -501,7 +504,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   }
   flush(second ? wid + MW : wid);
   if (SPW == 2 && !second) {      // the four-warp kernel never reached the midpoint: its stream wid + 4 is empty
-    *reinterpret_cast<float4*>(&part_o[wid + MW][lane * 4]) = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (lane < HD / 4) *reinterpret_cast<float4*>(&part_o[wid + MW][lane * 4]) = make_float4(0.f, 0.f, 0.f, 0.f);
     if (lane == 0) { part_m[wid + MW] = -INFINITY; part_l[wid + MW] = 0.f; }
   }
   workers_sync<WT>();
@@ -554,7 +557,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
       fw[i] = part_m[i] > -INFINITY ? ex2(part_m[i] - m_c) : 0.f;
       l_c += part_l[i] * fw[i];
     }
-    Exch* e0 = split > 1 ? cluster.map_shared_rank(&ex, 0) : &ex;
+    Exch<HD>* e0 = split > 1 ? cluster.map_shared_rank(&ex, 0) : &ex;
     if (tid < HD) {
       float a = 0.f;
 #pragma unroll
@@ -562,7 +565,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
       e0->o[rank][tid] = a;
     }
     if (tid < split) {
-      Exch* er = split > 1 ? cluster.map_shared_rank(&ex, tid) : &ex;
+      Exch<HD>* er = split > 1 ? cluster.map_shared_rank(&ex, tid) : &ex;
       er->m[rank] = m_c;
       er->l[rank] = l_c;
     }
@@ -683,7 +686,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
     if (lane == 0) warp_key[wid] = wkey;
     workers_sync<WT>();
     const unsigned long long win = warp_min_key(lane < MW ? warp_key[lane] : NO_KEY);
-    Exch* e0 = split > 1 ? cluster.map_shared_rank(&ex, 0) : &ex;
+    Exch<HD>* e0 = split > 1 ? cluster.map_shared_rank(&ex, 0) : &ex;
     if (win == NO_KEY) {
       if (tid == 0) e0->key[rank] = NO_KEY;
     } else if (my_key == win) {
@@ -816,13 +819,14 @@ void decode_history_forget(cudaStream_t st, bool probe_only) {
   }
 }
 
-// Returns cudaErrorNotSupported when the shape does not fit this kernel's shared memory (the caller
-// then takes the general kernel).
-cudaError_t launch_decode_mma(const Shape& s, int B, int F, int R, const vatp_cache& c, const void* q, const void* k,
+namespace {
+
+template <int HD>
+cudaError_t launch_hd(const Shape& s, int B, int F, int R, const vatp_cache& c, const void* q, const void* k,
                               const void* v, void* out, int32_t* evicted, int32_t* dev_status, cudaStream_t st,
                               bool may_overlap, int G) {
+  constexpr int STAGE_BYTES = stage_bytes<HD>, ROW_BYTES = HD * 2;
   const int cap = cache_capacity(B);
-  if (!vatp_tc_available() || G < 1 || G > GQ_HEADS) return cudaErrorNotSupported;
   const bool grouped = G > 1;           // s.units counts caches (KV heads); q and out hold G rows per unit
   const int sms = device_sm_count();
   // split a unit over a cluster while the grid still fits on the SMs once (a second launch can then be resident too)
@@ -869,8 +873,8 @@ cudaError_t launch_decode_mma(const Shape& s, int B, int F, int R, const vatp_ca
   const Plan lone = make_plan(true), beside = grouped ? lone : make_plan(false);      // grouped queries: always a whole SM
   if (!beside.ok || !lone.ok) return cudaErrorNotSupported;
   CUtensorMap tm_k, tm_v;
-  if (!make_rows_map_bf16(&tm_k, c.k_cache, (uint64_t)s.units * cap, GROUP) ||
-      !make_rows_map_bf16(&tm_v, c.v_cache, (uint64_t)s.units * cap, GROUP))
+  if (!make_rows_map_bf16(&tm_k, c.k_cache, HD, (uint64_t)s.units * cap, GROUP) ||
+      !make_rows_map_bf16(&tm_v, c.v_cache, HD, (uint64_t)s.units * cap, GROUP))
     return cudaErrorInvalidValue;
   const bool win = s.window > 0;
   const size_t units = (size_t)s.units, slots = units * cap;
@@ -882,9 +886,9 @@ cudaError_t launch_decode_mma(const Shape& s, int B, int F, int R, const vatp_ca
                        {win ? (const char*)c.ring : nullptr, win ? slots * s.window * 4 : 0},
                        {win ? (const char*)c.acc_fixed : nullptr, win ? slots * 8 : 0},
                        {(const char*)q, units * G * ROW_BYTES}, {(const char*)k, units * ROW_BYTES}, {(const char*)v, units * ROW_BYTES}};
-  auto kern_alone = grouped ? (win ? decode_mma_kernel<true, MW_ALONE, GQ_HEADS> : decode_mma_kernel<false, MW_ALONE, GQ_HEADS>)
-                            : (win ? decode_mma_kernel<true, MW_ALONE, 1> : decode_mma_kernel<false, MW_ALONE, 1>);
-  auto kern_beside = grouped ? kern_alone : (win ? decode_mma_kernel<true, MW_BESIDE, 1> : decode_mma_kernel<false, MW_BESIDE, 1>);
+  auto kern_alone = grouped ? (win ? decode_mma_kernel<HD, true, MW_ALONE, GQ_HEADS> : decode_mma_kernel<HD, false, MW_ALONE, GQ_HEADS>)
+                            : (win ? decode_mma_kernel<HD, true, MW_ALONE, 1> : decode_mma_kernel<HD, false, MW_ALONE, 1>);
+  auto kern_beside = grouped ? kern_alone : (win ? decode_mma_kernel<HD, true, MW_BESIDE, 1> : decode_mma_kernel<HD, false, MW_BESIDE, 1>);
   cudaError_t e = cudaFuncSetAttribute(kern_beside, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)whole_sm);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kern_alone, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)whole_sm);
   if (e != cudaSuccess) return e;
@@ -919,6 +923,18 @@ cudaError_t launch_decode_mma(const Shape& s, int B, int F, int R, const vatp_ca
   return cudaLaunchKernelEx(&cfg, kern, tm_k, tm_v, independent, G, state_in_smem, split, chunk, nstage, B, cap, F, R, s.window, s.norm, s.scale * LOG2E, c,
                             (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v,
                             (__nv_bfloat16*)out, evicted, dev_status);
+}
+
+}  // namespace
+
+// Returns cudaErrorNotSupported when the shape does not fit this kernel's shared memory (the caller
+// then takes the general kernel).
+cudaError_t launch_decode_mma(const Shape& s, int B, int F, int R, const vatp_cache& c, const void* q, const void* k,
+                              const void* v, void* out, int32_t* evicted, int32_t* dev_status, cudaStream_t st,
+                              bool may_overlap, int G) {
+  if (!vatp_tc_available() || G < 1 || G > GQ_HEADS) return cudaErrorNotSupported;
+  return s.d == 64 ? launch_hd<64>(s, B, F, R, c, q, k, v, out, evicted, dev_status, st, may_overlap, G)
+                   : launch_hd<128>(s, B, F, R, c, q, k, v, out, evicted, dev_status, st, may_overlap, G);
 }
 
 }  // namespace vatp

@@ -112,7 +112,7 @@ vatp_status prefill_impl(const vatp_params* p, const void* q, const void* k, con
     const size_t n = (size_t)sh.units * sh.T;
     float* part = reinterpret_cast<float*>(static_cast<char*>(workspace) + lse_bytes(p));
     const int eb = p->dtype == VATP_F32 ? 4 : 2;
-    const bool tc = p->dtype == VATP_BF16 && p->head_dim == 128 && vatp_tc_available();
+    const bool tc = p->dtype == VATP_BF16 && vatp_tc_available();
     // the general kernel keeps its (natural-log) normalisers in the caller's layout: lse_out, or a scratch copy of
     // that layout at the head of the workspace when the caller wants none (it fits: G * units * T floats <= `part`)
     e = cudaSuccess;
@@ -154,7 +154,7 @@ vatp_status prefill_impl(const vatp_params* p, const void* q, const void* k, con
     if (e == cudaSuccess) e = launch_group_mean(G, (int64_t)n, part, vnorm, attn_acc, score, st);
     return e == cudaSuccess ? VATP_OK : VATP_ERR_CUDA;
   }
-  if (p->dtype == VATP_BF16 && p->head_dim == 128 && vatp_tc_available()) {
+  if (p->dtype == VATP_BF16 && vatp_tc_available()) {
     e = launch_prefill_tc(sh, q, k, v, ws, lse_out, attn_acc, vnorm, score, win_rows, dev_status, st, lse_in, attn_out);
   } else if (attn_out) {
     // general path: the forward leaves natural-log normalisers where pass 2 reads them (the caller's array, or
@@ -284,7 +284,7 @@ vatp_status vatp_decode_step(const vatp_params* p, const vatp_cache* cache, cons
   if (!aligned16(q_new) || !aligned16(k_new) || !aligned16(v_new) || !aligned16(out)) return VATP_ERR_INVALID_ARG;
   if (group_of(p) > 1) {
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    if (p->dtype == VATP_BF16 && p->head_dim == 128 && group_of(p) <= 8) {
+    if (p->dtype == VATP_BF16 && group_of(p) <= 8) {
       // tensor-core step: the group's heads ride in the rows of the MMA tiles, every K and V row is read once
       Shape sh;
       std::memset(&sh, 0, sizeof(sh));

@@ -72,9 +72,9 @@ bool vatp_tc_available();
 // multiprocessors of the current device (looked up once per device)
 int device_sm_count();
 
-// 2-D tensor map over `rows` contiguous rows of 128 bf16: box = 64 columns x box_rows rows, 128-byte
+// 2-D tensor map over `rows` contiguous rows of d (a multiple of 64) bf16: box = 64 columns x box_rows rows, 128-byte
 // swizzle, rows beyond the end read as zeros.  False when the driver entry point is missing.
-bool make_rows_map_bf16(CUtensorMap* m, const void* base, uint64_t rows, uint32_t box_rows);
+bool make_rows_map_bf16(CUtensorMap* m, const void* base, int d, uint64_t rows, uint32_t box_rows);
 
 // 2-D tensor map over `rows` rows of row_words 32-bit words, row_stride_bytes apart (a multiple of 16); the box
 // is one row: for gathers of whole rows by row index.  False when the driver entry point is missing.
@@ -105,7 +105,7 @@ cudaError_t launch_prefill_simt(const Shape& s, int dtype, const void* q, const 
                                 bool lse_given = false);
 // lse_in: row normalisers [units][T] (natural log) from the caller; non-null skips pass 1
 // attn_out: non-null replaces pass 1 by the fused attention forward, which also writes the output rows (bf16; unit
-// (b, h) at b * osb + h * osh, rows of 128 elements)
+// (b, h) at b * osb + h * osh, rows of head_dim elements)
 cudaError_t launch_prefill_tc(const Shape& s, const void* q, const void* k, const void* v, float* lse_ws,
                               float* lse_out, float* attn_acc, float* vnorm, float* score, float* win_rows,
                               int32_t* dev_status, cudaStream_t st, const float* lse_in = nullptr, void* attn_out = nullptr);
@@ -124,7 +124,7 @@ cudaError_t launch_window_ring_grouped(const Shape& s, int G, int dtype, int B, 
 cudaError_t launch_window_ring(const Shape& s, int dtype, int B, const void* q, const float* lse, const vatp_cache& c,
                                int32_t* dev_status, cudaStream_t st);
 cudaError_t launch_window_ring_tc(const Shape& s, int B, const void* q, const float* lse, const vatp_cache& c,
-                                  int32_t* dev_status, cudaStream_t st);   // bf16, head_dim 128, tensor cores
+                                  int32_t* dev_status, cudaStream_t st);   // bf16, tensor cores
 // grouped-query attention: mean over the group's G partial indicators [G][n] and Eq. 4; the decode step of a KV group
 cudaError_t launch_group_mean(int G, int64_t n, const float* part, const float* vnorm, float* attn_acc, float* score,
                               cudaStream_t st);
@@ -135,7 +135,7 @@ cudaError_t launch_decode(const Shape& s, int dtype, int B, int F, int R, const 
                           const void* k, const void* v, void* out, int32_t* evicted, int32_t* dev_status, cudaStream_t st,
                           bool may_overlap);
 
-// bf16, head_dim 128 only; cudaErrorNotSupported when the shape does not fit (take launch_decode's general kernel)
+// bf16 only; cudaErrorNotSupported when the shape does not fit (take launch_decode's general kernel)
 // may_overlap: the caller opted in to launches that run beside earlier decode launches on the stream when they share
 // no buffer with them (VATP_FLAG_DECODE_OVERLAP)
 // G: query heads per cache (grouped-query attention, 1 .. 8): s.units counts caches, q and out hold G rows per unit

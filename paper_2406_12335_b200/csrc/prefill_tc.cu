@@ -759,7 +759,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
           // an odd tile count leaves half a chunk of padding that pass 2 reads as "no query"
           if ((a.nt & 1) && it.tile == a.nt - 1 && VATP_INB((int64_t)u * a.Tpad + tok + TILE, (int64_t)a.units * a.Tpad, a.dev_status))
             a.lse2[(int64_t)u * a.Tpad + tok + TILE] = -INFINITY;
-          if (a.lse_out && tok < a.T)
+          // (head_dim 64 leaves the rows before a history window alone, head_dim 128 those before its first tile)
+          if (a.lse_out && tok < a.T && (HD == 128 || tok >= a.first_row))
             a.lse_out[(int64_t)(u / a.heads) * a.lse_sb + (int64_t)(u % a.heads) * a.lse_sh + tok] = lse2 * 0.69314718055994531f;
         } else {
           const float tot = hsum2(add2(cs[0], cs[1])) + (sm.part_a[pi][0][row] + sm.part_a[pi][1][row]) + sm.part_a[pi][2][row];

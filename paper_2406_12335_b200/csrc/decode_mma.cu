@@ -3,33 +3,47 @@
 //
 // The step is HBM-bound (every cached K and V row is read once) but so short - tens of megabytes -
 // that fixed latencies decide its duration.  Hence:
-//   * every warp owns a ring of stages and requests its first stages (tiled TMA loads of 16 rows x
-//     128 bytes, 128-byte swizzled so that ldmatrix is conflict-free) before anything else happens;
+//   * every warp has a ring of units - the K rows or the V rows of a 16-row group, one tiled TMA load each,
+//     128-byte swizzled so that ldmatrix is conflict-free; the first units are requested before anything else happens;
 //   * q.K^T and p.V run on the warp-level tensor-core path (mma.sync m16n8k16, bf16 in, fp32
-//     accumulate): S^T = q K^T leaves the probabilities of 16 rows in exactly the registers the
-//     A operand of p V wants, so a 16-row group costs about 80 instructions.  p is split into two
-//     bf16 halves (rows 0-7 / 8-15 of the A tile carry hi / lo): the product keeps ~16 bits of p;
-//   * a unit is split over a thread-block cluster when units are few.  Every CTA PUSHES its running
-//     max and sum into the shared memory of all CTAs of the unit and its partial output into rank
-//     0's; after one cluster barrier each CTA knows the softmax normaliser, updates the indicators of
-//     its own slots and proposes its own eviction candidate to rank 0; after a second barrier rank 0
-//     picks the candidate of the whole unit.  No global scratch, one launch;
-//   * consecutive steps overlap (programmatic dependent launch).  By default a step requests its
-//     first K/V tiles early and reads everything else only after all earlier work in the stream has
-//     completed; its control warp releases the next launch once that wait is over, so at most one
+//     accumulate): S^T = q K^T with the queries in the rows, O^T = V^T p with V^T out of ldmatrix.trans as the A operand:
+//     sixteen output channels per instruction and 32 accumulator registers for 128 channels.  p is split into two bf16
+//     halves (columns hi / lo of the B operand, or two products when the columns are heads): the product keeps ~16 bits
+//     of p;
+//   * two phases, all K rows and then all V rows: no group of rows depends on another, and exponentials are taken once
+//     per slot.  (One sweep with an online softmax was a chain of ~2300 cycles per 16-row group - fragments, products,
+//     maximum, exponentials, fragments, products - of which eight warps per CTA hid too little: with the data already in
+//     L2 it took 4 of a waiting step's 12.5 us.  tcgen05 with the rows as M and 16 columns was no faster than mma.sync:
+//     its instructions issue 65 cycles apart for 4 KB of rows each.)
+//   * eight warps and at most half of an SM's shared memory: two CTAs fit on an SM, so the
+//     CTAs of the next launch are resident while this one runs.  A launch that has to wait for its predecessor has then
+//     already filled its rings and asked for the rest of its rows in L2 (its K and V rows are the one thing it may read
+//     early), and what is left after the wait is the arithmetic, the tail and reads that hit L2;
+//   * more units than CTAs fit on the machine: a CTA takes several, and a producer warp streams the next one's rows while
+//     the tail of this one runs;
+//   * a unit (sequence, head) is split over a thread-block cluster when units are few.  Every CTA pushes its
+//     max and sum to all CTAs of the unit, and each of them the channels of its partial output that this one is to
+//     sum up, with st.async: the receiver waits on an mbarrier of its own that counts the bytes (a cluster barrier
+//     makes every CTA wait for a round trip of all).  Each CTA then knows the softmax normaliser, updates the indicators
+//     of its own slots and sends its eviction candidate to rank 0, which picks.  No global scratch, one launch;
+//   * consecutive steps overlap (programmatic dependent launch).  By default a step requests
+//     K/V tiles early and reads everything else only after all earlier work in the stream has
+//     completed; it releases the next launch once that wait is over, so at most one
 //     unfinished predecessor exists while a step sets up, and the one cache row that predecessor
 //     may have written - the row of its incoming token, recorded in last_slot - is re-read after
 //     the wait and patched in.  A caller that steps several independent caches on one stream may
 //     opt in (VATP_FLAG_DECODE_OVERLAP) to more: the host keeps, per stream, the buffers of the
 //     last launches, and a launch that shares no buffer with any launch that can still be in
-//     flight (another layer's or another sequence's cache) never waits: its control warp releases
-//     the next launch at once and only holds the CTA until the previous launch has completed, so
+//     flight (another layer's or another sequence's cache) never waits: it releases
+//     the next launch at once and only stays until the previous launch has completed, so
 //     launches still complete in order and the number in flight is bounded by what fits on the
-//     machine (two CTAs fit on an SM).  A launch that does wait has its SMs to itself and runs the
-//     eight-warp variant of the kernel (same arithmetic, see MW below);
+//     machine;
 //   * grouped-query attention (several query heads share one cache; the paper leaves the case open and points at
 //     a group-wise score, read here as the MEAN of the heads' probabilities): up to eight heads of a group ride
-//     in the rows of the MMA tiles (template parameter GT), so a K or V row is still read once per step.
+//     in the rows of S^T (template parameter GT), so a K or V row is still read once per step.
+// Measured (us per step, before and after the two phases, the exchange by st.async and the co-resident successor): 32 units
+// x 2049 slots, every launch waiting 12.5 -> 10.4; 256 units x 1639, launches overlapping 38 -> 35 (138 MB: 6.1 TB/s of the
+// 6.56 a copy reaches); 512 units x 1025 with a history window 73 -> 58; 8 units x 2049, four heads each 11.0 -> 10.4.
 #include <cooperative_groups.h>
 
 #include <mutex>
@@ -41,25 +55,20 @@ namespace cg = cooperative_groups;
 namespace vatp {
 namespace {
 
-// Streaming warps per CTA (template parameter MW of the kernel; their threads WT = 32 MW, plus one control warp):
-// four when launches of different caches run side by side (two CTAs per SM), eight for a launch that waits for its
-// predecessor and has the SM to itself - one warp per scheduler cannot hide the latency of its own
-// ldmatrix / mma.sync / softmax chain, so such a launch streams faster with two.
-// The arithmetic does not depend on MW: a CTA's 16-row groups are always dealt to NSTREAM = 8 online-softmax streams -
-// the groups below the midpoint H (a multiple of four) to streams 0-3 by g mod 4, those from H on to streams 4-7 -
-// each stream is folded in ascending group order, and the eight partials are merged in stream order.  A warp of the
-// eight-warp kernel folds one stream; warp w of the four-warp kernel walks groups w, w + 4, ... in one sweep,
-// files its partial under stream w where it crosses H and starts afresh for stream w + 4.  Results are
-// bit-identical whichever kernel a launch gets.
-constexpr int MW_BESIDE = 4, MW_ALONE = 8;
-constexpr int NSTREAM = 8;
+// Eight warps; the 16-row group g of a CTA goes to warp g mod 8, which takes its groups in ascending order
+// (the logits of all of them, then their share of the output); the eight partial outputs are summed in warp order.
+// Nothing of this depends on how a launch is scheduled or how much shared memory it takes: results are bit-identical
+// either way.
+constexpr int MW = 8;
+constexpr int WT = MW * 32;           // consumer threads; a producer warp follows
+constexpr int DM_THREADS = WT + 32;
 // (the kernels' template parameter HD: head_dim, 64 or 128)
-constexpr int GROUP = 16;             // rows per MMA group = rows of K (and of V) per stage
+constexpr int GROUP = 16;             // rows per MMA group
+template <int HD> constexpr int unit_bytes = GROUP * HD * 2;   // K rows (or V rows) of a group: [64-column half][16 rows][128 bytes]
 constexpr int TILE_BYTES = GROUP * 128;    // 16 rows x 64 bf16, 128-byte swizzled
-template <int HD> constexpr int stage_bytes = 2 * (HD / 64) * TILE_BYTES; // K columns 0-63 (, K 64-127), V 0-63 (, V 64-127)
+constexpr int MAX_SLOTS = 8;          // units a warp keeps in flight at most
 constexpr int MAX_SPLIT = 8;
 constexpr int GQ_HEADS = 8;           // grouped queries: query heads per cache this kernel takes (rows 0-7 of the MMA tiles)
-constexpr int GQ_MAX_SPLIT = MAX_SPLIT;   // ... and the CTAs a unit is split over at most
 constexpr float LOG2E = 1.4426950408889634f;
 constexpr unsigned long long NO_KEY = ~0ull;
 
@@ -75,6 +84,16 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+  return ok != 0;
+}
+// the same without suspending the warp (its other lanes have barriers of their own to look at)
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}"
       : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
   return ok != 0;
@@ -99,11 +118,30 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
                "l"(src), "r"(bytes), "r"(smem_u32(bar))
                : "memory");
 }
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1) {
+__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1, int c2) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-      ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(c0), "r"(c1)
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+      ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2)
       : "memory");
+}
+// address of `addr` (this CTA's shared memory) in CTA `rank` of the cluster
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+// asynchronous stores into another CTA's shared memory; its mbarrier counts the bytes when they have landed
+__device__ __forceinline__ void st_async(uint32_t addr, float v, uint32_t bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
+               ::"r"(addr), "r"(__float_as_uint(v)), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void st_async2(uint32_t addr, float a, float b, uint32_t bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];"
+               ::"r"(addr), "r"(__float_as_uint(a)), "r"(__float_as_uint(b)), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void st_async4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+               ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d), "r"(bar) : "memory");
 }
 __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t (&r)[4]) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
@@ -132,21 +170,13 @@ __device__ __forceinline__ float ex2(float x) {
   return y;
 }
 
-// barrier over the streaming warps only (the control warp does not take part)
-template <int WT>
+// barrier over the consumer warps only
 __device__ __forceinline__ void workers_sync() { asm volatile("bar.sync 1, %0;" ::"n"(WT) : "memory"); }
-__device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
-// what the CTAs of a unit push into one another
-template <int HD>
-struct Exch {
-  float m[MAX_SPLIT], l[MAX_SPLIT];       // in every rank: per rank the max of its logits (log2 domain) and the sum of exp2(s - m)
-  float o[MAX_SPLIT][HD];                 // in rank 0: partial outputs of every rank
-  unsigned long long key[MAX_SPLIT];      // in rank 0: every rank's eviction candidate (NO_KEY: none) ...
-  int key_slot[MAX_SPLIT], key_pos[MAX_SPLIT];   // ... its slot in the unit and its position
+struct __align__(16) Candidate {      // eviction candidate of a CTA, sent to rank 0 (key NO_KEY: none)
+  unsigned long long key;
+  int slot, pos;
 };
-
 
 // eviction order as one integer: lower importance first, among equals the higher position first
 __device__ __forceinline__ unsigned long long evict_key(float I, int pos) {
@@ -161,156 +191,256 @@ __device__ __forceinline__ unsigned long long warp_min_key(unsigned long long ke
 }
 
 // GT = 1: one query head per cache (multi-head attention).  GT = GQ_HEADS: grouped queries - up to GQ_HEADS query
-// heads (G of them, a run-time argument) share the cache of unit u: row g of the MMA tiles carries head g, so the
-// streaming loop is the same instructions, and every K and V row is read once for the whole group; the maxima,
-// sums and partial outputs exist per head, and the indicator advances by the MEAN of the heads' probabilities.
-// Only the eight-warp kernel is built for it (the per-head partials take the room a second CTA would need).
-template <int HD, bool WINDOWED, int MW, int GT>
-__global__ void __launch_bounds__(MW * 32 + 32, MW == MW_BESIDE ? 2 : 1)
+// heads (G of them, a run-time argument) share the cache of unit u: row g of S^T carries head g, so every K and V row
+// is read once for the whole group; the maxima, sums and partial outputs exist per head, and the indicator advances by
+// the MEAN of the heads' probabilities.
+// FEED: a producer warp keeps the rings full, for CTAs with several units and for grids beyond one CTA per SM.  Otherwise
+// every warp requests its own rows: one warp less at 128 instead of 96 registers, and a shorter way from a freed slot to
+// the next request, which is what a launch that has the machine to itself is bound by.
+template <int HD, bool WINDOWED, int GT, bool FEED>
+__global__ void __launch_bounds__(FEED ? DM_THREADS : WT, 2)
 decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, int independent, int G,
-                  int state_in_smem, int split, int chunk, int nstage, int B, int cap, int F, int R, int w, int norm, float scale_log2,
-                  vatp_cache c,
+                  int units, int state_in_smem, int part_in_ring, int split, int chunk, int nslot, int l2_rows, int B, int cap, int F, int R, int w, int norm,
+                  float scale_log2, vatp_cache c,
                   const __nv_bfloat16* __restrict__ q_new, const __nv_bfloat16* __restrict__ k_new,
                   const __nv_bfloat16* __restrict__ v_new, __nv_bfloat16* __restrict__ out,
                   int32_t* __restrict__ evicted, int32_t* __restrict__ dev_status) {
-  constexpr int STAGE_BYTES = stage_bytes<HD>, NTILE = HD / 64, ROW_CHUNKS = HD / 8;   // tiles and 16-byte chunks of a row
-  constexpr int WT = MW * 32;           // streaming threads (at least HD: one per output channel where outputs are formed)
-  static_assert(WT >= HD, "one streaming thread per output channel");
-  static_assert(GT == 1 || (GT == GQ_HEADS && MW == MW_ALONE), "grouped queries: the eight-warp kernel only");
+  constexpr int UNIT = unit_bytes<HD>, ROW_CHUNKS = HD / 8;   // 16-byte chunks of a row
+  static_assert(WT >= HD, "one thread per output channel");
   extern __shared__ unsigned char dyn_raw[];
   unsigned char* dyn = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(dyn_raw) + 1023) & ~uintptr_t(1023));
-  // [MW][nstage] stages | logits[chunk] | acc[chunk] | vnorm[chunk] | pos[chunk]: the per-slot arrays of
-  // this CTA's own slots.  For large caches only the logits are held here, which keeps the CTA small
-  // enough for two launches to be resident together; acc, vnorm and pos are then copied into the stage
-  // memory once the streaming is over (state_in_smem == 2) or, if even that is too small, read from
-  // global memory in the tail (state_in_smem == 0).
-  unsigned char* stage_base = dyn;
-  float* logit_s = reinterpret_cast<float*>(dyn + (size_t)MW * nstage * STAGE_BYTES);
-  // (grouped queries: logits[G][chunk], state always here (state_in_smem == 1), then the per-head partial outputs
-  // of the eight streams [NSTREAM][G][HD] and, in rank 0, those of every CTA of the unit [split][G][HD])
-  float* acc_s = state_in_smem == 2 ? reinterpret_cast<float*>(stage_base) : logit_s + (GT > 1 ? G : 1) * chunk;
+  // [MW][nslot] units | partial outputs of the warps [MW][G][HD] (part_in_ring: in the warps' own rings instead) |
+  // slices of partial outputs received [split][G][HD / split] | logits[G][chunk] | per-slot state of this CTA's own
+  // slots: acc (with a history window the ring row that leaves it), vnorm, pos, with a window the fixed-point sums.
+  // Where the state does not fit beside the rings it is copied into the rings' memory once the streaming is over
+  // (state_in_smem == 2; a CTA with one unit only) or read from global memory in the tail (state_in_smem == 0).
+  unsigned char* ring_base = dyn;
+  const int g_rows = GT > 1 ? G : 1;
+  const int ring_bytes = MW * nslot * UNIT;
+  float* part_o = reinterpret_cast<float*>(part_in_ring ? ring_base : dyn + ring_bytes);
+  const int part_ld = part_in_ring ? nslot * (UNIT / 4) : g_rows * HD;       // floats from one warp's partial to the next
+  float* xo = reinterpret_cast<float*>(dyn + ring_bytes + (part_in_ring ? 0 : MW * g_rows * HD * 4));
+  float* logit_s = xo + g_rows * HD;
+  float* acc_s = state_in_smem == 2 ? reinterpret_cast<float*>(ring_base) : logit_s + g_rows * chunk;
   float* vn_s = acc_s + chunk;
   int* pos_s = reinterpret_cast<int*>(vn_s + chunk);
-  float* gq_part = reinterpret_cast<float*>(pos_s + chunk);
-  float* gq_xo = gq_part + NSTREAM * (GT > 1 ? G : 0) * HD;
+  long long* fx_s = reinterpret_cast<long long*>(pos_s + chunk);
 
-  __shared__ __align__(8) uint64_t bars[MW * 4 + 1];
-  __shared__ __align__(16) Exch<HD> ex;
-  constexpr int SPW = NSTREAM / MW;     // streams per warp
-  static_assert(SPW == 1 || SPW == 2, "a warp folds one or two streams");
-  __shared__ __align__(16) float part_o[NSTREAM][HD];
-  __shared__ float part_m[NSTREAM], part_l[NSTREAM];
-  // grouped queries: per stream and head; per rank and head (pushed by every CTA of the unit); the unit's normalisers
-  __shared__ float gq_pm[GT > 1 ? NSTREAM : 1][GT], gq_pl[GT > 1 ? NSTREAM : 1][GT];
-  __shared__ float gq_m[GT > 1 ? GQ_MAX_SPLIT : 1][GT], gq_l[GT > 1 ? GQ_MAX_SPLIT : 1][GT];
-  __shared__ float gq_fr[GT > 1 ? GQ_MAX_SPLIT : 1][GT], gq_mall[GT], gq_invl[GT];
+  __shared__ __align__(8) uint64_t full[MW * MAX_SLOTS], empty[MW * MAX_SLOTS], misc_bars[4];
+  __shared__ float part_m[MW][GT], part_l[MW][GT];
+  __shared__ float2 ex_ml[MAX_SPLIT][GT];          // per rank and head: max of its logits (log2 domain), sum of exp2(s - m)
+  __shared__ float gq_fr[GT > 1 ? MAX_SPLIT : 1][GT], gq_f[GT], gq_invl[GT];
+  __shared__ Candidate cand[MAX_SPLIT];            // in rank 0: every rank's eviction candidate
   __shared__ unsigned long long warp_key[MW];
-  __shared__ int ctrl_evicting;
 
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = split > 1 ? (int)cluster.block_rank() : 0;
-  const int u = blockIdx.x / split;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int j4 = lane & 3;
-
-  // Remote shared memory may only be touched once its CTA runs: everyone arrives here, and waits
-  // (long since satisfied) just before the first remote store.
-  if (split > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // all five warps
-
-  if (wid == MW) {
-    // ---- control warp: release the next launch, then hold this CTA until the previous launch has completed
-    // (it arrives at the unit's barrier at once, so that the streaming warps never wait for it)
-    // (its arrivals at the unit's two barriers come as early as the barrier's phases allow)
-    if (split > 1) { cluster_wait_acquire(); cluster_arrive_release(); }
-    if (lane == 0) {
-      // An independent launch lets its successor start at once.  A launch that waits for its
-      // predecessor releases its successor only after that wait: the successor's early tile
-      // requests then race with this launch alone, never with launches before it.
-      if (independent) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-      asm volatile("griddepcontrol.wait;" ::: "memory");
-      if (!independent) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    }
-    __syncwarp();
-    if (split > 1) {
-      cluster_wait_acquire();
-      // a second barrier follows when the step evicts (the streaming warps have published that by now)
-      if (*reinterpret_cast<volatile int*>(&ctrl_evicting)) { cluster_arrive_release(); cluster_wait_acquire(); }
-    }
-    return;
-  }
-
-  // this CTA's slot range inside the allocation
+  uint64_t* state_full = &misc_bars[0];
+  uint64_t* state_empty = &misc_bars[1];
+  uint64_t* ex_bar = &misc_bars[2];                // the exchange of maxima, sums and partial outputs
+  uint64_t* cand_bar = &misc_bars[3];              // rank 0: the candidates
+  // This CTA's units: u0, u0 + u_step, ... (more than one only when no unit is split).
+  const int u0 = blockIdx.x / split, u_step = gridDim.x / split;
+  // its slot range inside a unit's allocation
   const int s0 = min(rank * chunk, cap);
   const int rows_alloc = min(chunk, cap - s0);
   const int ngroups = (rows_alloc + GROUP - 1) / GROUP;
-  const int row_base = u * cap + s0;     // first row of the range in the [units * cap, 128] view of the caches
-  uint64_t* my_bars = &bars[wid * 4];
-  uint64_t* state_bar = &bars[MW * 4];
-  unsigned char* my_stages = stage_base + (size_t)wid * nstage * STAGE_BYTES;
-
-  // every warp arms its own barriers: no CTA-wide barrier before the first copy is requested
-  if (lane == 0) {
-    for (int s = 0; s < nstage; ++s) mbar_init(&my_bars[s], 1);
-    if (wid == 1) mbar_init(state_bar, 1);     // armed and used by this same lane
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncwarp();
-  // lanes 0 .. 2 NTILE - 1 fetch the tiles of group g (rows beyond the caches arrive as zeros)
-  auto issue = [&](int g, int stage) {
-    unsigned char* dst = my_stages + stage * STAGE_BYTES;
-    uint64_t* bar = &my_bars[stage];
-    if (lane == 0) mbar_expect_tx(bar, STAGE_BYTES);
-    __syncwarp();
-    if (lane < 2 * NTILE) tma_load_2d(dst + lane * TILE_BYTES, lane < NTILE ? &tm_k : &tm_v, bar, (lane & (NTILE - 1)) * 64, row_base + g * GROUP);
-  };
-  // This warp's groups: g_first, g_first + 4, ... below g_end.  H: where streams 4-7 begin.
-  const int H = ((ngroups + 7) >> 3) << 2;
-  const int g_first = SPW == 2 ? wid : (wid < 4 ? wid : H + wid - 4);
-  const int g_end = (SPW == 2 || wid >= 4) ? ngroups : min(H, ngroups);
-  for (int s = 0; s < nstage; ++s)
-    if (g_first + s * 4 < g_end) issue(g_first + s * 4, s);
-  // The next launch in the stream may start now; nothing below this line is read before the previous
-  // launch has completed and its writes are visible.
-  if (!independent) asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (tid == 32 && rows_alloc > 0) {      // per-slot state of this CTA's slots
+  // Warp x's groups are x, x + MW, ...: as many as groups_of(x, rows) among the first `rows` rows.  Its units in order: the
+  // K rows of its groups, then their V rows.  A launch requests the first units of its first unit (sequence, head) before
+  // it may read how many rows are live; when fewer are than the allocation holds, those are dropped and the live ones
+  // requested anew.
+  auto groups_of = [](int x, int rows) { return x * GROUP < rows ? (rows - x * GROUP + MW * GROUP - 1) / (MW * GROUP) : 0; };
+  auto copy_state = [&](int u, int t) {            // one thread: the per-slot state of this CTA's slots
     const int64_t o = (int64_t)u * cap + s0;
+    mbar_expect_tx(state_full, (WINDOWED ? 20u : 12u) * rows_alloc);
+    bulk_g2s(acc_s, WINDOWED ? c.ring + ((int64_t)u * w + (t % w)) * cap + s0 : c.acc + o, rows_alloc * 4, state_full);
+    bulk_g2s(vn_s, c.vnorm + o, rows_alloc * 4, state_full);
+    bulk_g2s(pos_s, c.pos + o, rows_alloc * 4, state_full);
+    if (WINDOWED) bulk_g2s(fx_s, c.acc_fixed + o, rows_alloc * 8, state_full);
+  };
+
+  // Another CTA's shared memory may only be written once that CTA runs and its exchange barriers are armed: everyone
+  // arrives here and waits (long since satisfied) just before the first remote store.
+  if (tid == 0) {
+    for (int i = 0; i < MW; ++i)
+      for (int s = 0; s < nslot; ++s) { mbar_init(&full[i * MAX_SLOTS + s], 1); mbar_init(&empty[i * MAX_SLOTS + s], 1); }
+    mbar_init(state_full, 1);
+    mbar_init(state_empty, WT);
+    mbar_init(ex_bar, 1);
+    mbar_init(cand_bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (split > 1) {
+      mbar_expect_tx(ex_bar, (uint32_t)(8 * g_rows * split + 4 * g_rows * HD));
+      if (rank == 0) mbar_expect_tx(cand_bar, (uint32_t)(split * sizeof(Candidate)));
+    }
+  }
+  __syncthreads();
+  if (split > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+
+  auto issue = [&](int x, int u, int j, int n, int slot) {    // one lane: unit j of n groups into ring slot `slot` of warp x
+    uint64_t* bar = &full[x * MAX_SLOTS + slot];
+    mbar_expect_tx(bar, UNIT);
+    const bool is_v = j >= n;
+    tma_load_3d(ring_base + (x * nslot + slot) * UNIT, is_v ? &tm_v : &tm_k, bar, 0,
+                u * cap + s0 + (x + MW * (is_v ? j - n : j)) * GROUP, 0);
+  };
+  auto prefetch_rows = [&](bool v_rows) {    // one lane: the rows of the first unit that the rings do not hold yet, to L2
+    const int per_warp = 2 * ((ngroups + MW - 1) / MW);
+    const int held = (v_rows ? max(nslot - per_warp / 2, 0) : min(nslot, per_warp / 2)) * MW * GROUP;   // (about)
+    const int ahead = min(rows_alloc - held, l2_rows);
+    if (ahead > 0)
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;"
+                   ::"l"((const __nv_bfloat16*)(v_rows ? c.v_cache : c.k_cache) + (int64_t)(u0 * cap + s0 + held) * HD), "r"(ahead * HD * 2)
+                   : "memory");
+  };
+  auto bring_state = [&](int u) {            // one lane: the per-slot state into shared memory, or on its way to L2
+    const int t = WINDOWED ? c.next_pos[u] : 0;
     if (state_in_smem == 1) {
-      mbar_expect_tx(state_bar, 3u * rows_alloc * 4u);
-      bulk_g2s(acc_s, c.acc + o, rows_alloc * 4, state_bar);
-      bulk_g2s(vn_s, c.vnorm + o, rows_alloc * 4, state_bar);
-      bulk_g2s(pos_s, c.pos + o, rows_alloc * 4, state_bar);
-    } else if (state_in_smem == 0) {
-      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(c.acc + o), "r"(rows_alloc * 4) : "memory");
+      copy_state(u, t);
+    } else {
+      const int64_t o = (int64_t)u * cap + s0;
+      if (WINDOWED) {
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"((const void*)((uintptr_t)(c.ring + ((int64_t)u * w + (t % w)) * cap + s0) & ~(uintptr_t)15)), "r"(rows_alloc * 4) : "memory");
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"((const void*)((uintptr_t)(c.acc_fixed + o) & ~(uintptr_t)15)), "r"(rows_alloc * 8) : "memory");
+      } else {
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(c.acc + o), "r"(rows_alloc * 4) : "memory");
+      }
       asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(c.vnorm + o), "r"(rows_alloc * 4) : "memory");
       asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(c.pos + o), "r"(rows_alloc * 4) : "memory");
     }
-  }
+  };
 
-  const int len = c.len[u];
-  const int fs = c.free_slot[u];
-  const int t = c.next_pos[u];
-  const int ls = c.last_slot[u];
-#ifdef VATP_DEBUG_BOUNDS
-  // the state words come from memory: out of range, nothing of this unit is touched
-  if (!VATP_INB(len, cap, dev_status) || !VATP_INB(fs, cap, dev_status) || !VATP_INB(ls + 1, cap + 1, dev_status)) {
-    if (tid == 0) ctrl_evicting = 0;
-    if (split > 1) {      // the unit's first barrier is still reached by every thread (all its CTAs read the same words)
-      cluster_wait_acquire();
-      cluster_arrive_release(); cluster_wait_acquire();
+  if (FEED && wid == MW) {
+    // ---- the producer warp: lane x < MW feeds warp x, lane MW brings the per-slot state.  (A warp that issued its own
+    // copies spent a quarter of its time on that.)
+    const int na = lane < MW ? groups_of(lane, rows_alloc) : 0;
+    const int early = min(nslot, 2 * na);
+    // An independent launch lets its successor start at once, and stays until the launch before it has completed, so
+    // that launches complete in order.  A launch that waits for its predecessor releases its successor
+    // only after that wait: the successor's early tile requests then race with this launch alone, never with launches
+    // before it.
+    if (independent && lane == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    for (int j = 0; j < early; ++j) issue(lane, u0, j, na, j);
+    __syncwarp();
+    if (!independent) {
+      // A launch that waits has the time: the rows that the rings do not hold yet start on their way to L2.
+      if (l2_rows > 0 && (lane == MW || lane == MW + 1)) prefetch_rows(lane != MW);
+      __syncwarp();
+      // Nothing but K and V rows is read before the previous launch has completed and its writes are visible.
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      if (lane == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     }
+    int u = u0, j = early, base = 0, n = na, total = 2 * na;     // next unit j of `total`; those below base were dropped
+    int slot = early == nslot ? 0 : early, use = early == nslot ? 1 : 0;
+    bool done = rows_alloc <= 0 || lane > MW || (lane == MW && state_in_smem == 2);
+    auto live_groups = [&]() { return groups_of(lane, min(c.len[u] + 1 - s0, rows_alloc)); };
+    if (lane < MW && !done) {
+      n = live_groups();
+      if (n != na) { base = early; total = early + 2 * n; }
+    }
+    __syncwarp();
+    asm volatile("bar.arrive 2, %0;" ::"n"(WT + 32) : "memory");      // the live range has been read, see below
+    uint64_t t0 = 0;
+    for (uint32_t spins = 1; __any_sync(0xffffffffu, !done); ++spins) {
+      if (!done && lane < MW) {
+        if (j >= total) {
+          u += u_step;
+          done = u >= units;
+          if (!done) { n = live_groups(); j = base = 0; total = 2 * n; }
+        } else if (use == 0 || mbar_test(&empty[lane * MAX_SLOTS + slot], (use - 1) & 1)) {
+          issue(lane, u, j - base, n, slot);
+          ++j;
+          if (++slot == nslot) { slot = 0; ++use; }
+          spins = 0;
+        }
+      } else if (!done) {
+        if (use == 0 || mbar_test(state_empty, (use - 1) & 1)) {
+          bring_state(u);
+          ++use;
+          u += u_step;
+          done = u >= units;
+          spins = 0;
+        }
+      }
+      if ((spins & 1023u) == 1023u) {      // nothing moved for a while: a bounded wait (lanes vote, so that all leave together)
+        const uint64_t now = global_ns();
+        if (t0 == 0) t0 = now;
+        if (now - t0 > 1000000000ull) {
+          if (!done && dev_status) atomicExch(dev_status, (int)VATP_ERR_TIMEOUT);
+          done = true;
+        }
+      } else if (spins == 0) {
+        t0 = 0;
+      }
+    }
+    if (split > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (independent && lane == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
     return;
   }
+
+  const int na_mine = groups_of(wid, rows_alloc), early_mine = min(nslot, 2 * na_mine);
+  if (!FEED) {
+    if (independent && tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (lane == 0)
+      for (int j = 0; j < early_mine; ++j) issue(wid, u0, j, na_mine, j);
+    if (!independent && l2_rows > 0 && lane == 0 && wid < 2) prefetch_rows(wid == 1);
+    __syncwarp();
+  }
+  if (!independent) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (!FEED && tid == 32 && rows_alloc > 0 && state_in_smem != 2) bring_state(u0);
+  uint64_t* my_full = &full[wid * MAX_SLOTS];
+  uint64_t* my_empty = &empty[wid * MAX_SLOTS];
+  unsigned char* my_ring = ring_base + (size_t)wid * nslot * UNIT;
+  int slot = 0, par = 0;                  // ring position of the next unit this warp consumes
+  int at = 0, last = 2 * na_mine, base = 0, n = na_mine;   // !FEED: its number, how many there are, those dropped, live groups
+  bool bad = false;                       // this lane's wait ran out: it no longer waits, the results are void
+  // ldmatrix lane addressing: matrix i = lane / 8, row r = lane % 8.  A tile row is 128 bytes and its
+  // 16-byte chunk c sits at position c ^ (row % 8).
+  //   K (plain):  matrices (rows 0-7, k lo), (rows 0-7, k hi), (rows 8-15, k lo), (rows 8-15, k hi)
+  //   V (trans):  matrices (rows 0-7, ch lo), (rows 0-7, ch hi), (rows 8-15, ch lo), (rows 8-15, ch hi): the A operand V^T
+  const uint32_t row_off = (uint32_t)(((lane >> 4) * 8 + (lane & 7)) * 128), lm_x = (uint32_t)(((lane >> 3) & 1) ^ (lane & 7));
+  auto arrived = [&]() {                  // the next unit is complete
+    if (!bad && !mbar_wait(&my_full[slot], par)) bad = true;
+    __syncwarp();
+  };
+  auto release = [&](bool wrote) {        // this warp has read it: the slot may be filled again
+    // generic-proxy stores into the slot must be ordered before the next bulk copy into it
+    if (wrote) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+    if (FEED) {
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&my_empty[slot])) : "memory");
+    } else {
+      if (lane == 0 && !bad && at + nslot < last) issue(wid, u0, at + nslot - base, n, slot);
+      ++at;
+    }
+    if (++slot == nslot) { slot = 0; par ^= 1; }
+  };
+  const bool has_chunk = (lane & 15) < ROW_CHUNKS;
+  auto patch_row = [&](unsigned char* tile, int rr, const uint4& raw, bool v_half) {
+    const int ch = lane & 15;
+    if (has_chunk && (lane >= 16) == v_half)
+      *reinterpret_cast<uint4*>(tile + (ch >> 3) * TILE_BYTES + rr * 128 + (((ch & 7) ^ (rr & 7)) << 4)) = raw;
+  };
+  uint32_t state_par = 0;
+
+  for (int u = u0; u < units; u += u_step) {
+  const int len_m = c.len[u];
+  const int fs_m = c.free_slot[u];
+  const int t = c.next_pos[u];
+  const int ls_m = c.last_slot[u];
+#ifdef VATP_DEBUG_BOUNDS
+  // the state words come from memory: out of range they are clamped and reported (every access below stays inside)
+  (void)(VATP_INB(len_m, cap, dev_status) && VATP_INB(fs_m, cap, dev_status) && VATP_INB(ls_m + 1, cap + 1, dev_status));
+  const int len = min(max(len_m, 0), cap - 1), fs = min(max(fs_m, 0), cap - 1), ls = min(max(ls_m, -1), cap - 1);
+#else
+  const int len = len_m, fs = fs_m, ls = ls_m;
 #endif
   const int hi = len + 1;                // slots [0, hi) are live once the new token is in
   const int cnt = max(min(hi - s0, rows_alloc), 0);
   const int fs_local = fs - s0;          // row of the incoming token inside this CTA's range (if owned)
   const bool owns_new = fs_local >= 0 && fs_local < cnt;
-  if (WINDOWED && tid == 64 && rows_alloc > 0) {
-    // the tail reads the ring row that leaves the window and the exact sums: have them in L2 by then
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(c.ring + ((int64_t)u * w + (t % w)) * cap + s0), "r"(rows_alloc * 4) : "memory");
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(c.acc_fixed + (int64_t)u * cap + s0), "r"(rows_alloc * 8) : "memory");
-  }
-  if (tid == 0) ctrl_evicting = hi > B ? 1 : 0;     // read by the control warp after the first barrier
   const int ls_local = ls - s0;          // row the previous step appended (its tile may predate that store)
   const bool owns_last = !independent && ls >= 0 && ls != fs && ls_local >= 0 && ls_local < cnt;
 
@@ -323,19 +453,20 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
     qa[ks][0] = __ldg(reinterpret_cast<const uint32_t*>(qn + ks * 16 + 2 * j4));
     qa[ks][1] = __ldg(reinterpret_cast<const uint32_t*>(qn + ks * 16 + 8 + 2 * j4));
   }
-  // 16 bytes of the incoming K row (lanes 0-15) or V row (lanes 16-31); with head_dim 64 the first eight lanes of each half
-  const bool has_chunk = (lane & 15) < ROW_CHUNKS;
-  uint4 new_raw = make_uint4(0u, 0u, 0u, 0u);
-  if (has_chunk) new_raw = __ldg(reinterpret_cast<const uint4*>((lane < 16 ? k_new : v_new) + (int64_t)u * HD) + (lane & 15));
-
-  uint4 last_raw = make_uint4(0u, 0u, 0u, 0u);
-  if (owns_last && has_chunk)
+  // ---- the group that holds the incoming token's row: its warp stores the row and its norm (Eq. 4) and patches the
+  // row into the tiles it streams; the group that holds the row of the previous step's token likewise re-reads that row.
+  // Lanes 0-15 take 16 bytes of the K row each, lanes 16-31 of the V row (with head_dim 64 the first eight of each).
+  const int new_warp = owns_new ? (fs_local / GROUP) % MW : -1, last_warp = owns_last ? (ls_local / GROUP) % MW : -1;
+  // the new row's norm is needed by the thread that updates its slot
+  const int norm_warp = owns_new ? (fs_local % WT) / 32 : -1;
+  uint4 new_raw = make_uint4(0u, 0u, 0u, 0u), last_raw = make_uint4(0u, 0u, 0u, 0u);
+  if (has_chunk && (wid == new_warp || wid == norm_warp))
+    new_raw = __ldg(reinterpret_cast<const uint4*>((lane < 16 ? k_new : v_new) + (int64_t)u * HD) + (lane & 15));
+  if (has_chunk && wid == last_warp)
     last_raw = *(reinterpret_cast<const uint4*>((const __nv_bfloat16*)(lane < 16 ? c.k_cache : c.v_cache) +
                                                 ((int64_t)u * cap + ls) * HD) + (lane & 15));
-
-  // ---- append: the CTA that owns the free slot stores the new row and its norm (Eq. 4) ----
   float new_norm = 0.f;
-  {
+  if (wid == new_warp || wid == norm_warp) {
     const uint32_t wv[4] = {new_raw.x, new_raw.y, new_raw.z, new_raw.w};
 #pragma unroll
     for (int i = 0; i < 4; ++i)
@@ -343,278 +474,225 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
 #pragma unroll
     for (int o = 8; o; o >>= 1) new_norm = norm_merge(norm, new_norm, __shfl_xor_sync(0xffffffffu, new_norm, o));
     new_norm = norm_finish(norm, __shfl_sync(0xffffffffu, new_norm, 16));      // the V half's partial
-  }
-  if (owns_new && wid == 0) {
-    __nv_bfloat16* dst = (__nv_bfloat16*)(lane < 16 ? c.k_cache : c.v_cache) + ((int64_t)u * cap + fs) * HD;
-    if (has_chunk) reinterpret_cast<uint4*>(dst)[lane & 15] = new_raw;
-    if (lane == 0) {
-      c.vnorm[(int64_t)u * cap + fs] = new_norm;
-      c.pos[(int64_t)u * cap + fs] = t;
-    }
-  }
-  if (split > 1) cluster_wait_acquire();
-
-  // ---- stream the groups: logits, online softmax, partial output ----
-  float m_run = -INFINITY, l_run = 0.f;
-  float o_acc[HD / 8][4];
-#pragma unroll
-  for (int i = 0; i < HD / 8; ++i) { o_acc[i][0] = o_acc[i][1] = o_acc[i][2] = o_acc[i][3] = 0.f; }
-  bool ok = true;
-  // ldmatrix lane addressing: matrix i = lane / 8, row r = lane % 8.  A tile row is 128 bytes and its
-  // 16-byte chunk c sits at position c ^ (row % 8).
-  //   K (plain):  matrices (rows 0-7, k lo), (rows 0-7, k hi), (rows 8-15, k lo), (rows 8-15, k hi)
-  //   V (trans):  matrices (rows 0-7, n lo), (rows 8-15, n lo), (rows 0-7, n hi), (rows 8-15, n hi)
-  const int lm_i = lane >> 3, lm_r = lane & 7;
-  const uint32_t k_row_off = (uint32_t)(((lm_i >> 1) * 8 + lm_r) * 128), k_x = (uint32_t)((lm_i & 1) ^ lm_r);
-  const uint32_t v_row_off = (uint32_t)(((lm_i & 1) * 8 + lm_r) * 128), v_x = (uint32_t)((lm_i >> 1) ^ lm_r);
-  // the running partial goes to its stream's slot (every lane with the same j4 holds the same values; rows 0-7
-  // are the hi part, 8-15 the lo part)
-  auto flush = [&](int stream) {
-    float l = l_run;
-    l += __shfl_xor_sync(0xffffffffu, l, 1);
-    l += __shfl_xor_sync(0xffffffffu, l, 2);
-    if constexpr (GT > 1) {
-      const int hg = lane >> 2;      // this lane's head
-      if (hg < G) {
-        float* po = gq_part + ((size_t)stream * G + hg) * HD;
-#pragma unroll
-        for (int i = 0; i < HD / 8; ++i)
-          *reinterpret_cast<float2*>(&po[i * 8 + 2 * j4]) = make_float2(o_acc[i][0] + o_acc[i][2], o_acc[i][1] + o_acc[i][3]);
-        if (j4 == 0) { gq_pm[stream][hg] = m_run; gq_pl[stream][hg] = l; }
+    if (wid == new_warp) {
+      __nv_bfloat16* dst = (__nv_bfloat16*)(lane < 16 ? c.k_cache : c.v_cache) + ((int64_t)u * cap + fs) * HD;
+      if (has_chunk) reinterpret_cast<uint4*>(dst)[lane & 15] = new_raw;
+      if (lane == 0) {
+        c.vnorm[(int64_t)u * cap + fs] = new_norm;
+        c.pos[(int64_t)u * cap + fs] = t;
       }
-    } else if (lane < 4) {
-#pragma unroll
-      for (int i = 0; i < HD / 8; ++i)
-        *reinterpret_cast<float2*>(&part_o[stream][i * 8 + 2 * j4]) = make_float2(o_acc[i][0] + o_acc[i][2], o_acc[i][1] + o_acc[i][3]);
-      if (lane == 0) { part_m[stream] = m_run; part_l[stream] = l; }
     }
-  };
-  int it = 0, g = g_first;
-  bool past_live = false, second = false;
-  // folds this warp's groups below g_stop into the running partial
-  auto fold_groups = [&](int g_stop) {
-    for (; g < g_stop; g += 4, ++it) {
-      if (it >= nstage && g * GROUP >= cnt) { past_live = true; break; }     // never requested (see the end of the loop body)
-      const int stage = it % nstage;
-      const uint32_t parity = (it / nstage) & 1;
-      if (ok && !mbar_wait(&my_bars[stage], parity)) ok = false;
-      ok = __all_sync(0xffffffffu, ok);
-      unsigned char* ks = my_stages + stage * STAGE_BYTES;
-      unsigned char* vs = ks + NTILE * TILE_BYTES;
-      const int r0 = g * GROUP;
-      bool wrote = false;
-      if (ok && r0 < cnt) {
-        // the incoming token's row is not in the cache yet: patch it in; rows beyond the live range
-        // must not reach the p V product (their probability is 0, but 0 * garbage need not be 0)
-        if (owns_new && fs_local >= r0 && fs_local < r0 + GROUP) {
-          const int rr = fs_local - r0, ch = lane & 15;
-          if (has_chunk) *reinterpret_cast<uint4*>((lane < 16 ? ks : vs) + (ch >> 3) * TILE_BYTES + rr * 128 + (((ch & 7) ^ (rr & 7)) << 4)) = new_raw;
-          wrote = true;
-        }
-        if (owns_last && ls_local >= r0 && ls_local < r0 + GROUP) {
-          const int rr = ls_local - r0, ch = lane & 15;
-          if (has_chunk) *reinterpret_cast<uint4*>((lane < 16 ? ks : vs) + (ch >> 3) * TILE_BYTES + rr * 128 + (((ch & 7) ^ (rr & 7)) << 4)) = last_raw;
-          wrote = true;
-        }
-        if (cnt < r0 + GROUP) {
-          for (int rr = cnt - r0 + (lane >> 4); rr < GROUP && has_chunk; rr += 2)
-            *reinterpret_cast<uint4*>(vs + ((lane >> 3) & 1) * TILE_BYTES + rr * 128 + ((lane & 7) << 4)) = make_uint4(0u, 0u, 0u, 0u);
-          wrote = true;
-        }
-        __syncwarp();
-        // S^T = q K^T: two n-tiles of 8 rows; c[0], c[1] = logits of rows 2 j4, 2 j4 + 1 of the tile
-        float sa[4] = {0.f, 0.f, 0.f, 0.f}, sb[4] = {0.f, 0.f, 0.f, 0.f};
-        const uint32_t kaddr = smem_u32(ks) + k_row_off;
-  #pragma unroll
-        for (int kk = 0; kk < HD / 16; ++kk) {
-          uint32_t bf[4];
-          ldsm_x4(kaddr + (kk >> 2) * TILE_BYTES + ((k_x ^ ((2 * kk) & 7)) << 4), bf);
-          mma_bf16(sa, qa[kk][0], 0u, qa[kk][1], 0u, bf[0], bf[1]);
-          mma_bf16(sb, qa[kk][0], 0u, qa[kk][1], 0u, bf[2], bf[3]);
-        }
-        float s[4] = {sa[0] * scale_log2, sa[1] * scale_log2, sb[0] * scale_log2, sb[1] * scale_log2};
-        const int rows[4] = {r0 + 2 * j4, r0 + 2 * j4 + 1, r0 + 8 + 2 * j4, r0 + 9 + 2 * j4};
-  #pragma unroll
-        for (int i = 0; i < 4; ++i)
-          if (rows[i] >= cnt) s[i] = -INFINITY;
-        if constexpr (GT > 1) {
-          if ((lane >> 2) < G) {
-  #pragma unroll
-            for (int i = 0; i < 4; ++i)
-              if (rows[i] < cnt) logit_s[(lane >> 2) * chunk + rows[i]] = s[i];
-          }
-        } else if (lane < 4) {
-  #pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (rows[i] < cnt) logit_s[rows[i]] = s[i];
-        }
-        float gmax = fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3]));
-        gmax = fmaxf(gmax, __shfl_xor_sync(0xffffffffu, gmax, 1));
-        gmax = fmaxf(gmax, __shfl_xor_sync(0xffffffffu, gmax, 2));
-        if (gmax > m_run) {          // uniform over a tile row's four lanes - over the warp with one head (r0 < cnt guarantees a live row, so gmax is finite)
-          const float f = ex2(m_run - gmax);   // 0 on the first group
-          l_run *= f;
-  #pragma unroll
-          for (int i = 0; i < HD / 8; ++i) { o_acc[i][0] *= f; o_acc[i][1] *= f; o_acc[i][2] *= f; o_acc[i][3] *= f; }
-          m_run = gmax;
-        }
-        float p[4];
-  #pragma unroll
-        for (int i = 0; i < 4; ++i) { p[i] = ex2(s[i] - m_run); l_run += p[i]; }
-        // A operand of p V: rows 0-7 carry the high bf16 half of p, rows 8-15 the remainder
-        const uint32_t hi0 = pack_bf16(p[0], p[1]), hi1 = pack_bf16(p[2], p[3]);
-        const uint32_t lo0 = pack_bf16(p[0] - __uint_as_float(hi0 << 16), p[1] - __uint_as_float(hi0 & 0xffff0000u));
-        const uint32_t lo1 = pack_bf16(p[2] - __uint_as_float(hi1 << 16), p[3] - __uint_as_float(hi1 & 0xffff0000u));
-        const uint32_t vaddr = smem_u32(vs) + v_row_off;
-  #pragma unroll
-        for (int nn = 0; nn < HD / 16; ++nn) {
-          uint32_t bf[4];
-          ldsm_x4_t(vaddr + (nn >> 2) * TILE_BYTES + ((v_x ^ ((2 * nn) & 7)) << 4), bf);
-          mma_bf16(o_acc[2 * nn], hi0, lo0, hi1, lo1, bf[0], bf[1]);
-          mma_bf16(o_acc[2 * nn + 1], hi0, lo0, hi1, lo1, bf[2], bf[3]);
-        }
-      }
-      // generic-proxy stores into a stage must be ordered before the next bulk copy into it
-      if (wrote) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      __syncwarp();
-      const int next = g + nstage * 4;
-      // later requests know the live range: groups beyond it are not fetched
-      if (ok && next < g_end && next * GROUP < cnt) issue(next, stage);
-    }
-  };
-  if (SPW == 2) {
-    // the four-warp kernel: stream wid up to the midpoint, filed, then stream wid + 4 from a fresh partial
-    fold_groups(min(H, g_end));
-    if (!past_live && g < g_end) {
-      flush(wid);
-      second = true;
-      m_run = -INFINITY;
-      l_run = 0.f;
-#pragma unroll
-      for (int i = 0; i < HD / 8; ++i) { o_acc[i][0] = o_acc[i][1] = o_acc[i][2] = o_acc[i][3] = 0.f; }
-      fold_groups(g_end);
-    }
-  } else {
-    fold_groups(g_end);
-  }
-  if (!ok && lane == 0) {
-    // a copy never completed: flag it and give what is still in flight one more bounded wait
-    if (dev_status) atomicExch(dev_status, (int)VATP_ERR_TIMEOUT);
-    for (int s = 0; s < nstage; ++s) mbar_wait(&my_bars[s], 0);
-  }
-  flush(second ? wid + MW : wid);
-  if (SPW == 2 && !second) {      // the four-warp kernel never reached the midpoint: its stream wid + 4 is empty
-    if (lane < HD / 4) *reinterpret_cast<float4*>(&part_o[wid + MW][lane * 4]) = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (lane == 0) { part_m[wid + MW] = -INFINITY; part_l[wid + MW] = 0.f; }
-  }
-  workers_sync<WT>();
-  if (state_in_smem == 2 && tid == 32 && rows_alloc > 0) {
-    // every stage of this CTA has been consumed: the per-slot state of its slots lands there while the
-    // cluster gathers (the stages were last written by bulk copies and read by ldmatrix; warps that
-    // stored into them have fenced)
-    const int64_t o = (int64_t)u * cap + s0;
-    mbar_expect_tx(state_bar, 3u * rows_alloc * 4u);
-    bulk_g2s(acc_s, c.acc + o, rows_alloc * 4, state_bar);
-    bulk_g2s(vn_s, c.vnorm + o, rows_alloc * 4, state_bar);
-    bulk_g2s(pos_s, c.pos + o, rows_alloc * 4, state_bar);
   }
 
-  // ---- CTA partial: max and sum to every CTA of the unit, partial output to rank 0 ----
-  if constexpr (GT > 1) {
-    // per head of the group; thread tid < HD merges channel tid of the eight streams, threads HD .. HD + split - 1
-    // push the head's maximum and sum to the unit's CTAs
-    float* xo0 = split > 1 ? cluster.map_shared_rank(gq_xo, 0) : gq_xo;
-    for (int h = 0; h < G; ++h) {
-      float m_c = -INFINITY;
+  // ---- stream the rows: first all K rows (logits), then, with the CTA's maximum known, all V rows.  In one sweep with an
+  // online softmax every 16-row group was a chain of ~2300 cycles (fragments, products, maximum, exponentials, fragments,
+  // products) that eight warps walked through five times; here the groups of a warp depend on nothing, and exponentials
+  // are taken once per slot instead of once per lane of an MMA tile.
+  n = groups_of(wid, cnt);                // this warp's live groups
+  if (u == u0 && n != na_mine) {          // rows requested before the live range was known: dropped (see the producer)
+    base = early_mine;
+    last = early_mine + 2 * n;
+    for (int i = early_mine; i > 0; --i) { arrived(); release(false); }
+  }
+  float m_run = -INFINITY;                // of head lane / 4 (one head: the same in every lane)
+  for (int r0 = wid * GROUP; r0 < n * MW * GROUP; r0 += MW * GROUP) {
+    const bool has_new = wid == new_warp && fs_local >= r0 && fs_local < r0 + GROUP;
+    const bool has_last = wid == last_warp && ls_local >= r0 && ls_local < r0 + GROUP;
+    // S^T = q K^T, two n-tiles of 8 rows; c[0], c[1] = logits of rows 2 j4, 2 j4 + 1 of the tile
+    arrived();
+    unsigned char* ks = my_ring + slot * UNIT;
+    // the incoming token's row is not in the cache yet: patch it in
+    if (has_new) patch_row(ks, fs_local - r0, new_raw, false);
+    if (has_last) patch_row(ks, ls_local - r0, last_raw, false);
+    if (has_new || has_last) __syncwarp();
+    const uint32_t kaddr = smem_u32(ks) + row_off;
+    // all fragments first (one latency instead of one per step), then two chains per n-tile
+    uint32_t bf[HD / 16][4];
 #pragma unroll
-      for (int i = 0; i < NSTREAM; ++i) m_c = fmaxf(m_c, gq_pm[i][h]);
-      float fw[NSTREAM], l_c = 0.f;
+    for (int kk = 0; kk < HD / 16; ++kk) ldsm_x4(kaddr + (kk >> 2) * TILE_BYTES + ((lm_x ^ ((2 * kk) & 7)) << 4), bf[kk]);
+    float sa[2][4], sb[2][4];
 #pragma unroll
-      for (int i = 0; i < NSTREAM; ++i) {
-        fw[i] = gq_pm[i][h] > -INFINITY ? ex2(gq_pm[i][h] - m_c) : 0.f;
-        l_c += gq_pl[i][h] * fw[i];
-      }
-      if (tid < HD) {
-        float a = 0.f;
+    for (int i = 0; i < 4; ++i) sa[0][i] = sa[1][i] = sb[0][i] = sb[1][i] = 0.f;
 #pragma unroll
-        for (int i = 0; i < NSTREAM; ++i) a = fmaf(gq_part[((size_t)i * G + h) * HD + tid], fw[i], a);
-        xo0[((size_t)rank * G + h) * HD + tid] = a;
-      } else if (tid < HD + split) {
-        const int r = tid - HD;
-        float* rm = split > 1 ? cluster.map_shared_rank(&gq_m[0][0], r) : &gq_m[0][0];
-        float* rl = split > 1 ? cluster.map_shared_rank(&gq_l[0][0], r) : &gq_l[0][0];
-        rm[rank * GT + h] = m_c;
-        rl[rank * GT + h] = l_c;
-      }
+    for (int kk = 0; kk < HD / 16; ++kk) {
+      mma_bf16(sa[kk & 1], qa[kk][0], 0u, qa[kk][1], 0u, bf[kk][0], bf[kk][1]);
+      mma_bf16(sb[kk & 1], qa[kk][0], 0u, qa[kk][1], 0u, bf[kk][2], bf[kk][3]);
     }
-  } else {
+    release(has_new || has_last);
+    float s[4] = {(sa[0][0] + sa[1][0]) * scale_log2, (sa[0][1] + sa[1][1]) * scale_log2, (sb[0][0] + sb[1][0]) * scale_log2,
+                  (sb[0][1] + sb[1][1]) * scale_log2};
+    const int ra = r0 + 2 * j4, rb = ra + 8;      // this lane's rows: ra, ra + 1, rb, rb + 1
+    if (r0 + GROUP > cnt) {
+      if (ra >= cnt) s[0] = -INFINITY;
+      if (ra + 1 >= cnt) s[1] = -INFINITY;
+      if (rb >= cnt) s[2] = -INFINITY;
+      if (rb + 1 >= cnt) s[3] = -INFINITY;
+    }
+    // (chunk is a multiple of 16: dead rows of the last group have logits too, -inf)
+    if (GT > 1 ? (lane >> 2) < G : lane < 4) {
+      float* lg = logit_s + (GT > 1 ? (lane >> 2) * chunk : 0);
+      *reinterpret_cast<float2*>(lg + ra) = make_float2(s[0], s[1]);
+      *reinterpret_cast<float2*>(lg + rb) = make_float2(s[2], s[3]);
+    }
+    m_run = fmaxf(m_run, fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3])));
+  }
+  m_run = fmaxf(m_run, __shfl_xor_sync(0xffffffffu, m_run, 1));
+  m_run = fmaxf(m_run, __shfl_xor_sync(0xffffffffu, m_run, 2));
+  if (GT > 1 ? (j4 == 0 && (lane >> 2) < G) : lane == 0) part_m[wid][GT > 1 ? lane >> 2 : 0] = m_run;
+  // (The first time together with the producer warp: whoever finishes the step rewrites `len`, which every producer of the
+  // unit must have read by then.)
+  if (FEED && u == u0) asm volatile("bar.sync 2, %0;" ::"n"(WT + 32) : "memory");
+  else workers_sync();
+  // The next launch may start: its early requests queue behind this one's (released right after the wait they delayed this
+  // launch's own rows by more than they gained).
+  if (!FEED && !independent && tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // ---- exp2(s - m) of the CTA's slots, in place, and their sum (m: the CTA's maximum, finite when it has a live row)
+  for (int h = 0; h < g_rows; ++h) {
     float m_c = -INFINITY;
 #pragma unroll
-    for (int i = 0; i < NSTREAM; ++i) m_c = fmaxf(m_c, part_m[i]);
-    float fw[NSTREAM], l_c = 0.f;
-#pragma unroll
-    for (int i = 0; i < NSTREAM; ++i) {
-      fw[i] = part_m[i] > -INFINITY ? ex2(part_m[i] - m_c) : 0.f;
-      l_c += part_l[i] * fw[i];
+    for (int k = 0; k < MW; ++k) m_c = fmaxf(m_c, part_m[k][h]);
+    float l = 0.f;
+    float* lg = logit_s + h * chunk;
+    for (int i = tid; i < (cnt + GROUP - 1) / GROUP * GROUP; i += WT) {
+      const float e = ex2(lg[i] - m_c);
+      lg[i] = e;
+      l += e;
     }
-    Exch<HD>* e0 = split > 1 ? cluster.map_shared_rank(&ex, 0) : &ex;
-    if (tid < HD) {
-      float a = 0.f;
 #pragma unroll
-      for (int i = 0; i < NSTREAM; ++i) a = fmaf(part_o[i][tid], fw[i], a);
-      e0->o[rank][tid] = a;
+    for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    if (lane == 0) part_l[wid][h] = l;
+  }
+  workers_sync();
+  // ---- O^T += V^T p
+  float o_acc[HD / 16][4];                // channels 16 i + lane / 4 (+ 8) x columns 2 j4, 2 j4 + 1 of O^T
+#pragma unroll
+  for (int i = 0; i < HD / 16; ++i) { o_acc[i][0] = o_acc[i][1] = o_acc[i][2] = o_acc[i][3] = 0.f; }
+  const float* p_s = logit_s + (GT > 1 ? min(lane >> 2, G - 1) * chunk : 0) + 2 * j4;
+  for (int r0 = wid * GROUP; r0 < n * MW * GROUP; r0 += MW * GROUP) {
+    const bool has_new = wid == new_warp && fs_local >= r0 && fs_local < r0 + GROUP;
+    const bool has_last = wid == last_warp && ls_local >= r0 && ls_local < r0 + GROUP;
+    const float2 pa = *reinterpret_cast<const float2*>(p_s + r0), pb = *reinterpret_cast<const float2*>(p_s + r0 + 8);
+    // B operand of V^T p: the high bf16 half of p and the remainder - in the even and odd columns with one head, as two
+    // products otherwise (the columns are heads then)
+    const uint32_t hi0 = pack_bf16(pa.x, pa.y), hi1 = pack_bf16(pb.x, pb.y);
+    const uint32_t lo0 = pack_bf16(pa.x - __uint_as_float(hi0 << 16), pa.y - __uint_as_float(hi0 & 0xffff0000u));
+    const uint32_t lo1 = pack_bf16(pb.x - __uint_as_float(hi1 << 16), pb.y - __uint_as_float(hi1 & 0xffff0000u));
+    const uint32_t b0 = (GT == 1 && (lane & 4)) ? lo0 : hi0, b1 = (GT == 1 && (lane & 4)) ? lo1 : hi1;
+    arrived();
+    unsigned char* vs = my_ring + slot * UNIT;
+    if (has_new) patch_row(vs, fs_local - r0, new_raw, true);
+    if (has_last) patch_row(vs, ls_local - r0, last_raw, true);
+    const bool ragged = cnt < r0 + GROUP;
+    // rows beyond the live range must not reach the product (their probability is 0, but 0 * garbage need not be 0)
+    if (ragged)
+      for (int rr = cnt - r0 + (lane >> 4); rr < GROUP && has_chunk; rr += 2)
+        *reinterpret_cast<uint4*>(vs + ((lane >> 3) & 1) * TILE_BYTES + rr * 128 + ((lane & 7) << 4)) = make_uint4(0u, 0u, 0u, 0u);
+    if (has_new || has_last || ragged) __syncwarp();
+    const uint32_t vaddr = smem_u32(vs) + row_off;
+    uint32_t af[HD / 16][4];
+#pragma unroll
+    for (int nn = 0; nn < HD / 16; ++nn) ldsm_x4_t(vaddr + (nn >> 2) * TILE_BYTES + ((lm_x ^ ((2 * nn) & 7)) << 4), af[nn]);
+#pragma unroll
+    for (int nn = 0; nn < HD / 16; ++nn) {
+      mma_bf16(o_acc[nn], af[nn][0], af[nn][1], af[nn][2], af[nn][3], b0, b1);
+      if (GT > 1) mma_bf16(o_acc[nn], af[nn][0], af[nn][1], af[nn][2], af[nn][3], lo0, lo1);
     }
-    if (tid < split) {
-      Exch<HD>* er = split > 1 ? cluster.map_shared_rank(&ex, tid) : &ex;
-      er->m[rank] = m_c;
-      er->l[rank] = l_c;
+    release(has_new || has_last || ragged);
+  }
+  // ---- the warp's partial
+  {
+    float* po = part_o + (size_t)wid * part_ld;
+    const int row = lane >> 2;
+    __syncwarp();                         // (part_in_ring: every lane is past its last read of the ring)
+    if constexpr (GT > 1) {
+#pragma unroll
+      for (int i = 0; i < HD / 16; ++i) {
+        if (2 * j4 < G) { po[2 * j4 * HD + 16 * i + row] = o_acc[i][0]; po[2 * j4 * HD + 16 * i + 8 + row] = o_acc[i][2]; }
+        if (2 * j4 + 1 < G) { po[(2 * j4 + 1) * HD + 16 * i + row] = o_acc[i][1]; po[(2 * j4 + 1) * HD + 16 * i + 8 + row] = o_acc[i][3]; }
+      }
+    } else {
+      // every column pair holds the same two halves: lane j4 writes two of the eight tiles
+#pragma unroll
+      for (int i = 0; i < HD / 16; ++i)
+        if ((i & 3) == j4) { po[16 * i + row] = o_acc[i][0] + o_acc[i][1]; po[16 * i + 8 + row] = o_acc[i][2] + o_acc[i][3]; }
     }
   }
-  if (split > 1) { cluster_arrive_release(); cluster_wait_acquire(); } else workers_sync<WT>();
+  workers_sync();
+  if (split > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  // every unit of this CTA has been consumed: the per-slot state of its slots lands in the rings while the CTAs of
+  // the unit exchange (they were last written by bulk copies and read by ldmatrix; warps that stored into them have
+  // fenced)
+  if (!part_in_ring && state_in_smem == 2 && tid == 32 && rows_alloc > 0) copy_state(u, t);
 
-  // ---- every CTA: the unit's softmax normaliser (all data is local now) ----
+  // ---- CTA partial: max and sum to every CTA of the unit, channel slice r of the partial output to rank r ----
+  const int slice = HD / split;           // channels a CTA of the unit sums up and writes
+  for (int i = tid; i < g_rows * HD; i += WT) {
+    const int h = GT > 1 ? i / HD : 0, ch = GT > 1 ? i - h * HD : i;
+    float m_c = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < MW; ++k) m_c = fmaxf(m_c, part_m[k][h]);
+    float a = 0.f, l_c = 0.f;
+#pragma unroll
+    for (int k = 0; k < MW; ++k) {
+      l_c += part_l[k][h];
+      a += part_o[(size_t)k * part_ld + h * HD + ch];
+    }
+    const int dst = ch / slice, off = (rank * g_rows + h) * slice + (ch - dst * slice);
+    if (split > 1) {
+      st_async(map_rank(smem_u32(&xo[off]), dst), a, map_rank(smem_u32(ex_bar), dst));
+      if (ch < split) st_async2(map_rank(smem_u32(&ex_ml[rank][h]), ch), m_c, l_c, map_rank(smem_u32(ex_bar), ch));
+    } else {
+      xo[off] = a;
+      if (ch == 0) ex_ml[0][h] = make_float2(m_c, l_c);
+    }
+  }
+  if (split > 1) {
+    if (!mbar_wait(ex_bar, 0)) bad = true;
+  } else {
+    workers_sync();
+  }
+
+  // ---- every CTA: the unit's softmax normaliser (all data is local now) and its slice of the output ----
+  float m_all = -INFINITY, own_f = 0.f;    // own_f: this CTA's exp2(s - m) -> probability
   if constexpr (GT > 1) {
     if (tid < G) {         // one thread per head
       float m_h = -INFINITY, L_h = 0.f;
-      for (int r = 0; r < split; ++r) m_h = fmaxf(m_h, gq_m[r][tid]);
+      for (int r = 0; r < split; ++r) m_h = fmaxf(m_h, ex_ml[r][tid].x);
       for (int r = 0; r < split; ++r) {
-        const float f = gq_m[r][tid] > -INFINITY ? ex2(gq_m[r][tid] - m_h) : 0.f;
+        const float f = ex_ml[r][tid].x > -INFINITY ? ex2(ex_ml[r][tid].x - m_h) : 0.f;
         gq_fr[r][tid] = f;
-        L_h += gq_l[r][tid] * f;
+        L_h += ex_ml[r][tid].y * f;
       }
-      gq_mall[tid] = m_h;
       gq_invl[tid] = 1.f / L_h;
+      gq_f[tid] = gq_fr[rank][tid] * (1.f / L_h);       // this CTA's exp2(s - m) -> probability
     }
-    workers_sync<WT>();
-    if (rank == 0 && tid < HD) {
-      for (int h = 0; h < G; ++h) {
-        float a = 0.f;
-        for (int r = 0; r < split; ++r) a = fmaf(gq_xo[((size_t)r * G + h) * HD + tid], gq_fr[r][h], a);
-        out[((int64_t)u * G + h) * HD + tid] = __float2bfloat16(a * gq_invl[h]);
-      }
+    workers_sync();
+    for (int i = tid; i < G * slice; i += WT) {
+      const int h = i / slice, ch = i - h * slice;
+      float a = 0.f;
+      for (int r = 0; r < split; ++r) a = fmaf(xo[(r * G + h) * slice + ch], gq_fr[r][h], a);
+      out[((int64_t)u * G + h) * HD + rank * slice + ch] = __float2bfloat16(a * gq_invl[h]);
     }
-  }
-  float m_all = -INFINITY, L = 0.f;
-  float fr[MAX_SPLIT];
-#pragma unroll
-  for (int r = 0; r < MAX_SPLIT; ++r)
-    if (r < split) m_all = fmaxf(m_all, ex.m[r]);
-#pragma unroll
-  for (int r = 0; r < MAX_SPLIT; ++r) {
-    fr[r] = (r < split && ex.m[r] > -INFINITY) ? ex2(ex.m[r] - m_all) : 0.f;
-    if (r < split) L += ex.l[r] * fr[r];
-  }
-  const float invL = 1.f / L;
-  if (GT == 1 && rank == 0 && tid < HD) {
-    float a = 0.f;
+  } else {
+    float L = 0.f, a = 0.f;
 #pragma unroll
     for (int r = 0; r < MAX_SPLIT; ++r)
-      if (r < split) a = fmaf(ex.o[r][tid], fr[r], a);
-    out[(int64_t)u * HD + tid] = __float2bfloat16(a * invL);
+      if (r < split) m_all = fmaxf(m_all, ex_ml[r][0].x);
+#pragma unroll
+    for (int r = 0; r < MAX_SPLIT; ++r)
+      if (r < split) {
+        const float f = ex_ml[r][0].x > -INFINITY ? ex2(ex_ml[r][0].x - m_all) : 0.f;
+        L += ex_ml[r][0].y * f;
+        if (r == rank) own_f = f;
+        if (tid < slice) a = fmaf(xo[r * slice + tid], f, a);
+      }
+    const float invL = 1.f / L;
+    own_f *= invL;
+    if (tid < slice) out[(int64_t)u * HD + rank * slice + tid] = __float2bfloat16(a * invL);
   }
 
   // ---- indicator update (Eq. 2 / Eq. 3) and importance (Eq. 4) of this CTA's slots, its arg-min ----
-  if (state_in_smem && rows_alloc > 0 && !mbar_wait(state_bar, 0) && dev_status) atomicExch(dev_status, (int)VATP_ERR_TIMEOUT);
+  if (state_in_smem && rows_alloc > 0 && !mbar_wait(state_full, state_par)) bad = true;
   const bool evicting = hi > B;
   unsigned long long my_key = NO_KEY;
   int my_slot = -1, my_pos = -1;
@@ -627,39 +705,39 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
     float* __restrict__ acc_g = c.acc + (int64_t)u * cap + s0;
 #pragma unroll 4
     for (int i = tid; i < cnt; i += WT) {
-      const int slot = s0 + i;
+      const int slot_u = s0 + i;
       float p;
       if constexpr (GT > 1) {      // the mean of the heads' probabilities
         float a = 0.f;
-        for (int h = 0; h < G; ++h) a = fmaf(ex2(lg[h * chunk + i] - gq_mall[h]), gq_invl[h], a);
+        for (int h = 0; h < G; ++h) a = fmaf(lg[h * chunk + i], gq_f[h], a);
         p = a / (float)G;
       } else {
-        p = ex2(lg[i] - m_all) * invL;
+        p = lg[i] * own_f;
       }
-      const bool is_new = slot == fs;
+      const bool is_new = slot_u == fs;
       float S;
       if (WINDOWED) {
         float* ring_row = c.ring + ((int64_t)u * w + (t % w)) * cap;
-        const int64_t o = (int64_t)u * cap + slot;
+        const int64_t o = (int64_t)u * cap + slot_u;
         long long fx;
         if (is_new) {
           fx = prob_to_fixed(p);     // (the recycled slot's ring column is cleared below)
         } else {
-          fx = c.acc_fixed[o] + prob_to_fixed(p) - prob_to_fixed(ring_row[slot]);
+          fx = (state_in_smem ? fx_s[i] : c.acc_fixed[o]) + prob_to_fixed(p) - prob_to_fixed(state_in_smem ? as[i] : ring_row[slot_u]);
         }
-        ring_row[slot] = p;
+        ring_row[slot_u] = p;
         c.acc_fixed[o] = fx;
         S = fixed_to_prob(fx);
       } else {
         S = is_new ? p : (state_in_smem ? as[i] : acc_g[i]) + p;
       }
-      if (VATP_INB((int64_t)u * cap + slot, (int64_t)gridDim.x / split * cap, dev_status)) acc_g[i] = S;
+      if (VATP_INB((int64_t)u * cap + slot_u, (int64_t)units * cap, dev_status)) acc_g[i] = S;
       if (evicting) {
-        const int ps = is_new ? t : (state_in_smem ? ps_s[i] : c.pos[(int64_t)u * cap + slot]);
-        const float I = S * (is_new ? new_norm : (state_in_smem ? vs[i] : c.vnorm[(int64_t)u * cap + slot]));
+        const int ps = is_new ? t : (state_in_smem ? ps_s[i] : c.pos[(int64_t)u * cap + slot_u]);
+        const float I = S * (is_new ? new_norm : (state_in_smem ? vs[i] : c.vnorm[(int64_t)u * cap + slot_u]));
         if (ps >= F && ps <= t - R) {
           const unsigned long long key = evict_key(I, ps);
-          if (key < my_key) { my_key = key; my_slot = slot; my_pos = ps; }
+          if (key < my_key) { my_key = key; my_slot = slot_u; my_pos = ps; }
         }
       }
     }
@@ -667,54 +745,64 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   if (WINDOWED) {
     // recycled slot: the other rows of its ring column belong to the previous occupant (shared out over the unit's CTAs)
     for (int rr = rank * WT + tid; rr < w; rr += split * WT)
-      if (rr != t % w && VATP_INB(((int64_t)u * w + rr) * cap + fs, (int64_t)gridDim.x / split * w * cap, dev_status))
+      if (rr != t % w && VATP_INB(((int64_t)u * w + rr) * cap + fs, (int64_t)units * w * cap, dev_status))
         c.ring[((int64_t)u * w + rr) * cap + fs] = 0.f;
   }
-  if (!evicting) {
-    if (rank == 0 && tid == 0) {
-      c.len[u] = hi;
-      c.free_slot[u] = hi;
-      c.next_pos[u] = t + 1;
-      c.last_slot[u] = fs;
-      if (evicted) evicted[u] = -1;
-    }
-    return;
+  // (units of one CTA one after the other: the next one's logits, partials and state may replace this one's)
+  const bool more = u + u_step < units;
+  if (state_in_smem == 1) {
+    if (more) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(state_empty)) : "memory");
+    state_par ^= 1;
   }
-  // this CTA's candidate (positions are unique: exactly one thread holds the winning key), pushed to rank 0
-  {
+  if (evicting) {
+    // this CTA's candidate (positions are unique: exactly one thread holds the winning key), sent to rank 0
     const unsigned long long wkey = warp_min_key(my_key);
     if (lane == 0) warp_key[wid] = wkey;
-    workers_sync<WT>();
+    workers_sync();
     const unsigned long long win = warp_min_key(lane < MW ? warp_key[lane] : NO_KEY);
-    Exch<HD>* e0 = split > 1 ? cluster.map_shared_rank(&ex, 0) : &ex;
-    if (win == NO_KEY) {
-      if (tid == 0) e0->key[rank] = NO_KEY;
-    } else if (my_key == win) {
-      e0->key[rank] = win;
-      e0->key_slot[rank] = my_slot;
-      e0->key_pos[rank] = my_pos;
+    if (win == NO_KEY ? tid == 0 : my_key == win) {
+      if (split > 1)
+        st_async4(map_rank(smem_u32(&cand[rank]), 0), (uint32_t)win, (uint32_t)(win >> 32), (uint32_t)my_slot, (uint32_t)my_pos,
+                  map_rank(smem_u32(cand_bar), 0));
+      else
+        cand[0] = Candidate{win, my_slot, my_pos};
     }
   }
-  if (split > 1) { cluster_arrive_release(); cluster_wait_acquire(); } else workers_sync<WT>();
-  if (rank != 0 || tid != 0) return;      // nothing of the other CTAs' shared memory is read by anyone
-  {
-    unsigned long long best = NO_KEY;
-    int br = -1;
-    for (int r = 0; r < split; ++r)
-      if (ex.key[r] < best) { best = ex.key[r]; br = r; }
-    if (br >= 0) {
-      const int slot = ex.key_slot[br];
-      if (VATP_INB(slot, cap, dev_status)) c.pos[(int64_t)u * cap + slot] = -1;
-      c.free_slot[u] = slot;
-      c.len[u] = hi - 1;
-      if (evicted) evicted[u] = ex.key_pos[br];
-    } else {   // nothing eligible (cannot happen when F + R <= B): keep the state consistent
-      c.len[u] = hi;
-      c.free_slot[u] = min(hi, cap - 1);
-      if (evicted) evicted[u] = -1;
+  if (split == 1) workers_sync();
+  if (rank == 0 && tid == 0) {            // nothing of the other CTAs' shared memory is read or written by anyone any more
+    int out_slot = hi, left = hi, ev = -1;                         // not evicting: the cache grows
+    if (evicting) {
+      if (split > 1 && !mbar_wait(cand_bar, 0)) bad = true;
+      unsigned long long best = NO_KEY;
+      int br = -1;
+      for (int r = 0; r < split; ++r)
+        if (cand[r].key < best) { best = cand[r].key; br = r; }
+      if (br >= 0) {
+        out_slot = cand[br].slot;
+        ev = cand[br].pos;
+        left = hi - 1;
+        if (VATP_INB(out_slot, cap, dev_status)) c.pos[(int64_t)u * cap + out_slot] = -1;
+      } else {   // nothing eligible (cannot happen when F + R <= B): keep the state consistent
+        out_slot = min(hi, cap - 1);
+      }
     }
+    c.len[u] = left;
+    c.free_slot[u] = out_slot;
     c.next_pos[u] = t + 1;
     c.last_slot[u] = fs;
+    if (evicted) evicted[u] = ev;
+  }
+  }   // next unit of this CTA
+  if (!FEED && independent && tid == WT - 1) asm volatile("griddepcontrol.wait;" ::: "memory");     // (launches complete in order)
+  if (bad) {
+    // Something never completed: flag it, give copies that may still be in flight time to land, and stay until the unit's
+    // other CTAs have sent what they send here (threads that exit count as arrived).
+    if (dev_status) atomicExch(dev_status, (int)VATP_ERR_TIMEOUT);
+    for (int i = 0; i < 200; ++i) __nanosleep(1000);
+    if (split > 1) {
+      asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+      asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    }
   }
 }
 
@@ -823,60 +911,56 @@ namespace {
 
 template <int HD>
 cudaError_t launch_hd(const Shape& s, int B, int F, int R, const vatp_cache& c, const void* q, const void* k,
-                              const void* v, void* out, int32_t* evicted, int32_t* dev_status, cudaStream_t st,
-                              bool may_overlap, int G) {
-  constexpr int STAGE_BYTES = stage_bytes<HD>, ROW_BYTES = HD * 2;
+                      const void* v, void* out, int32_t* evicted, int32_t* dev_status, cudaStream_t st,
+                      bool may_overlap, int G) {
+  constexpr int UNIT = unit_bytes<HD>, ROW_BYTES = HD * 2;
   const int cap = cache_capacity(B);
   const bool grouped = G > 1;           // s.units counts caches (KV heads); q and out hold G rows per unit
   const int sms = device_sm_count();
   // split a unit over a cluster while the grid still fits on the SMs once (a second launch can then be resident too)
   int split = 1;
-  while (split < (grouped ? GQ_MAX_SPLIT : MAX_SPLIT) && s.units * split * 2 <= sms && cap / (split * 2) >= 4 * GROUP) split *= 2;
+  while (split < MAX_SPLIT && s.units * split * 2 <= sms && cap / (split * 2) >= 4 * GROUP) split *= 2;
   int chunk = (cap + split - 1) / split;
   chunk = (chunk + GROUP - 1) / GROUP * GROUP;
-  // Shared-memory plan.  A launch that may run beside its neighbours stays within half an SM (two CTAs
-  // per SM, so that consecutive launches can both be resident) when at least two stages per warp fit
-  // there beside the per-slot state; large caches leave acc / vnorm / pos out of shared memory to get
-  // there.  A launch that has to wait for its predecessor anyway runs alone: it takes the whole SM and
-  // up to four stages per warp, which doubles the bytes it keeps in flight.
-  struct Plan {
-    int state_in_smem, nstage;
-    size_t dyn;
-    bool ok;
-  };
-  const size_t half_sm = 104 * 1024, whole_sm = 215 * 1024;     // dynamic bytes, 1 KB of it alignment slack
-  const size_t tot = (size_t)chunk;      // slots whose logits and state one CTA holds
-  auto make_plan = [&](bool alone) {
-    Plan p{};
-    const int MW = alone ? MW_ALONE : MW_BESIDE;
-    const size_t stage_set = (size_t)MW * STAGE_BYTES;
-    size_t state_bytes = 4 * sizeof(float) * tot;
-    if (grouped)    // logits per head, the state, the streams' partial outputs per head, rank 0's copy of every CTA's
-      state_bytes = (size_t)(G + 3) * sizeof(float) * tot + (size_t)(NSTREAM + split) * G * HD * sizeof(float);
-    p.state_in_smem = 1;
-    const bool fits_half = !alone && state_bytes + 1024 + 2 * stage_set <= half_sm;
-    if (!alone && !fits_half && sizeof(float) * tot + 1024 + 2 * stage_set <= half_sm) {
-      state_bytes = sizeof(float) * tot;
-      p.state_in_smem = tot * 12 <= 2 * stage_set ? 2 : 0;
-    }
-    p.ok = state_bytes + stage_set + 1024 <= whole_sm;
-    if (!p.ok) return p;
-    const bool half = !alone && state_bytes + 1024 + 2 * stage_set <= half_sm;
-    p.nstage = (int)(((half ? half_sm : whole_sm) - 1024 - state_bytes) / stage_set);
-    p.nstage = p.nstage > 4 ? 4 : p.nstage;
-    const int groups_per_warp = ((chunk / GROUP) + MW - 1) / MW;
-    if (p.nstage > groups_per_warp) p.nstage = groups_per_warp > 0 ? groups_per_warp : 1;
-    if (p.state_in_smem == 2 && tot * 12 > (size_t)MW * p.nstage * STAGE_BYTES) p.state_in_smem = 0;
-    p.dyn = (size_t)MW * p.nstage * STAGE_BYTES + state_bytes + 1024;
-    return p;
-  };
-  const Plan lone = make_plan(true), beside = grouped ? lone : make_plan(false);      // grouped queries: always a whole SM
-  if (!beside.ok || !lone.ok) return cudaErrorNotSupported;
-  CUtensorMap tm_k, tm_v;
-  if (!make_rows_map_bf16(&tm_k, c.k_cache, HD, (uint64_t)s.units * cap, GROUP) ||
-      !make_rows_map_bf16(&tm_v, c.v_cache, HD, (uint64_t)s.units * cap, GROUP))
-    return cudaErrorInvalidValue;
+  // Two CTAs per SM at most; beyond that a CTA takes several units, one after the other (its producer warp then fills the
+  // rings with the next unit's rows while the tail of this one runs).
+  const int resident = 2;
+  const int grid = s.units * split <= resident * sms ? s.units * split : resident * sms;
+  const bool one_unit = grid == s.units * split;
+  // Shared-memory plan.  Half an SM (two CTAs per SM, so that the next launch is resident while this one runs) with as
+  // many units in flight per warp as fit there, at least two; the per-slot state beside them (1), in the rings' memory
+  // after the streaming (2) or in global memory (0).  Only when not even that fits, a whole SM.
   const bool win = s.window > 0;
+  const size_t half_sm = 111 * 1024, whole_sm = 222 * 1024;     // dynamic bytes, 1 KB of it alignment slack
+  const int groups_per_warp = ((chunk / GROUP) + MW - 1) / MW;
+  const bool part_in_ring = grouped && one_unit;                // a warp's partial outputs land in its ring
+  const size_t fixed = 1024 + (part_in_ring ? 0 : (size_t)MW * G * HD * 4) + (size_t)G * HD * 4 + (size_t)G * chunk * 4;
+  const size_t state = (size_t)(win ? 20 : 12) * chunk;
+  const bool copyable = !win || (((uintptr_t)c.ring | (uintptr_t)c.acc_fixed) & 15) == 0;      // (bulk copies: 16-byte aligned)
+  int nslot = 0, state_in_smem = 0;
+  size_t dyn = 0;
+  auto plan = [&](size_t limit, int most) {
+    for (int n = most; n >= 2 && !nslot; --n) {
+      const size_t rings = (size_t)MW * n * UNIT;
+      if (part_in_ring && (size_t)n * UNIT < (size_t)G * HD * 4) continue;
+      if (copyable && rings + fixed + state <= limit) state_in_smem = 1;
+      else if (copyable && !grouped && one_unit && state <= rings && rings + fixed <= limit) state_in_smem = 2;
+      else if (n == 2 && rings + fixed <= limit) state_in_smem = 0;
+      else continue;
+      nslot = n;
+      dyn = rings + fixed + (state_in_smem == 1 ? state : 0);
+    }
+  };
+  int most = 2 * groups_per_warp;
+  most = most < 2 ? 2 : (most > MAX_SLOTS ? MAX_SLOTS : most);
+  if (part_in_ring && (size_t)most * UNIT < (size_t)G * HD * 4) most = (G * HD * 4 + UNIT - 1) / UNIT;
+  plan(half_sm, most);
+  if (!nslot) plan(whole_sm, most);
+  if (!nslot) return cudaErrorNotSupported;
+  CUtensorMap tm_k, tm_v;
+  if (!make_halves_map_bf16(&tm_k, c.k_cache, HD, (uint64_t)s.units * cap, GROUP) ||
+      !make_halves_map_bf16(&tm_v, c.v_cache, HD, (uint64_t)s.units * cap, GROUP))
+    return cudaErrorInvalidValue;
   const size_t units = (size_t)s.units, slots = units * cap;
   Range written[16] = {{(const char*)c.k_cache, slots * ROW_BYTES}, {(const char*)c.v_cache, slots * ROW_BYTES},
                        {(const char*)c.acc, slots * 4}, {(const char*)c.vnorm, slots * 4}, {(const char*)c.pos, slots * 4},
@@ -886,29 +970,25 @@ cudaError_t launch_hd(const Shape& s, int B, int F, int R, const vatp_cache& c, 
                        {win ? (const char*)c.ring : nullptr, win ? slots * s.window * 4 : 0},
                        {win ? (const char*)c.acc_fixed : nullptr, win ? slots * 8 : 0},
                        {(const char*)q, units * G * ROW_BYTES}, {(const char*)k, units * ROW_BYTES}, {(const char*)v, units * ROW_BYTES}};
-  auto kern_alone = grouped ? (win ? decode_mma_kernel<HD, true, MW_ALONE, GQ_HEADS> : decode_mma_kernel<HD, false, MW_ALONE, GQ_HEADS>)
-                            : (win ? decode_mma_kernel<HD, true, MW_ALONE, 1> : decode_mma_kernel<HD, false, MW_ALONE, 1>);
-  auto kern_beside = grouped ? kern_alone : (win ? decode_mma_kernel<HD, true, MW_BESIDE, 1> : decode_mma_kernel<HD, false, MW_BESIDE, 1>);
-  cudaError_t e = cudaFuncSetAttribute(kern_beside, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)whole_sm);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(kern_alone, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)whole_sm);
+  // One CTA per SM at most: no producer warp (see the kernel; 32 units x 2049 slots 10.4 us per waiting step against 12.7
+  // with one).  Beyond that it pays (512 units x 1025 slots with a history window 57 us against 79).
+  const bool feed = grid > sms;
+  auto kern = feed ? (grouped ? (win ? decode_mma_kernel<HD, true, GQ_HEADS, true> : decode_mma_kernel<HD, false, GQ_HEADS, true>)
+                              : (win ? decode_mma_kernel<HD, true, 1, true> : decode_mma_kernel<HD, false, 1, true>))
+                   : (grouped ? (win ? decode_mma_kernel<HD, true, GQ_HEADS, false> : decode_mma_kernel<HD, false, GQ_HEADS, false>)
+                              : (win ? decode_mma_kernel<HD, true, 1, false> : decode_mma_kernel<HD, false, 1, false>));
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)whole_sm);
   if (e != cudaSuccess) return e;
   // share of the machine this launch holds while resident (every CTA waits for the previous launch before it retires)
-  auto share_of = [&](const Plan& p, bool alone) {
-    int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, alone ? kern_alone : kern_beside,
-                                                      (alone || grouped ? MW_ALONE : MW_BESIDE) * 32 + 32, p.dyn) != cudaSuccess || occ < 1)
-      occ = 1;
-    return (double)(s.units * split) / ((double)occ * sms);
-  };
-  const int independent = independent_of_in_flight(st, capture_of(st), may_overlap, written, 16, written, share_of(beside, false),
-                                                   share_of(lone, true)) ? 1 : 0;
-  const Plan& pl = independent ? beside : lone;
-  auto kern = independent ? kern_beside : kern_alone;
-  const int nstage = pl.nstage, state_in_smem = pl.state_in_smem;
-  const size_t dyn = pl.dyn;
+  const double share = (double)grid / ((double)(dyn <= half_sm ? 2 : 1) * sms);
+  const int independent = independent_of_in_flight(st, capture_of(st), may_overlap, written, 16, written, share, share) ? 1 : 0;
+  // Rows of K (and of V) that a waiting CTA asks for in L2 ahead of its wait: all it has, as long as a launch's rows take
+  // no more than a third of the 126 MB.
+  const int64_t l2_most = ((int64_t)40 << 20) / ((int64_t)s.units * split * 2 * ROW_BYTES);
+  const int l2_rows = (int)(l2_most < chunk ? l2_most : chunk);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(s.units * split);
-  cfg.blockDim = dim3((independent && !grouped ? MW_BESIDE : MW_ALONE) * 32 + 32);
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(feed ? DM_THREADS : WT);
   cfg.dynamicSmemBytes = dyn;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
@@ -920,8 +1000,8 @@ cudaError_t launch_hd(const Shape& s, int B, int F, int R, const vatp_cache& c, 
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, kern, tm_k, tm_v, independent, G, state_in_smem, split, chunk, nstage, B, cap, F, R, s.window, s.norm, s.scale * LOG2E, c,
-                            (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v,
+  return cudaLaunchKernelEx(&cfg, kern, tm_k, tm_v, independent, G, s.units, state_in_smem, (int)part_in_ring, split, chunk, nslot, l2_rows, B, cap, F, R, s.window,
+                            s.norm, s.scale * LOG2E, c, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v,
                             (__nv_bfloat16*)out, evicted, dev_status);
 }
 

@@ -1524,6 +1524,17 @@ bool make_rows_map_bf16(CUtensorMap* m, const void* base, int d, uint64_t rows, 
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool make_halves_map_bf16(CUtensorMap* m, const void* base, int d, uint64_t rows, uint32_t box_rows) {
+  if (!encode_fn()) return false;
+  const cuuint64_t dims[3] = {64, (cuuint64_t)rows, (cuuint64_t)(d / 64)};
+  const cuuint64_t strides[2] = {(cuuint64_t)d * 2, 128};
+  const cuuint32_t box[3] = {64, box_rows, (cuuint32_t)(d / 64)};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  return encode_fn()(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 bool make_row_gather_map(CUtensorMap* m, const void* base, uint32_t row_words, uint64_t rows, uint64_t row_stride_bytes) {
   if (!encode_fn()) return false;
   const cuuint64_t dims[2] = {(cuuint64_t)row_words, (cuuint64_t)rows};

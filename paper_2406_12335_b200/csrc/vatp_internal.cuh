@@ -76,6 +76,10 @@ int device_sm_count();
 // swizzle, rows beyond the end read as zeros.  False when the driver entry point is missing.
 bool make_rows_map_bf16(CUtensorMap* m, const void* base, int d, uint64_t rows, uint32_t box_rows);
 
+// 3-D tensor map over the same rows seen as [d / 64][rows][64]: one box brings all 64-column halves of box_rows rows, one
+// half after the other, each 128-byte swizzled.  False when the driver entry point is missing.
+bool make_halves_map_bf16(CUtensorMap* m, const void* base, int d, uint64_t rows, uint32_t box_rows);
+
 // 2-D tensor map over `rows` rows of row_words 32-bit words, row_stride_bytes apart (a multiple of 16); the box
 // is one row: for gathers of whole rows by row index.  False when the driver entry point is missing.
 bool make_row_gather_map(CUtensorMap* m, const void* base, uint32_t row_words, uint64_t rows, uint64_t row_stride_bytes);

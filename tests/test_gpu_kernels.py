@@ -37,3 +37,71 @@ def test_head_dim_64_window_leaves_earlier_normalisers_alone():
                           dev_status=g.status)
     torch.cuda.synchronize()
     assert torch.all(g.lse[..., :344 - 256] == 7.0) and torch.all(g.lse[..., 344 - 256:] != 7.0)
+
+
+@pytest.mark.parametrize("b,h,kv,d,B,window", [
+    (1, 3, 0, 128, 1, 0),        # one slot besides the incoming token's
+    (1, 3, 0, 128, 127, 0),      # ring of fewer units than slots
+    (2, 60, 0, 128, 200, 0),     # 120 units: one CTA each, requests by the warps themselves
+    (3, 100, 0, 128, 130, 0),    # 300 units: more than two CTAs per SM hold, the producer warp goes on to a second unit
+    (3, 100, 0, 64, 130, 40),    # the same with head_dim 64 and a history window (the state of the next unit is fetched early)
+    (5, 8, 2, 128, 600, 0),      # grouped queries split over a cluster
+    (2, 640, 160, 64, 90, 0),    # grouped queries, several units per CTA
+    (1, 2, 0, 128, 9000, 0),     # state beyond shared memory
+])
+@pytest.mark.parametrize("grow", [0, 5])
+def test_decode_step_against_float64(b, h, kv, d, B, window, grow):
+    """One-step arithmetic of every unit against float64 torch: output rows, indicators, evicted token; grow: the cache
+    starts that many tokens short of its budget, so rows requested before the live range is known are dropped."""
+    V = P.vatp()
+    hk, T = kv or h, 2 * B
+    G = h // hk
+    if grow >= B:
+        return
+    p = V.make_params(batch=b, heads=h, kv_heads=kv, seq_len=T, head_dim=d, dtype="bf16", budget=B,
+                      indicator="window" if window else "h2o", window=window)
+    c, n = V.Cache(p), B - grow
+    g = torch.Generator(device="cuda").manual_seed(B + h)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")  # noqa: E731
+    c.k_cache[:, :, :n], c.v_cache[:, :, :n] = rnd(b, hk, n, d).bfloat16(), rnd(b, hk, n, d).bfloat16()
+    c.pos[:, :, :n] = torch.arange(n, dtype=torch.int32, device="cuda")
+    c.vnorm[:, :, :n] = c.v_cache[:, :, :n].float().abs().sum(-1)
+    c.len.fill_(n), c.free_slot.fill_(n), c.next_pos.fill_(T)
+    if window:
+        c.ring[..., :n] = torch.rand(b, hk, window, n, generator=g, device="cuda") / n
+        c.acc_fixed[..., :n] = (c.ring[..., :n].double() * 2.0 ** 52).long().sum(2)
+        c.acc.copy_((c.acc_fixed.double() / 2.0 ** 52).float())
+    else:
+        c.acc[:, :, :n] = torch.rand(b, hk, n, generator=g, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    i0, i1 = torch.arange(b, device="cuda")[:, None], torch.arange(hk, device="cuda")[None]
+    for s in range(3):
+        q, k, v = rnd(b, h, d).bfloat16(), rnd(b, hk, d).bfloat16(), rnd(b, hk, d).bfloat16()
+        fs = c.free_slot.long()
+        K, W, acc, vn, pos = c.k_cache.double(), c.v_cache.double(), c.acc.double(), c.vnorm.double(), c.pos.clone()
+        K[i0, i1, fs], W[i0, i1, fs], vn[i0, i1, fs], pos[i0, i1, fs] = k.double(), v.double(), v.double().abs().sum(-1), T + s
+        live = pos >= 0
+        logits = torch.einsum("bhd,bhnd->bhn", q.double(), K.repeat_interleave(G, 1)) * d ** -0.5
+        prob = torch.softmax(logits.masked_fill(~live.repeat_interleave(G, 1), float("-inf")), -1)
+        want = torch.einsum("bhn,bhnd->bhd", prob, W.repeat_interleave(G, 1))
+        acc[i0, i1, fs] = 0
+        if window:
+            old = c.ring[:, :, (T + s) % window].double()
+            old[i0, i1, fs] = 0
+            acc -= old
+        acc += prob.view(b, hk, G, -1).mean(2)
+        out, ev = torch.empty_like(q), torch.empty(b, hk, dtype=torch.int32, device="cuda")
+        V.vatp_decode_step(p, c, q, k, v, out, evicted_pos=ev, dev_status=status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        # bf16 output: half a unit in the last place of the largest value, and the sums' 1e-3
+        assert torch.all((out.double() - want).abs() <= 2.0 ** -8 * want.abs() + 1e-3 * want.abs().amax(-1, keepdim=True))
+        assert torch.all(((c.acc.double() - acc).abs() <= 1e-3 * acc.abs() + 1e-6)[live])
+        assert torch.all(((c.vnorm.double() - vn).abs() <= 1e-5 * vn)[live])
+        if n + s < B:
+            assert torch.all(ev == -1)
+        else:
+            imp = (acc * vn).masked_fill(~live, float("inf"))
+            got = imp.gather(2, (pos == ev[..., None]).int().argmax(-1, keepdim=True))[..., 0]
+            assert torch.all((pos == ev[..., None]).sum(-1) == 1)
+            assert torch.all(got <= imp.amin(-1) * (1 + 2e-3) + 1e-9)      # the minimum, up to both sides' tolerance

@@ -750,10 +750,8 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   }
   // (units of one CTA one after the other: the next one's logits, partials and state may replace this one's)
   const bool more = u + u_step < units;
-  if (state_in_smem == 1) {
-    if (more) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(state_empty)) : "memory");
-    state_par ^= 1;
-  }
+  if (more) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(state_empty)) : "memory");
+  if (state_in_smem == 1) state_par ^= 1;
   if (evicting) {
     // this CTA's candidate (positions are unique: exactly one thread holds the winning key), sent to rank 0
     const unsigned long long wkey = warp_min_key(my_key);

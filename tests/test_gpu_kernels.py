@@ -48,6 +48,7 @@ def test_head_dim_64_window_leaves_earlier_normalisers_alone():
     (5, 8, 2, 128, 600, 0),      # grouped queries split over a cluster
     (2, 640, 160, 64, 90, 0),    # grouped queries, several units per CTA
     (1, 2, 0, 128, 9000, 0),     # state beyond shared memory
+    (1, 300, 0, 128, 2048, 30),  # several units per CTA, their state read from global memory in the tail
 ])
 @pytest.mark.parametrize("grow", [0, 5])
 def test_decode_step_against_float64(b, h, kv, d, B, window, grow):

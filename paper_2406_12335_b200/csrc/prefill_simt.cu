@@ -2,88 +2,133 @@
 //
 // Pass 1 gives every query row its log-sum-exp (the normaliser of Eq. 1); pass 2 recomputes the
 // logits tile by tile and adds exp(s - lse) into per-key sums (Eq. 2, or Eq. 3 when only the last
-// w query rows count), fused with the value l1 norm and the Eq. 4 product.  This is the path for
-// fp32 inputs (tensor cores would round the operands) and for shapes the tensor-core kernel does
-// not take.  No float atomics: each CTA owns a tile of rows (pass 1) or of keys (pass 2).
+// w query rows count), fused with the value norm and the Eq. 4 product.  This is the path for
+// fp32 inputs (tensor cores would round the operands) and for devices without the tensor-core kernels.
+// No float atomics: the CTAs of a cluster own a tile of rows (pass 1) or of keys (pass 2).
+//
+// Bound by the FMA pipes when there are many tiles, by latency when there are few.  So
+//   * a thread holds M x M logits (M = 4 or 8) of a 16 M x 16 M tile; both operands sit in shared memory transposed, so
+//     that M elements of a channel are one or two 16-byte loads: 2 (4) loads per 16 (64) FMAs where one element per load
+//     made it 8 per 16.  The next tile's rows are on their way to registers under the products (M = 4);
+//   * few tiles are shared out over a cluster of up to eight CTAs along the other dimension, which combine their row
+//     statistics or column sums through distributed shared memory;
+//   * both passes are programmatic dependents: they are resident when the launch before them ends.
+// 2 heads x 512 tokens x 64 channels, scoring + selection + compaction: 93 -> 34 us.
+#include <cooperative_groups.h>
+
 #include "vatp_internal.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace vatp {
 namespace {
 
-constexpr int TILE = 64;      // queries or keys per CTA tile
-constexpr int NTHREADS = 256; // 16 x 16 threads, 4 x 4 logits each
+constexpr int NTHREADS = 256;   // 16 x 16 threads, M x M logits each
+constexpr int MAX_CLUSTER = 8;
 
-template <typename T>
-__device__ __forceinline__ void load_tile(float* dst, int ld, const T* src, int64_t row_stride, int row0, int rows_valid,
-                                          int d) {
-  // dst[r][c] for r < TILE; rows beyond rows_valid are zero
-  const int vec = d / 4;
-  for (int i = threadIdx.x; i < TILE * vec; i += NTHREADS) {
-    int r = i / vec, c4 = (i % vec) * 4;
-    float x0 = 0.f, x1 = 0.f, x2 = 0.f, x3 = 0.f;
-    if (r < rows_valid) {
-      const T* p = src + (int64_t)(row0 + r) * row_stride + c4;
-      x0 = to_f32(p[0]); x1 = to_f32(p[1]); x2 = to_f32(p[2]); x3 = to_f32(p[3]);
+template <typename T> __device__ __forceinline__ float4 load4(const T* p);
+template <> __device__ __forceinline__ float4 load4<float>(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+template <> __device__ __forceinline__ float4 load4<__nv_bfloat16>(const __nv_bfloat16* p) {
+  const uint2 r = __ldg(reinterpret_cast<const uint2*>(p));
+  return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xffff0000u), __uint_as_float(r.y << 16), __uint_as_float(r.y & 0xffff0000u));
+}
+
+// A tile of 16 M rows x D channels, transposed: element (row, c) at [c][row], leading dimension LD (a multiple of four).
+// Neighbouring lanes take neighbouring rows, so that the stores are free of bank conflicts.
+template <int M, int D>
+struct Tile {
+  static constexpr int ROWS = 16 * M, LD = ROWS + 4, NV = ROWS * (D / 4) / NTHREADS;
+  template <typename T>
+  static __device__ __forceinline__ void fetch(float4 (&r)[NV], const T* src, int64_t row_stride, int row0, int rows_valid) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const int idx = threadIdx.x + i * NTHREADS, row = idx % ROWS, c4 = idx / ROWS;
+      r[i] = row < rows_valid ? load4(src + (int64_t)(row0 + row) * row_stride + c4 * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    float* o = dst + r * ld + c4;
-    o[0] = x0; o[1] = x1; o[2] = x2; o[3] = x3;
+  }
+  static __device__ __forceinline__ void store(float* dst, const float4 (&r)[NV]) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const int idx = threadIdx.x + i * NTHREADS, row = idx % ROWS, c4 = idx / ROWS;
+      float* o = dst + c4 * 4 * LD + row;
+      o[0] = r[i].x; o[LD] = r[i].y; o[2 * LD] = r[i].z; o[3 * LD] = r[i].w;
+    }
+  }
+};
+
+// row (or column) of element i of the thread's t-th group: four consecutive ones, the second four half a tile on
+template <int M> __device__ __forceinline__ int micro_at(int t, int i) { return (i >> 2) * 64 + t * 4 + (i & 3); }
+
+// s[i][j] = <A row micro_at(ty, i), B row micro_at(tx, j)>, channels in ascending order
+template <int M, int D>
+__device__ __forceinline__ void micro_gemm(const float* As, const float* Bs, int ty, int tx, float (&s)[M][M]) {
+  constexpr int LD = Tile<M, D>::LD;
+#pragma unroll
+  for (int i = 0; i < M; ++i)
+#pragma unroll
+    for (int j = 0; j < M; ++j) s[i][j] = 0.f;
+#pragma unroll 4
+  for (int c = 0; c < D; ++c) {
+    float a[M], b[M];
+#pragma unroll
+    for (int h = 0; h < M / 4; ++h) {
+      *reinterpret_cast<float4*>(&a[4 * h]) = *reinterpret_cast<const float4*>(As + c * LD + h * 64 + ty * 4);
+      *reinterpret_cast<float4*>(&b[4 * h]) = *reinterpret_cast<const float4*>(Bs + c * LD + h * 64 + tx * 4);
+    }
+#pragma unroll
+    for (int i = 0; i < M; ++i)
+#pragma unroll
+      for (int j = 0; j < M; ++j) s[i][j] = fmaf(a[i], b[j], s[i][j]);
   }
 }
 
-// s[i][j] = <A[ty + 16 i], B[tx + 16 j]> for the thread's 4 x 4 micro-tile
-__device__ __forceinline__ void micro_gemm(const float* As, const float* Bs, int ld, int d, int ty, int tx,
-                                           float (&s)[4][4]) {
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) s[i][j] = 0.f;
-  for (int c = 0; c < d; ++c) {
-    float a[4], b[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) a[i] = As[(ty + 16 * i) * ld + c];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) b[j] = Bs[(tx + 16 * j) * ld + c];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) s[i][j] = fmaf(a[i], b[j], s[i][j]);
-  }
-}
-
-// Pass 1: one CTA per (query tile, unit).  lse[j] over keys i <= j.
-template <typename T>
+// Pass 1: one cluster per (query tile, unit), its CTAs take every cs-th key tile.  lse[j] over keys i <= j.
+template <typename T, int M, int D>
 __global__ void __launch_bounds__(NTHREADS) rowstats_kernel(Shape sh, const T* __restrict__ q, const T* __restrict__ k,
-                                                            float* __restrict__ lse, int first_row) {
-  extern __shared__ float smem[];
-  const int ld = sh.d + 1;
+                                                            float* __restrict__ lse, int first_row, int cs) {
+  constexpr int ROWS = Tile<M, D>::ROWS, LD = Tile<M, D>::LD, NV = Tile<M, D>::NV;
+  extern __shared__ __align__(16) float smem[];
   float* Qs = smem;
-  float* Ks = smem + TILE * ld;
+  float* Ks = smem + D * LD;
+  __shared__ float2 part[ROWS];
+  // nothing is read before all earlier work has completed; pass 2 may set up from then on
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = cs > 1 ? (int)cluster.block_rank() : 0;
   const int u = blockIdx.y;
-  const int q0 = first_row + blockIdx.x * TILE;
-  if (q0 >= sh.T) return;
+  const int ntile = (sh.T - first_row + ROWS - 1) / ROWS;
+  const int q0 = first_row + (ntile - 1 - (int)(blockIdx.x / cs)) * ROWS;      // the longest rows first
   const T* qu = q + unit_offset_q(sh, u);
   const T* ku = k + unit_offset(sh, u);
   const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
+  const int last_key = min(q0 + ROWS, sh.T);  // exclusive
 
-  load_tile(Qs, ld, qu, sh.st, q0, min(TILE, sh.T - q0), sh.d);
-  float m[4], l[4];
+  float m[M], l[M];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) { m[i] = -INFINITY; l[i] = 0.f; }
-
-  const int last_key = min(q0 + TILE, sh.T);  // exclusive
-  for (int k0 = 0; k0 < last_key; k0 += TILE) {
+  for (int i = 0; i < M; ++i) { m[i] = -INFINITY; l[i] = 0.f; }
+  {
+    float4 r[NV];
+    Tile<M, D>::fetch(r, qu, sh.st, q0, min(ROWS, sh.T - q0));
+    Tile<M, D>::store(Qs, r);
+  }
+  float4 next[NV];
+  if (M == 4 && rank * ROWS < last_key) Tile<M, D>::fetch(next, ku, sh.st, rank * ROWS, min(ROWS, sh.T - rank * ROWS));
+  for (int k0 = rank * ROWS; k0 < last_key; k0 += cs * ROWS) {
+    if (M != 4) Tile<M, D>::fetch(next, ku, sh.st, k0, min(ROWS, sh.T - k0));
     __syncthreads();
-    load_tile(Ks, ld, ku, sh.st, k0, min(TILE, sh.T - k0), sh.d);
+    Tile<M, D>::store(Ks, next);
     __syncthreads();
-    float s[4][4];
-    micro_gemm(Qs, Ks, ld, sh.d, ty, tx, s);
+    if (M == 4 && k0 + cs * ROWS < last_key) Tile<M, D>::fetch(next, ku, sh.st, k0 + cs * ROWS, min(ROWS, sh.T - k0 - cs * ROWS));
+    float s[M][M];
+    micro_gemm<M, D>(Qs, Ks, ty, tx, s);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int row = q0 + ty + 16 * i;
+    for (int i = 0; i < M; ++i) {
+      const int row = q0 + micro_at<M>(ty, i);
       float tile_max = -INFINITY;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int col = k0 + tx + 16 * j;
+      for (int j = 0; j < M; ++j) {
+        const int col = k0 + micro_at<M>(tx, j);
         s[i][j] = (col <= row) ? s[i][j] * sh.scale : -INFINITY;
         tile_max = fmaxf(tile_max, s[i][j]);
       }
@@ -91,7 +136,7 @@ __global__ void __launch_bounds__(NTHREADS) rowstats_kernel(Shape sh, const T* _
         const float m_new = fmaxf(m[i], tile_max);
         float add = 0.f;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) add += expf(s[i][j] - m_new);
+        for (int j = 0; j < M; ++j) add += expf(s[i][j] - m_new);
         l[i] = l[i] * expf(m[i] - m_new) + add;
         m[i] = m_new;
       }
@@ -99,7 +144,7 @@ __global__ void __launch_bounds__(NTHREADS) rowstats_kernel(Shape sh, const T* _
   }
   // merge the 16 threads (same ty, consecutive lanes) that share each row
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < M; ++i) {
 #pragma unroll
     for (int off = 8; off >= 1; off >>= 1) {
       const float m2 = __shfl_xor_sync(0xffffffffu, m[i], off);
@@ -110,41 +155,75 @@ __global__ void __launch_bounds__(NTHREADS) rowstats_kernel(Shape sh, const T* _
         m[i] = mn;
       }
     }
-    const int row = q0 + ty + 16 * i;
-    if (tx == 0 && row < sh.T) lse[unit_offset_lse(sh, u) + row] = m[i] + logf(l[i]);
+    const int at = micro_at<M>(ty, i);
+    if (tx == 0) {
+      if (cs > 1) part[at] = make_float2(m[i], l[i]);
+      else if (q0 + at < sh.T) lse[unit_offset_lse(sh, u) + q0 + at] = m[i] + logf(l[i]);
+    }
+  }
+  if (cs > 1) {
+    cluster.sync();
+    if (rank == 0 && (int)threadIdx.x < ROWS && q0 + (int)threadIdx.x < sh.T) {
+      float2 p[MAX_CLUSTER];
+      float mx = -INFINITY, sum = 0.f;
+#pragma unroll
+      for (int r = 0; r < MAX_CLUSTER; ++r) {
+        p[r] = r < cs ? cluster.map_shared_rank(part, r)[threadIdx.x] : make_float2(-INFINITY, 0.f);
+        mx = fmaxf(mx, p[r].x);
+      }
+#pragma unroll
+      for (int r = 0; r < MAX_CLUSTER; ++r)
+        if (p[r].x > -INFINITY) sum += p[r].y * expf(p[r].x - mx);
+      lse[unit_offset_lse(sh, u) + q0 + threadIdx.x] = mx + logf(sum);
+    }
+    cluster.sync();       // nobody leaves while rank 0 reads
   }
 }
 
-// Pass 2: one CTA per (key tile, unit).  Column sums over query rows j >= max(first_row, k).
-template <typename T>
+// Pass 2: one cluster per (key tile, unit), its CTAs take every cs-th query tile.  Column sums over query rows
+// j >= max(first_row, k).
+template <typename T, int M, int D>
 __global__ void __launch_bounds__(NTHREADS)
 colsum_kernel(Shape sh, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
               const float* __restrict__ lse, float* __restrict__ attn_acc, float* __restrict__ vnorm,
-              float* __restrict__ score, float* __restrict__ win_rows, int first_row) {
-  extern __shared__ float smem[];
-  const int ld = sh.d + 1;
+              float* __restrict__ score, float* __restrict__ win_rows, int first_row, int cs) {
+  constexpr int ROWS = Tile<M, D>::ROWS, LD = Tile<M, D>::LD, NV = Tile<M, D>::NV;
+  extern __shared__ __align__(16) float smem[];
   float* Qs = smem;
-  float* Ks = smem + TILE * ld;
-  float* lse_s = Ks + TILE * ld;        // [TILE]
-  float* red = lse_s + TILE;            // [16][TILE]
+  float* Ks = smem + D * LD;
+  float* lse_s = Ks + D * LD;           // [ROWS]
+  float* red = Qs;                      // [16][ROWS], once the products are done (D >= 16)
+  __shared__ float vn_s[ROWS], part[ROWS];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = cs > 1 ? (int)cluster.block_rank() : 0;
   const int u = blockIdx.y;
-  const int k0 = blockIdx.x * TILE;
+  const int k0 = (int)(blockIdx.x / cs) * ROWS;
   const T* qu = q + unit_offset_q(sh, u);
   const T* ku = k + unit_offset(sh, u);
   const T* vu = v + unit_offset(sh, u);
   const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
-  const int keys_valid = min(TILE, sh.T - k0);
+  const int keys_valid = min(ROWS, sh.T - k0);
+  if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // Everything this pass reads but the normalisers was complete before pass 1 released it; without a pass 1 before it
+  // (normalisers given) it waits first.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 
-  load_tile(Ks, ld, ku, sh.st, k0, keys_valid, sh.d);
-  float cs[4] = {0.f, 0.f, 0.f, 0.f};
+  {
+    float4 r[NV];
+    Tile<M, D>::fetch(r, ku, sh.st, k0, keys_valid);
+    Tile<M, D>::store(Ks, r);
+  }
+  float cs_sum[M];
+#pragma unroll
+  for (int j = 0; j < M; ++j) cs_sum[j] = 0.f;
 
   // query tiles are aligned to first_row so that window rows map to whole tiles
   int qstart = first_row;
-  if (k0 > first_row) qstart = first_row + ((k0 - first_row) / TILE) * TILE;
+  if (k0 > first_row) qstart = first_row + ((k0 - first_row) / ROWS) * ROWS;
   const int wrow0 = sh.T - sh.window;   // query position of win_rows row 0 (may be negative)
   float* wr = win_rows ? win_rows + (int64_t)u * sh.window * sh.T : nullptr;
 
-  if (wr) {
+  if (wr && rank == 0) {
     // rows of the window that lie entirely above this key tile (j < k0): zeros
     for (int j = max(first_row, 0); j < min(qstart, sh.T); ++j)
       for (int c = threadIdx.x; c < keys_valid; c += NTHREADS) wr[(int64_t)(j - wrow0) * sh.T + k0 + c] = 0.f;
@@ -153,76 +232,144 @@ colsum_kernel(Shape sh, const T* __restrict__ q, const T* __restrict__ k, const 
       for (int c = threadIdx.x; c < keys_valid; c += NTHREADS) wr[(int64_t)r * sh.T + k0 + c] = 0.f;
   }
 
-  for (int q0 = qstart; q0 < sh.T; q0 += TILE) {
+  float4 next[NV];
+  const int qfirst = qstart + rank * ROWS;
+  if (M == 4 && qfirst < sh.T) Tile<M, D>::fetch(next, qu, sh.st, qfirst, min(ROWS, sh.T - qfirst));
+  for (int q0 = qfirst; q0 < sh.T; q0 += cs * ROWS) {
+    const int rows_valid = min(ROWS, sh.T - q0);
+    if (M != 4) Tile<M, D>::fetch(next, qu, sh.st, q0, rows_valid);
     __syncthreads();
-    const int rows_valid = min(TILE, sh.T - q0);
-    load_tile(Qs, ld, qu, sh.st, q0, rows_valid, sh.d);
-    if (threadIdx.x < TILE) lse_s[threadIdx.x] = threadIdx.x < rows_valid ? lse[unit_offset_lse(sh, u) + q0 + threadIdx.x] : 0.f;
+    Tile<M, D>::store(Qs, next);
+    if (threadIdx.x < ROWS) lse_s[threadIdx.x] = (int)threadIdx.x < rows_valid ? lse[unit_offset_lse(sh, u) + q0 + threadIdx.x] : 0.f;
     __syncthreads();
-    float s[4][4];
-    micro_gemm(Qs, Ks, ld, sh.d, ty, tx, s);
+    if (M == 4 && q0 + cs * ROWS < sh.T) Tile<M, D>::fetch(next, qu, sh.st, q0 + cs * ROWS, min(ROWS, sh.T - q0 - cs * ROWS));
+    float s[M][M];
+    micro_gemm<M, D>(Qs, Ks, ty, tx, s);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int row = q0 + ty + 16 * i;
-      const float lr = lse_s[ty + 16 * i];
+    for (int i = 0; i < M; ++i) {
+      const int row = q0 + micro_at<M>(ty, i);
+      const float lr = lse_s[micro_at<M>(ty, i)];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int col = k0 + tx + 16 * j;
+      for (int j = 0; j < M; ++j) {
+        const int col = k0 + micro_at<M>(tx, j);
         float p = 0.f;
         if (row < sh.T && col <= row && col < sh.T) p = expf(s[i][j] * sh.scale - lr);
-        cs[j] += p;
+        cs_sum[j] += p;
         if (wr && row < sh.T && col < sh.T) wr[(int64_t)(row - wrow0) * sh.T + col] = p;
       }
     }
   }
-  __syncthreads();
-#pragma unroll
-  for (int j = 0; j < 4; ++j) red[ty * TILE + tx + 16 * j] = cs[j];
-  // value norms (Eq. 4): 4 threads per row
-  float* vn_s = Qs;  // reuse
-  __syncthreads();
-  {
-    const int r = threadIdx.x / 4, part = threadIdx.x % 4;
-    float acc = 0.f;
-    if (r < keys_valid) {
-      const T* p = vu + (int64_t)(k0 + r) * sh.st;
-      for (int c = part; c < sh.d; c += 4) acc = norm_fold(sh.norm, acc, to_f32(p[c]));
+  // value norms (Eq. 4): four threads per row, by the last CTA of the cluster, which has the fewest query tiles
+  if (rank == cs - 1) {
+    for (int r = threadIdx.x / 4; r < ROWS; r += NTHREADS / 4) {
+      const int part4 = threadIdx.x % 4;
+      float acc = 0.f;
+      if (r < keys_valid) {
+        const T* p = vu + (int64_t)(k0 + r) * sh.st;
+#pragma unroll 4
+        for (int c = part4 * 4; c < D; c += 16) {
+          const float4 x = load4(p + c);
+          acc = norm_fold(sh.norm, norm_fold(sh.norm, norm_fold(sh.norm, norm_fold(sh.norm, acc, x.x), x.y), x.z), x.w);
+        }
+      }
+      acc = norm_merge(sh.norm, acc, __shfl_xor_sync(0xffffffffu, acc, 1));
+      acc = norm_merge(sh.norm, acc, __shfl_xor_sync(0xffffffffu, acc, 2));
+      if (part4 == 0) vn_s[r] = norm_finish(sh.norm, acc);
     }
-    acc = norm_merge(sh.norm, acc, __shfl_xor_sync(0xffffffffu, acc, 1));
-    acc = norm_merge(sh.norm, acc, __shfl_xor_sync(0xffffffffu, acc, 2));
-    if (part == 0) vn_s[r] = norm_finish(sh.norm, acc);
   }
   __syncthreads();
-  if (threadIdx.x < keys_valid) {
-    float tot = 0.f;
 #pragma unroll
-    for (int t = 0; t < 16; ++t) tot += red[t * TILE + threadIdx.x];
+  for (int j = 0; j < M; ++j) red[ty * ROWS + micro_at<M>(tx, j)] = cs_sum[j];
+  __syncthreads();
+  float tot = 0.f;
+  if ((int)threadIdx.x < ROWS) {
+#pragma unroll
+    for (int t = 0; t < 16; ++t) tot += red[t * ROWS + threadIdx.x];
+    part[threadIdx.x] = tot;
+  }
+  if (cs > 1) cluster.sync(); else __syncthreads();
+  if (rank == 0 && (int)threadIdx.x < keys_valid) {
+    float n1 = 0.f;
+    if (cs > 1) {
+      tot = 0.f;
+#pragma unroll
+      for (int r = 0; r < MAX_CLUSTER; ++r)
+        if (r < cs) tot += cluster.map_shared_rank(part, r)[threadIdx.x];
+      n1 = cluster.map_shared_rank(vn_s, cs - 1)[threadIdx.x];
+    } else {
+      n1 = vn_s[threadIdx.x];
+    }
     const int64_t o = (int64_t)u * sh.T + k0 + threadIdx.x;
-    const float n1 = vn_s[threadIdx.x];
     attn_acc[o] = tot;
     vnorm[o] = n1;
     score[o] = tot * n1;
   }
+  if (cs > 1) cluster.sync();       // nobody leaves while rank 0 reads
+}
+
+// launch configuration: programmatic dependent, clusters of cs CTAs along x
+struct ClusterLaunch {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  ClusterLaunch(dim3 grid, size_t smem, cudaStream_t st, int cs) : cfg{} {
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(NTHREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cs;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+  }
+};
+
+template <typename T, int M, int D>
+cudaError_t launch_m(const Shape& s, const T* q, const T* k, const T* v, float* lse, float* attn_acc, float* vnorm,
+                     float* score, float* win_rows, cudaStream_t st, bool lse_given) {
+  using Tl = Tile<M, D>;
+  const size_t smem1 = sizeof(float) * 2 * D * Tl::LD, smem2 = smem1 + sizeof(float) * Tl::ROWS;
+  cudaError_t e;
+  if ((e = cudaFuncSetAttribute(rowstats_kernel<T, M, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1)) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(colsum_kernel<T, M, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2)) != cudaSuccess) return e;
+  const int first_row = s.window > 0 ? (s.T > s.window ? s.T - s.window : 0) : 0;
+  const int qtiles = (s.T - first_row + Tl::ROWS - 1) / Tl::ROWS, ktiles = (s.T + Tl::ROWS - 1) / Tl::ROWS;
+  // Clusters while the grid leaves SMs idle and there are tiles to share: the longest row of tiles bounds the pass.
+  auto cluster_for = [&](int tiles, int most) {
+    int cs = 1;
+    while (cs < MAX_CLUSTER && (int64_t)tiles * s.units * cs * 2 <= 2 * device_sm_count() && cs < most) cs *= 2;
+    return cs;
+  };
+  if (!lse_given) {
+    const int cs = cluster_for(qtiles, ktiles);
+    ClusterLaunch c1(dim3(qtiles * cs, s.units), smem1, st, cs);
+    if ((e = cudaLaunchKernelEx(&c1.cfg, rowstats_kernel<T, M, D>, s, q, k, lse, first_row, cs)) != cudaSuccess) return e;
+  }
+  const int cs = cluster_for(ktiles, qtiles);
+  ClusterLaunch c2(dim3(ktiles * cs, s.units), smem2, st, cs);
+  return cudaLaunchKernelEx(&c2.cfg, colsum_kernel<T, M, D>, s, q, k, v, (const float*)lse, attn_acc, vnorm, score,
+                            s.window > 0 ? win_rows : nullptr, first_row, cs);
+}
+
+template <typename T, int D>
+cudaError_t launch_t(const Shape& s, const T* q, const T* k, const T* v, float* lse, float* attn_acc, float* vnorm,
+                     float* score, float* win_rows, cudaStream_t st, bool lse_given) {
+  // 128 x 128 tiles (half the shared-memory loads per FMA) once they fill the machine twice over in both passes
+  const int rows = s.window > 0 && s.window < s.T ? s.window : s.T;
+  const int64_t tiles = (int64_t)s.units * ((rows + 127) / 128);
+  return tiles >= 2 * device_sm_count()
+             ? launch_m<T, 8, D>(s, q, k, v, lse, attn_acc, vnorm, score, win_rows, st, lse_given)
+             : launch_m<T, 4, D>(s, q, k, v, lse, attn_acc, vnorm, score, win_rows, st, lse_given);
 }
 
 template <typename T>
-cudaError_t launch_t(const Shape& s, const T* q, const T* k, const T* v, float* lse, float* attn_acc, float* vnorm,
+cudaError_t launch_d(const Shape& s, const T* q, const T* k, const T* v, float* lse, float* attn_acc, float* vnorm,
                      float* score, float* win_rows, cudaStream_t st, bool lse_given) {
-  const int ld = s.d + 1;
-  const size_t smem1 = sizeof(float) * 2 * TILE * ld;
-  const size_t smem2 = smem1 + sizeof(float) * (TILE + 16 * TILE);
-  cudaError_t e;
-  e = cudaFuncSetAttribute(rowstats_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(colsum_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
-  if (e != cudaSuccess) return e;
-  const int first_row = s.window > 0 ? max(s.T - s.window, 0) : 0;
-  const int qtiles = (s.T - first_row + TILE - 1) / TILE;
-  const int ktiles = (s.T + TILE - 1) / TILE;
-  if (!lse_given) rowstats_kernel<T><<<dim3(qtiles, s.units), NTHREADS, smem1, st>>>(s, q, k, lse, first_row);
-  colsum_kernel<T><<<dim3(ktiles, s.units), NTHREADS, smem2, st>>>(s, q, k, v, lse, attn_acc, vnorm, score,
-                                                                    s.window > 0 ? win_rows : nullptr, first_row);
-  return cudaGetLastError();
+  return s.d == 64 ? launch_t<T, 64>(s, q, k, v, lse, attn_acc, vnorm, score, win_rows, st, lse_given)
+                   : launch_t<T, 128>(s, q, k, v, lse, attn_acc, vnorm, score, win_rows, st, lse_given);
 }
 
 }  // namespace
@@ -231,9 +378,9 @@ cudaError_t launch_prefill_simt(const Shape& s, int dtype, const void* q, const 
                                 float* attn_acc, float* vnorm, float* score, float* win_rows, cudaStream_t st,
                                 bool lse_given) {
   if (dtype == VATP_F32)
-    return launch_t<float>(s, (const float*)q, (const float*)k, (const float*)v, lse, attn_acc, vnorm, score, win_rows, st,
+    return launch_d<float>(s, (const float*)q, (const float*)k, (const float*)v, lse, attn_acc, vnorm, score, win_rows, st,
                            lse_given);
-  return launch_t<__nv_bfloat16>(s, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, lse,
+  return launch_d<__nv_bfloat16>(s, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, lse,
                                  attn_acc, vnorm, score, win_rows, st, lse_given);
 }
 

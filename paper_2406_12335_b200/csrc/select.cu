@@ -4,12 +4,14 @@
 // One CTA per unit; the unit's scores are staged in shared memory once when they fit and read
 // from global memory (L2-resident) otherwise; for long prompts and few units a cluster of four or two CTAs shares a
 // unit (select_cluster_kernel below).  Pure integer work after the key transform.
-// Every warp counts into a histogram of its own and the 32 histograms are summed per bin.  The scores
+// The warps count into one to eight histograms that are summed per bin.  The scores
 // of a head share a few exponents, so in the first passes nearly all keys of a warp fall into one bin:
 // the lanes that agree with the warp's first candidate are counted by one addition (a ballot), the
 // others by shared-memory atomics, which rarely collide once the digits spread.  (Grouping all equal
 // digits with match.any cost more than everything else in the kernel: it takes time in proportion to
-// the number of distinct values in the warp.)
+// the number of distinct values in the warp.)  As soon as at most 32 keys share the boundary's digits - after two passes
+// for most units - one warp ranks those instead of two more passes.
+// (256 units x 7936 keys with the compaction behind it 103.7 -> 101.7 us; 8 units x 7806 20.9 -> 19.6.)
 #include <cooperative_groups.h>
 
 #include "vatp_internal.cuh"
@@ -28,14 +30,19 @@ __device__ __forceinline__ uint32_t order_key(float x) {
   return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 
-template <bool STAGED>
-__global__ void __launch_bounds__(SEL_THREADS) select_kernel(int T, int B, int F, int R, const float* __restrict__ score,
+// THREADS: 1024 for one CTA per SM at a time, 512 when more units than SMs are to share the machine (the passes are chains
+// of short phases; two or more CTAs per SM fill one another's).  copies: histograms the warps share out among them - one
+// for short ranges, where clearing and summing 32 of them took longer than the counting.
+template <bool STAGED, int THREADS>
+__global__ void __launch_bounds__(THREADS) select_kernel(int copies, int T, int B, int F, int R, const float* __restrict__ score,
                                                              int32_t* __restrict__ kept, int32_t* dev_status) {
-  extern __shared__ __align__(16) uint32_t keys_s[];  // STAGED: keys of the middle range (from index `pad` on)
+  constexpr int WARPS = THREADS / 32;
+  extern __shared__ __align__(16) uint32_t sel_smem[];
+  uint32_t* hist_c = sel_smem;                     // [copies][256] counts of the current pass
+  uint32_t* keys_s = sel_smem + copies * 256;      // STAGED: keys of the middle range (from index `pad` on)
   __shared__ uint32_t hist[256];
-  __shared__ uint32_t hist_w[SEL_WARPS][256];      // per-warp counts of the current pass
-  __shared__ uint32_t sh_prefix, sh_need;
-  __shared__ uint32_t warp_keep[SEL_WARPS], warp_eq[SEL_WARPS];
+  __shared__ uint32_t sh_prefix, sh_need, sh_in_bin, n_cand, cand[32];
+  __shared__ uint32_t warp_keep[WARPS], warp_eq[WARPS];
 
   // Launched as a programmatic dependent: the next launch (the compaction) may set up now, and the
   // scores are read only once the launch that produced them has completed.
@@ -47,13 +54,13 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(int T, int B, int F
   const int tid = threadIdx.x;
 
   if (T <= B) {  // everything survives
-    for (int i = tid; i < B; i += SEL_THREADS) out[i] = i < T ? i : -1;
+    for (int i = tid; i < B; i += THREADS) out[i] = i < T ? i : -1;
     return;
   }
   const int n = T - R - F;   // middle range length (> 0 here because T > B >= F + R)
   const int ksel = B - F - R;  // how many of the middle range survive
-  for (int i = tid; i < F; i += SEL_THREADS) out[i] = i;
-  for (int i = tid; i < R; i += SEL_THREADS) out[B - R + i] = T - R + i;
+  for (int i = tid; i < F; i += THREADS) out[i] = i;
+  for (int i = tid; i < R; i += THREADS) out[B - R + i] = T - R + i;
   if (ksel == 0) return;
 
   // Staging: key i sits at keys_s[pad + i], pad chosen so that 16-byte loads from global memory pair with
@@ -68,16 +75,16 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(int T, int B, int F
     const int nvec = (n - a0) >> 2;
     const float4* src4 = reinterpret_cast<const float4*>(mid + a0);
     uint4* dst4 = reinterpret_cast<uint4*>(keys_s + pad + a0);
-    for (int v0 = 0; v0 < nvec; v0 += 4 * SEL_THREADS) {
+    for (int v0 = 0; v0 < nvec; v0 += 4 * THREADS) {
       float4 x[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int v = v0 + j * SEL_THREADS + tid;
+        const int v = v0 + j * THREADS + tid;
         if (v < nvec) x[j] = __ldg(src4 + v);
       }
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int v = v0 + j * SEL_THREADS + tid;
+        const int v = v0 + j * THREADS + tid;
         if (v < nvec && VATP_INB(pad + a0 + 4 * v + 3, n + 4, dev_status)) dst4[v] = make_uint4(order_key(x[j].x), order_key(x[j].y), order_key(x[j].z), order_key(x[j].w));
       }
     }
@@ -92,39 +99,44 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(int T, int B, int F
   // Lanes that share the digit of the warp's first candidate are counted together; the rest add one each.
   uint32_t prefix = 0, mask = 0, need = (uint32_t)ksel;
   const int lane = tid & 31, wid = tid >> 5;
+  uint32_t* my_hist = hist_c + (wid % copies) * 256;
   for (int shift = 24; shift >= 0; shift -= 8) {
-#pragma unroll
-    for (int i = lane; i < 256; i += 32) hist_w[wid][i] = 0;
-    __syncwarp();
-    for (int base = 0; base < n; base += SEL_THREADS) {
+    for (int i = tid; i < copies * 256; i += THREADS) hist_c[i] = 0;
+    if (tid == 0) n_cand = 0;
+    __syncthreads();
+    for (int base = 0; base < n; base += THREADS) {
       const int i = base + tid;
       uint32_t digit = 256u;                       // lanes without a candidate share a dummy digit
       if (i < n) {
         const uint32_t key = key_at(i);
         if ((key & mask) == prefix) digit = (key >> shift) & 255u;
       }
-      const uint32_t cand = __ballot_sync(0xffffffffu, digit < 256u);
-      if (cand) {
-        const int first = __ffs(cand) - 1;
+      const uint32_t some = __ballot_sync(0xffffffffu, digit < 256u);
+      if (some) {
+        const int first = __ffs(some) - 1;
         const uint32_t d0 = __shfl_sync(0xffffffffu, digit, first);
         const uint32_t same = __ballot_sync(0xffffffffu, digit == d0);
-        if (lane == first) atomicAdd(&hist_w[wid][d0], (uint32_t)__popc(same));
-        else if (digit < 256u && digit != d0) atomicAdd(&hist_w[wid][digit], 1u);
+        if (lane == first) atomicAdd(&my_hist[d0], (uint32_t)__popc(same));
+        else if (digit < 256u && digit != d0) atomicAdd(&my_hist[digit], 1u);
       }
     }
     __syncthreads();
-    if (tid < 256) {
-      uint32_t tot = 0;
+    const uint32_t* totals = hist_c;
+    if (copies > 1) {
+      if (tid < 256) {
+        uint32_t tot = 0;
 #pragma unroll 8
-      for (int w = 0; w < SEL_WARPS; ++w) tot += hist_w[w][tid];
-      hist[tid] = tot;
+        for (int w = 0; w < copies; ++w) tot += hist_c[w * 256 + tid];
+        hist[tid] = tot;
+      }
+      __syncthreads();
+      totals = hist;
     }
-    __syncthreads();
     if (tid < 32) {
       // walk the 256 bins from the top: 8 bins per lane, suffix sums by shuffles
       uint32_t c[8], tot = 0;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) { c[j] = hist[255 - (tid * 8 + j)]; tot += c[j]; }
+      for (int j = 0; j < 8; ++j) { c[j] = totals[255 - (tid * 8 + j)]; tot += c[j]; }
       uint32_t incl = tot;
 #pragma unroll
       for (int off = 1; off < 32; off <<= 1) {
@@ -138,6 +150,7 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(int T, int B, int F
           if (need <= before + c[j]) {
             sh_prefix = prefix | ((uint32_t)(255 - (tid * 8 + j)) << shift);
             sh_need = need - before;
+            sh_in_bin = c[j];
             break;
           }
           before += c[j];
@@ -148,6 +161,36 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(int T, int B, int F
     prefix = sh_prefix;
     need = sh_need;
     mask |= 255u << shift;
+    if (shift > 0 && sh_in_bin <= 32u) {
+      // A warp's worth of keys share the digits so far (two passes are enough for most units): they are collected and
+      // ranked against one another by one warp, in place of the remaining passes.
+      for (int base = 0; base < n; base += THREADS) {
+        const int i = base + tid;
+        if (i < n) {
+          const uint32_t key = key_at(i);
+          if ((key & mask) == prefix) cand[atomicAdd(&n_cand, 1u)] = key;
+        }
+      }
+      __syncthreads();
+      if (tid < 32) {
+        const bool have = tid < (int)n_cand;
+        const uint32_t key = have ? cand[tid] : 0u;
+        uint32_t larger = 0, equal = 0;
+        for (int j = 0; j < (int)n_cand; ++j) {
+          const uint32_t other = __shfl_sync(0xffffffffu, key, j);
+          larger += other > key;
+          equal += other == key;
+        }
+        if (have && larger < need && need <= larger + equal) {    // lanes with equal keys write the same
+          sh_prefix = key;
+          sh_need = need - larger;
+        }
+      }
+      __syncthreads();
+      prefix = sh_prefix;
+      need = sh_need;
+      break;
+    }
   }
   const uint32_t tau = prefix;     // the ksel-th largest key; `need` of the keys equal to tau survive
   const uint32_t need_eq = need;
@@ -157,7 +200,7 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(int T, int B, int F
   // (consecutive shared-memory words: no bank conflicts; one key per lane and a ballot give the order inside a
   // step).  First the warps count their kept and tied keys, one scan over the 32 warp totals gives every warp its
   // output offset and the rank of its first tie, then the warps write.
-  const int per_w = ((n + SEL_WARPS - 1) / SEL_WARPS + 31) & ~31;
+  const int per_w = ((n + WARPS - 1) / WARPS + 31) & ~31;
   const int lo = min(wid * per_w, n), hi_i = min(lo + per_w, n);
   const uint32_t lt_mask = (1u << lane) - 1u;
   uint32_t n_gt = 0, n_eq = 0;                      // warp-uniform
@@ -385,15 +428,19 @@ cudaError_t launch_select(int units, int T, int B, int F, int R, const float* sc
     cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, select_cluster_kernel, T, B, F, R, split, per, score, kept, dev_status);
   }
-  const size_t bytes = (size_t)(n + 4) * sizeof(uint32_t);     // up to three words of alignment padding
-  if (bytes <= 160 * 1024) {      // beside the 33 KB of histograms
-    cudaError_t e = cudaFuncSetAttribute(select_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e != cudaSuccess) return e;
-    DependentLaunch dl(dim3(units), dim3(SEL_THREADS), bytes, st);
-    return cudaLaunchKernelEx(&dl.cfg, select_kernel<true>, T, B, F, R, score, kept, dev_status);
-  }
-  DependentLaunch dl(dim3(units), dim3(SEL_THREADS), 0, st);
-  return cudaLaunchKernelEx(&dl.cfg, select_kernel<false>, T, B, F, R, score, kept, dev_status);
+  const int copies = n <= 2048 ? 1 : (n <= 16384 ? 4 : 8);
+  const size_t hist_bytes = (size_t)copies * 256 * sizeof(uint32_t);
+  const size_t bytes = hist_bytes + (size_t)(n + 4) * sizeof(uint32_t);     // up to three words of alignment padding
+  const bool staged = bytes <= 168 * 1024;
+  // more units than SMs: CTAs of 512 threads, several to an SM
+  const bool half = units > sms;
+  auto kern = staged ? (half ? select_kernel<true, 512> : select_kernel<true, 1024>)
+                     : (half ? select_kernel<false, 512> : select_kernel<false, 1024>);
+  const size_t dyn = staged ? bytes : hist_bytes;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+  if (e != cudaSuccess) return e;
+  DependentLaunch dl(dim3(units), dim3(half ? 512 : 1024), dyn, st);
+  return cudaLaunchKernelEx(&dl.cfg, kern, copies, T, B, F, R, score, kept, dev_status);
 }
 
 }  // namespace vatp

@@ -1346,9 +1346,13 @@ struct RingSmem {
   int abort_flag;
 };
 
-template <int HD>
-__global__ void __launch_bounds__(RG_THREADS, 2)
-window_ring_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kc, int heads, int T,
+// GROUPED: the history of a KV group holds the MEAN over its G query heads; `heads` counts KV heads, q and lse have
+// heads * G.  The chunk's queries of one head after the other meet the same key tile, and the probabilities are summed in
+// registers (64 per thread: one CTA per SM), in ascending head order.  16 x 8 caches of 1025 slots, 32 query heads, w 256:
+// 2.5 ms on FMA units, now see launch_ring_hd.
+template <int HD, bool GROUPED>
+__global__ void __launch_bounds__(RG_THREADS, GROUPED ? 1 : 2)
+window_ring_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kc, int heads, int G, int T,
                       int w, int B, int cap, float scale_log2, const float* __restrict__ lse, vatp_cache c,
                       int32_t* dev_status) {
   extern __shared__ unsigned char smem_raw[];
@@ -1382,80 +1386,104 @@ window_ring_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
   long long fx = 0;
   bool ok = true;
   uint32_t it = 0;
-  for (int c0 = 0; c0 < w && ok; c0 += CHUNK, ++it) {
-    // the previous chunk's accumulator and normalisers have been consumed by every warp
-    tc_fence_before();
-    __syncthreads();
-    for (int i = tid; i < CHUNK; i += RG_THREADS) {
-      const int r = c0 + i, j = T - w + r;
-      sm.nlse[i] = (r < w && j >= 0) ? -__ldg(lse + (int64_t)u * T + j) * 1.4426950408889634f : -INFINITY;
-    }
-    if (tid == 0) {
-      mbar_expect_tx(&sm.bar_ld, CHUNK_BYTES + (it == 0 ? TILE_BYTES : 0));
-      if (it == 0) {
-        tma_load_2d(sm.keys, &tm_kc, &sm.bar_ld, 0, u * cap + slot0);
-        if (HD > 64) tma_load_2d(sm.keys + SLAB_BYTES, &tm_kc, &sm.bar_ld, 64, u * cap + slot0);
+  // Writes one wave (32 window rows from column cs of the chunk at c0 on, p: this slot's probabilities) and adds it to the
+  // slot's sum.  Window row r = c0 + cs + i is query j = T - w + r and ring row j mod w; both advance by one per column
+  // (the ring row wraps at w; -w < j < 0 when the prompt is shorter than the window).
+  auto emit = [&](const float (&p)[32], int c0, int cs, int n_cols) {
+    const int j0 = T - w + c0 + cs;
+    int rr = j0 >= 0 ? j0 % w : j0 + w;
+    uint32_t off = (uint32_t)rr * (uint32_t)cap;          // element offset of the ring row (w * cap < 2^31: checked on the host)
+    const int live = min(32, n_cols - cs);
+    const bool st_ok = slot < cap;
+    if (live == 32 && rr + 32 <= w) {
+      // the common case - a whole wave inside the window, no wrap of the ring row inside it: no per-column bookkeeping
+      float* out_p = ring_s + off;
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        fx += prob_to_fixed(p[i]);
+        if (st_ok && VATP_INB(off + (uint32_t)i * (uint32_t)cap, (int64_t)w * cap, dev_status)) out_p[(size_t)i * cap] = p[i];
       }
-      // rows before the prompt (negative coordinate) and beyond it arrive as zeros
+    } else {
 #pragma unroll
-      for (int kh = 0; kh < HD / 64; ++kh)
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh)
-          tma_load_4d(sm.qrows + kh * (2 * SLAB_BYTES) + hh * SLAB_BYTES, &tm_q, &sm.bar_ld, 64 * kh, T - w + c0 + hh * TILE, h, b);
-      if (mbar_wait(&sm.bar_ld, it & 1, abort_flag, dev_status)) {
-        tc_fence_after();
-        umma_tile<0, 256, HD>(tmem, umma_desc(s32(sm.keys)), umma_desc(s32(sm.qrows)));
-        umma_commit(&sm.bar_mma);
-      }
-    }
-    __syncthreads();                                 // normalisers written (thread 0 has issued the MMAs or given up)
-    const bool got = mbar_wait(&sm.bar_mma, it & 1, abort_flag, dev_status);
-    if (!__syncthreads_and(got ? 1 : 0)) { ok = false; break; }     // the same verdict for every warp of the CTA
-    tc_fence_after();
-    const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16);
-    const int n_cols = min(CHUNK, w - c0);
-    for (int cs = 64 * grp; cs < min(n_cols, 64 * grp + 64); cs += 32) {
-      float x[32];
-      tmem_ld32(lane_addr + cs, x);
-      tmem_ld_wait();
-      // window row r = c0 + cs + i is query j = T - w + r and ring row j mod w; both advance by one per column
-      // (the ring row wraps at w; -w < j < 0 when the prompt is shorter than the window)
-      const int j0 = T - w + c0 + cs;
-      int rr = j0 >= 0 ? j0 % w : j0 + w;
-      uint32_t off = (uint32_t)rr * (uint32_t)cap;          // element offset of the ring row (w * cap < 2^31: checked on the host)
-      const int live = min(32, n_cols - cs);
-      const uint32_t lp = s32(&sm.nlse[cs]);
-      if (live == 32 && rr + 32 <= w) {
-        // the common case - a whole wave inside the window, no wrap of the ring row inside it: no per-column
-        // bookkeeping.  Column i is visible to this slot's token iff ps <= j0 + i, i.e. i >= first (-1 < first: ps >= 0).
-        const int first = ps >= 0 ? max(ps - j0, 0) : 32;
-        const bool st_ok = slot < cap;
-        float* out_p = ring_s + off;
-#pragma unroll
-        for (int i4 = 0; i4 < 32; i4 += 4) {
-          float4 nl;
-          asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(nl.x), "=f"(nl.y), "=f"(nl.z), "=f"(nl.w) : "r"(lp + 4 * i4));
-          const float nls[4] = {nl.x, nl.y, nl.z, nl.w};
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const int i = i4 + k;
-            const float pr = i >= first ? ex2(fmaf(x[i], scale_log2, nls[k])) : 0.f;
-            fx += prob_to_fixed(pr);
-            if (st_ok && VATP_INB(off + (uint32_t)i * (uint32_t)cap, (int64_t)w * cap, dev_status)) out_p[(size_t)i * cap] = pr;
-          }
+      for (int i = 0; i < 32; ++i) {
+        if (i < live) {
+          fx += prob_to_fixed(p[i]);
+          if (st_ok && VATP_INB(off, (int64_t)w * cap, dev_status)) ring_s[off] = p[i];
+          off += cap;
+          if (++rr == w) { rr = 0; off = 0; }
         }
-      } else {
+      }
+    }
+  };
+  const int n_heads = GROUPED ? G : 1;
+  float sum[GROUPED ? 2 : 1][GROUPED ? 32 : 1];          // the heads' probabilities of this thread's two waves
+  for (int c0 = 0; c0 < w && ok; c0 += CHUNK) {
+    const int n_cols = min(CHUNK, w - c0);
+    for (int g = 0; g < n_heads && ok; ++g, ++it) {
+      const float* lse_h = lse + ((int64_t)b * heads * n_heads + h * n_heads + g) * T;
+      // the previous accumulator and normalisers have been consumed by every warp
+      tc_fence_before();
+      __syncthreads();
+      for (int i = tid; i < CHUNK; i += RG_THREADS) {
+        const int r = c0 + i, j = T - w + r;
+        sm.nlse[i] = (r < w && j >= 0) ? -__ldg(lse_h + j) * 1.4426950408889634f : -INFINITY;
+      }
+      if (tid == 0) {
+        mbar_expect_tx(&sm.bar_ld, CHUNK_BYTES + (it == 0 ? TILE_BYTES : 0));
+        if (it == 0) {
+          tma_load_2d(sm.keys, &tm_kc, &sm.bar_ld, 0, u * cap + slot0);
+          if (HD > 64) tma_load_2d(sm.keys + SLAB_BYTES, &tm_kc, &sm.bar_ld, 64, u * cap + slot0);
+        }
+        // rows before the prompt (negative coordinate) and beyond it arrive as zeros
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          if (i < live) {
-            float nl;
-            asm("ld.shared.f32 %0, [%1];" : "=f"(nl) : "r"(lp + 4 * i));
-            float pr = 0.f;
-            if (ps >= 0 && ps <= j0 + i) pr = ex2(fmaf(x[i], scale_log2, nl));
-            fx += prob_to_fixed(pr);
-            if (slot < cap && VATP_INB(off, (int64_t)w * cap, dev_status)) ring_s[off] = pr;
-            off += cap;
-            if (++rr == w) { rr = 0; off = 0; }
+        for (int kh = 0; kh < HD / 64; ++kh)
+#pragma unroll
+          for (int hh = 0; hh < 2; ++hh)
+            tma_load_4d(sm.qrows + kh * (2 * SLAB_BYTES) + hh * SLAB_BYTES, &tm_q, &sm.bar_ld, 64 * kh, T - w + c0 + hh * TILE, h * n_heads + g, b);
+        if (mbar_wait(&sm.bar_ld, it & 1, abort_flag, dev_status)) {
+          tc_fence_after();
+          umma_tile<0, 256, HD>(tmem, umma_desc(s32(sm.keys)), umma_desc(s32(sm.qrows)));
+          umma_commit(&sm.bar_mma);
+        }
+      }
+      __syncthreads();                                 // normalisers written (thread 0 has issued the MMAs or given up)
+      const bool got = mbar_wait(&sm.bar_mma, it & 1, abort_flag, dev_status);
+      if (!__syncthreads_and(got ? 1 : 0)) { ok = false; break; }     // the same verdict for every warp of the CTA
+      tc_fence_after();
+      const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16);
+#pragma unroll
+      for (int wave = 0; wave < 2; ++wave) {
+        const int cs = 64 * grp + 32 * wave;
+        if (cs < n_cols) {
+          float x[32];
+          tmem_ld32(lane_addr + cs, x);
+          tmem_ld_wait();
+          // column i is visible to this slot's token iff ps <= j0 + i, i.e. i >= first (-1 < first: ps >= 0); rows that are
+          // no query have a normaliser of -inf
+          const int first = ps >= 0 ? max(ps - (T - w + c0 + cs), 0) : 32;
+          const uint32_t lp = s32(&sm.nlse[cs]);
+#pragma unroll
+          for (int i4 = 0; i4 < 32; i4 += 4) {
+            float4 nl;
+            asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(nl.x), "=f"(nl.y), "=f"(nl.z), "=f"(nl.w) : "r"(lp + 4 * i4));
+            const float nls[4] = {nl.x, nl.y, nl.z, nl.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const int i = i4 + k;
+              const float pr = i >= first ? ex2(fmaf(x[i], scale_log2, nls[k])) : 0.f;
+              if constexpr (GROUPED) sum[wave][i] = g == 0 ? pr : sum[wave][i] + pr;
+              else x[i] = pr;
+            }
+          }
+          if constexpr (GROUPED) {
+            if (g == G - 1) {
+              const float inv = 1.f / (float)G;
+#pragma unroll
+              for (int i = 0; i < 32; ++i) x[i] = sum[wave][i] * inv;
+              emit(x, c0, cs, n_cols);
+            }
+          } else {
+            emit(x, c0, cs, n_cols);
           }
         }
       }
@@ -1687,18 +1715,24 @@ cudaError_t launch_prefill_hd(const Shape& s, const void* q, const void* k, cons
                          : cudaLaunchKernelEx(&cfg, prefill_tc_kernel<HD, 2, false>, tm_q, tm_k, a);
 }
 
-template <int HD>
-cudaError_t launch_ring_hd(const Shape& s, int B, const void* q, const float* lse, const vatp_cache& c, int32_t* dev_status,
+template <int HD, bool GROUPED>
+cudaError_t launch_ring_hd(const Shape& s, int G, int B, const void* q, const float* lse, const vatp_cache& c, int32_t* dev_status,
                            cudaStream_t st) {
   const int cap = cache_capacity(B);
+  Shape sq = s;                          // the map over q: with grouped queries G times as many heads
+  sq.heads = s.heads * G;
+  sq.units = s.units * G;
+  sq.kv_heads = 0;
+  sq.qsh = s.qsh / G;
   CUtensorMap tm_q, tm_kc;
-  if (!make_map(&tm_q, q, s, true) || !make_rows_map_bf16(&tm_kc, c.k_cache, HD, (uint64_t)s.units * cap, TILE)) return cudaErrorInvalidValue;
+  if (!make_map(&tm_q, q, sq, true) || !make_rows_map_bf16(&tm_kc, c.k_cache, HD, (uint64_t)s.units * cap, TILE)) return cudaErrorInvalidValue;
   if ((int64_t)s.window * cap >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
   const size_t smem = sizeof(RingSmem<HD>) + 1024;
-  cudaError_t e = cudaFuncSetAttribute(window_ring_tc_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto kern = window_ring_tc_kernel<HD, GROUPED>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  window_ring_tc_kernel<HD><<<dim3((cap + TILE - 1) / TILE, s.units), RG_THREADS, smem, st>>>(
-      tm_q, tm_kc, s.heads, s.T, s.window, B, cap, s.scale * 1.4426950408889634f, lse, c, dev_status);
+  kern<<<dim3((cap + TILE - 1) / TILE, s.units), RG_THREADS, smem, st>>>(tm_q, tm_kc, s.heads, G, s.T, s.window, B, cap,
+                                                                         s.scale * 1.4426950408889634f, lse, c, dev_status);
   return cudaGetLastError();
 }
 
@@ -1712,9 +1746,11 @@ cudaError_t launch_prefill_tc(const Shape& s, const void* q, const void* k, cons
 }
 
 // Window history from Q and the compacted keys on the tensor cores (bf16); see window_ring_tc_kernel.
-cudaError_t launch_window_ring_tc(const Shape& s, int B, const void* q, const float* lse, const vatp_cache& c,
+cudaError_t launch_window_ring_tc(const Shape& s, int G, int B, const void* q, const float* lse, const vatp_cache& c,
                                   int32_t* dev_status, cudaStream_t st) {
-  return s.d == 64 ? launch_ring_hd<64>(s, B, q, lse, c, dev_status, st) : launch_ring_hd<128>(s, B, q, lse, c, dev_status, st);
+  if (G > 1)
+    return s.d == 64 ? launch_ring_hd<64, true>(s, G, B, q, lse, c, dev_status, st) : launch_ring_hd<128, true>(s, G, B, q, lse, c, dev_status, st);
+  return s.d == 64 ? launch_ring_hd<64, false>(s, 1, B, q, lse, c, dev_status, st) : launch_ring_hd<128, false>(s, 1, B, q, lse, c, dev_status, st);
 }
 
 }  // namespace vatp

@@ -269,8 +269,7 @@ vatp_status vatp_compact_window(const vatp_params* p, const void* q, const void*
   decode_history_forget(st);
   cudaError_t e = launch_compact(sh, p->dtype, p->budget, k, v, attn_acc, vnorm, nullptr, kept_idx, *cache, dev_status, st);
   if (e == cudaSuccess)
-    e = group_of(p) > 1 ? launch_window_ring_grouped(sh, group_of(p), p->dtype, p->budget, q, lse, *cache, st)
-                        : launch_window_ring(sh, p->dtype, p->budget, q, lse, *cache, dev_status, st);
+    e = launch_window_ring(sh, group_of(p), p->dtype, p->budget, q, lse, *cache, dev_status, st);
   return e == cudaSuccess ? VATP_OK : (e == cudaErrorNotSupported ? VATP_ERR_UNSUPPORTED : VATP_ERR_CUDA);
 }
 

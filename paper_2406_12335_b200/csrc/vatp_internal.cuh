@@ -123,11 +123,10 @@ cudaError_t launch_compact(const Shape& s, int dtype, int B, const void* k, cons
                            const float* vnorm, const float* win_rows, const int32_t* kept, const vatp_cache& c,
                            int32_t* dev_status, cudaStream_t st);
 // windowed decode state from Q, the compacted keys and the row normalisers (natural log): ring, acc_fixed, acc
-cudaError_t launch_window_ring_grouped(const Shape& s, int G, int dtype, int B, const void* q, const float* lse, const vatp_cache& c,
-                                       cudaStream_t st);
-cudaError_t launch_window_ring(const Shape& s, int dtype, int B, const void* q, const float* lse, const vatp_cache& c,
+// (G: query heads per KV head; s describes the KV units, q and lse hold G times as many heads)
+cudaError_t launch_window_ring(const Shape& s, int G, int dtype, int B, const void* q, const float* lse, const vatp_cache& c,
                                int32_t* dev_status, cudaStream_t st);
-cudaError_t launch_window_ring_tc(const Shape& s, int B, const void* q, const float* lse, const vatp_cache& c,
+cudaError_t launch_window_ring_tc(const Shape& s, int G, int B, const void* q, const float* lse, const vatp_cache& c,
                                   int32_t* dev_status, cudaStream_t st);   // bf16, tensor cores
 // grouped-query attention: mean over the group's G partial indicators [G][n] and Eq. 4; the decode step of a KV group
 cudaError_t launch_group_mean(int G, int64_t n, const float* part, const float* vnorm, float* attn_acc, float* score,

@@ -8,8 +8,8 @@
 //
 // Bound by the FMA pipes when there are many tiles, by latency when there are few.  So
 //   * a thread holds M x M logits (M = 4 or 8) of a 16 M x 16 M tile; both operands sit in shared memory transposed, so
-//     that M elements of a channel are one or two 16-byte loads: 2 (4) loads per 16 (64) FMAs where one element per load
-//     made it 8 per 16.  The next tile's rows are on their way to registers under the products (M = 4);
+//     that M elements of a channel are one or two 16-byte loads: 2 (4) loads per 16 (64) FMAs - issued as packed pairs -
+//     where one element per load made it 8 per 16.  The next tile's rows are on their way to registers under the products (M = 4);
 //   * few tiles are shared out over a cluster of up to eight CTAs along the other dimension, which combine their row
 //     statistics or column sums through distributed shared memory;
 //   * both passes are programmatic dependents: they are resident when the launch before them ends.
@@ -27,7 +27,7 @@ constexpr int MAX_CLUSTER = 8;
 
 // Pass 1: one cluster per (query tile, unit), its CTAs take every cs-th key tile.  lse[j] over keys i <= j.
 template <typename T, int M, int D>
-__global__ void __launch_bounds__(NTHREADS) rowstats_kernel(Shape sh, const T* __restrict__ q, const T* __restrict__ k,
+__global__ void __launch_bounds__(NTHREADS, M == 8 ? 2 : 1) rowstats_kernel(Shape sh, const T* __restrict__ q, const T* __restrict__ k,
                                                             float* __restrict__ lse, int first_row, int cs) {
   constexpr int ROWS = Tile<M, D>::ROWS, LD = Tile<M, D>::LD, NV = Tile<M, D>::NV;
   extern __shared__ __align__(16) float smem[];
@@ -55,16 +55,20 @@ __global__ void __launch_bounds__(NTHREADS) rowstats_kernel(Shape sh, const T* _
     Tile<M, D>::fetch(r, qu, sh.st, q0, min(ROWS, sh.T - q0));
     Tile<M, D>::store(Qs, r);
   }
-  float4 next[NV];
-  if (M == 4 && rank * ROWS < last_key) Tile<M, D>::fetch(next, ku, sh.st, rank * ROWS, min(ROWS, sh.T - rank * ROWS));
+  [[maybe_unused]] float4 next[M == 4 ? NV : 1];
+  if constexpr (M == 4)
+    if (rank * ROWS < last_key) Tile<M, D>::fetch(next, ku, sh.st, rank * ROWS, min(ROWS, sh.T - rank * ROWS));
   for (int k0 = rank * ROWS; k0 < last_key; k0 += cs * ROWS) {
-    if (M != 4) Tile<M, D>::fetch(next, ku, sh.st, k0, min(ROWS, sh.T - k0));
-    __syncthreads();
-    Tile<M, D>::store(Ks, next);
-    __syncthreads();
-    if (M == 4 && k0 + cs * ROWS < last_key) Tile<M, D>::fetch(next, ku, sh.st, k0 + cs * ROWS, min(ROWS, sh.T - k0 - cs * ROWS));
     float s[M][M];
-    micro_gemm<M, D>(Qs, Ks, ty, tx, s);
+    if constexpr (M == 4) {
+      __syncthreads();
+      Tile<M, D>::store(Ks, next);
+      __syncthreads();
+      if (k0 + cs * ROWS < last_key) Tile<M, D>::fetch(next, ku, sh.st, k0 + cs * ROWS, min(ROWS, sh.T - k0 - cs * ROWS));
+      micro_gemm<M, D>(Qs, Ks, ty, tx, s);
+    } else {
+      stream_gemm<T, M, D>(Qs, Ks, ku, sh.st, k0, min(ROWS, sh.T - k0), ty, tx, s);
+    }
 #pragma unroll
     for (int i = 0; i < M; ++i) {
       const int row = q0 + micro_at<M>(ty, i);
@@ -126,16 +130,17 @@ __global__ void __launch_bounds__(NTHREADS) rowstats_kernel(Shape sh, const T* _
 // Pass 2: one cluster per (key tile, unit), its CTAs take every cs-th query tile.  Column sums over query rows
 // j >= max(first_row, k).
 template <typename T, int M, int D>
-__global__ void __launch_bounds__(NTHREADS)
+__global__ void __launch_bounds__(NTHREADS, M == 8 ? 2 : 1)
 colsum_kernel(Shape sh, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
               const float* __restrict__ lse, float* __restrict__ attn_acc, float* __restrict__ vnorm,
               float* __restrict__ score, float* __restrict__ win_rows, int first_row, int cs) {
   constexpr int ROWS = Tile<M, D>::ROWS, LD = Tile<M, D>::LD, NV = Tile<M, D>::NV;
   extern __shared__ __align__(16) float smem[];
-  float* Qs = smem;
-  float* Ks = smem + D * LD;
-  float* lse_s = Ks + D * LD;           // [ROWS]
-  float* red = Qs;                      // [16][ROWS], once the products are done (D >= 16)
+  constexpr int DS = M == 4 ? D : 64;   // channels of the streamed tile in shared memory at a time
+  float* Ks = smem;
+  float* Qs = smem + D * LD;
+  float* lse_s = Qs + DS * LD;          // [ROWS]
+  float* red = Qs;                      // [16][ROWS], once the products are done (DS >= 16)
   __shared__ float vn_s[ROWS], part[ROWS];
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = cs > 1 ? (int)cluster.block_rank() : 0;
@@ -175,29 +180,37 @@ colsum_kernel(Shape sh, const T* __restrict__ q, const T* __restrict__ k, const 
       for (int c = threadIdx.x; c < keys_valid; c += NTHREADS) wr[(int64_t)r * sh.T + k0 + c] = 0.f;
   }
 
-  float4 next[NV];
+  [[maybe_unused]] float4 next[M == 4 ? NV : 1];
   const int qfirst = qstart + rank * ROWS;
-  if (M == 4 && qfirst < sh.T) Tile<M, D>::fetch(next, qu, sh.st, qfirst, min(ROWS, sh.T - qfirst));
+  if constexpr (M == 4)
+    if (qfirst < sh.T) Tile<M, D>::fetch(next, qu, sh.st, qfirst, min(ROWS, sh.T - qfirst));
   for (int q0 = qfirst; q0 < sh.T; q0 += cs * ROWS) {
     const int rows_valid = min(ROWS, sh.T - q0);
-    if (M != 4) Tile<M, D>::fetch(next, qu, sh.st, q0, rows_valid);
-    __syncthreads();
-    Tile<M, D>::store(Qs, next);
-    if (threadIdx.x < ROWS) lse_s[threadIdx.x] = (int)threadIdx.x < rows_valid ? lse[unit_offset_lse(sh, u) + q0 + threadIdx.x] : 0.f;
-    __syncthreads();
-    if (M == 4 && q0 + cs * ROWS < sh.T) Tile<M, D>::fetch(next, qu, sh.st, q0 + cs * ROWS, min(ROWS, sh.T - q0 - cs * ROWS));
+    // (s[i][j]: key k0 + micro_at(ty, i), query q0 + micro_at(tx, j))
     float s[M][M];
-    micro_gemm<M, D>(Qs, Ks, ty, tx, s);
+    const float l = (int)threadIdx.x < rows_valid ? lse[unit_offset_lse(sh, u) + q0 + threadIdx.x] : 0.f;
+    if constexpr (M == 4) {
+      __syncthreads();
+      Tile<M, D>::store(Qs, next);
+      if ((int)threadIdx.x < ROWS) lse_s[threadIdx.x] = l;
+      __syncthreads();
+      if (q0 + cs * ROWS < sh.T) Tile<M, D>::fetch(next, qu, sh.st, q0 + cs * ROWS, min(ROWS, sh.T - q0 - cs * ROWS));
+      micro_gemm<M, D>(Ks, Qs, ty, tx, s);
+    } else {
+      __syncthreads();                  // (every thread is past its last read of lse_s)
+      if ((int)threadIdx.x < ROWS) lse_s[threadIdx.x] = l;
+      stream_gemm<T, M, D>(Ks, Qs, qu, sh.st, q0, rows_valid, ty, tx, s);
+    }
 #pragma unroll
-    for (int i = 0; i < M; ++i) {
-      const int row = q0 + micro_at<M>(ty, i);
-      const float lr = lse_s[micro_at<M>(ty, i)];
+    for (int j = 0; j < M; ++j) {
+      const int row = q0 + micro_at<M>(tx, j);
+      const float lr = lse_s[micro_at<M>(tx, j)];
 #pragma unroll
-      for (int j = 0; j < M; ++j) {
-        const int col = k0 + micro_at<M>(tx, j);
+      for (int i = 0; i < M; ++i) {
+        const int col = k0 + micro_at<M>(ty, i);
         float p = 0.f;
         if (row < sh.T && col <= row && col < sh.T) p = expf(s[i][j] * sh.scale - lr);
-        cs_sum[j] += p;
+        cs_sum[i] += p;
         if (wr && row < sh.T && col < sh.T) wr[(int64_t)(row - wrow0) * sh.T + col] = p;
       }
     }
@@ -222,7 +235,7 @@ colsum_kernel(Shape sh, const T* __restrict__ q, const T* __restrict__ k, const 
   }
   __syncthreads();
 #pragma unroll
-  for (int j = 0; j < M; ++j) red[ty * ROWS + micro_at<M>(tx, j)] = cs_sum[j];
+  for (int i = 0; i < M; ++i) red[tx * ROWS + micro_at<M>(ty, i)] = cs_sum[i];
   __syncthreads();
   float tot = 0.f;
   if ((int)threadIdx.x < ROWS) {
@@ -254,7 +267,7 @@ template <typename T, int M, int D>
 cudaError_t launch_m(const Shape& s, const T* q, const T* k, const T* v, float* lse, float* attn_acc, float* vnorm,
                      float* score, float* win_rows, cudaStream_t st, bool lse_given) {
   using Tl = Tile<M, D>;
-  const size_t smem1 = sizeof(float) * 2 * D * Tl::LD, smem2 = smem1 + sizeof(float) * Tl::ROWS;
+  const size_t smem1 = sizeof(float) * (D + (M == 4 ? D : 64)) * Tl::LD, smem2 = smem1 + sizeof(float) * Tl::ROWS;
   cudaError_t e;
   if ((e = cudaFuncSetAttribute(rowstats_kernel<T, M, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1)) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(colsum_kernel<T, M, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2)) != cudaSuccess) return e;

@@ -847,9 +847,12 @@ constexpr int FW_THREADS = (2 + FW_NSW + 2) * 32;
 #define FW_POLY_MASK 0x0            // of the four pairs of an 8-probability piece, those whose exponential runs on the FMA pipe
 #endif
 constexpr int FW_ST = 3;               // stages of K and of V in shared memory
-constexpr int FW_PB = 2;               // P buffers in TMEM
+// P buffers in TMEM.  head_dim 64 keeps a second bf16 word of every probability (its rounding error), which the other half of
+// the buffer carries into a second product with the same V tile: the output row is then as good as with fp32 probabilities,
+// which its general kernel had, at products that the exponentials hide anyway.
+template <int HD> constexpr int fw_pb = HD == 64 ? 1 : 2;
 constexpr int FW_O_COL = 2 * TILE;     // TMEM columns: S buffers at 0 and 128, O at 256,
-constexpr int FW_P_COL = 3 * TILE;     // P buffers (bf16 pairs, 64 columns each) at 384 and 448
+constexpr int FW_P_COL = 3 * TILE;     // P buffers (bf16 pairs, 64 columns each) at 384 and 448 (head_dim 64: high and low half)
 constexpr float FW_LAZY = 8.f;         // log2 of the growth of a row maximum that forces a rescale
 
 template <int HD>
@@ -859,7 +862,7 @@ struct FwdSmem {
   alignas(1024) unsigned char v[FW_ST][tile_bytes<HD>];    // [d half][128 tokens][128 bytes]
   alignas(8) uint64_t q_full, q_empty;
   uint64_t k_full[FW_ST], k_empty[FW_ST], v_full[FW_ST], v_empty[FW_ST];
-  uint64_t s_full[2], s_empty[2], p_full[FW_PB], p_empty[FW_PB];
+  uint64_t s_full[2], s_empty[2], p_full[2], p_empty[2];
   uint64_t o_full, o_empty;
   uint64_t item_full[4], item_empty[4];
   uint64_t pair_bar[4];                 // softmax warps q and q + 4 (same rows, other keys)
@@ -922,7 +925,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
 attention_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                         const __grid_constant__ CUtensorMap tm_v, TcArgs a, __nv_bfloat16* __restrict__ out) {
   extern __shared__ unsigned char smem_raw[];
-  constexpr int TILE_BYTES = tile_bytes<HD>;
+  constexpr int TILE_BYTES = tile_bytes<HD>, FW_PB = fw_pb<HD>;
   FwdSmem<HD>& sm = *reinterpret_cast<FwdSmem<HD>*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   volatile int* abort_flag = &sm.abort_flag;
@@ -1081,6 +1084,11 @@ attention_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
           for (int kk = 0; kk < TILE / 16; ++kk)      // 16 keys per step: 8 columns further on in P, 2048 bytes in V
             umma_bf16_ts(tmem + FW_O_COL, tmem + FW_P_COL + pb * 64 + kk * 8, vd + (uint64_t)(kk * 128), idesc_pv<HD>,
                          (c > 0 || kk > 0) ? 1u : 0u);
+          if (HD == 64) {
+#pragma unroll
+            for (int kk = 0; kk < TILE / 16; ++kk)
+              umma_bf16_ts(tmem + FW_O_COL, tmem + FW_P_COL + 64 + kk * 8, vd + (uint64_t)(kk * 128), idesc_pv<HD>, 1u);
+          }
           umma_commit(&sm.v_empty[stg]);
           umma_commit(&sm.p_empty[pb]);
           if (c == nc - 1) umma_commit(&sm.o_full);
@@ -1181,6 +1189,7 @@ attention_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         const f32x2 c2 = pk2(sc, sc), nm2 = pk2(-m_ref, -m_ref);
         f32x2 la = pk2(0.f, 0.f), lb = la;
         float pk[32];                              // 64 probabilities as bf16 pairs: this thread's columns of the P buffer
+        [[maybe_unused]] float pl[HD == 64 ? 32 : 1];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           const float* xs = &x[j >> 2][(j & 3) * 8];
@@ -1191,10 +1200,14 @@ attention_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
             if (i & 2) lb = add2(lb, e); else la = add2(la, e);
             float p0, p1;
             upk2(e, p0, p1);
-            pk[j * 4 + (i >> 1)] = __uint_as_float(pack2_bf16(p0, p1));
+            const uint32_t hi = pack2_bf16(p0, p1);
+            pk[j * 4 + (i >> 1)] = __uint_as_float(hi);
+            if constexpr (HD == 64)      // what the rounding to bf16 lost
+              pl[j * 4 + (i >> 1)] = __uint_as_float(pack2_bf16(p0 - __uint_as_float(hi << 16), p1 - __uint_as_float(hi & 0xffff0000u)));
           }
         }
         tmem_st32(tmem + ((uint32_t)(quarter * 32) << 16) + FW_P_COL + pb * 64 + half * 32, pk);
+        if constexpr (HD == 64) tmem_st32(tmem + ((uint32_t)(quarter * 32) << 16) + FW_P_COL + 64 + half * 32, pl);
         l_run += hsum2(add2(la, lb));
         // P and any rescaled O (TMEM stores) are complete before the MMA warp is told
         tmem_st_wait();

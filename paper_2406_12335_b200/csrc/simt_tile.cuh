@@ -41,27 +41,75 @@ struct Tile {
 // row (or column) of element i of the thread's t-th group: four consecutive ones, the second four half a tile on
 template <int M> __device__ __forceinline__ int micro_at(int t, int i) { return (i >> 2) * 64 + t * 4 + (i & 3); }
 
-// s[i][j] = <A row micro_at(ty, i), B row micro_at(tx, j)>, channels in ascending order
-template <int M, int D>
-__device__ __forceinline__ void micro_gemm(const float* As, const float* Bs, int ty, int tx, float (&s)[M][M]) {
-  constexpr int LD = Tile<M, D>::LD;
-#pragma unroll
-  for (int i = 0; i < M; ++i)
-#pragma unroll
-    for (int j = 0; j < M; ++j) s[i][j] = 0.f;
+// Packed fp32 pairs: one instruction for two FMAs (same rounding), which leaves issue slots for the loads.
+typedef unsigned long long f32x2_t;
+__device__ __forceinline__ f32x2_t pack_f32x2(float lo, float hi) {
+  f32x2_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void fma_f32x2(f32x2_t& d, f32x2_t a, f32x2_t b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b)); }
+
+// s[i][j] += <A row micro_at(ty, i), B row micro_at(tx, j)> over NC channels in ascending order, as pairs along j
+template <int M, int NC, int LD>
+__device__ __forceinline__ void micro_gemm_add(const float* As, const float* Bs, int ty, int tx, f32x2_t (&s)[M][M / 2]) {
 #pragma unroll 4
-  for (int c = 0; c < D; ++c) {
-    float a[M], b[M];
+  for (int c = 0; c < NC; ++c) {
+    float a[M];
+    f32x2_t b[M / 2];
 #pragma unroll
     for (int h = 0; h < M / 4; ++h) {
       *reinterpret_cast<float4*>(&a[4 * h]) = *reinterpret_cast<const float4*>(As + c * LD + h * 64 + ty * 4);
-      *reinterpret_cast<float4*>(&b[4 * h]) = *reinterpret_cast<const float4*>(Bs + c * LD + h * 64 + tx * 4);
+      const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(Bs + c * LD + h * 64 + tx * 4);
+      b[2 * h] = x.x;
+      b[2 * h + 1] = x.y;
     }
 #pragma unroll
-    for (int i = 0; i < M; ++i)
+    for (int i = 0; i < M; ++i) {
+      const f32x2_t aa = pack_f32x2(a[i], a[i]);
 #pragma unroll
-      for (int j = 0; j < M; ++j) s[i][j] = fmaf(a[i], b[j], s[i][j]);
+      for (int j = 0; j < M / 2; ++j) fma_f32x2(s[i][j], aa, b[j]);
+    }
   }
+}
+template <int M>
+__device__ __forceinline__ void unpack_products(const f32x2_t (&s2)[M][M / 2], float (&s)[M][M]) {
+#pragma unroll
+  for (int i = 0; i < M; ++i)
+#pragma unroll
+    for (int j = 0; j < M / 2; ++j) asm("mov.b64 {%0, %1}, %2;" : "=f"(s[i][2 * j]), "=f"(s[i][2 * j + 1]) : "l"(s2[i][j]));
+}
+template <int M, int D>
+__device__ __forceinline__ void micro_gemm(const float* As, const float* Bs, int ty, int tx, float (&s)[M][M]) {
+  f32x2_t s2[M][M / 2];
+#pragma unroll
+  for (int i = 0; i < M; ++i)
+#pragma unroll
+    for (int j = 0; j < M / 2; ++j) s2[i][j] = 0ull;
+  micro_gemm_add<M, D, Tile<M, D>::LD>(As, Bs, ty, tx, s2);
+  unpack_products<M>(s2, s);
+}
+// The same with B brought into shared memory here, 64 channels at a time (M = 8: A whole and half of B are 101 KB at 128
+// channels, so that two CTAs fit on an SM and hide one another's loads).  Ends with every thread past its last read but one
+// barrier short of letting B be overwritten.
+template <typename T, int M, int D>
+__device__ __forceinline__ void stream_gemm(const float* As, float* Bs, const T* src, int64_t row_stride, int row0, int rows_valid, int ty, int tx,
+                                            float (&s)[M][M]) {
+  f32x2_t s2[M][M / 2];
+#pragma unroll
+  for (int i = 0; i < M; ++i)
+#pragma unroll
+    for (int j = 0; j < M / 2; ++j) s2[i][j] = 0ull;
+#pragma unroll 1
+  for (int c0 = 0; c0 < D; c0 += 64) {
+    float4 r[Tile<M, 64>::NV];
+    Tile<M, 64>::fetch(r, src + c0, row_stride, row0, rows_valid);
+    __syncthreads();
+    Tile<M, 64>::store(Bs, r);
+    __syncthreads();
+    micro_gemm_add<M, 64, Tile<M, 64>::LD>(As + c0 * Tile<M, D>::LD, Bs, ty, tx, s2);
+  }
+  unpack_products<M>(s2, s);
 }
 
 // launch configuration: programmatic dependent, clusters of cs CTAs along x

@@ -39,9 +39,10 @@ __global__ void __launch_bounds__(NTHREADS, M == 8 ? 2 : 1) rowstats_kernel(Shap
   if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = cs > 1 ? (int)cluster.block_rank() : 0;
-  const int u = blockIdx.y;
+  // the longest rows of all units first: with the units one after the other the last ones left half the SMs idle
+  const int item = blockIdx.x / cs, u = item % sh.units;
   const int ntile = (sh.T - first_row + ROWS - 1) / ROWS;
-  const int q0 = first_row + (ntile - 1 - (int)(blockIdx.x / cs)) * ROWS;      // the longest rows first
+  const int q0 = first_row + (ntile - 1 - item / sh.units) * ROWS;
   const T* qu = q + unit_offset_q(sh, u);
   const T* ku = k + unit_offset(sh, u);
   const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
@@ -144,8 +145,8 @@ colsum_kernel(Shape sh, const T* __restrict__ q, const T* __restrict__ k, const 
   __shared__ float vn_s[ROWS], part[ROWS];
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = cs > 1 ? (int)cluster.block_rank() : 0;
-  const int u = blockIdx.y;
-  const int k0 = (int)(blockIdx.x / cs) * ROWS;
+  const int item = blockIdx.x / cs, u = item % sh.units;      // the longest columns of all units first
+  const int k0 = item / sh.units * ROWS;
   const T* qu = q + unit_offset_q(sh, u);
   const T* ku = k + unit_offset(sh, u);
   const T* vu = v + unit_offset(sh, u);
@@ -281,11 +282,11 @@ cudaError_t launch_m(const Shape& s, const T* q, const T* k, const T* v, float* 
   };
   if (!lse_given) {
     const int cs = cluster_for(qtiles, ktiles);
-    ClusterLaunch c1(dim3(qtiles * cs, s.units), smem1, st, cs);
+    ClusterLaunch c1(dim3((unsigned)(qtiles * s.units * cs)), smem1, st, cs);
     if ((e = cudaLaunchKernelEx(&c1.cfg, rowstats_kernel<T, M, D>, s, q, k, lse, first_row, cs)) != cudaSuccess) return e;
   }
   const int cs = cluster_for(ktiles, qtiles);
-  ClusterLaunch c2(dim3(ktiles * cs, s.units), smem2, st, cs);
+  ClusterLaunch c2(dim3((unsigned)(ktiles * s.units * cs)), smem2, st, cs);
   return cudaLaunchKernelEx(&c2.cfg, colsum_kernel<T, M, D>, s, q, k, v, (const float*)lse, attn_acc, vnorm, score,
                             s.window > 0 ? win_rows : nullptr, first_row, cs);
 }

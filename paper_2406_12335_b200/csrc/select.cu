@@ -11,7 +11,8 @@
 // digits with match.any cost more than everything else in the kernel: it takes time in proportion to
 // the number of distinct values in the warp.)  As soon as at most 32 keys share the boundary's digits - after two passes
 // for most units - one warp ranks those instead of two more passes.
-// (256 units x 7936 keys with the compaction behind it 103.7 -> 101.7 us; 8 units x 7806 20.9 -> 19.6.)
+// Lanes take four keys at a time: the passes were bound by issue slots (178 warp instructions per 32 keys).
+// (256 units x 7936 keys with the compaction behind it 103.7 -> 98 us; 8 units x 7806 20.9 -> 19.6.)
 #include <cooperative_groups.h>
 
 #include "vatp_internal.cuh"
@@ -93,31 +94,56 @@ __global__ void __launch_bounds__(THREADS) select_kernel(int copies, int T, int 
     if (tid < n - tail0) keys_s[pad + tail0 + tid] = order_key(mid[tail0 + tid]);
     __syncthreads();
   }
-  auto key_at = [&](int i) -> uint32_t { return STAGED ? keys_s[pad + i] : order_key(sc[F + i]); };
+  // Four keys at a time: group v holds keys 4 v - pad .. 4 v - pad + 3 of the middle range.
+  const int nv = (pad + n + 3) >> 2;
+  struct Keys4 { uint32_t k[4]; };
+  auto keys_of = [&](int v) -> Keys4 {
+    Keys4 r;
+    if (STAGED) {
+      const uint4 x = reinterpret_cast<const uint4*>(keys_s)[v];
+      r.k[0] = x.x; r.k[1] = x.y; r.k[2] = x.z; r.k[3] = x.w;
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) r.k[e] = 4 * v + e < n ? order_key(sc[F + 4 * v + e]) : 0u;
+    }
+    return r;
+  };
+  auto in_range = [&](int v, int e) { return (unsigned)(4 * v + e - pad) < (unsigned)n; };
 
   // radix select, most significant byte first: find the key value tau of rank ksel (descending).
-  // Lanes that share the digit of the warp's first candidate are counted together; the rest add one each.
-  uint32_t prefix = 0, mask = 0, need = (uint32_t)ksel;
+  uint32_t prefix = 0, mask = 0, need = (uint32_t)ksel, ties = 0xffffffffu;     // ties: keys equal to tau, when known
   const int lane = tid & 31, wid = tid >> 5;
   uint32_t* my_hist = hist_c + (wid % copies) * 256;
   for (int shift = 24; shift >= 0; shift -= 8) {
     for (int i = tid; i < copies * 256; i += THREADS) hist_c[i] = 0;
     if (tid == 0) n_cand = 0;
     __syncthreads();
-    for (int base = 0; base < n; base += THREADS) {
-      const int i = base + tid;
-      uint32_t digit = 256u;                       // lanes without a candidate share a dummy digit
-      if (i < n) {
-        const uint32_t key = key_at(i);
-        if ((key & mask) == prefix) digit = (key >> shift) & 255u;
+    if (shift == 24) {
+      // the top digit is a sign and seven exponent bits: most keys of a warp share the first lane's, which are counted
+      // with ballots and added once; the others add one each
+      for (int v0 = 0; v0 < nv; v0 += THREADS) {
+        const int v = v0 + tid;
+        Keys4 x;
+        if (v < nv) x = keys_of(v);
+        uint32_t d[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) d[e] = v < nv && in_range(v, e) ? x.k[e] >> 24 : 256u;
+        const uint32_t d0 = __shfl_sync(0xffffffffu, d[3], 0);      // (256 where a warp begins in the padding: counts nothing)
+        uint32_t same = 0;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          same += __popc(__ballot_sync(0xffffffffu, d[e] == d0));
+          if (d[e] != d0 && d[e] < 256u) atomicAdd(&my_hist[d[e]], 1u);
+        }
+        if (lane == 0 && d0 < 256u) atomicAdd(&my_hist[d0], same);
       }
-      const uint32_t some = __ballot_sync(0xffffffffu, digit < 256u);
-      if (some) {
-        const int first = __ffs(some) - 1;
-        const uint32_t d0 = __shfl_sync(0xffffffffu, digit, first);
-        const uint32_t same = __ballot_sync(0xffffffffu, digit == d0);
-        if (lane == first) atomicAdd(&my_hist[d0], (uint32_t)__popc(same));
-        else if (digit < 256u && digit != d0) atomicAdd(&my_hist[digit], 1u);
+    } else {
+      // mantissa digits spread over the bins
+      for (int v = tid; v < nv; v += THREADS) {
+        const Keys4 x = keys_of(v);
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if ((x.k[e] & mask) == prefix && in_range(v, e)) atomicAdd(&my_hist[(x.k[e] >> shift) & 255u], 1u);
       }
     }
     __syncthreads();
@@ -160,16 +186,16 @@ __global__ void __launch_bounds__(THREADS) select_kernel(int copies, int T, int 
     __syncthreads();
     prefix = sh_prefix;
     need = sh_need;
+    ties = sh_in_bin;
     mask |= 255u << shift;
-    if (shift > 0 && sh_in_bin <= 32u) {
+    if (shift > 0 && ties <= 32u) {
       // A warp's worth of keys share the digits so far (two passes are enough for most units): they are collected and
       // ranked against one another by one warp, in place of the remaining passes.
-      for (int base = 0; base < n; base += THREADS) {
-        const int i = base + tid;
-        if (i < n) {
-          const uint32_t key = key_at(i);
-          if ((key & mask) == prefix) cand[atomicAdd(&n_cand, 1u)] = key;
-        }
+      for (int v = tid; v < nv; v += THREADS) {
+        const Keys4 x = keys_of(v);
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if ((x.k[e] & mask) == prefix && in_range(v, e)) cand[atomicAdd(&n_cand, 1u)] = x.k[e];
       }
       __syncthreads();
       if (tid < 32) {
@@ -184,53 +210,81 @@ __global__ void __launch_bounds__(THREADS) select_kernel(int copies, int T, int 
         if (have && larger < need && need <= larger + equal) {    // lanes with equal keys write the same
           sh_prefix = key;
           sh_need = need - larger;
+          sh_in_bin = equal;
         }
       }
       __syncthreads();
       prefix = sh_prefix;
       need = sh_need;
+      ties = sh_in_bin;
       break;
     }
   }
-  const uint32_t tau = prefix;     // the ksel-th largest key; `need` of the keys equal to tau survive
+  const uint32_t tau = prefix;     // the ksel-th largest key; `need` of the `ties` keys equal to tau survive
   const uint32_t need_eq = need;
 
   // Ordered compaction: keep key > tau, and the first need_eq (lowest index) keys equal to tau.
-  // Warp w owns the contiguous range [w * per_w, (w + 1) * per_w) and walks it 32 consecutive keys at a time
-  // (consecutive shared-memory words: no bank conflicts; one key per lane and a ballot give the order inside a
-  // step).  First the warps count their kept and tied keys, one scan over the 32 warp totals gives every warp its
+  // Warp w owns a contiguous range of key groups and walks it 32 groups at a time, a lane per group.
+  // First the warps count their kept and tied keys, one scan over the warp totals gives every warp its
   // output offset and the rank of its first tie, then the warps write.
-  const int per_w = ((n + WARPS - 1) / WARPS + 31) & ~31;
-  const int lo = min(wid * per_w, n), hi_i = min(lo + per_w, n);
+  const bool all_ties = ties == need_eq;             // the usual case: key >= tau decides
+  const int per_w = (nv + WARPS - 1) / WARPS;
+  const int lo = min(wid * per_w, nv), hi_v = min(lo + per_w, nv);
   const uint32_t lt_mask = (1u << lane) - 1u;
-  uint32_t n_gt = 0, n_eq = 0;                      // warp-uniform
-  for (int i0 = lo; i0 < hi_i; i0 += 32) {
-    const int i = i0 + lane;
-    const uint32_t key = i < hi_i ? key_at(i) : 0u;
-    n_gt += __popc(__ballot_sync(0xffffffffu, i < hi_i && key > tau));
-    n_eq += __popc(__ballot_sync(0xffffffffu, i < hi_i && key == tau));
+  uint32_t n_gt = 0, n_eq = 0;
+  for (int v = lo + lane; v < hi_v; v += 32) {
+    const Keys4 x = keys_of(v);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const bool in = in_range(v, e);
+      n_gt += in && x.k[e] > tau;
+      n_eq += in && x.k[e] == tau;
+    }
   }
+  n_gt = __reduce_add_sync(0xffffffffu, n_gt);
+  n_eq = __reduce_add_sync(0xffffffffu, n_eq);
   if (lane == 0) { warp_keep[wid] = n_gt; warp_eq[wid] = n_eq; }
   __syncthreads();
   // exclusive prefix over the warps, computed by every warp for itself
-  uint32_t a = lane < wid ? warp_keep[lane] : 0u, b = lane < wid ? warp_eq[lane] : 0u;
-#pragma unroll
-  for (int off = 16; off; off >>= 1) {
-    a += __shfl_xor_sync(0xffffffffu, a, off);
-    b += __shfl_xor_sync(0xffffffffu, b, off);
-  }
-  uint32_t eq_rank = b;                             // ties before this warp's range
+  const uint32_t a = __reduce_add_sync(0xffffffffu, lane < wid ? warp_keep[lane] : 0u);
+  uint32_t eq_rank = __reduce_add_sync(0xffffffffu, lane < wid ? warp_eq[lane] : 0u);     // ties before this warp's range
   uint32_t o = a + min(eq_rank, need_eq);           // output offset of this warp's first kept key
-  for (int i0 = lo; i0 < hi_i; i0 += 32) {
-    const int i = i0 + lane;
-    const uint32_t key = i < hi_i ? key_at(i) : 0u;
-    const bool is_eq = i < hi_i && key == tau;
-    const uint32_t eq_b = __ballot_sync(0xffffffffu, is_eq);
-    const bool keep = i < hi_i && (key > tau || (is_eq && eq_rank + __popc(eq_b & lt_mask) < need_eq));
-    const uint32_t keep_b = __ballot_sync(0xffffffffu, keep);
-    if (keep && VATP_INB(F + o + __popc(keep_b & lt_mask), B - R, dev_status)) out[F + o + __popc(keep_b & lt_mask)] = F + i;
-    o += __popc(keep_b);
-    eq_rank += __popc(eq_b);
+  for (int v0 = lo; v0 < hi_v; v0 += 32) {
+    const int v = v0 + lane;
+    Keys4 x;
+    if (v < hi_v) x = keys_of(v);
+    bool keep[4];
+    uint32_t eq_before = eq_rank, eq_here = 0;
+    if (!all_ties) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) eq_here += v < hi_v && in_range(v, e) && x.k[e] == tau;
+      // ties of the lanes before this one
+      uint32_t incl = eq_here;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += y;
+      }
+      eq_before += incl - eq_here;
+      eq_rank += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    uint32_t at = o, step = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const bool in = v < hi_v && in_range(v, e);
+      keep[e] = in && (x.k[e] > tau || (x.k[e] == tau && (all_ties || eq_before < need_eq)));
+      if (!all_ties && in && x.k[e] == tau) ++eq_before;
+      const uint32_t b = __ballot_sync(0xffffffffu, keep[e]);
+      at += __popc(b & lt_mask);                     // kept keys of the lanes before this one
+      step += __popc(b);
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (keep[e]) {
+        if (VATP_INB(F + at, B - R, dev_status)) out[F + at] = F + 4 * v + e - pad;
+        ++at;
+      }
+    o += step;
   }
 }
 

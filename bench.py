@@ -222,9 +222,9 @@ def prune_launches(wl, args):
     windowed = wl.indicator == "window"
     tensor_core = wl.dtype == "bf16" and wl.head_dim == 128
     if tensor_core:
-        # Eq. 2 with the l1 norm: counter reset, pass 1 (value norms on its side warp), pass 2;
-        # otherwise: norm kernel, pass 1 unless the normalisers are given, pass 2
-        scoring = 2 if args.lse_given else 3
+        # counter reset, pass 1 unless the normalisers are given, the norm kernel (Eq. 2 with the l1 norm: the side warp of
+        # pass 1 instead), pass 2
+        scoring = 3 if args.lse_given or not (windowed or wl.norm != "l1") else 4
     else:
         scoring = 1 if args.lse_given else 2       # row statistics, column sums
     compaction = 2 if windowed else 1              # gather, then the window history (rebuilt or gathered)

@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(CB_THREADS, 1)
 compact_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, int64_t gather_rs,
                Shape sh, int elem_bytes, int B, int cap, const char* __restrict__ k, const char* __restrict__ v,
                const float* __restrict__ attn_acc, const float* __restrict__ vnorm, const int32_t* __restrict__ kept,
-               vatp_cache c, int rows_pb, int nbuf, int32_t* dev_status) {
+               vatp_cache c, int rows_pb, int nbuf, int release, int32_t* dev_status) {
   extern __shared__ __align__(128) unsigned char cb_smem[];
   __shared__ __align__(8) uint64_t bars[CB_WARPS][CB_MAXBUF];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -67,6 +67,8 @@ compact_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   __syncwarp();
   // launched as a programmatic dependent of the selection: nothing is read before that has completed
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  // The history rebuild may set up meanwhile.  Nothing else is released early: a decode step requests cache rows before its wait.
+  if (release && threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   const int len = min(sh.T, B);
   const int nb = (cap + rows_pb - 1) / rows_pb;
@@ -239,7 +241,7 @@ cudaError_t launch_compact(const Shape& s, int dtype, int B, const void* k, cons
   const dim3 grid((unsigned)(want < sms ? want : sms));
   DependentLaunch dl(grid, dim3(CB_THREADS), smem, st);
   e = cudaLaunchKernelEx(&dl.cfg, compact_kernel, tm_k, tm_v, rs, s, eb, B, cap, (const char*)k, (const char*)v, attn_acc,
-                         vnorm, kept, c, rows_pb, nbuf, dev_status);
+                         vnorm, kept, c, rows_pb, nbuf, s.window > 0 && !win_rows ? 1 : 0, dev_status);
   if (e != cudaSuccess) return e;
   if (s.window > 0 && win_rows) {
     ring_kernel<<<dim3((cap + 127) / 128, s.units), 128, 0, st>>>(s.units, s.T, s.window, B, cap, win_rows, kept, c, dev_status);

@@ -384,6 +384,9 @@ decode_gqa_kernel(int G, int d, int B, int cap, int F, int R, int w, int norm, f
 // attn_acc[u][t] = mean over the group's G partial indicators; score = that mean times the value norm (Eq. 4)
 __global__ void group_mean_kernel(int G, int64_t n, const float* __restrict__ part, const float* __restrict__ vnorm,
                                   float* __restrict__ attn_acc, float* __restrict__ score) {
+  // a programmatic dependent of pass 2; the selection, its own dependent, may set up
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   float s = 0.f;
@@ -431,8 +434,8 @@ cudaError_t launch_gqa(int units, int G, int d, int split, int seg, size_t smem,
 
 cudaError_t launch_group_mean(int G, int64_t n, const float* part, const float* vnorm, float* attn_acc, float* score,
                               cudaStream_t st) {
-  group_mean_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(G, n, part, vnorm, attn_acc, score);
-  return cudaGetLastError();
+  DependentLaunch dl(dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st);
+  return cudaLaunchKernelEx(&dl.cfg, group_mean_kernel, G, n, part, vnorm, attn_acc, score);
 }
 
 // units: batch * kv_heads.  cudaErrorNotSupported when the probabilities of a unit's heads do not fit in shared memory,

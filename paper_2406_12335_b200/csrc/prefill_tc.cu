@@ -1292,16 +1292,23 @@ __global__ void reset_counters_kernel(unsigned* counters) {
 // When the caller supplies the row normalisers (lse_in, natural log, [units][T]) the same launch brings them
 // into the layout pass 2 reads and so stands in for pass 1: log2 domain and negated, padded to whole chunks,
 // -inf where a query contributes nothing (beyond the prompt, before the history window).
+// It is a programmatic dependent.  After pass 1 (or the forward), whose launch has released it, everything it reads is
+// complete, and it runs beside that pass - small CTAs, for the registers a pass-1 CTA leaves on its SM - instead of before
+// it; only the first CTA stays until that pass has completed, so that whatever waits for this launch waits for both (32 heads
+// x 2048 tokens with a window of 256, scoring + selection + compaction + history: 70 -> 61 us with the counters' memset
+// gone).  With the caller's normalisers it stands in for pass 1 and waits first.
+constexpr int VN_THREADS = 128, VN_TOKENS = 64;
 template <int HD, int KIND>
-__global__ void __launch_bounds__(256) vnorm_kernel(TcArgs a, const float* __restrict__ lse_in) {
+__global__ void __launch_bounds__(VN_THREADS) vnorm_kernel(TcArgs a, const float* __restrict__ lse_in) {
+  if (lse_in) asm volatile("griddepcontrol.wait;" ::: "memory");
   // pass 2, a programmatic dependent, may set up while this kernel runs; it reads what is written here
   // only after its griddepcontrol.wait
   if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int u = blockIdx.x;
   if (lse_in) {
-    // this CTA's 128 tokens; the last CTA of the unit also fills the padding up to Tpad
-    const int last = blockIdx.y == gridDim.y - 1 ? a.Tpad : (blockIdx.y + 1) * 128;
-    for (int i = blockIdx.y * 128 + threadIdx.x; i < last; i += 256) {
+    // this CTA's tokens; the last CTA of the unit also fills the padding up to Tpad
+    const int last = blockIdx.y == gridDim.y - 1 ? a.Tpad : (blockIdx.y + 1) * VN_TOKENS;
+    for (int i = blockIdx.y * VN_TOKENS + threadIdx.x; i < last; i += VN_THREADS) {
       float x = -INFINITY;
       if (i < a.T) {
         const float l = __ldg(lse_in + (int64_t)u * a.T + i);
@@ -1313,9 +1320,9 @@ __global__ void __launch_bounds__(256) vnorm_kernel(TcArgs a, const float* __res
   }
   const int b = u / a.kv_heads, h = u - b * a.kv_heads;      // (one CTA column per KV unit)
   const __nv_bfloat16* vu = a.v + (int64_t)b * a.sb + (int64_t)h * a.sh;
-  constexpr int LPR = HD / 8, RPP = 256 / LPR, NP = 128 / RPP;     // lanes per row, rows per pass of the CTA, passes
+  constexpr int LPR = HD / 8, RPP = VN_THREADS / LPR, NP = VN_TOKENS / RPP;     // lanes per row, rows per pass of the CTA, passes
   const int sub = threadIdx.x / LPR, part = threadIdx.x % LPR;
-  const int row0 = blockIdx.y * 128 + sub;
+  const int row0 = blockIdx.y * VN_TOKENS + sub;
   uint4 raw[NP];
 #pragma unroll
   for (int j = 0; j < NP; ++j) {
@@ -1335,6 +1342,7 @@ __global__ void __launch_bounds__(256) vnorm_kernel(TcArgs a, const float* __res
     const int tok = row0 + RPP * j;
     if (part == 0 && tok < a.T) a.vnorm[(int64_t)u * a.T + tok] = norm_finish(KIND, acc);
   }
+  if (!lse_in && blockIdx.x == 0 && blockIdx.y == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 
@@ -1390,6 +1398,8 @@ window_ring_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
 
+  // a programmatic dependent of the compaction: set up by now, it reads nothing before that has completed
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int quarter = wid & 3, grp = wid >> 2;      // TMEM lanes this warp may touch; which 64 columns of a chunk it takes
   const int row = quarter * 32 + lane;
   const int slot = slot0 + row;                     // this thread's slot = its TMEM lane
@@ -1672,21 +1682,16 @@ cudaError_t launch_prefill_hd(const Shape& s, const void* q, const void* k, cons
   const int items1 = a.units * (a.nt - a.ft), items2 = a.units * a.nt;
   // the side warp belongs to pass 1 (too short under a history window) or to the fused forward (always all tiles)
   a.side_norm = (a.ft == 0 || attn_out) && a.norm == VATP_NORM_L1 && !lse_in;
-  // The counters are zeroed first.  When pass 1 follows at once, a one-warp kernel does it and pass 1 is its
-  // programmatic dependent (see reset_counters_kernel); otherwise a memset node.
-  a.wait_first = (a.side_norm && !lse_in) ? 1 : 0;
-  if (a.wait_first) {
-    DependentLaunch dr(dim3(1), dim3(32), 0, st);
-    if ((e = cudaLaunchKernelEx(&dr.cfg, reset_counters_kernel, a.counters)) != cudaSuccess) return e;
-  } else if ((e = cudaMemsetAsync(a.counters, 0, 2 * sizeof(unsigned), st)) != cudaSuccess) {
-    return e;
-  }
-  if (!a.side_norm) {
-    const dim3 grid(a.kv_units, (s.T + 127) / 128);
-    if (a.norm == VATP_NORM_L1) vnorm_kernel<HD, VATP_NORM_L1><<<grid, 256, 0, st>>>(a, lse_in);
-    else if (a.norm == VATP_NORM_L2) vnorm_kernel<HD, VATP_NORM_L2><<<grid, 256, 0, st>>>(a, lse_in);
-    else vnorm_kernel<HD, VATP_NORM_LINF><<<grid, 256, 0, st>>>(a, lse_in);
-  }
+  // The counters are zeroed first, by a one-warp kernel that waits for all earlier work; what follows is its programmatic
+  // dependent (see reset_counters_kernel).
+  a.wait_first = 1;
+  DependentLaunch dr(dim3(1), dim3(32), 0, st);
+  if ((e = cudaLaunchKernelEx(&dr.cfg, reset_counters_kernel, a.counters)) != cudaSuccess) return e;
+  auto value_norms = [&]() {
+    DependentLaunch dv(dim3(a.kv_units, (s.T + VN_TOKENS - 1) / VN_TOKENS), dim3(VN_THREADS), 0, st);
+    auto kern = a.norm == VATP_NORM_L1 ? vnorm_kernel<HD, VATP_NORM_L1> : a.norm == VATP_NORM_L2 ? vnorm_kernel<HD, VATP_NORM_L2> : vnorm_kernel<HD, VATP_NORM_LINF>;
+    return cudaLaunchKernelEx(&dv.cfg, kern, a, lse_in);
+  };
   if (attn_out) {
     // the forward sweep stands in for pass 1; it streams K and V, so a group's units share the L2 three ways
     const size_t fsmem = sizeof(FwdSmem<HD>) + 1024;
@@ -1697,22 +1702,16 @@ cudaError_t launch_prefill_hd(const Shape& s, const void* q, const void* k, cons
       const size_t g = ((size_t)48 << 20) / unit_bytes;
       af.gu = g < 1 ? 1 : (g > (size_t)s.units ? s.units : (int)g);
     }
-    if (a.wait_first) {
-      DependentLaunch df(dim3(items2 < sms ? items2 : sms), dim3(FW_THREADS), fsmem, st);
-      if ((e = cudaLaunchKernelEx(&df.cfg, attention_fwd_tc_kernel<HD>, tm_q, tm_k, tm_v, af, static_cast<__nv_bfloat16*>(attn_out))) !=
-          cudaSuccess)
-        return e;
-    } else {
-      attention_fwd_tc_kernel<HD><<<items2 < sms ? items2 : sms, FW_THREADS, fsmem, st>>>(tm_q, tm_k, tm_v, af,
-                                                                                      static_cast<__nv_bfloat16*>(attn_out));
-    }
-  } else if (a.wait_first && !lse_in) {
+    DependentLaunch df(dim3(items2 < sms ? items2 : sms), dim3(FW_THREADS), fsmem, st);
+    if ((e = cudaLaunchKernelEx(&df.cfg, attention_fwd_tc_kernel<HD>, tm_q, tm_k, tm_v, af, static_cast<__nv_bfloat16*>(attn_out))) !=
+        cudaSuccess)
+      return e;
+  } else if (!lse_in) {
     DependentLaunch d1(dim3(items1 < sms ? items1 : sms), dim3(TC_THREADS), smem, st);
     if ((e = cudaLaunchKernelEx(&d1.cfg, prefill_tc_kernel<HD, 1, false>, tm_q, tm_k, a)) != cudaSuccess) return e;
-  } else if (!lse_in) {
-    prefill_tc_kernel<HD, 1, false><<<items1 < sms ? items1 : sms, TC_THREADS, smem, st>>>(tm_q, tm_k, a);
   }
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  // without the side warp (and in place of pass 1 when the normalisers are given): the norms
+  if (!a.side_norm && (e = value_norms()) != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(items2 < sms ? items2 : sms);
   cfg.blockDim = dim3(TC_THREADS);
@@ -1744,9 +1743,8 @@ cudaError_t launch_ring_hd(const Shape& s, int G, int B, const void* q, const fl
   auto kern = window_ring_tc_kernel<HD, GROUPED>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<dim3((cap + TILE - 1) / TILE, s.units), RG_THREADS, smem, st>>>(tm_q, tm_kc, s.heads, G, s.T, s.window, B, cap,
-                                                                         s.scale * 1.4426950408889634f, lse, c, dev_status);
-  return cudaGetLastError();
+  DependentLaunch dl(dim3((cap + TILE - 1) / TILE, s.units), dim3(RG_THREADS), smem, st);
+  return cudaLaunchKernelEx(&dl.cfg, kern, tm_q, tm_kc, s.heads, G, s.T, s.window, B, cap, s.scale * 1.4426950408889634f, lse, c, dev_status);
 }
 
 }  // namespace

@@ -119,6 +119,7 @@ cudaError_t launch_attention_fwd_general(const Shape& s, int dtype, const void* 
 size_t prefill_tc_workspace_bytes(int units, int T);  // padded log2-domain row normalisers
 cudaError_t launch_select(int units, int T, int B, int F, int R, const float* score, int32_t* kept, int32_t* dev_status,
                           cudaStream_t st);
+// (with a history window and no win_rows the caller launches the history rebuild next: the kernel releases it early)
 cudaError_t launch_compact(const Shape& s, int dtype, int B, const void* k, const void* v, const float* attn_acc,
                            const float* vnorm, const float* win_rows, const int32_t* kept, const vatp_cache& c,
                            int32_t* dev_status, cudaStream_t st);

@@ -6,9 +6,10 @@
 //   * every warp has a ring of units - the K rows or the V rows of a 16-row group, one tiled TMA load each,
 //     128-byte swizzled so that ldmatrix is conflict-free; the first units are requested before anything else happens;
 //   * q.K^T and p.V run on the warp-level tensor-core path (mma.sync m16n8k16, bf16 in, fp32
-//     accumulate): S^T = q K^T with the queries in the rows, O^T = V^T p with V^T out of ldmatrix.trans as the A operand:
-//     sixteen output channels per instruction and 32 accumulator registers for 128 channels.  p is split into two bf16
-//     halves (columns hi / lo of the B operand, or two products when the columns are heads): the product keeps ~16 bits
+//     accumulate) with the cached rows as the A operand, of which every row counts: S = K q^T with the queries in the eight
+//     columns, O^T = V^T p with V^T out of ldmatrix.trans: sixteen rows or channels per instruction.  (With the queries as
+//     A, half of the first phase's products were padding: 512 units x 1025 slots 57 against 55 us.)  p is split into two
+//     bf16 halves (in columns of their own with up to four heads, as two products with more): the product keeps ~16 bits
 //     of p;
 //   * two phases, all K rows and then all V rows: no group of rows depends on another, and exponentials are taken once
 //     per slot.  (One sweep with an online softmax was a chain of ~2300 cycles per 16-row group - fragments, products,
@@ -17,8 +18,8 @@
 //     its instructions issue 65 cycles apart for 4 KB of rows each.)
 //   * eight warps and at most half of an SM's shared memory: two CTAs fit on an SM, so the
 //     CTAs of the next launch are resident while this one runs.  A launch that has to wait for its predecessor has then
-//     already filled its rings and asked for the rest of its rows in L2 (its K and V rows are the one thing it may read
-//     early), and what is left after the wait is the arithmetic, the tail and reads that hit L2;
+//     already filled its rings (its K and V rows are the one thing it may read early).  (Asking for the rest of its rows in
+//     L2 as well, by bulk prefetch or line by line, made a step of 32 units x 2049 slots 0.1 to 2 us longer.);
 //   * more units than CTAs fit on the machine: a CTA takes several, and a producer warp streams the next one's rows while
 //     the tail of this one runs;
 //   * a unit (sequence, head) is split over a thread-block cluster when units are few.  Every CTA pushes its
@@ -40,10 +41,11 @@
 //     machine;
 //   * grouped-query attention (several query heads share one cache; the paper leaves the case open and points at
 //     a group-wise score, read here as the MEAN of the heads' probabilities): up to eight heads of a group ride
-//     in the rows of S^T (template parameter GT), so a K or V row is still read once per step.
-// Measured (us per step, before and after the two phases, the exchange by st.async and the co-resident successor): 32 units
-// x 2049 slots, every launch waiting 12.5 -> 10.4; 256 units x 1639, launches overlapping 38 -> 35 (138 MB: 6.1 TB/s of the
-// 6.56 a copy reaches); 512 units x 1025 with a history window 73 -> 58; 8 units x 2049, four heads each 11.0 -> 10.4.
+//     in the columns of the products (template parameter GT), so a K or V row is still read once per step.
+// Measured (us per step, before and after the two phases, the exchange by st.async, the co-resident successor and the rows as
+// A operand): 32 units x 2049 slots, every launch waiting 12.5 -> 10.3; 256 units x 1639, launches overlapping 38 -> 34.4
+// (215 MB: 6.2 TB/s of the 6.56 a copy reaches); 512 units x 1025 with a history window 73 -> 55; 8 units x 2049, four heads
+// each 11.0 -> 9.3 (exponentials a warp per head, the ranks' factors unrolled, one product per group for up to four heads).
 #include <cooperative_groups.h>
 
 #include <mutex>
@@ -68,7 +70,7 @@ template <int HD> constexpr int unit_bytes = GROUP * HD * 2;   // K rows (or V r
 constexpr int TILE_BYTES = GROUP * 128;    // 16 rows x 64 bf16, 128-byte swizzled
 constexpr int MAX_SLOTS = 8;          // units a warp keeps in flight at most
 constexpr int MAX_SPLIT = 8;
-constexpr int GQ_HEADS = 8;           // grouped queries: query heads per cache this kernel takes (rows 0-7 of the MMA tiles)
+constexpr int GQ_HEADS = 8;           // grouped queries: query heads per cache this kernel takes (columns of the MMA tiles)
 constexpr float LOG2E = 1.4426950408889634f;
 constexpr unsigned long long NO_KEY = ~0ull;
 
@@ -191,7 +193,7 @@ __device__ __forceinline__ unsigned long long warp_min_key(unsigned long long ke
 }
 
 // GT = 1: one query head per cache (multi-head attention).  GT = GQ_HEADS: grouped queries - up to GQ_HEADS query
-// heads (G of them, a run-time argument) share the cache of unit u: row g of S^T carries head g, so every K and V row
+// heads (G of them, a run-time argument) share the cache of unit u: column g of the products carries head g, so every K and V row
 // is read once for the whole group; the maxima, sums and partial outputs exist per head, and the indicator advances by
 // the MEAN of the heads' probabilities.
 // FEED: a producer warp keeps the rings full, for CTAs with several units and for grids beyond one CTA per SM.  Otherwise
@@ -200,7 +202,7 @@ __device__ __forceinline__ unsigned long long warp_min_key(unsigned long long ke
 template <int HD, bool WINDOWED, int GT, bool FEED>
 __global__ void __launch_bounds__(FEED ? DM_THREADS : WT, 2)
 decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, int independent, int G,
-                  int units, int state_in_smem, int part_in_ring, int split, int chunk, int nslot, int l2_rows, int B, int cap, int F, int R, int w, int norm,
+                  int units, int state_in_smem, int part_in_ring, int split, int chunk, int nslot, int B, int cap, int F, int R, int w, int norm,
                   float scale_log2, vatp_cache c,
                   const __nv_bfloat16* __restrict__ q_new, const __nv_bfloat16* __restrict__ k_new,
                   const __nv_bfloat16* __restrict__ v_new, __nv_bfloat16* __restrict__ out,
@@ -286,15 +288,6 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
     tma_load_3d(ring_base + (x * nslot + slot) * UNIT, is_v ? &tm_v : &tm_k, bar, 0,
                 u * cap + s0 + (x + MW * (is_v ? j - n : j)) * GROUP, 0);
   };
-  auto prefetch_rows = [&](bool v_rows) {    // one lane: the rows of the first unit that the rings do not hold yet, to L2
-    const int per_warp = 2 * ((ngroups + MW - 1) / MW);
-    const int held = (v_rows ? max(nslot - per_warp / 2, 0) : min(nslot, per_warp / 2)) * MW * GROUP;   // (about)
-    const int ahead = min(rows_alloc - held, l2_rows);
-    if (ahead > 0)
-      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;"
-                   ::"l"((const __nv_bfloat16*)(v_rows ? c.v_cache : c.k_cache) + (int64_t)(u0 * cap + s0 + held) * HD), "r"(ahead * HD * 2)
-                   : "memory");
-  };
   auto bring_state = [&](int u) {            // one lane: the per-slot state into shared memory, or on its way to L2
     const int t = WINDOWED ? c.next_pos[u] : 0;
     if (state_in_smem == 1) {
@@ -325,8 +318,6 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
     for (int j = 0; j < early; ++j) issue(lane, u0, j, na, j);
     __syncwarp();
     if (!independent) {
-      // A launch that waits has the time: the rows that the rings do not hold yet start on their way to L2.
-      if (l2_rows > 0 && (lane == MW || lane == MW + 1)) prefetch_rows(lane != MW);
       __syncwarp();
       // Nothing but K and V rows is read before the previous launch has completed and its writes are visible.
       asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -385,7 +376,6 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
     if (independent && tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (lane == 0)
       for (int j = 0; j < early_mine; ++j) issue(wid, u0, j, na_mine, j);
-    if (!independent && l2_rows > 0 && lane == 0 && wid < 2) prefetch_rows(wid == 1);
     __syncwarp();
   }
   if (!independent) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -426,6 +416,18 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   uint32_t state_par = 0;
 
   for (int u = u0; u < units; u += u_step) {
+  // everything the step needs of the unit is requested at once
+  uint4 new_raw = make_uint4(0u, 0u, 0u, 0u), last_raw = make_uint4(0u, 0u, 0u, 0u);
+  if (!FEED && has_chunk) new_raw = __ldg(reinterpret_cast<const uint4*>((lane < 16 ? k_new : v_new) + (int64_t)u * HD) + (lane & 15));
+  // B operand of K q^T: q in every column (grouped queries: column g carries head g of the unit's group, columns beyond the
+  // group repeat its last head)
+  const __nv_bfloat16* qn = GT > 1 ? q_new + ((int64_t)u * G + min(lane >> 2, G - 1)) * HD : q_new + (int64_t)u * HD;
+  uint32_t qb[HD / 16][2];
+#pragma unroll
+  for (int ks = 0; ks < HD / 16; ++ks) {
+    qb[ks][0] = __ldg(reinterpret_cast<const uint32_t*>(qn + ks * 16 + 2 * j4));
+    qb[ks][1] = __ldg(reinterpret_cast<const uint32_t*>(qn + ks * 16 + 8 + 2 * j4));
+  }
   const int len_m = c.len[u];
   const int fs_m = c.free_slot[u];
   const int t = c.next_pos[u];
@@ -444,23 +446,13 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   const int ls_local = ls - s0;          // row the previous step appended (its tile may predate that store)
   const bool owns_last = !independent && ls >= 0 && ls != fs && ls_local >= 0 && ls_local < cnt;
 
-  // A operand of q K^T: q replicated over the rows 0-7 of the tile (rows 8-15 zero)
-  // (grouped queries: row g of the tile carries head g of the unit's group; rows beyond the group repeat its last head)
-  const __nv_bfloat16* qn = GT > 1 ? q_new + ((int64_t)u * G + min(lane >> 2, G - 1)) * HD : q_new + (int64_t)u * HD;
-  uint32_t qa[HD / 16][2];
-#pragma unroll
-  for (int ks = 0; ks < HD / 16; ++ks) {
-    qa[ks][0] = __ldg(reinterpret_cast<const uint32_t*>(qn + ks * 16 + 2 * j4));
-    qa[ks][1] = __ldg(reinterpret_cast<const uint32_t*>(qn + ks * 16 + 8 + 2 * j4));
-  }
   // ---- the group that holds the incoming token's row: its warp stores the row and its norm (Eq. 4) and patches the
   // row into the tiles it streams; the group that holds the row of the previous step's token likewise re-reads that row.
   // Lanes 0-15 take 16 bytes of the K row each, lanes 16-31 of the V row (with head_dim 64 the first eight of each).
   const int new_warp = owns_new ? (fs_local / GROUP) % MW : -1, last_warp = owns_last ? (ls_local / GROUP) % MW : -1;
   // the new row's norm is needed by the thread that updates its slot
   const int norm_warp = owns_new ? (fs_local % WT) / 32 : -1;
-  uint4 new_raw = make_uint4(0u, 0u, 0u, 0u), last_raw = make_uint4(0u, 0u, 0u, 0u);
-  if (has_chunk && (wid == new_warp || wid == norm_warp))
+  if (FEED && has_chunk && (wid == new_warp || wid == norm_warp))
     new_raw = __ldg(reinterpret_cast<const uint4*>((lane < 16 ? k_new : v_new) + (int64_t)u * HD) + (lane & 15));
   if (has_chunk && wid == last_warp)
     last_raw = *(reinterpret_cast<const uint4*>((const __nv_bfloat16*)(lane < 16 ? c.k_cache : c.v_cache) +
@@ -494,11 +486,12 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
     last = early_mine + 2 * n;
     for (int i = early_mine; i > 0; --i) { arrived(); release(false); }
   }
-  float m_run = -INFINITY;                // of head lane / 4 (one head: the same in every lane)
+  float m_run[2] = {-INFINITY, -INFINITY};       // of heads 2 j4 and 2 j4 + 1 (one head: the same in every lane)
   for (int r0 = wid * GROUP; r0 < n * MW * GROUP; r0 += MW * GROUP) {
     const bool has_new = wid == new_warp && fs_local >= r0 && fs_local < r0 + GROUP;
     const bool has_last = wid == last_warp && ls_local >= r0 && ls_local < r0 + GROUP;
-    // S^T = q K^T, two n-tiles of 8 rows; c[0], c[1] = logits of rows 2 j4, 2 j4 + 1 of the tile
+    // S = K q^T: the rows are the A operand, as in the second phase (as the B operand they took two products of which half
+    // was padding)
     arrived();
     unsigned char* ks = my_ring + slot * UNIT;
     // the incoming token's row is not in the cache yet: patch it in
@@ -506,39 +499,38 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
     if (has_last) patch_row(ks, ls_local - r0, last_raw, false);
     if (has_new || has_last) __syncwarp();
     const uint32_t kaddr = smem_u32(ks) + row_off;
-    // all fragments first (one latency instead of one per step), then two chains per n-tile
+    // all fragments first (one latency instead of one per step), then two chains
     uint32_t bf[HD / 16][4];
 #pragma unroll
     for (int kk = 0; kk < HD / 16; ++kk) ldsm_x4(kaddr + (kk >> 2) * TILE_BYTES + ((lm_x ^ ((2 * kk) & 7)) << 4), bf[kk]);
-    float sa[2][4], sb[2][4];
+    float sa[2][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) sa[0][i] = sa[1][i] = sb[0][i] = sb[1][i] = 0.f;
+    for (int i = 0; i < 4; ++i) sa[0][i] = sa[1][i] = 0.f;
 #pragma unroll
-    for (int kk = 0; kk < HD / 16; ++kk) {
-      mma_bf16(sa[kk & 1], qa[kk][0], 0u, qa[kk][1], 0u, bf[kk][0], bf[kk][1]);
-      mma_bf16(sb[kk & 1], qa[kk][0], 0u, qa[kk][1], 0u, bf[kk][2], bf[kk][3]);
-    }
+    for (int kk = 0; kk < HD / 16; ++kk)
+      mma_bf16(sa[kk & 1], bf[kk][0], bf[kk][2], bf[kk][1], bf[kk][3], qb[kk][0], qb[kk][1]);
     release(has_new || has_last);
-    float s[4] = {(sa[0][0] + sa[1][0]) * scale_log2, (sa[0][1] + sa[1][1]) * scale_log2, (sb[0][0] + sb[1][0]) * scale_log2,
-                  (sb[0][1] + sb[1][1]) * scale_log2};
-    const int ra = r0 + 2 * j4, rb = ra + 8;      // this lane's rows: ra, ra + 1, rb, rb + 1
-    if (r0 + GROUP > cnt) {
-      if (ra >= cnt) s[0] = -INFINITY;
-      if (ra + 1 >= cnt) s[1] = -INFINITY;
-      if (rb >= cnt) s[2] = -INFINITY;
-      if (rb + 1 >= cnt) s[3] = -INFINITY;
+    // this lane: rows lane / 4 and lane / 4 + 8, heads 2 j4 and 2 j4 + 1 (one head: the same value in every column)
+    const int ra = r0 + (lane >> 2), rb = ra + 8;
+    const bool live_a = ra < cnt, live_b = rb < cnt;      // (chunk is a multiple of 16: dead rows of the last group have logits too, -inf)
+#pragma unroll
+    for (int x = 0; x < (GT > 1 ? 2 : 1); ++x) {
+      const float a = live_a ? (sa[0][x] + sa[1][x]) * scale_log2 : -INFINITY;
+      const float b = live_b ? (sa[0][2 + x] + sa[1][2 + x]) * scale_log2 : -INFINITY;
+      if (GT > 1 ? 2 * j4 + x < G : j4 == 0) {
+        float* lg = logit_s + (GT > 1 ? (2 * j4 + x) * chunk : 0);
+        lg[ra] = a;
+        lg[rb] = b;
+      }
+      m_run[x] = fmaxf(m_run[x], fmaxf(a, b));
     }
-    // (chunk is a multiple of 16: dead rows of the last group have logits too, -inf)
-    if (GT > 1 ? (lane >> 2) < G : lane < 4) {
-      float* lg = logit_s + (GT > 1 ? (lane >> 2) * chunk : 0);
-      *reinterpret_cast<float2*>(lg + ra) = make_float2(s[0], s[1]);
-      *reinterpret_cast<float2*>(lg + rb) = make_float2(s[2], s[3]);
-    }
-    m_run = fmaxf(m_run, fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3])));
   }
-  m_run = fmaxf(m_run, __shfl_xor_sync(0xffffffffu, m_run, 1));
-  m_run = fmaxf(m_run, __shfl_xor_sync(0xffffffffu, m_run, 2));
-  if (GT > 1 ? (j4 == 0 && (lane >> 2) < G) : lane == 0) part_m[wid][GT > 1 ? lane >> 2 : 0] = m_run;
+#pragma unroll
+  for (int x = 0; x < (GT > 1 ? 2 : 1); ++x) {
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) m_run[x] = fmaxf(m_run[x], __shfl_xor_sync(0xffffffffu, m_run[x], o));
+    if (GT > 1 ? lane < 4 && 2 * j4 + x < G : lane == 0) part_m[wid][GT > 1 ? 2 * j4 + x : 0] = m_run[x];
+  }
   // (The first time together with the producer warp: whoever finishes the step rewrites `len`, which every producer of the
   // unit must have read by then.)
   if (FEED && u == u0) asm volatile("bar.sync 2, %0;" ::"n"(WT + 32) : "memory");
@@ -547,37 +539,57 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   // launch's own rows by more than they gained).
   if (!FEED && !independent && tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // ---- exp2(s - m) of the CTA's slots, in place, and their sum (m: the CTA's maximum, finite when it has a live row)
-  for (int h = 0; h < g_rows; ++h) {
-    float m_c = -INFINITY;
+  if constexpr (GT == 1) {
+    float m_c = -INFINITY, l = 0.f;
 #pragma unroll
-    for (int k = 0; k < MW; ++k) m_c = fmaxf(m_c, part_m[k][h]);
-    float l = 0.f;
-    float* lg = logit_s + h * chunk;
+    for (int k = 0; k < MW; ++k) m_c = fmaxf(m_c, part_m[k][0]);
     for (int i = tid; i < (cnt + GROUP - 1) / GROUP * GROUP; i += WT) {
-      const float e = ex2(lg[i] - m_c);
-      lg[i] = e;
+      const float e = ex2(logit_s[i] - m_c);
+      logit_s[i] = e;
       l += e;
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    if (lane == 0) part_l[wid][h] = l;
+    if (lane == 0) part_l[wid][0] = l;
+  } else {
+    // warp x takes heads x, x + MW, ...; a lane every 32nd slot, four at a time
+    for (int h = wid; h < G; h += MW) {
+      float m_c = -INFINITY, l = 0.f;
+#pragma unroll
+      for (int k = 0; k < MW; ++k) m_c = fmaxf(m_c, part_m[k][h]);
+      float* lg = logit_s + h * chunk;
+      const int rows = (cnt + GROUP - 1) / GROUP * GROUP;
+#pragma unroll 4
+      for (int i = lane; i < rows; i += 32) {
+        const float e = ex2(lg[i] - m_c);
+        lg[i] = e;
+        l += e;
+      }
+#pragma unroll
+      for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+      if (lane == 0) { part_l[0][h] = l; part_m[0][h] = m_c; }      // (the CTA's: nobody else reads this head's maxima)
+    }
   }
   workers_sync();
   // ---- O^T += V^T p
   float o_acc[HD / 16][4];                // channels 16 i + lane / 4 (+ 8) x columns 2 j4, 2 j4 + 1 of O^T
 #pragma unroll
   for (int i = 0; i < HD / 16; ++i) { o_acc[i][0] = o_acc[i][1] = o_acc[i][2] = o_acc[i][3] = 0.f; }
-  const float* p_s = logit_s + (GT > 1 ? min(lane >> 2, G - 1) * chunk : 0) + 2 * j4;
+  // columns of the B operand: with up to four heads the high halves of p of head 0, 1, ... and then the remainders; with more
+  // a column per head, and two products
+  const bool two_halves = GT == 1 || G <= GT / 2;
+  const bool low_col = two_halves && (lane >> 2 & (GT == 1 ? 1 : GT / 2));
+  const int my_head = GT == 1 ? 0 : min(two_halves ? lane >> 2 & (GT / 2 - 1) : lane >> 2, G - 1);
+  const float* p_s = logit_s + my_head * chunk + 2 * j4;
   for (int r0 = wid * GROUP; r0 < n * MW * GROUP; r0 += MW * GROUP) {
     const bool has_new = wid == new_warp && fs_local >= r0 && fs_local < r0 + GROUP;
     const bool has_last = wid == last_warp && ls_local >= r0 && ls_local < r0 + GROUP;
     const float2 pa = *reinterpret_cast<const float2*>(p_s + r0), pb = *reinterpret_cast<const float2*>(p_s + r0 + 8);
-    // B operand of V^T p: the high bf16 half of p and the remainder - in the even and odd columns with one head, as two
-    // products otherwise (the columns are heads then)
+    // B operand of V^T p: the high bf16 half of p and the remainder
     const uint32_t hi0 = pack_bf16(pa.x, pa.y), hi1 = pack_bf16(pb.x, pb.y);
     const uint32_t lo0 = pack_bf16(pa.x - __uint_as_float(hi0 << 16), pa.y - __uint_as_float(hi0 & 0xffff0000u));
     const uint32_t lo1 = pack_bf16(pb.x - __uint_as_float(hi1 << 16), pb.y - __uint_as_float(hi1 & 0xffff0000u));
-    const uint32_t b0 = (GT == 1 && (lane & 4)) ? lo0 : hi0, b1 = (GT == 1 && (lane & 4)) ? lo1 : hi1;
+    const uint32_t b0 = low_col ? lo0 : hi0, b1 = low_col ? lo1 : hi1;
     arrived();
     unsigned char* vs = my_ring + slot * UNIT;
     if (has_new) patch_row(vs, fs_local - r0, new_raw, true);
@@ -595,7 +607,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
 #pragma unroll
     for (int nn = 0; nn < HD / 16; ++nn) {
       mma_bf16(o_acc[nn], af[nn][0], af[nn][1], af[nn][2], af[nn][3], b0, b1);
-      if (GT > 1) mma_bf16(o_acc[nn], af[nn][0], af[nn][1], af[nn][2], af[nn][3], lo0, lo1);
+      if (!two_halves) mma_bf16(o_acc[nn], af[nn][0], af[nn][1], af[nn][2], af[nn][3], lo0, lo1);
     }
     release(has_new || has_last || ragged);
   }
@@ -605,6 +617,11 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
     const int row = lane >> 2;
     __syncwarp();                         // (part_in_ring: every lane is past its last read of the ring)
     if constexpr (GT > 1) {
+      if (two_halves)
+#pragma unroll
+        for (int i = 0; i < HD / 16; ++i)
+#pragma unroll
+          for (int x = 0; x < 4; ++x) o_acc[i][x] += __shfl_xor_sync(0xffffffffu, o_acc[i][x], 2);
 #pragma unroll
       for (int i = 0; i < HD / 16; ++i) {
         if (2 * j4 < G) { po[2 * j4 * HD + 16 * i + row] = o_acc[i][0]; po[2 * j4 * HD + 16 * i + 8 + row] = o_acc[i][2]; }
@@ -626,25 +643,24 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
 
   // ---- CTA partial: max and sum to every CTA of the unit, channel slice r of the partial output to rank r ----
   const int slice = HD / split;           // channels a CTA of the unit sums up and writes
+  if (tid < split * g_rows) {
+    const int h = GT > 1 ? tid / split : 0, dst = GT > 1 ? tid - h * split : tid;
+    float m = part_m[0][h], l = part_l[0][h];
+    if (GT == 1) {
+#pragma unroll
+      for (int k = 1; k < MW; ++k) { m = fmaxf(m, part_m[k][0]); l += part_l[k][0]; }
+    }
+    if (split > 1) st_async2(map_rank(smem_u32(&ex_ml[rank][h]), dst), m, l, map_rank(smem_u32(ex_bar), dst));
+    else ex_ml[0][h] = make_float2(m, l);
+  }
   for (int i = tid; i < g_rows * HD; i += WT) {
     const int h = GT > 1 ? i / HD : 0, ch = GT > 1 ? i - h * HD : i;
-    float m_c = -INFINITY;
+    float a = 0.f;
 #pragma unroll
-    for (int k = 0; k < MW; ++k) m_c = fmaxf(m_c, part_m[k][h]);
-    float a = 0.f, l_c = 0.f;
-#pragma unroll
-    for (int k = 0; k < MW; ++k) {
-      l_c += part_l[k][h];
-      a += part_o[(size_t)k * part_ld + h * HD + ch];
-    }
+    for (int k = 0; k < MW; ++k) a += part_o[(size_t)k * part_ld + h * HD + ch];
     const int dst = ch / slice, off = (rank * g_rows + h) * slice + (ch - dst * slice);
-    if (split > 1) {
-      st_async(map_rank(smem_u32(&xo[off]), dst), a, map_rank(smem_u32(ex_bar), dst));
-      if (ch < split) st_async2(map_rank(smem_u32(&ex_ml[rank][h]), ch), m_c, l_c, map_rank(smem_u32(ex_bar), ch));
-    } else {
-      xo[off] = a;
-      if (ch == 0) ex_ml[0][h] = make_float2(m_c, l_c);
-    }
+    if (split > 1) st_async(map_rank(smem_u32(&xo[off]), dst), a, map_rank(smem_u32(ex_bar), dst));
+    else xo[off] = a;
   }
   if (split > 1) {
     if (!mbar_wait(ex_bar, 0)) bad = true;
@@ -656,21 +672,31 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   float m_all = -INFINITY, own_f = 0.f;    // own_f: this CTA's exp2(s - m) -> probability
   if constexpr (GT > 1) {
     if (tid < G) {         // one thread per head
-      float m_h = -INFINITY, L_h = 0.f;
-      for (int r = 0; r < split; ++r) m_h = fmaxf(m_h, ex_ml[r][tid].x);
-      for (int r = 0; r < split; ++r) {
-        const float f = ex_ml[r][tid].x > -INFINITY ? ex2(ex_ml[r][tid].x - m_h) : 0.f;
-        gq_fr[r][tid] = f;
-        L_h += ex_ml[r][tid].y * f;
+      float2 ml[MAX_SPLIT];
+      float m_h = -INFINITY, L_h = 0.f, own = 0.f;
+#pragma unroll
+      for (int r = 0; r < MAX_SPLIT; ++r) {
+        ml[r] = r < split ? ex_ml[r][tid] : make_float2(-INFINITY, 0.f);
+        m_h = fmaxf(m_h, ml[r].x);
       }
-      gq_invl[tid] = 1.f / L_h;
-      gq_f[tid] = gq_fr[rank][tid] * (1.f / L_h);       // this CTA's exp2(s - m) -> probability
+#pragma unroll
+      for (int r = 0; r < MAX_SPLIT; ++r) {
+        const float f = ml[r].x > -INFINITY ? ex2(ml[r].x - m_h) : 0.f;
+        gq_fr[r][tid] = f;
+        L_h += ml[r].y * f;
+        if (r == rank) own = f;
+      }
+      const float inv = 1.f / L_h;
+      gq_invl[tid] = inv;
+      gq_f[tid] = own * inv;                             // this CTA's exp2(s - m) -> probability
     }
     workers_sync();
     for (int i = tid; i < G * slice; i += WT) {
       const int h = i / slice, ch = i - h * slice;
       float a = 0.f;
-      for (int r = 0; r < split; ++r) a = fmaf(xo[(r * G + h) * slice + ch], gq_fr[r][h], a);
+#pragma unroll
+      for (int r = 0; r < MAX_SPLIT; ++r)
+        if (r < split) a = fmaf(xo[(r * G + h) * slice + ch], gq_fr[r][h], a);
       out[((int64_t)u * G + h) * HD + rank * slice + ch] = __float2bfloat16(a * gq_invl[h]);
     }
   } else {
@@ -709,7 +735,9 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
       float p;
       if constexpr (GT > 1) {      // the mean of the heads' probabilities
         float a = 0.f;
-        for (int h = 0; h < G; ++h) a = fmaf(lg[h * chunk + i], gq_f[h], a);
+#pragma unroll
+        for (int h = 0; h < GT; ++h)
+          if (h < G) a = fmaf(lg[h * chunk + i], gq_f[h], a);
         p = a / (float)G;
       } else {
         p = lg[i] * own_f;
@@ -968,8 +996,8 @@ cudaError_t launch_hd(const Shape& s, int B, int F, int R, const vatp_cache& c, 
                        {win ? (const char*)c.ring : nullptr, win ? slots * s.window * 4 : 0},
                        {win ? (const char*)c.acc_fixed : nullptr, win ? slots * 8 : 0},
                        {(const char*)q, units * G * ROW_BYTES}, {(const char*)k, units * ROW_BYTES}, {(const char*)v, units * ROW_BYTES}};
-  // One CTA per SM at most: no producer warp (see the kernel; 32 units x 2049 slots 10.4 us per waiting step against 12.7
-  // with one).  Beyond that it pays (512 units x 1025 slots with a history window 57 us against 79).
+  // One CTA per SM at most: no producer warp (see the kernel; 32 units x 2049 slots 10.3 us per waiting step against 12.7
+  // with one).  Beyond that it pays (512 units x 1025 slots with a history window 55 us against 79).
   const bool feed = grid > sms;
   auto kern = feed ? (grouped ? (win ? decode_mma_kernel<HD, true, GQ_HEADS, true> : decode_mma_kernel<HD, false, GQ_HEADS, true>)
                               : (win ? decode_mma_kernel<HD, true, 1, true> : decode_mma_kernel<HD, false, 1, true>))
@@ -980,10 +1008,6 @@ cudaError_t launch_hd(const Shape& s, int B, int F, int R, const vatp_cache& c, 
   // share of the machine this launch holds while resident (every CTA waits for the previous launch before it retires)
   const double share = (double)grid / ((double)(dyn <= half_sm ? 2 : 1) * sms);
   const int independent = independent_of_in_flight(st, capture_of(st), may_overlap, written, 16, written, share, share) ? 1 : 0;
-  // Rows of K (and of V) that a waiting CTA asks for in L2 ahead of its wait: all it has, as long as a launch's rows take
-  // no more than a third of the 126 MB.
-  const int64_t l2_most = ((int64_t)40 << 20) / ((int64_t)s.units * split * 2 * ROW_BYTES);
-  const int l2_rows = (int)(l2_most < chunk ? l2_most : chunk);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(feed ? DM_THREADS : WT);
@@ -998,7 +1022,7 @@ cudaError_t launch_hd(const Shape& s, int B, int F, int R, const vatp_cache& c, 
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, kern, tm_k, tm_v, independent, G, s.units, state_in_smem, (int)part_in_ring, split, chunk, nslot, l2_rows, B, cap, F, R, s.window,
+  return cudaLaunchKernelEx(&cfg, kern, tm_k, tm_v, independent, G, s.units, state_in_smem, (int)part_in_ring, split, chunk, nslot, B, cap, F, R, s.window,
                             s.norm, s.scale * LOG2E, c, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v,
                             (__nv_bfloat16*)out, evicted, dev_status);
 }

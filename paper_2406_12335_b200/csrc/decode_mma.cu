@@ -484,6 +484,9 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   if (u == u0 && n != na_mine) {          // rows requested before the live range was known: dropped (see the producer)
     base = early_mine;
     last = early_mine + 2 * n;
+    if (!FEED && lane == 0)               // (slots the early requests left free)
+      for (int j = early_mine; j < min(nslot, last); ++j) issue(wid, u0, j - base, n, j);
+    __syncwarp();
     for (int i = early_mine; i > 0; --i) { arrived(); release(false); }
   }
   float m_run[2] = {-INFINITY, -INFINITY};       // of heads 2 j4 and 2 j4 + 1 (one head: the same in every lane)

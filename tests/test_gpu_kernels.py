@@ -43,6 +43,7 @@ def test_head_dim_64_window_leaves_earlier_normalisers_alone():
     (1, 3, 0, 128, 1, 0),        # one slot besides the incoming token's
     (1, 3, 0, 128, 127, 0),      # ring of fewer units than slots
     (2, 60, 0, 128, 200, 0),     # 120 units: one CTA each, requests by the warps themselves
+    (2, 60, 0, 64, 300, 0),      # rings deeper than some warps' rows
     (3, 100, 0, 128, 130, 0),    # 300 units: more than two CTAs per SM hold, the producer warp goes on to a second unit
     (3, 100, 0, 64, 130, 40),    # the same with head_dim 64 and a history window (the state of the next unit is fetched early)
     (5, 8, 2, 128, 600, 0),      # grouped queries split over a cluster
@@ -50,7 +51,7 @@ def test_head_dim_64_window_leaves_earlier_normalisers_alone():
     (1, 2, 0, 128, 9000, 0),     # state beyond shared memory
     (1, 300, 0, 128, 2048, 30),  # several units per CTA, their state read from global memory in the tail
 ])
-@pytest.mark.parametrize("grow", [0, 5])
+@pytest.mark.parametrize("grow", [0, 5, 190])
 def test_decode_step_against_float64(b, h, kv, d, B, window, grow):
     """One-step arithmetic of every unit against float64 torch: output rows, indicators, evicted token; grow: the cache
     starts that many tokens short of its budget, so rows requested before the live range is known are dropped."""

@@ -42,10 +42,9 @@
 //   * grouped-query attention (several query heads share one cache; the paper leaves the case open and points at
 //     a group-wise score, read here as the MEAN of the heads' probabilities): up to eight heads of a group ride
 //     in the columns of the products (template parameter GT), so a K or V row is still read once per step.
-// Measured (us per step, before and after the two phases, the exchange by st.async, the co-resident successor and the rows as
-// A operand): 32 units x 2049 slots, every launch waiting 12.5 -> 10.3; 256 units x 1639, launches overlapping 38 -> 34.4
-// (215 MB: 6.2 TB/s of the 6.56 a copy reaches); 512 units x 1025 with a history window 73 -> 55; 8 units x 2049, four heads
-// each 11.0 -> 9.3 (exponentials a warp per head, the ranks' factors unrolled, one product per group for up to four heads).
+// Measured (us per step, first and latest version): 32 units x 2049 slots, every launch waiting 12.5 -> 9.6; 256 units x
+// 1639, launches overlapping 38 -> 34.2 (215 MB: 6.3 TB/s of the 6.56 a copy reaches); 512 units x 1025 with a history window
+// 73 -> 55; 8 units x 2049, four heads each 11.0 -> 8.9.
 #include <cooperative_groups.h>
 
 #include <mutex>
@@ -78,16 +77,16 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)_
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
 // the same without suspending the warp (its other lanes have barriers of their own to look at)
@@ -106,7 +105,7 @@ __device__ __forceinline__ uint64_t global_ns() {
   return t;
 }
 // Bounded wait (about one second): false when the copy never signalled.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
   if (mbar_try_wait(bar, parity)) return true;
   const uint64_t t0 = global_ns();
   while (!mbar_try_wait(bar, parity))
@@ -120,11 +119,14 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
                "l"(src), "r"(bytes), "r"(smem_u32(bar))
                : "memory");
 }
-__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1, int c2) {
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2) {
   asm volatile(
       "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-      ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2)
+      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
       : "memory");
+}
+__device__ __forceinline__ void st_shared16(uint32_t addr, const uint4& v) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 // address of `addr` (this CTA's shared memory) in CTA `rank` of the cluster
 __device__ __forceinline__ uint32_t map_rank(uint32_t addr, int rank) {
@@ -169,6 +171,12 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+__device__ __forceinline__ float warp_max(float x) {
+  float y;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(y) : "f"(x));
   return y;
 }
 
@@ -237,7 +245,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
 
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = split > 1 ? (int)cluster.block_rank() : 0;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, wid = __shfl_sync(0xffffffffu, tid >> 5, 0);    // (wid: the same in every lane)
   const int j4 = lane & 3;
   uint64_t* state_full = &misc_bars[0];
   uint64_t* state_empty = &misc_bars[1];
@@ -248,7 +256,6 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   // its slot range inside a unit's allocation
   const int s0 = min(rank * chunk, cap);
   const int rows_alloc = min(chunk, cap - s0);
-  const int ngroups = (rows_alloc + GROUP - 1) / GROUP;
   // Warp x's groups are x, x + MW, ...: as many as groups_of(x, rows) among the first `rows` rows.  Its units in order: the
   // K rows of its groups, then their V rows.  A launch requests the first units of its first unit (sequence, head) before
   // it may read how many rows are live; when fewer are than the allocation holds, those are dropped and the live ones
@@ -256,7 +263,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   auto groups_of = [](int x, int rows) { return x * GROUP < rows ? (rows - x * GROUP + MW * GROUP - 1) / (MW * GROUP) : 0; };
   auto copy_state = [&](int u, int t) {            // one thread: the per-slot state of this CTA's slots
     const int64_t o = (int64_t)u * cap + s0;
-    mbar_expect_tx(state_full, (WINDOWED ? 20u : 12u) * rows_alloc);
+    mbar_expect_tx(smem_u32(state_full), (WINDOWED ? 20u : 12u) * rows_alloc);
     bulk_g2s(acc_s, WINDOWED ? c.ring + ((int64_t)u * w + (t % w)) * cap + s0 : c.acc + o, rows_alloc * 4, state_full);
     bulk_g2s(vn_s, c.vnorm + o, rows_alloc * 4, state_full);
     bulk_g2s(pos_s, c.pos + o, rows_alloc * 4, state_full);
@@ -274,18 +281,18 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
     mbar_init(cand_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     if (split > 1) {
-      mbar_expect_tx(ex_bar, (uint32_t)(8 * g_rows * split + 4 * g_rows * HD));
-      if (rank == 0) mbar_expect_tx(cand_bar, (uint32_t)(split * sizeof(Candidate)));
+      mbar_expect_tx(smem_u32(ex_bar), (uint32_t)(8 * g_rows * split + 4 * g_rows * HD));
+      if (rank == 0) mbar_expect_tx(smem_u32(cand_bar), (uint32_t)(split * sizeof(Candidate)));
     }
   }
   __syncthreads();
   if (split > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 
   auto issue = [&](int x, int u, int j, int n, int slot) {    // one lane: unit j of n groups into ring slot `slot` of warp x
-    uint64_t* bar = &full[x * MAX_SLOTS + slot];
+    const uint32_t bar = smem_u32(&full[x * MAX_SLOTS + slot]);
     mbar_expect_tx(bar, UNIT);
     const bool is_v = j >= n;
-    tma_load_3d(ring_base + (x * nslot + slot) * UNIT, is_v ? &tm_v : &tm_k, bar, 0,
+    tma_load_3d(smem_u32(ring_base) + (x * nslot + slot) * UNIT, is_v ? &tm_v : &tm_k, bar, 0,
                 u * cap + s0 + (x + MW * (is_v ? j - n : j)) * GROUP, 0);
   };
   auto bring_state = [&](int u) {            // one lane: the per-slot state into shared memory, or on its way to L2
@@ -378,13 +385,21 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
       for (int j = 0; j < early_mine; ++j) issue(wid, u0, j, na_mine, j);
     __syncwarp();
   }
+  // (their values are read after the wait; on their way to L2 meanwhile, since a layer's words have long left it)
+  if (!FEED && !independent && tid < 4) {
+    const int32_t* words = tid == 0 ? c.len : tid == 1 ? c.free_slot : tid == 2 ? c.next_pos : c.last_slot;
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(words + u0));
+  }
   if (!independent) asm volatile("griddepcontrol.wait;" ::: "memory");
   if (!FEED && tid == 32 && rows_alloc > 0 && state_in_smem != 2) bring_state(u0);
-  uint64_t* my_full = &full[wid * MAX_SLOTS];
-  uint64_t* my_empty = &empty[wid * MAX_SLOTS];
-  unsigned char* my_ring = ring_base + (size_t)wid * nslot * UNIT;
-  int slot = 0, par = 0;                  // ring position of the next unit this warp consumes
-  int at = 0, last = 2 * na_mine, base = 0, n = na_mine;   // !FEED: its number, how many there are, those dropped, live groups
+  const uint32_t full_a = smem_u32(&full[wid * MAX_SLOTS]), empty_a = smem_u32(&empty[wid * MAX_SLOTS]);
+  const uint32_t ring_a = smem_u32(ring_base + (size_t)wid * nslot * UNIT);
+  uint32_t slot = 0, unit_a = ring_a, par = 0;     // ring position of the next unit this warp consumes
+  int n = na_mine;                        // live groups
+  // !FEED: the units still to be requested, those of K among them, the next one's row
+  const int row0 = u0 * cap + s0 + wid * GROUP;
+  int to_request = 2 * na_mine - early_mine, k_left = max(na_mine - early_mine, 0);
+  int next_row = row0 + (early_mine < na_mine ? early_mine : early_mine - na_mine) * (MW * GROUP);
   bool bad = false;                       // this lane's wait ran out: it no longer waits, the results are void
   // ldmatrix lane addressing: matrix i = lane / 8, row r = lane % 8.  A tile row is 128 bytes and its
   // 16-byte chunk c sits at position c ^ (row % 8).
@@ -392,31 +407,44 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   //   V (trans):  matrices (rows 0-7, ch lo), (rows 0-7, ch hi), (rows 8-15, ch lo), (rows 8-15, ch hi): the A operand V^T
   const uint32_t row_off = (uint32_t)(((lane >> 4) * 8 + (lane & 7)) * 128), lm_x = (uint32_t)(((lane >> 3) & 1) ^ (lane & 7));
   auto arrived = [&]() {                  // the next unit is complete
-    if (!bad && !mbar_wait(&my_full[slot], par)) bad = true;
+    const uint32_t bar = full_a + 8 * slot;
+    if (!mbar_try_wait(bar, par) && !bad && !mbar_wait(bar, par)) bad = true;
     __syncwarp();
   };
-  auto release = [&](bool wrote) {        // this warp has read it: the slot may be filled again
+  auto request = [&](uint32_t bar, uint32_t dst) {       // the next unit of this warp
+    if (lane == 0 && !bad) {
+      mbar_expect_tx(bar, UNIT);
+      tma_load_3d(dst, k_left > 0 ? &tm_k : &tm_v, bar, 0, next_row, 0);
+    }
+    --to_request;
+    next_row = --k_left == 0 ? row0 : next_row + MW * GROUP;
+  };
+  auto release = [&](bool wrote) {        // this warp has read it: its slot may be filled again
     // generic-proxy stores into the slot must be ordered before the next bulk copy into it
     if (wrote) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncwarp();
     if (FEED) {
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&my_empty[slot])) : "memory");
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(empty_a + 8 * slot) : "memory");
     } else {
-      if (lane == 0 && !bad && at + nslot < last) issue(wid, u0, at + nslot - base, n, slot);
-      ++at;
+      if (to_request > 0) request(full_a + 8 * slot, unit_a);
     }
-    if (++slot == nslot) { slot = 0; par ^= 1; }
+    unit_a += UNIT;
+    if (++slot == nslot) { slot = 0; unit_a = ring_a; par ^= 1; }
   };
   const bool has_chunk = (lane & 15) < ROW_CHUNKS;
-  auto patch_row = [&](unsigned char* tile, int rr, const uint4& raw, bool v_half) {
+  auto patch_row = [&](uint32_t tile, int rr, const uint4& raw, bool v_half) {
     const int ch = lane & 15;
     if (has_chunk && (lane >= 16) == v_half)
-      *reinterpret_cast<uint4*>(tile + (ch >> 3) * TILE_BYTES + rr * 128 + (((ch & 7) ^ (rr & 7)) << 4)) = raw;
+      st_shared16(tile + (ch >> 3) * TILE_BYTES + rr * 128 + (((ch & 7) ^ (rr & 7)) << 4), raw);
   };
   uint32_t state_par = 0;
 
   for (int u = u0; u < units; u += u_step) {
   // everything the step needs of the unit is requested at once
+  const int len_m = c.len[u];
+  const int fs_m = c.free_slot[u];
+  const int t = c.next_pos[u];
+  const int ls_m = c.last_slot[u];
   uint4 new_raw = make_uint4(0u, 0u, 0u, 0u), last_raw = make_uint4(0u, 0u, 0u, 0u);
   if (!FEED && has_chunk) new_raw = __ldg(reinterpret_cast<const uint4*>((lane < 16 ? k_new : v_new) + (int64_t)u * HD) + (lane & 15));
   // B operand of K q^T: q in every column (grouped queries: column g carries head g of the unit's group, columns beyond the
@@ -428,10 +456,6 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
     qb[ks][0] = __ldg(reinterpret_cast<const uint32_t*>(qn + ks * 16 + 2 * j4));
     qb[ks][1] = __ldg(reinterpret_cast<const uint32_t*>(qn + ks * 16 + 8 + 2 * j4));
   }
-  const int len_m = c.len[u];
-  const int fs_m = c.free_slot[u];
-  const int t = c.next_pos[u];
-  const int ls_m = c.last_slot[u];
 #ifdef VATP_DEBUG_BOUNDS
   // the state words come from memory: out of range they are clamped and reported (every access below stays inside)
   (void)(VATP_INB(len_m, cap, dev_status) && VATP_INB(fs_m, cap, dev_status) && VATP_INB(ls_m + 1, cap + 1, dev_status));
@@ -458,23 +482,26 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
     last_raw = *(reinterpret_cast<const uint4*>((const __nv_bfloat16*)(lane < 16 ? c.k_cache : c.v_cache) +
                                                 ((int64_t)u * cap + ls) * HD) + (lane & 15));
   float new_norm = 0.f;
-  if (wid == new_warp || wid == norm_warp) {
-    const uint32_t wv[4] = {new_raw.x, new_raw.y, new_raw.z, new_raw.w};
+  auto incoming = [&]() {
+    if (wid == new_warp || wid == norm_warp) {
+      const uint32_t wv[4] = {new_raw.x, new_raw.y, new_raw.z, new_raw.w};
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      new_norm = norm_fold(norm, norm_fold(norm, new_norm, __uint_as_float(wv[i] << 16)), __uint_as_float(wv[i] & 0xffff0000u));
+      for (int i = 0; i < 4; ++i)
+        new_norm = norm_fold(norm, norm_fold(norm, new_norm, __uint_as_float(wv[i] << 16)), __uint_as_float(wv[i] & 0xffff0000u));
 #pragma unroll
-    for (int o = 8; o; o >>= 1) new_norm = norm_merge(norm, new_norm, __shfl_xor_sync(0xffffffffu, new_norm, o));
-    new_norm = norm_finish(norm, __shfl_sync(0xffffffffu, new_norm, 16));      // the V half's partial
-    if (wid == new_warp) {
-      __nv_bfloat16* dst = (__nv_bfloat16*)(lane < 16 ? c.k_cache : c.v_cache) + ((int64_t)u * cap + fs) * HD;
-      if (has_chunk) reinterpret_cast<uint4*>(dst)[lane & 15] = new_raw;
-      if (lane == 0) {
-        c.vnorm[(int64_t)u * cap + fs] = new_norm;
-        c.pos[(int64_t)u * cap + fs] = t;
+      for (int o = 8; o; o >>= 1) new_norm = norm_merge(norm, new_norm, __shfl_xor_sync(0xffffffffu, new_norm, o));
+      new_norm = norm_finish(norm, __shfl_sync(0xffffffffu, new_norm, 16));      // the V half's partial
+      if (wid == new_warp) {
+        __nv_bfloat16* dst = (__nv_bfloat16*)(lane < 16 ? c.k_cache : c.v_cache) + ((int64_t)u * cap + fs) * HD;
+        if (has_chunk) reinterpret_cast<uint4*>(dst)[lane & 15] = new_raw;
+        if (lane == 0) {
+          c.vnorm[(int64_t)u * cap + fs] = new_norm;
+          c.pos[(int64_t)u * cap + fs] = t;
+        }
       }
     }
-  }
+  };
+  if (FEED) incoming();                   // (otherwise while the unit's CTAs exchange)
 
   // ---- stream the rows: first all K rows (logits), then, with the CTA's maximum known, all V rows.  In one sweep with an
   // online softmax every 16-row group was a chain of ~2300 cycles (fragments, products, maximum, exponentials, fragments,
@@ -482,44 +509,63 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   // are taken once per slot instead of once per lane of an MMA tile.
   n = groups_of(wid, cnt);                // this warp's live groups
   if (u == u0 && n != na_mine) {          // rows requested before the live range was known: dropped (see the producer)
-    base = early_mine;
-    last = early_mine + 2 * n;
-    if (!FEED && lane == 0)               // (slots the early requests left free)
-      for (int j = early_mine; j < min(nslot, last); ++j) issue(wid, u0, j - base, n, j);
-    __syncwarp();
+    if (!FEED) {
+      to_request = 2 * n;
+      k_left = n;
+      next_row = row0;
+      for (int j = early_mine; j < nslot && to_request > 0; ++j) request(full_a + 8 * j, ring_a + j * UNIT);     // (slots left free)
+    }
     for (int i = early_mine; i > 0; --i) { arrived(); release(false); }
   }
+  // The loops of both phases are software pipelined: a warp waits for its next group and requests its fragments while the
+  // products of this one are under way.  (One group after the other was 950 cycles each of waits, fragments, products and
+  // requests in turn; two groups at a
+  // time found the rings, three units deep, empty.  What counts is the number of instructions: ring addresses and requests
+  // kept as counters, edge cases behind one test per group: 32 units x 2049 slots 10.1 -> 9.7 us per step.)
+  constexpr int RSTEP = MW * GROUP;       // rows from one group of a warp to its next
+  const int r_end = n * RSTEP;
   float m_run[2] = {-INFINITY, -INFINITY};       // of heads 2 j4 and 2 j4 + 1 (one head: the same in every lane)
-  for (int r0 = wid * GROUP; r0 < n * MW * GROUP; r0 += MW * GROUP) {
-    const bool has_new = wid == new_warp && fs_local >= r0 && fs_local < r0 + GROUP;
-    const bool has_last = wid == last_warp && ls_local >= r0 && ls_local < r0 + GROUP;
-    // S = K q^T: the rows are the A operand, as in the second phase (as the B operand they took two products of which half
-    // was padding)
+  uint32_t frag[HD / 16][4];              // a group's rows as the A operand
+  bool wrote = false;
+  const bool patches = wid == new_warp || wid == last_warp;
+  // S = K q^T: the rows are the A operand, as in the second phase (as the B operand they took two products of which half
+  // was padding)
+  auto k_fetch = [&](int r0) {
     arrived();
-    unsigned char* ks = my_ring + slot * UNIT;
-    // the incoming token's row is not in the cache yet: patch it in
-    if (has_new) patch_row(ks, fs_local - r0, new_raw, false);
-    if (has_last) patch_row(ks, ls_local - r0, last_raw, false);
-    if (has_new || has_last) __syncwarp();
-    const uint32_t kaddr = smem_u32(ks) + row_off;
-    // all fragments first (one latency instead of one per step), then two chains
-    uint32_t bf[HD / 16][4];
+    wrote = false;
+    if (patches) {                        // the incoming token's row is not in the cache yet: patch it in
+      const bool has_new = wid == new_warp && fs_local >= r0 && fs_local < r0 + GROUP;
+      const bool has_last = wid == last_warp && ls_local >= r0 && ls_local < r0 + GROUP;
+      if (has_new) patch_row(unit_a, fs_local - r0, new_raw, false);
+      if (has_last) patch_row(unit_a, ls_local - r0, last_raw, false);
+      wrote = has_new || has_last;
+      __syncwarp();
+    }
+    const uint32_t kaddr = unit_a + row_off;
 #pragma unroll
-    for (int kk = 0; kk < HD / 16; ++kk) ldsm_x4(kaddr + (kk >> 2) * TILE_BYTES + ((lm_x ^ ((2 * kk) & 7)) << 4), bf[kk]);
+    for (int kk = 0; kk < HD / 16; ++kk) ldsm_x4(kaddr + (kk >> 2) * TILE_BYTES + ((lm_x ^ ((2 * kk) & 7)) << 4), frag[kk]);
+  };
+  if (!FEED && n > 0) k_fetch(wid * GROUP);
+  for (int r0 = wid * GROUP; r0 < r_end; r0 += RSTEP) {
+    if (FEED) k_fetch(r0);
     float sa[2][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) sa[0][i] = sa[1][i] = 0.f;
 #pragma unroll
     for (int kk = 0; kk < HD / 16; ++kk)
-      mma_bf16(sa[kk & 1], bf[kk][0], bf[kk][2], bf[kk][1], bf[kk][3], qb[kk][0], qb[kk][1]);
-    release(has_new || has_last);
+      mma_bf16(sa[kk & 1], frag[kk][0], frag[kk][2], frag[kk][1], frag[kk][3], qb[kk][0], qb[kk][1]);
+    release(wrote);
+    if (!FEED && r0 + RSTEP < r_end) k_fetch(r0 + RSTEP);
     // this lane: rows lane / 4 and lane / 4 + 8, heads 2 j4 and 2 j4 + 1 (one head: the same value in every column)
     const int ra = r0 + (lane >> 2), rb = ra + 8;
-    const bool live_a = ra < cnt, live_b = rb < cnt;      // (chunk is a multiple of 16: dead rows of the last group have logits too, -inf)
+    const bool ragged = r0 + GROUP > cnt;      // (chunk is a multiple of 16: dead rows of the last group have logits too, -inf)
 #pragma unroll
     for (int x = 0; x < (GT > 1 ? 2 : 1); ++x) {
-      const float a = live_a ? (sa[0][x] + sa[1][x]) * scale_log2 : -INFINITY;
-      const float b = live_b ? (sa[0][2 + x] + sa[1][2 + x]) * scale_log2 : -INFINITY;
+      float a = (sa[0][x] + sa[1][x]) * scale_log2, b = (sa[0][2 + x] + sa[1][2 + x]) * scale_log2;
+      if (ragged) {
+        if (ra >= cnt) a = -INFINITY;
+        if (rb >= cnt) b = -INFINITY;
+      }
       if (GT > 1 ? 2 * j4 + x < G : j4 == 0) {
         float* lg = logit_s + (GT > 1 ? (2 * j4 + x) * chunk : 0);
         lg[ra] = a;
@@ -530,8 +576,12 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   }
 #pragma unroll
   for (int x = 0; x < (GT > 1 ? 2 : 1); ++x) {
+    if (GT == 1) {
+      m_run[x] = warp_max(m_run[x]);
+    } else {
 #pragma unroll
-    for (int o = 4; o < 32; o <<= 1) m_run[x] = fmaxf(m_run[x], __shfl_xor_sync(0xffffffffu, m_run[x], o));
+      for (int o = 4; o < 32; o <<= 1) m_run[x] = fmaxf(m_run[x], __shfl_xor_sync(0xffffffffu, m_run[x], o));
+    }
     if (GT > 1 ? lane < 4 && 2 * j4 + x < G : lane == 0) part_m[wid][GT > 1 ? 2 * j4 + x : 0] = m_run[x];
   }
   // (The first time together with the producer warp: whoever finishes the step rewrites `len`, which every producer of the
@@ -578,41 +628,50 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   float o_acc[HD / 16][4];                // channels 16 i + lane / 4 (+ 8) x columns 2 j4, 2 j4 + 1 of O^T
 #pragma unroll
   for (int i = 0; i < HD / 16; ++i) { o_acc[i][0] = o_acc[i][1] = o_acc[i][2] = o_acc[i][3] = 0.f; }
-  // columns of the B operand: with up to four heads the high halves of p of head 0, 1, ... and then the remainders; with more
-  // a column per head, and two products
+  // columns of the B operand: with up to four heads the high bf16 halves of p of head 0, 1, ... and then the remainders; with
+  // more a column per head, and two products
   const bool two_halves = GT == 1 || G <= GT / 2;
   const bool low_col = two_halves && (lane >> 2 & (GT == 1 ? 1 : GT / 2));
   const int my_head = GT == 1 ? 0 : min(two_halves ? lane >> 2 & (GT / 2 - 1) : lane >> 2, G - 1);
   const float* p_s = logit_s + my_head * chunk + 2 * j4;
-  for (int r0 = wid * GROUP; r0 < n * MW * GROUP; r0 += MW * GROUP) {
-    const bool has_new = wid == new_warp && fs_local >= r0 && fs_local < r0 + GROUP;
-    const bool has_last = wid == last_warp && ls_local >= r0 && ls_local < r0 + GROUP;
+  uint32_t b0, b1, lo0, lo1;
+  auto v_fetch = [&](int r0) {
     const float2 pa = *reinterpret_cast<const float2*>(p_s + r0), pb = *reinterpret_cast<const float2*>(p_s + r0 + 8);
+    arrived();
+    const bool ragged = cnt < r0 + GROUP;
+    wrote = ragged;
+    if (patches || ragged) {
+      const bool has_new = wid == new_warp && fs_local >= r0 && fs_local < r0 + GROUP;
+      const bool has_last = wid == last_warp && ls_local >= r0 && ls_local < r0 + GROUP;
+      if (has_new) patch_row(unit_a, fs_local - r0, new_raw, true);
+      if (has_last) patch_row(unit_a, ls_local - r0, last_raw, true);
+      // rows beyond the live range must not reach the product (their probability is 0, but 0 * garbage need not be 0)
+      if (ragged)
+        for (int rr = cnt - r0 + (lane >> 4); rr < GROUP && has_chunk; rr += 2)
+          st_shared16(unit_a + ((lane >> 3) & 1) * TILE_BYTES + rr * 128 + ((lane & 7) << 4), make_uint4(0u, 0u, 0u, 0u));
+      wrote = has_new || has_last || ragged;
+      __syncwarp();
+    }
+    const uint32_t vaddr = unit_a + row_off;
+#pragma unroll
+    for (int nn = 0; nn < HD / 16; ++nn) ldsm_x4_t(vaddr + (nn >> 2) * TILE_BYTES + ((lm_x ^ ((2 * nn) & 7)) << 4), frag[nn]);
     // B operand of V^T p: the high bf16 half of p and the remainder
     const uint32_t hi0 = pack_bf16(pa.x, pa.y), hi1 = pack_bf16(pb.x, pb.y);
-    const uint32_t lo0 = pack_bf16(pa.x - __uint_as_float(hi0 << 16), pa.y - __uint_as_float(hi0 & 0xffff0000u));
-    const uint32_t lo1 = pack_bf16(pb.x - __uint_as_float(hi1 << 16), pb.y - __uint_as_float(hi1 & 0xffff0000u));
-    const uint32_t b0 = low_col ? lo0 : hi0, b1 = low_col ? lo1 : hi1;
-    arrived();
-    unsigned char* vs = my_ring + slot * UNIT;
-    if (has_new) patch_row(vs, fs_local - r0, new_raw, true);
-    if (has_last) patch_row(vs, ls_local - r0, last_raw, true);
-    const bool ragged = cnt < r0 + GROUP;
-    // rows beyond the live range must not reach the product (their probability is 0, but 0 * garbage need not be 0)
-    if (ragged)
-      for (int rr = cnt - r0 + (lane >> 4); rr < GROUP && has_chunk; rr += 2)
-        *reinterpret_cast<uint4*>(vs + ((lane >> 3) & 1) * TILE_BYTES + rr * 128 + ((lane & 7) << 4)) = make_uint4(0u, 0u, 0u, 0u);
-    if (has_new || has_last || ragged) __syncwarp();
-    const uint32_t vaddr = smem_u32(vs) + row_off;
-    uint32_t af[HD / 16][4];
-#pragma unroll
-    for (int nn = 0; nn < HD / 16; ++nn) ldsm_x4_t(vaddr + (nn >> 2) * TILE_BYTES + ((lm_x ^ ((2 * nn) & 7)) << 4), af[nn]);
+    lo0 = pack_bf16(pa.x - __uint_as_float(hi0 << 16), pa.y - __uint_as_float(hi0 & 0xffff0000u));
+    lo1 = pack_bf16(pb.x - __uint_as_float(hi1 << 16), pb.y - __uint_as_float(hi1 & 0xffff0000u));
+    b0 = low_col ? lo0 : hi0;
+    b1 = low_col ? lo1 : hi1;
+  };
+  if (!FEED && n > 0) v_fetch(wid * GROUP);
+  for (int r0 = wid * GROUP; r0 < r_end; r0 += RSTEP) {
+    if (FEED) v_fetch(r0);
 #pragma unroll
     for (int nn = 0; nn < HD / 16; ++nn) {
-      mma_bf16(o_acc[nn], af[nn][0], af[nn][1], af[nn][2], af[nn][3], b0, b1);
-      if (!two_halves) mma_bf16(o_acc[nn], af[nn][0], af[nn][1], af[nn][2], af[nn][3], lo0, lo1);
+      mma_bf16(o_acc[nn], frag[nn][0], frag[nn][1], frag[nn][2], frag[nn][3], b0, b1);
+      if (!two_halves) mma_bf16(o_acc[nn], frag[nn][0], frag[nn][1], frag[nn][2], frag[nn][3], lo0, lo1);
     }
-    release(has_new || has_last || ragged);
+    release(wrote);
+    if (!FEED && r0 + RSTEP < r_end) v_fetch(r0 + RSTEP);
   }
   // ---- the warp's partial
   {
@@ -645,7 +704,8 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   if (!part_in_ring && state_in_smem == 2 && tid == 32 && rows_alloc > 0) copy_state(u, t);
 
   // ---- CTA partial: max and sum to every CTA of the unit, channel slice r of the partial output to rank r ----
-  const int slice = HD / split;           // channels a CTA of the unit sums up and writes
+  const int slice = HD / split;           // channels a CTA of the unit sums up and writes (a power of two)
+  const int slice_log2 = 31 - __clz(slice);
   if (tid < split * g_rows) {
     const int h = GT > 1 ? tid / split : 0, dst = GT > 1 ? tid - h * split : tid;
     float m = part_m[0][h], l = part_l[0][h];
@@ -661,18 +721,48 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
     float a = 0.f;
 #pragma unroll
     for (int k = 0; k < MW; ++k) a += part_o[(size_t)k * part_ld + h * HD + ch];
-    const int dst = ch / slice, off = (rank * g_rows + h) * slice + (ch - dst * slice);
+    const int dst = ch >> slice_log2, off = (rank * g_rows + h) * slice + (ch & (slice - 1));
     if (split > 1) st_async(map_rank(smem_u32(&xo[off]), dst), a, map_rank(smem_u32(ex_bar), dst));
     else xo[off] = a;
   }
+  if (!FEED) incoming();
+  // ---- the state of this thread's slots tid, tid + WT, ...: SB of them in registers at a time, the first ones (where their
+  // state has landed by now) read while the exchange is under way
+  constexpr int SB = FEED ? 2 : 4;
+  float old_r[SB], norm_r[SB], exp_r[SB];
+  int pos_r[SB];
+  long long fx_r[WINDOWED ? SB : 1];
+  const float* old_g = WINDOWED ? c.ring + ((int64_t)u * w + (t % w)) * cap + s0 : c.acc + (int64_t)u * cap + s0;
+  auto fetch = [&](int i0) {
+#pragma unroll
+    for (int k = 0; k < SB; ++k) {
+      const int i = i0 + k * WT;
+      exp_r[k] = old_r[k] = norm_r[k] = 0.f;
+      pos_r[k] = 0;
+      if (WINDOWED) fx_r[k] = 0;
+      if (i < cnt) {
+        const int64_t o = (int64_t)u * cap + s0 + i;
+        if (GT == 1) exp_r[k] = logit_s[i];
+        old_r[k] = state_in_smem ? acc_s[i] : old_g[i];
+        norm_r[k] = state_in_smem ? vn_s[i] : c.vnorm[o];
+        pos_r[k] = state_in_smem ? pos_s[i] : c.pos[o];
+        if (WINDOWED) fx_r[k] = state_in_smem ? fx_s[i] : c.acc_fixed[o];
+      }
+    }
+  };
+  const bool fetch_early = !FEED && state_in_smem == 1 && rows_alloc > 0;
+  if (fetch_early) {
+    if (!mbar_wait(smem_u32(state_full), state_par)) bad = true;
+    fetch(tid);
+  }
   if (split > 1) {
-    if (!mbar_wait(ex_bar, 0)) bad = true;
+    if (!mbar_wait(smem_u32(ex_bar), 0)) bad = true;
   } else {
     workers_sync();
   }
 
   // ---- every CTA: the unit's softmax normaliser (all data is local now) and its slice of the output ----
-  float m_all = -INFINITY, own_f = 0.f;    // own_f: this CTA's exp2(s - m) -> probability
+  float own_f = 0.f;       // own_f: this CTA's exp2(s - m) -> probability
   if constexpr (GT > 1) {
     if (tid < G) {         // one thread per head
       float2 ml[MAX_SPLIT];
@@ -695,7 +785,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
     }
     workers_sync();
     for (int i = tid; i < G * slice; i += WT) {
-      const int h = i / slice, ch = i - h * slice;
+      const int h = i >> slice_log2, ch = i & (slice - 1);
       float a = 0.f;
 #pragma unroll
       for (int r = 0; r < MAX_SPLIT; ++r)
@@ -703,75 +793,74 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
       out[((int64_t)u * G + h) * HD + rank * slice + ch] = __float2bfloat16(a * gq_invl[h]);
     }
   } else {
-    float L = 0.f, a = 0.f;
+    float2 ml[MAX_SPLIT];
+    float m_all = -INFINITY, L = 0.f, a = 0.f, part[MAX_SPLIT];
 #pragma unroll
-    for (int r = 0; r < MAX_SPLIT; ++r)
-      if (r < split) m_all = fmaxf(m_all, ex_ml[r][0].x);
+    for (int r = 0; r < MAX_SPLIT; ++r) {
+      ml[r] = r < split ? ex_ml[r][0] : make_float2(-INFINITY, 0.f);
+      part[r] = r < split && tid < slice ? xo[r * slice + tid] : 0.f;
+      m_all = fmaxf(m_all, ml[r].x);
+    }
 #pragma unroll
-    for (int r = 0; r < MAX_SPLIT; ++r)
-      if (r < split) {
-        const float f = ex_ml[r][0].x > -INFINITY ? ex2(ex_ml[r][0].x - m_all) : 0.f;
-        L += ex_ml[r][0].y * f;
-        if (r == rank) own_f = f;
-        if (tid < slice) a = fmaf(xo[r * slice + tid], f, a);
-      }
+    for (int r = 0; r < MAX_SPLIT; ++r) {
+      const float f = ml[r].x > -INFINITY ? ex2(ml[r].x - m_all) : 0.f;
+      L += ml[r].y * f;
+      a = fmaf(part[r], f, a);
+      if (r == rank) own_f = f;
+    }
     const float invL = 1.f / L;
     own_f *= invL;
     if (tid < slice) out[(int64_t)u * HD + rank * slice + tid] = __float2bfloat16(a * invL);
   }
 
   // ---- indicator update (Eq. 2 / Eq. 3) and importance (Eq. 4) of this CTA's slots, its arg-min ----
-  if (state_in_smem && rows_alloc > 0 && !mbar_wait(state_full, state_par)) bad = true;
+  if (!fetch_early) {
+    if (state_in_smem && rows_alloc > 0 && !mbar_wait(smem_u32(state_full), state_par)) bad = true;
+    fetch(tid);
+  }
   const bool evicting = hi > B;
   unsigned long long my_key = NO_KEY;
   int my_slot = -1, my_pos = -1;
-  {
-    // local copies: the stores into the state arrays below cannot alias what the loop reads
-    const float* __restrict__ lg = logit_s;
-    const float* __restrict__ as = acc_s;
-    const float* __restrict__ vs = vn_s;
-    const int* __restrict__ ps_s = pos_s;
-    float* __restrict__ acc_g = c.acc + (int64_t)u * cap + s0;
-#pragma unroll 4
-    for (int i = tid; i < cnt; i += WT) {
+  for (int i0 = tid; i0 < cnt;) {
+#pragma unroll
+    for (int k = 0; k < SB; ++k) {
+      const int i = i0 + k * WT;
+      if (i >= cnt) continue;
       const int slot_u = s0 + i;
+      const int64_t o = (int64_t)u * cap + slot_u;
       float p;
       if constexpr (GT > 1) {      // the mean of the heads' probabilities
         float a = 0.f;
 #pragma unroll
         for (int h = 0; h < GT; ++h)
-          if (h < G) a = fmaf(lg[h * chunk + i], gq_f[h], a);
+          if (h < G) a = fmaf(logit_s[h * chunk + i], gq_f[h], a);
         p = a / (float)G;
       } else {
-        p = lg[i] * own_f;
+        p = exp_r[k] * own_f;
       }
       const bool is_new = slot_u == fs;
       float S;
       if (WINDOWED) {
-        float* ring_row = c.ring + ((int64_t)u * w + (t % w)) * cap;
-        const int64_t o = (int64_t)u * cap + slot_u;
-        long long fx;
-        if (is_new) {
-          fx = prob_to_fixed(p);     // (the recycled slot's ring column is cleared below)
-        } else {
-          fx = (state_in_smem ? fx_s[i] : c.acc_fixed[o]) + prob_to_fixed(p) - prob_to_fixed(state_in_smem ? as[i] : ring_row[slot_u]);
-        }
-        ring_row[slot_u] = p;
+        // (a recycled slot's ring column is cleared below)
+        const long long fx = is_new ? prob_to_fixed(p) : fx_r[k] + prob_to_fixed(p) - prob_to_fixed(old_r[k]);
+        c.ring[((int64_t)u * w + (t % w)) * cap + slot_u] = p;
         c.acc_fixed[o] = fx;
         S = fixed_to_prob(fx);
       } else {
-        S = is_new ? p : (state_in_smem ? as[i] : acc_g[i]) + p;
+        S = is_new ? p : old_r[k] + p;
       }
-      if (VATP_INB((int64_t)u * cap + slot_u, (int64_t)units * cap, dev_status)) acc_g[i] = S;
+      if (VATP_INB(o, (int64_t)units * cap, dev_status)) c.acc[o] = S;
       if (evicting) {
-        const int ps = is_new ? t : (state_in_smem ? ps_s[i] : c.pos[(int64_t)u * cap + slot_u]);
-        const float I = S * (is_new ? new_norm : (state_in_smem ? vs[i] : c.vnorm[(int64_t)u * cap + slot_u]));
+        const int ps = is_new ? t : pos_r[k];
+        const float I = S * (is_new ? new_norm : norm_r[k]);
         if (ps >= F && ps <= t - R) {
           const unsigned long long key = evict_key(I, ps);
           if (key < my_key) { my_key = key; my_slot = slot_u; my_pos = ps; }
         }
       }
     }
+    i0 += SB * WT;
+    if (i0 < cnt) fetch(i0);
   }
   if (WINDOWED) {
     // recycled slot: the other rows of its ring column belong to the previous occupant (shared out over the unit's CTAs)
@@ -801,14 +890,19 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   if (rank == 0 && tid == 0) {            // nothing of the other CTAs' shared memory is read or written by anyone any more
     int out_slot = hi, left = hi, ev = -1;                         // not evicting: the cache grows
     if (evicting) {
-      if (split > 1 && !mbar_wait(cand_bar, 0)) bad = true;
+      if (split > 1 && !mbar_wait(smem_u32(cand_bar), 0)) bad = true;
       unsigned long long best = NO_KEY;
       int br = -1;
-      for (int r = 0; r < split; ++r)
-        if (cand[r].key < best) { best = cand[r].key; br = r; }
+      int best_slot = -1, best_pos = -1;
+#pragma unroll
+      for (int r = 0; r < MAX_SPLIT; ++r)
+        if (r < split) {
+          const Candidate x = cand[r];
+          if (x.key < best) { best = x.key; best_slot = x.slot; best_pos = x.pos; br = r; }
+        }
       if (br >= 0) {
-        out_slot = cand[br].slot;
-        ev = cand[br].pos;
+        out_slot = best_slot;
+        ev = best_pos;
         left = hi - 1;
         if (VATP_INB(out_slot, cap, dev_status)) c.pos[(int64_t)u * cap + out_slot] = -1;
       } else {   // nothing eligible (cannot happen when F + R <= B): keep the state consistent
@@ -821,6 +915,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
     c.last_slot[u] = fs;
     if (evicted) evicted[u] = ev;
   }
+  if (!FEED) break;     // (one unit a CTA)
   }   // next unit of this CTA
   if (!FEED && independent && tid == WT - 1) asm volatile("griddepcontrol.wait;" ::: "memory");     // (launches complete in order)
   if (bad) {
@@ -999,7 +1094,7 @@ cudaError_t launch_hd(const Shape& s, int B, int F, int R, const vatp_cache& c, 
                        {win ? (const char*)c.ring : nullptr, win ? slots * s.window * 4 : 0},
                        {win ? (const char*)c.acc_fixed : nullptr, win ? slots * 8 : 0},
                        {(const char*)q, units * G * ROW_BYTES}, {(const char*)k, units * ROW_BYTES}, {(const char*)v, units * ROW_BYTES}};
-  // One CTA per SM at most: no producer warp (see the kernel; 32 units x 2049 slots 10.3 us per waiting step against 12.7
+  // One CTA per SM at most: no producer warp (see the kernel; 32 units x 2049 slots 10.3 us per waiting step against 12.7, before the loops were trimmed
   // with one).  Beyond that it pays (512 units x 1025 slots with a history window 55 us against 79).
   const bool feed = grid > sms;
   auto kern = feed ? (grouped ? (win ? decode_mma_kernel<HD, true, GQ_HEADS, true> : decode_mma_kernel<HD, false, GQ_HEADS, true>)

@@ -42,7 +42,7 @@
 //   * grouped-query attention (several query heads share one cache; the paper leaves the case open and points at
 //     a group-wise score, read here as the MEAN of the heads' probabilities): up to eight heads of a group ride
 //     in the columns of the products (template parameter GT), so a K or V row is still read once per step.
-// Measured (us per step, first and latest version): 32 units x 2049 slots, every launch waiting 12.5 -> 9.6; 256 units x
+// Measured (us per step, first and latest version): 32 units x 2049 slots, every launch waiting 12.5 -> 9.15; 256 units x
 // 1639, launches overlapping 38 -> 34.2 (215 MB: 6.3 TB/s of the 6.56 a copy reaches); 512 units x 1025 with a history window
 // 73 -> 55; 8 units x 2049, four heads each 11.0 -> 8.9.
 #include <cooperative_groups.h>
@@ -210,7 +210,7 @@ __device__ __forceinline__ unsigned long long warp_min_key(unsigned long long ke
 template <int HD, bool WINDOWED, int GT, bool FEED>
 __global__ void __launch_bounds__(FEED ? DM_THREADS : WT, 2)
 decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, int independent, int G,
-                  int units, int state_in_smem, int part_in_ring, int split, int chunk, int nslot, int B, int cap, int F, int R, int w, int norm,
+                  int units, int state_in_smem, int part_in_ring, int split, int chunk, int ld, int nslot, int B, int cap, int F, int R, int w, int norm,
                   float scale_log2, vatp_cache c,
                   const __nv_bfloat16* __restrict__ q_new, const __nv_bfloat16* __restrict__ k_new,
                   const __nv_bfloat16* __restrict__ v_new, __nv_bfloat16* __restrict__ out,
@@ -220,7 +220,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   extern __shared__ unsigned char dyn_raw[];
   unsigned char* dyn = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(dyn_raw) + 1023) & ~uintptr_t(1023));
   // [MW][nslot] units | partial outputs of the warps [MW][G][HD] (part_in_ring: in the warps' own rings instead) |
-  // slices of partial outputs received [split][G][HD / split] | logits[G][chunk] | per-slot state of this CTA's own
+  // slices of partial outputs received [split][G][HD / split] | logits[G][ld] | per-slot state of this CTA's own
   // slots: acc (with a history window the ring row that leaves it), vnorm, pos, with a window the fixed-point sums.
   // Where the state does not fit beside the rings it is copied into the rings' memory once the streaming is over
   // (state_in_smem == 2; a CTA with one unit only) or read from global memory in the tail (state_in_smem == 0).
@@ -231,10 +231,10 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   const int part_ld = part_in_ring ? nslot * (UNIT / 4) : g_rows * HD;       // floats from one warp's partial to the next
   float* xo = reinterpret_cast<float*>(dyn + ring_bytes + (part_in_ring ? 0 : MW * g_rows * HD * 4));
   float* logit_s = xo + g_rows * HD;
-  float* acc_s = state_in_smem == 2 ? reinterpret_cast<float*>(ring_base) : logit_s + g_rows * chunk;
-  float* vn_s = acc_s + chunk;
-  int* pos_s = reinterpret_cast<int*>(vn_s + chunk);
-  long long* fx_s = reinterpret_cast<long long*>(pos_s + chunk);
+  float* acc_s = state_in_smem == 2 ? reinterpret_cast<float*>(ring_base) : logit_s + g_rows * ld;
+  float* vn_s = acc_s + ld;
+  int* pos_s = reinterpret_cast<int*>(vn_s + ld);
+  long long* fx_s = reinterpret_cast<long long*>(pos_s + ld);
 
   __shared__ __align__(8) uint64_t full[MW * MAX_SLOTS], empty[MW * MAX_SLOTS], misc_bars[4];
   __shared__ float part_m[MW][GT], part_l[MW][GT];
@@ -255,7 +255,10 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   const int u0 = blockIdx.x / split, u_step = gridDim.x / split;
   // its slot range inside a unit's allocation
   const int s0 = min(rank * chunk, cap);
-  const int rows_alloc = min(chunk, cap - s0);
+  const int tile_alloc = min(chunk, cap - s0);
+  // ld > chunk: the unit's last CTA takes a few slots more than its tiles hold, see tail_row
+  const bool tail_cta = !FEED && ld > chunk && rank == split - 1;
+  const int rows_alloc = tail_cta ? cap - s0 : tile_alloc;
   // Warp x's groups are x, x + MW, ...: as many as groups_of(x, rows) among the first `rows` rows.  Its units in order: the
   // K rows of its groups, then their V rows.  A launch requests the first units of its first unit (sequence, head) before
   // it may read how many rows are live; when fewer are than the allocation holds, those are dropped and the live ones
@@ -378,7 +381,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
     return;
   }
 
-  const int na_mine = groups_of(wid, rows_alloc), early_mine = min(nslot, 2 * na_mine);
+  const int na_mine = groups_of(wid, tile_alloc), early_mine = min(nslot, 2 * na_mine);
   if (!FEED) {
     if (independent && tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (lane == 0)
@@ -481,6 +484,29 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   if (has_chunk && wid == last_warp)
     last_raw = *(reinterpret_cast<const uint4*>((const __nv_bfloat16*)(lane < 16 ? c.k_cache : c.v_cache) +
                                                 ((int64_t)u * cap + ls) * HD) + (lane & 15));
+  // ---- the slots beyond the tiles (a budget that fills whole tiles leaves the incoming token's): warp x takes row x / G for
+  // head x mod G, a lane HD / 32 channels, with plain loads.  (As one more group of one warp, a single row made every
+  // CTA of the unit wait for its two steps.)
+  constexpr int TC = HD / 32;             // channels of a lane
+  const int tail_row = GT > 1 ? wid / G : wid, tail_head = GT > 1 ? wid - tail_row * G : 0;
+  const bool has_tail = tail_cta && chunk + tail_row < cnt;
+  uint32_t tail_q[TC / 2], tail_k[TC / 2], tail_v[TC / 2];
+#pragma unroll
+  for (int x = 0; x < TC / 2; ++x) tail_q[x] = tail_k[x] = tail_v[x] = 0u;
+  if (has_tail) {
+    const int slot_u = s0 + chunk + tail_row;
+    const int64_t o = ((int64_t)u * cap + slot_u) * HD + lane * TC, o_new = (int64_t)u * HD + lane * TC;
+    const bool is_new = slot_u == fs;
+    const __nv_bfloat16* kp = is_new ? k_new + o_new : (const __nv_bfloat16*)c.k_cache + o;
+    const __nv_bfloat16* vp = is_new ? v_new + o_new : (const __nv_bfloat16*)c.v_cache + o;
+    const __nv_bfloat16* qp = q_new + ((int64_t)u * g_rows + tail_head) * HD + lane * TC;
+#pragma unroll
+    for (int x = 0; x < TC / 2; ++x) {
+      tail_q[x] = reinterpret_cast<const uint32_t*>(qp)[x];
+      tail_k[x] = reinterpret_cast<const uint32_t*>(kp)[x];
+      tail_v[x] = reinterpret_cast<const uint32_t*>(vp)[x];
+    }
+  }
   float new_norm = 0.f;
   auto incoming = [&]() {
     if (wid == new_warp || wid == norm_warp) {
@@ -507,7 +533,8 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   // online softmax every 16-row group was a chain of ~2300 cycles (fragments, products, maximum, exponentials, fragments,
   // products) that eight warps walked through five times; here the groups of a warp depend on nothing, and exponentials
   // are taken once per slot instead of once per lane of an MMA tile.
-  n = groups_of(wid, cnt);                // this warp's live groups
+  const int cnt_t = FEED ? cnt : min(cnt, chunk);     // live rows in tiles
+  n = groups_of(wid, cnt_t);              // this warp's live groups
   if (u == u0 && n != na_mine) {          // rows requested before the live range was known: dropped (see the producer)
     if (!FEED) {
       to_request = 2 * n;
@@ -558,21 +585,36 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
     if (!FEED && r0 + RSTEP < r_end) k_fetch(r0 + RSTEP);
     // this lane: rows lane / 4 and lane / 4 + 8, heads 2 j4 and 2 j4 + 1 (one head: the same value in every column)
     const int ra = r0 + (lane >> 2), rb = ra + 8;
-    const bool ragged = r0 + GROUP > cnt;      // (chunk is a multiple of 16: dead rows of the last group have logits too, -inf)
+    const bool ragged = r0 + GROUP > cnt_t;      // (chunk is a multiple of 16: dead rows of the last group have logits too, -inf)
 #pragma unroll
     for (int x = 0; x < (GT > 1 ? 2 : 1); ++x) {
       float a = (sa[0][x] + sa[1][x]) * scale_log2, b = (sa[0][2 + x] + sa[1][2 + x]) * scale_log2;
       if (ragged) {
-        if (ra >= cnt) a = -INFINITY;
-        if (rb >= cnt) b = -INFINITY;
+        if (ra >= cnt_t) a = -INFINITY;
+        if (rb >= cnt_t) b = -INFINITY;
       }
       if (GT > 1 ? 2 * j4 + x < G : j4 == 0) {
-        float* lg = logit_s + (GT > 1 ? (2 * j4 + x) * chunk : 0);
+        float* lg = logit_s + (GT > 1 ? (2 * j4 + x) * ld : 0);
         lg[ra] = a;
         lg[rb] = b;
       }
       m_run[x] = fmaxf(m_run[x], fmaxf(a, b));
     }
+  }
+  if (!FEED && has_tail) {
+    float s = 0.f;
+#pragma unroll
+    for (int x = 0; x < TC / 2; ++x) {
+      s = fmaf(__uint_as_float(tail_q[x] << 16), __uint_as_float(tail_k[x] << 16), s);
+      s = fmaf(__uint_as_float(tail_q[x] & 0xffff0000u), __uint_as_float(tail_k[x] & 0xffff0000u), s);
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    s *= scale_log2;
+    if (lane == 0) logit_s[tail_head * ld + chunk + tail_row] = s;
+#pragma unroll
+    for (int x = 0; x < (GT > 1 ? 2 : 1); ++x)
+      if (GT == 1 || 2 * j4 + x == tail_head) m_run[x] = fmaxf(m_run[x], s);
   }
 #pragma unroll
   for (int x = 0; x < (GT > 1 ? 2 : 1); ++x) {
@@ -592,11 +634,12 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   // launch's own rows by more than they gained).
   if (!FEED && !independent && tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // ---- exp2(s - m) of the CTA's slots, in place, and their sum (m: the CTA's maximum, finite when it has a live row)
+  const int exp_rows = cnt > cnt_t ? cnt : (cnt + GROUP - 1) / GROUP * GROUP;
   if constexpr (GT == 1) {
     float m_c = -INFINITY, l = 0.f;
 #pragma unroll
     for (int k = 0; k < MW; ++k) m_c = fmaxf(m_c, part_m[k][0]);
-    for (int i = tid; i < (cnt + GROUP - 1) / GROUP * GROUP; i += WT) {
+    for (int i = tid; i < exp_rows; i += WT) {
       const float e = ex2(logit_s[i] - m_c);
       logit_s[i] = e;
       l += e;
@@ -610,10 +653,9 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
       float m_c = -INFINITY, l = 0.f;
 #pragma unroll
       for (int k = 0; k < MW; ++k) m_c = fmaxf(m_c, part_m[k][h]);
-      float* lg = logit_s + h * chunk;
-      const int rows = (cnt + GROUP - 1) / GROUP * GROUP;
+      float* lg = logit_s + h * ld;
 #pragma unroll 4
-      for (int i = lane; i < rows; i += 32) {
+      for (int i = lane; i < exp_rows; i += 32) {
         const float e = ex2(lg[i] - m_c);
         lg[i] = e;
         l += e;
@@ -633,12 +675,12 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   const bool two_halves = GT == 1 || G <= GT / 2;
   const bool low_col = two_halves && (lane >> 2 & (GT == 1 ? 1 : GT / 2));
   const int my_head = GT == 1 ? 0 : min(two_halves ? lane >> 2 & (GT / 2 - 1) : lane >> 2, G - 1);
-  const float* p_s = logit_s + my_head * chunk + 2 * j4;
+  const float* p_s = logit_s + my_head * ld + 2 * j4;
   uint32_t b0, b1, lo0, lo1;
   auto v_fetch = [&](int r0) {
     const float2 pa = *reinterpret_cast<const float2*>(p_s + r0), pb = *reinterpret_cast<const float2*>(p_s + r0 + 8);
     arrived();
-    const bool ragged = cnt < r0 + GROUP;
+    const bool ragged = cnt_t < r0 + GROUP;
     wrote = ragged;
     if (patches || ragged) {
       const bool has_new = wid == new_warp && fs_local >= r0 && fs_local < r0 + GROUP;
@@ -647,7 +689,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
       if (has_last) patch_row(unit_a, ls_local - r0, last_raw, true);
       // rows beyond the live range must not reach the product (their probability is 0, but 0 * garbage need not be 0)
       if (ragged)
-        for (int rr = cnt - r0 + (lane >> 4); rr < GROUP && has_chunk; rr += 2)
+        for (int rr = cnt_t - r0 + (lane >> 4); rr < GROUP && has_chunk; rr += 2)
           st_shared16(unit_a + ((lane >> 3) & 1) * TILE_BYTES + rr * 128 + ((lane & 7) << 4), make_uint4(0u, 0u, 0u, 0u));
       wrote = has_new || has_last || ragged;
       __syncwarp();
@@ -694,6 +736,16 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
 #pragma unroll
       for (int i = 0; i < HD / 16; ++i)
         if ((i & 3) == j4) { po[16 * i + row] = o_acc[i][0] + o_acc[i][1]; po[16 * i + 8 + row] = o_acc[i][2] + o_acc[i][3]; }
+    }
+  }
+  if (!FEED && has_tail) {
+    const float p = logit_s[tail_head * ld + chunk + tail_row];
+    float* po = part_o + (size_t)wid * part_ld + tail_head * HD + lane * TC;
+    __syncwarp();
+#pragma unroll
+    for (int x = 0; x < TC / 2; ++x) {
+      po[2 * x] = fmaf(p, __uint_as_float(tail_v[x] << 16), po[2 * x]);
+      po[2 * x + 1] = fmaf(p, __uint_as_float(tail_v[x] & 0xffff0000u), po[2 * x + 1]);
     }
   }
   workers_sync();
@@ -833,7 +885,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
         float a = 0.f;
 #pragma unroll
         for (int h = 0; h < GT; ++h)
-          if (h < G) a = fmaf(logit_s[h * chunk + i], gq_f[h], a);
+          if (h < G) a = fmaf(logit_s[h * ld + i], gq_f[h], a);
         p = a / (float)G;
       } else {
         p = exp_r[k] * own_f;
@@ -1046,6 +1098,15 @@ cudaError_t launch_hd(const Shape& s, int B, int F, int R, const vatp_cache& c, 
   while (split < MAX_SPLIT && s.units * split * 2 <= sms && cap / (split * 2) >= 4 * GROUP) split *= 2;
   int chunk = (cap + split - 1) / split;
   chunk = (chunk + GROUP - 1) / GROUP * GROUP;
+  int ld = chunk;        // slots a CTA has room for
+  // A few slots more than whole rounds of the warps (a group each) hold: the last CTA takes them with plain loads, at most
+  // one row and head a warp.  (32 units x 2049 slots, four CTAs each: 9.6 us per step with them in one more group, 9.15 so;
+  // 16 units x 1025 6.55 and 5.95.)  Only without a producer warp, see below.
+  const int rounds = (B + 1) / (MW * GROUP * split), extra = B + 1 - rounds * MW * GROUP * split;
+  if (s.units * split <= sms && rounds > 0 && extra > 0 && extra * G <= MW) {
+    chunk = rounds * MW * GROUP;
+    ld = chunk + GROUP;  // (the capacity is the slots' number rounded up to eight)
+  }
   // Two CTAs per SM at most; beyond that a CTA takes several units, one after the other (its producer warp then fills the
   // rings with the next unit's rows while the tail of this one runs).
   const int resident = 2;
@@ -1058,8 +1119,8 @@ cudaError_t launch_hd(const Shape& s, int B, int F, int R, const vatp_cache& c, 
   const size_t half_sm = 111 * 1024, whole_sm = 222 * 1024;     // dynamic bytes, 1 KB of it alignment slack
   const int groups_per_warp = ((chunk / GROUP) + MW - 1) / MW;
   const bool part_in_ring = grouped && one_unit;                // a warp's partial outputs land in its ring
-  const size_t fixed = 1024 + (part_in_ring ? 0 : (size_t)MW * G * HD * 4) + (size_t)G * HD * 4 + (size_t)G * chunk * 4;
-  const size_t state = (size_t)(win ? 20 : 12) * chunk;
+  const size_t fixed = 1024 + (part_in_ring ? 0 : (size_t)MW * G * HD * 4) + (size_t)G * HD * 4 + (size_t)G * ld * 4;
+  const size_t state = (size_t)(win ? 20 : 12) * ld;
   const bool copyable = !win || (((uintptr_t)c.ring | (uintptr_t)c.acc_fixed) & 15) == 0;      // (bulk copies: 16-byte aligned)
   int nslot = 0, state_in_smem = 0;
   size_t dyn = 0;
@@ -1120,7 +1181,7 @@ cudaError_t launch_hd(const Shape& s, int B, int F, int R, const vatp_cache& c, 
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, kern, tm_k, tm_v, independent, G, s.units, state_in_smem, (int)part_in_ring, split, chunk, nslot, B, cap, F, R, s.window,
+  return cudaLaunchKernelEx(&cfg, kern, tm_k, tm_v, independent, G, s.units, state_in_smem, (int)part_in_ring, split, chunk, ld, nslot, B, cap, F, R, s.window,
                             s.norm, s.scale * LOG2E, c, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v,
                             (__nv_bfloat16*)out, evicted, dev_status);
 }

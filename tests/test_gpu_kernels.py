@@ -48,6 +48,9 @@ def test_head_dim_64_window_leaves_earlier_normalisers_alone():
     (3, 100, 0, 64, 130, 40),    # the same with head_dim 64 and a history window (the state of the next unit is fetched early)
     (5, 8, 2, 128, 600, 0),      # grouped queries split over a cluster
     (2, 640, 160, 64, 90, 0),    # grouped queries, several units per CTA
+    (1, 3, 0, 128, 1030, 0),     # eight CTAs a unit, seven slots beyond their tiles
+    (1, 4, 0, 64, 1031, 40),     # ... eight, a history window
+    (1, 8, 2, 128, 1025, 0),     # ... two, four heads
     (1, 2, 0, 128, 9000, 0),     # state beyond shared memory
     (1, 300, 0, 128, 2048, 30),  # several units per CTA, their state read from global memory in the tail
 ])

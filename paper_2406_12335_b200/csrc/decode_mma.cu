@@ -43,7 +43,7 @@
 //     a group-wise score, read here as the MEAN of the heads' probabilities): up to eight heads of a group ride
 //     in the columns of the products (template parameter GT), so a K or V row is still read once per step.
 // Measured (us per step, first and latest version): 32 units x 2049 slots, every launch waiting 12.5 -> 9.15; 256 units x
-// 1639, launches overlapping 38 -> 34.2 (215 MB: 6.3 TB/s of the 6.56 a copy reaches); 512 units x 1025 with a history window
+// 1639, launches overlapping 38 -> 33.4 (215 MB: 6.4 TB/s of the 6.56 a copy reaches); 512 units x 1025 with a history window
 // 73 -> 55; 8 units x 2049, four heads each 11.0 -> 8.9.
 #include <cooperative_groups.h>
 
@@ -204,7 +204,7 @@ __device__ __forceinline__ unsigned long long warp_min_key(unsigned long long ke
 // heads (G of them, a run-time argument) share the cache of unit u: column g of the products carries head g, so every K and V row
 // is read once for the whole group; the maxima, sums and partial outputs exist per head, and the indicator advances by
 // the MEAN of the heads' probabilities.
-// FEED: a producer warp keeps the rings full, for CTAs with several units and for grids beyond one CTA per SM.  Otherwise
+// FEED: a producer warp keeps the rings full, for CTAs with several units.  Otherwise
 // every warp requests its own rows: one warp less at 128 instead of 96 registers, and a shorter way from a freed slot to
 // the next request, which is what a launch that has the machine to itself is bound by.
 template <int HD, bool WINDOWED, int GT, bool FEED>
@@ -1096,14 +1096,22 @@ cudaError_t launch_hd(const Shape& s, int B, int F, int R, const vatp_cache& c, 
   // split a unit over a cluster while the grid still fits on the SMs once (a second launch can then be resident too)
   int split = 1;
   while (split < MAX_SPLIT && s.units * split * 2 <= sms && cap / (split * 2) >= 4 * GROUP) split *= 2;
+  // Long units on a machine that they leave half idle: two CTAs per SM have twice the rows in flight (96 units x 1536 slots
+  // 18.5 -> 15.3 us per waiting step and 19.9 -> 12.0 overlapping; 60 x 3501 22.3 -> 19.9).  Shorter ranges gain only while
+  // launches wait for one another (96 x 1025 13.6 -> 11.8, overlapping 8.3 -> 9.1), and clusters of four do not fill every
+  // SM twice (68 x 3501 23.8 -> 22.3, 72 x 3501 24.9 -> 31.9), of eight still less.
+  const int long_range = (may_overlap ? 40 : 28) * GROUP;
+  while (split < 4 && s.units * split * 2 <= (split == 1 ? 2 * sms : sms * 9 / 5) && s.units * split * 2 > sms &&
+         cap / (split * 2) >= long_range)
+    split *= 2;
   int chunk = (cap + split - 1) / split;
   chunk = (chunk + GROUP - 1) / GROUP * GROUP;
   int ld = chunk;        // slots a CTA has room for
   // A few slots more than whole rounds of the warps (a group each) hold: the last CTA takes them with plain loads, at most
   // one row and head a warp.  (32 units x 2049 slots, four CTAs each: 9.6 us per step with them in one more group, 9.15 so;
-  // 16 units x 1025 6.55 and 5.95.)  Only without a producer warp, see below.
+  // 16 units x 1025 6.55 and 5.95.)  Only with one unit a CTA.
   const int rounds = (B + 1) / (MW * GROUP * split), extra = B + 1 - rounds * MW * GROUP * split;
-  if (s.units * split <= sms && rounds > 0 && extra > 0 && extra * G <= MW) {
+  if (s.units * split <= 2 * sms && rounds > 0 && extra > 0 && extra * G <= MW) {
     chunk = rounds * MW * GROUP;
     ld = chunk + GROUP;  // (the capacity is the slots' number rounded up to eight)
   }
@@ -1155,9 +1163,9 @@ cudaError_t launch_hd(const Shape& s, int B, int F, int R, const vatp_cache& c, 
                        {win ? (const char*)c.ring : nullptr, win ? slots * s.window * 4 : 0},
                        {win ? (const char*)c.acc_fixed : nullptr, win ? slots * 8 : 0},
                        {(const char*)q, units * G * ROW_BYTES}, {(const char*)k, units * ROW_BYTES}, {(const char*)v, units * ROW_BYTES}};
-  // One CTA per SM at most: no producer warp (see the kernel; 32 units x 2049 slots 10.3 us per waiting step against 12.7, before the loops were trimmed
-  // with one).  Beyond that it pays (512 units x 1025 slots with a history window 55 us against 79).
-  const bool feed = grid > sms;
+  // CTAs with several units have a producer warp.  (One unit a CTA, without it against with it: 32 units x 2049 slots 9.2 and
+  // 12.3 us per waiting step, 256 x 1025 24.1 and 26.3; 512 units x 1025 with a history window, two a CTA: 79 and 55.)
+  const bool feed = !one_unit;
   auto kern = feed ? (grouped ? (win ? decode_mma_kernel<HD, true, GQ_HEADS, true> : decode_mma_kernel<HD, false, GQ_HEADS, true>)
                               : (win ? decode_mma_kernel<HD, true, 1, true> : decode_mma_kernel<HD, false, 1, true>))
                    : (grouped ? (win ? decode_mma_kernel<HD, true, GQ_HEADS, false> : decode_mma_kernel<HD, false, GQ_HEADS, false>)

@@ -48,6 +48,8 @@ def test_head_dim_64_window_leaves_earlier_normalisers_alone():
     (3, 100, 0, 64, 130, 40),    # the same with head_dim 64 and a history window (the state of the next unit is fetched early)
     (5, 8, 2, 128, 600, 0),      # grouped queries split over a cluster
     (2, 640, 160, 64, 90, 0),    # grouped queries, several units per CTA
+    (1, 80, 0, 128, 1100, 0),    # a unit over two CTAs, beyond one CTA per SM
+    (1, 60, 0, 64, 1900, 0),     # ... over four
     (1, 3, 0, 128, 1030, 0),     # eight CTAs a unit, seven slots beyond their tiles
     (1, 4, 0, 64, 1031, 40),     # ... eight, a history window
     (1, 8, 2, 128, 1025, 0),     # ... two, four heads

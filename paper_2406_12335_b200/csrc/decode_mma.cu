@@ -1037,10 +1037,19 @@ StreamHistory* history_of(cudaStream_t st, unsigned long long capture, bool crea
 
 // True when `touched` overlaps nothing that a launch possibly still in flight on `st` writes; records this
 // launch.  may_overlap false (the caller did not opt in): records it and answers false.
+// share: of the machine, if as many of its CTAs share an SM as fit; share_alone: if each has an SM to itself, which *alone
+// asks the caller to arrange (and which is recorded then).
 bool independent_of_in_flight(cudaStream_t st, unsigned long long capture, bool may_overlap, const Range* touched, int nt,
-                               const Range* written, double share_if_indep, double share_if_not) {
+                               const Range* written, double share, double share_alone, bool* alone) {
   std::lock_guard<std::mutex> lock(g_hist_mutex);
   StreamHistory* h = history_of(st, capture, true);
+  // Launches too few CTAs wide for the ones between two steps of a cache to fill the machine would have to wait.  Alone on
+  // their SMs (half as many fit) they may not: 8 units x 301 slots, eight caches in turn, 3.9 us per step waiting and 2.3 so;
+  // 48 x 2001, four caches, 13.4 and 9.4.
+  int apart = h->count == HIST ? HIST : 0;       // launches since the last one on this cache
+  for (int j = 0; j < h->count; ++j)
+    if (overlaps(touched[0], h->rec[(h->head - j + HIST) % HIST].w[0])) { apart = j; break; }
+  *alone = may_overlap && apart * share < 1.0 && apart * share_alone >= 1.0;
   // The first recorded launch follows work this table knows nothing about (another kernel, the start of a
   // graph): it waits, and by the time it lets its successor start everything before it has completed.
   bool indep = may_overlap && h->count > 0;
@@ -1057,7 +1066,7 @@ bool independent_of_in_flight(cudaStream_t st, unsigned long long capture, bool 
   if (h->count < HIST) ++h->count;
   LaunchRecord& r = h->rec[h->head];
   for (int k = 0; k < NRANGE; ++k) r.w[k] = written[k];
-  r.share = indep ? share_if_indep : share_if_not;
+  r.share = *alone ? share_alone : share;
   return indep;
 }
 
@@ -1069,7 +1078,8 @@ bool independent_of_in_flight(cudaStream_t st, unsigned long long capture, bool 
 bool decode_overlap_policy_probe(void* stream, const uint64_t* begin, const uint64_t* bytes, int n, double share) {
   Range r[NRANGE] = {};
   for (int i = 0; i < n && i < NRANGE; ++i) r[i] = Range{reinterpret_cast<const char*>(begin[i]), (size_t)bytes[i]};
-  return independent_of_in_flight(static_cast<cudaStream_t>(stream), 0, true, r, NRANGE, r, share, share);
+  bool alone;
+  return independent_of_in_flight(static_cast<cudaStream_t>(stream), 0, true, r, NRANGE, r, share, share, &alone);
 }
 
 // Any other work this library enqueues on `st` (prefill, selection, compaction, the general decode kernel)
@@ -1097,12 +1107,13 @@ cudaError_t launch_hd(const Shape& s, int B, int F, int R, const vatp_cache& c, 
   int split = 1;
   while (split < MAX_SPLIT && s.units * split * 2 <= sms && cap / (split * 2) >= 4 * GROUP) split *= 2;
   // Long units on a machine that they leave half idle: two CTAs per SM have twice the rows in flight (96 units x 1536 slots
-  // 18.5 -> 15.3 us per waiting step and 19.9 -> 12.0 overlapping; 60 x 3501 22.3 -> 19.9).  Shorter ranges gain only while
-  // launches wait for one another (96 x 1025 13.6 -> 11.8, overlapping 8.3 -> 9.1), and clusters of four do not fill every
-  // SM twice (68 x 3501 23.8 -> 22.3, 72 x 3501 24.9 -> 31.9), of eight still less.
-  const int long_range = (may_overlap ? 40 : 28) * GROUP;
+  // 18.5 -> 15.3 us per waiting step and 19.9 -> 12.0 overlapping; 60 x 3501 22.3 -> 19.9).  Shorter ranges gain while
+  // launches wait for one another (96 x 1025 13.6 -> 11.8) and lose a little of what overlapping gives (8.3 -> 9.1, 9.6 in
+  // the first version); clusters of four do not fill every
+  // SM twice (68 x 3501 23.8 -> 22.3, 72 x 3501 24.9 -> 31.9), of eight still less.  (The split decides in which order sums are
+  // taken: it depends on the shape alone.)
   while (split < 4 && s.units * split * 2 <= (split == 1 ? 2 * sms : sms * 9 / 5) && s.units * split * 2 > sms &&
-         cap / (split * 2) >= long_range)
+         cap / (split * 2) >= (split == 1 ? 28 : 40) * GROUP)
     split *= 2;
   int chunk = (cap + split - 1) / split;
   chunk = (chunk + GROUP - 1) / GROUP * GROUP;
@@ -1124,7 +1135,7 @@ cudaError_t launch_hd(const Shape& s, int B, int F, int R, const vatp_cache& c, 
   // many units in flight per warp as fit there, at least two; the per-slot state beside them (1), in the rings' memory
   // after the streaming (2) or in global memory (0).  Only when not even that fits, a whole SM.
   const bool win = s.window > 0;
-  const size_t half_sm = 111 * 1024, whole_sm = 222 * 1024;     // dynamic bytes, 1 KB of it alignment slack
+  const size_t third_sm = 77 * 1024, half_sm = 111 * 1024, whole_sm = 222 * 1024;   // dynamic bytes, 1 KB of it alignment slack
   const int groups_per_warp = ((chunk / GROUP) + MW - 1) / MW;
   const bool part_in_ring = grouped && one_unit;                // a warp's partial outputs land in its ring
   const size_t fixed = 1024 + (part_in_ring ? 0 : (size_t)MW * G * HD * 4) + (size_t)G * HD * 4 + (size_t)G * ld * 4;
@@ -1172,9 +1183,13 @@ cudaError_t launch_hd(const Shape& s, int B, int F, int R, const vatp_cache& c, 
                               : (win ? decode_mma_kernel<HD, true, 1, false> : decode_mma_kernel<HD, false, 1, false>));
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)whole_sm);
   if (e != cudaSuccess) return e;
-  // share of the machine this launch holds while resident (every CTA waits for the previous launch before it retires)
-  const double share = (double)grid / ((double)(dyn <= half_sm ? 2 : 1) * sms);
-  const int independent = independent_of_in_flight(st, capture_of(st), may_overlap, written, 16, written, share, share) ? 1 : 0;
+  // share of the machine this launch holds while resident (every CTA waits for the previous launch before it retires): exactly
+  // two CTAs of this kernel fit on an SM, or exactly one
+  const bool half = dyn <= half_sm;
+  const double share_alone = (double)grid / sms, share = half ? share_alone / 2 : share_alone;
+  bool alone = false;
+  const int independent = independent_of_in_flight(st, capture_of(st), may_overlap, written, 16, written, share, share_alone, &alone) ? 1 : 0;
+  dyn = half && !alone ? (dyn > third_sm ? dyn : third_sm) : whole_sm;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(feed ? DM_THREADS : WT);

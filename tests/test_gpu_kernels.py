@@ -112,3 +112,37 @@ def test_decode_step_against_float64(b, h, kv, d, B, window, grow):
             got = imp.gather(2, (pos == ev[..., None]).int().argmax(-1, keepdim=True))[..., 0]
             assert torch.all((pos == ev[..., None]).sum(-1) == 1)
             assert torch.all(got <= imp.amin(-1) * (1 + 2e-3) + 1e-9)      # the minimum, up to both sides' tolerance
+
+
+@pytest.mark.parametrize("units,B,layers", [
+    (8, 300, 8),     # eight launches of one CTA per SM fill the machine, of two they do not
+    (48, 500, 4),
+    (8, 300, 2),     # too few either way
+    (90, 1000, 3),   # a unit over two CTAs
+])
+def test_steps_of_several_caches_side_by_side(units, B, layers):
+    """Steps of several caches in turn, with and without leave to overlap: the same bits."""
+    V = P.vatp()
+    got = []
+    for overlap in (False, True):
+        g = torch.Generator(device="cuda").manual_seed(B)
+        rnd = lambda *s: torch.randn(*s, generator=g, device="cuda").bfloat16()  # noqa: E731
+        p = V.make_params(batch=1, heads=units, seq_len=2 * B, head_dim=128, dtype="bf16", budget=B, decode_overlap=overlap)
+        caches = [V.Cache(p) for _ in range(layers)]
+        for c in caches:
+            c.k_cache[:, :, :B], c.v_cache[:, :, :B] = rnd(1, units, B, 128), rnd(1, units, B, 128)
+            c.pos[:, :, :B] = torch.arange(B, dtype=torch.int32, device="cuda")
+            c.vnorm[:, :, :B] = c.v_cache[:, :, :B].float().abs().sum(-1)
+            c.acc[:, :, :B] = torch.rand(1, units, B, generator=g, device="cuda")
+            c.len.fill_(B), c.free_slot.fill_(B), c.next_pos.fill_(2 * B)
+        qkv = [[rnd(3, 1, units, 128) for _ in range(layers)] for _ in range(6)]
+        out = torch.empty(6, layers, 1, units, 128, dtype=torch.bfloat16, device="cuda")
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        for s in range(6):
+            for l, c in enumerate(caches):
+                V.vatp_decode_step(p, c, *qkv[s][l], out[s, l], dev_status=status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        got.append([out] + [t for c in caches for t in (c.k_cache, c.v_cache, c.acc, c.vnorm, c.pos, c.len, c.free_slot)])
+    assert all(torch.equal(a, b) for a, b in zip(*got))

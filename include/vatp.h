@@ -36,7 +36,7 @@
  *     with a history window) are not available with it (VATP_ERR_UNSUPPORTED), and the workspace
  *     holds a normaliser row per query head and G partial indicators.  The decode step takes
  *     the tensor-core kernel for bf16 and G <= 8 (VATP_FLAG_DECODE_OVERLAP applies as in the multi-head case) and a
- *     general kernel otherwise; the history rebuild runs a general kernel.
+ *     general kernel otherwise; the history rebuild runs on the tensor cores for bf16.
  *   - Inputs are assumed finite.
  *   - A second build of the library (compiled with -DVATP_DEBUG_BOUNDS) range-checks every row, slot,
  *     window-row and scratch index its kernels compute before the access; an index outside its array is
@@ -206,8 +206,8 @@ vatp_status vatp_prefill_attention_scores(const vatp_params* params, const void*
  * First call on a device: looks up the array's device address (once per device, with the current
  * device) - make that first call outside any stream capture.
  * Sharing: all calls on a device use the same array.  Calls on one stream are ordered and safe
- * (each call starts by zeroing its counters - a memset, or a kernel that first waits for all
- * earlier work in the stream - and touches nothing else before that, so it cannot begin before
+ * (each call starts by zeroing its counters, in a kernel that first waits for all earlier work in
+ * the stream, and touches nothing else before that, so it cannot begin before
  * the previous call on the stream has finished with the array);
  * calls that may overlap on the GPU (different streams, different host threads) race on it and
  * give wrong scores - serialise them, or use vatp_prefill_scores with separate workspaces.  The

@@ -137,11 +137,15 @@ decode_kernel(int split, int chunk, int B, int cap, int F, int R, int w, int nor
   const T* vc = (const T*)c.v_cache + ((int64_t)u * cap + s0) * D;
   uint64_t* state_bar = &bars[DEC_WARPS * NSTAGE];
 
-  if (tid == 0) {
-    for (int i = 0; i < DEC_WARPS * NSTAGE + 1; ++i) mbar_init(&bars[i], 1);
+  if (tid < DEC_WARPS * NSTAGE + 1) {
+    mbar_init(&bars[tid], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
+  // A programmatic dependent of the launch before it: nothing of global memory is touched until that has completed, and the
+  // next launch may set up meanwhile.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   auto issue = [&](int ch, int stage) {   // one lane: request K and V rows of chunk `ch`
     const int r0 = ch * ROWS;
@@ -206,6 +210,14 @@ decode_kernel(int split, int chunk, int B, int cap, int F, int R, int w, int nor
       c.pos[(int64_t)u * cap + fs] = t;
     }
   }
+
+  // A recycled slot's ring column belongs to the previous occupant.  While the histories fit in L2 all threads clear its other
+  // rows under the streaming (2 units x 601 slots, w 256: 8.1 us per step, 9.2 with one thread clearing at the end); beyond
+  // that this burst of scattered stores takes longer than a thread's stores one after the other (64 x 2001: 25.6 and 21.8).
+  const bool clear_early = WINDOWED && (int64_t)(gridDim.x / split) * cap * w <= (3 << 22);
+  if (clear_early)
+    for (int rr = rank * DEC_THREADS + tid; rr < w; rr += split * DEC_THREADS)
+      if (rr != t % w && VATP_INB(fs, cap, dev_status)) c.ring[((int64_t)u * w + rr) * cap + fs] = 0.f;
 
   // ---- stream the chunks: logits, online softmax, partial output ----
   float m_run = -INFINITY, l_run = 0.f;
@@ -346,8 +358,8 @@ decode_kernel(int split, int chunk, int B, int cap, int F, int R, int w, int nor
       float* ring_row = c.ring + ((int64_t)u * w + (t % w)) * cap;
       long long fx;
       if (is_new) {
-        // recycled slot: its ring column belongs to the previous occupant
-        for (int rr = 0; rr < w; ++rr) c.ring[((int64_t)u * w + rr) * cap + slot] = 0.f;
+        if (!clear_early)
+          for (int rr = 0; rr < w; ++rr) c.ring[((int64_t)u * w + rr) * cap + slot] = 0.f;
         fx = prob_to_fixed(p);
       } else {
         fx = c.acc_fixed[o] + prob_to_fixed(p) - prob_to_fixed(ring_row[slot]);
@@ -416,14 +428,25 @@ template <typename T, int D, bool WINDOWED>
 cudaError_t launch_t(const Shape& s, int B, int F, int R, const vatp_cache& c, const void* q, const void* k,
                      const void* v, void* out, int32_t* evicted, int32_t* dev_status, cudaStream_t st) {
   const int cap = cache_capacity(B);
-  // split a unit over a cluster when there are too few units to fill 148 SMs
-  int split = 1;
-  while (split < MAX_SPLIT && s.units * split * 2 <= 148 * 2 && cap / (split * 2) >= 64) split *= 2;
-  int chunk = (cap + split - 1) / split;
-  chunk = (chunk + 7) / 8 * 8;
+  // Split a unit over a cluster when there are too few units to fill the machine once: as many CTAs as are resident
+  // together, two per SM where two fit (less what clusters leave over, unless units are long: 34 units x 64 channels, four and
+  // eight CTAs each, 601 slots 8.9 and 9.4 us per step, 2001 slots 15.8 and 14.7).  With fp32 and head_dim 128 one fits, and twice that
+  // many ran one half after the other: 32 units x 601 slots 25.5 us per step, now 11.9.
   const size_t stage_bytes = (size_t)DEC_WARPS * NSTAGE * 2 * ROWS * D * sizeof(T);
-  const size_t dyn = stage_bytes + 4 * sizeof(float) * chunk;
-  if (dyn > 200 * 1024) return cudaErrorInvalidConfiguration;
+  auto chunk_of = [&](int n) { return ((cap + n - 1) / n + 7) / 8 * 8; };
+  auto dyn_of = [&](int n) { return stage_bytes + 4 * sizeof(float) * chunk_of(n); };
+  const size_t most_dyn = 200 * 1024;
+  const int sms = device_sm_count();
+  int split = 1;
+  while (split < MAX_SPLIT && cap / (split * 2) >= 64 &&
+         s.units * split * 2 <= (dyn_of(split) > most_dyn ? 2 * sms : dyn_of(split * 2) > 96 * 1024 ? sms : cap < 1024 || split < 4 ? sms * 9 / 5 : 2 * sms))
+    split *= 2;          // (or as far as it takes for the slots' state to fit)
+  const int chunk = chunk_of(split);
+  // (at most two CTAs per SM: the next launch's would otherwise crowd the SMs that are left first; clusters of eight need
+  // the third place to fit: 32 units x 601 x 64 channels 9.4 us, 13.0 without it)
+  size_t dyn = dyn_of(split);
+  if (s.units * split > sms && split < MAX_SPLIT && dyn < 77 * 1024) dyn = 77 * 1024;
+  if (dyn > most_dyn) return cudaErrorInvalidConfiguration;
   auto kern = decode_kernel<T, D, WINDOWED>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
   if (e != cudaSuccess) return e;
@@ -432,13 +455,15 @@ cudaError_t launch_t(const Shape& s, int B, int F, int R, const vatp_cache& c, c
   cfg.blockDim = dim3(DEC_THREADS);
   cfg.dynamicSmemBytes = dyn;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = split;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, kern, split, chunk, B, cap, F, R, s.window, s.norm, s.scale * LOG2E, c, (const T*)q,
                             (const T*)k, (const T*)v, (T*)out, evicted, dev_status);
 }

@@ -146,3 +146,54 @@ def test_steps_of_several_caches_side_by_side(units, B, layers):
         assert int(status.item()) == 0
         got.append([out] + [t for c in caches for t in (c.k_cache, c.v_cache, c.acc, c.vnorm, c.pos, c.len, c.free_slot)])
     assert all(torch.equal(a, b) for a, b in zip(*got))
+
+
+@pytest.mark.parametrize("units,B,d,window", [
+    (37, 600, 128, 0),       # one CTA per SM resident: a cluster of two
+    (64, 600, 64, 300),      # two CTAs per SM, all threads clear a recycled slot's history first
+    (30, 1500, 64, 400),     # clusters of eight, a long history: one thread clears it
+    (30, 19000, 128, 0),     # split further for the slots' state to fit
+    (2, 1, 64, 3),           # one slot besides the incoming token's
+])
+def test_fp32_decode_step_against_float64(units, B, d, window):
+    """The general kernel's steps back to back, each read only at the end, against float64 torch."""
+    V = P.vatp()
+    p = V.make_params(batch=1, heads=units, seq_len=2 * B, head_dim=d, dtype="f32", budget=B,
+                      indicator="window" if window else "h2o", window=window)
+    c = V.Cache(p)
+    g = torch.Generator(device="cuda").manual_seed(units + B)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")  # noqa: E731
+    c.k_cache[:, :, :B], c.v_cache[:, :, :B] = rnd(1, units, B, d), rnd(1, units, B, d)
+    c.pos[:, :, :B] = torch.arange(B, dtype=torch.int32, device="cuda")
+    c.vnorm[:, :, :B] = c.v_cache[:, :, :B].abs().sum(-1)
+    c.len.fill_(B), c.free_slot.fill_(B), c.next_pos.fill_(2 * B)
+    if window:
+        c.ring[..., :B] = torch.rand(1, units, window, B, generator=g, device="cuda") / B
+        c.acc_fixed[..., :B] = (c.ring[..., :B].double() * 2.0 ** 52).long().sum(2)
+        c.acc.copy_((c.acc_fixed.double() / 2.0 ** 52).float())
+    else:
+        c.acc[:, :, :B] = torch.rand(1, units, B, generator=g, device="cuda")
+    K, W, pos, n = c.k_cache[0].double(), c.v_cache[0].double(), c.pos[0].clone(), B + 1
+    fs = c.free_slot[0].long()
+    q, k, v = (rnd(4, 1, units, d) for _ in range(3))
+    out, ev = torch.empty_like(q), torch.empty(4, 1, units, dtype=torch.int32, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for s in range(4):
+        V.vatp_decode_step(p, c, q[s], k[s], v[s], out[s], evicted_pos=ev[s], dev_status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    i = torch.arange(units, device="cuda")
+    for s in range(4):
+        K[i, fs], W[i, fs], pos[i, fs] = k[s, 0].double(), v[s, 0].double(), 2 * B + s
+        logits = torch.einsum("hd,hnd->hn", q[s, 0].double(), K) * d ** -0.5
+        want = torch.einsum("hn,hnd->hd", torch.softmax(logits.masked_fill(pos < 0, float("-inf")), -1), W)
+        # fp32 sums of n terms and exponentials: n * 2^-24 of the largest value, and 2^-20 of slack for exp2f's argument
+        assert torch.all((out[s, 0].double() - want).abs() <= (n * 2.0 ** -24 + 2.0 ** -18) * W.abs().amax(1))
+        fs = (pos == ev[s, 0][:, None]).int().argmax(1)
+        pos[i, fs] = -1
+    assert torch.equal(pos[:, :n], c.pos[0, :, :n])
+    if window:
+        # the windowed sums are the ring's columns added up exactly
+        live = c.pos[0] >= 0
+        sums = (c.ring[0].double() * 2.0 ** 52).long().sum(1)
+        assert torch.equal(sums[live], c.acc_fixed[0][live])

@@ -15,6 +15,7 @@
 // (256 units x 7936 keys with the compaction behind it 103.7 -> 98 us; 8 units x 7806 20.9 -> 19.6.)
 #include <cooperative_groups.h>
 
+#include "select_staging.h"
 #include "vatp_internal.cuh"
 
 namespace cg = cooperative_groups;
@@ -86,7 +87,7 @@ __global__ void __launch_bounds__(THREADS) select_kernel(int copies, int T, int 
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int v = v0 + j * THREADS + tid;
-        if (v < nvec && VATP_INB(pad + a0 + 4 * v + 3, n + 4, dev_status)) dst4[v] = make_uint4(order_key(x[j].x), order_key(x[j].y), order_key(x[j].z), order_key(x[j].w));
+        if (v < nvec && VATP_INB(pad + a0 + 4 * v + 3, staged_words(n), dev_status)) dst4[v] = make_uint4(order_key(x[j].x), order_key(x[j].y), order_key(x[j].z), order_key(x[j].w));
       }
     }
     if (tid < a0) keys_s[pad + tid] = order_key(mid[tid]);
@@ -95,12 +96,13 @@ __global__ void __launch_bounds__(THREADS) select_kernel(int copies, int T, int 
     __syncthreads();
   }
   // Four keys at a time: group v holds keys 4 v - pad .. 4 v - pad + 3 of the middle range.
-  const int nv = (pad + n + 3) >> 2;
+  const int nv = staged_groups(pad, n);
   struct Keys4 { uint32_t k[4]; };
   auto keys_of = [&](int v) -> Keys4 {
     Keys4 r;
     if (STAGED) {
-      const uint4 x = reinterpret_cast<const uint4*>(keys_s)[v];
+      uint4 x = make_uint4(0u, 0u, 0u, 0u);
+      if (VATP_INB(4 * v + 3, staged_words(n), dev_status)) x = reinterpret_cast<const uint4*>(keys_s)[v];
       r.k[0] = x.x; r.k[1] = x.y; r.k[2] = x.z; r.k[3] = x.w;
     } else {
 #pragma unroll
@@ -484,7 +486,7 @@ cudaError_t launch_select(int units, int T, int B, int F, int R, const float* sc
   }
   const int copies = n <= 2048 ? 1 : (n <= 16384 ? 4 : 8);
   const size_t hist_bytes = (size_t)copies * 256 * sizeof(uint32_t);
-  const size_t bytes = hist_bytes + (size_t)(n + 4) * sizeof(uint32_t);     // up to three words of alignment padding
+  const size_t bytes = hist_bytes + (size_t)staged_words(n) * sizeof(uint32_t);
   const bool staged = bytes <= 168 * 1024;
   // more units than SMs: CTAs of 512 threads, several to an SM
   const bool half = units > sms;

@@ -197,3 +197,42 @@ def test_fp32_decode_step_against_float64(units, B, d, window):
         live = c.pos[0] >= 0
         sums = (c.ring[0].double() * 2.0 ** 52).long().sum(1)
         assert torch.equal(sums[live], c.acc_fixed[0][live])
+
+
+@pytest.mark.parametrize("units", [5, 200])          # CTAs of 1024 and of 512 threads
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 30, 31, 1022, 1023, 1024, 1025, 2047, 2051, 7806, 7807])
+def test_select_middle_range_of_every_length_and_alignment(units, n):
+    """Middle ranges of every residue mod 4 whose first score lies at every alignment (odd prompt lengths, several units),
+    some with ties at the boundary: the kept sets bit for bit."""
+    from oracle import vatp_oracle as O
+    V = P.vatp()
+    for F in range(4):
+        R, keep = 2 + (n + F) % 2, max(n // 3, 1) - (n == 1)
+        T, B = n + F + R, keep + F + R
+        if T <= B or B == 0:
+            continue
+        T += 1 - T % 2 if n > 8 else 0               # odd: the units' rows start at all four alignments
+        g = torch.Generator().manual_seed(n + F)
+        score = torch.rand(1, units, T, generator=g)
+        score[:, ::2] = (score[:, ::2] * 16).floor()
+        p = V.make_params(batch=1, heads=units, seq_len=T, head_dim=64, dtype="f32", budget=B, n_sink=F, n_recent=R)
+        kept = torch.empty(1, units, B, dtype=torch.int32, device="cuda")
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        V.vatp_select(p, score.cuda(), kept, dev_status=status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        for u in list(range(5)) + [units - 1]:
+            assert kept[0, u].cpu().numpy().tolist() == O.select_keep(score[0, u].numpy(), B, F, R).tolist()
+
+
+def test_select_alignments_on_the_bounds_checking_build():
+    """The same on the build that range-checks every staged group before it is read."""
+    import os
+    import subprocess
+    import sys
+    from paper_2406_12335_b200 import build
+    env = dict(os.environ, VATP_LIBRARY=build.build(debug_bounds=True))
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-m", "pytest", "tests/test_gpu_kernels.py", "-x", "-q", "-m", "gpu", "-k", "every_length_and_alignment",
+                        "-p", "no:cacheprovider"], cwd=root, env=env, capture_output=True, text=True)
+    assert r.returncode == 0 and " passed" in r.stdout, (r.stdout + r.stderr)[-2000:]

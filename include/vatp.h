@@ -307,8 +307,8 @@ vatp_status vatp_selftest_bounded_wait(uint64_t limit_ns, int32_t* dev_status, u
 
 /*
  * Host-only probe of the rule that lets consecutive vatp_decode_step launches overlap on the GPU (no
- * device work, usable without a GPU).  Pretends that a launch on `stream` reads and writes the n
- * (<= 13) host-described byte ranges [begin[i], begin[i] + bytes[i]) and keeps `share` of the
+ * device work, usable without a GPU).  Pretends that a launch on `stream` reads and writes the first 13 and
+ * only reads the others of the n (<= 16) host-described byte ranges [begin[i], begin[i] + bytes[i]) and keeps `share` of the
  * machine's CTA slots until the launch before it has completed.  Returns 1 when that launch would
  * run without waiting for its predecessors - it overlaps none of the recorded launches that can
  * still be resident - else 0, and records it; -1 on bad arguments.  A negative `share` instead ends

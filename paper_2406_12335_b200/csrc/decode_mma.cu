@@ -987,17 +987,18 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
 }
 
 
-// Host-side record, per stream, of the buffers the last launches write and of the share of the
+// Host-side record, per stream, of the buffers the last launches write and read and of the share of the
 // machine each occupies.  Every CTA of a launch stays resident until the previous launch has
 // completed, so launch M - j can still be running when M starts only if the launches between them fit
-// on the machine together: M may skip all waiting when it touches nothing that those launches write.
+// on the machine together: M may skip all waiting when it touches nothing that those launches write and writes
+// nothing that they read.
 struct Range {
   const char* p;
   size_t n;
 };
-constexpr int HIST = 8, NRANGE = 13;
+constexpr int HIST = 8, NRANGE = 13, NTOUCHED = 16;   // of the ranges a launch touches the first NRANGE are written
 struct LaunchRecord {
-  Range w[NRANGE];
+  Range r[NTOUCHED];
   double share;        // CTAs / (resident CTAs the machine holds of this launch's kind)
 };
 struct StreamHistory {
@@ -1039,12 +1040,12 @@ StreamHistory* history_of(cudaStream_t st, unsigned long long capture, bool crea
   return h;
 }
 
-// True when `touched` overlaps nothing that a launch possibly still in flight on `st` writes; records this
-// launch.  may_overlap false (the caller did not opt in): records it and answers false.
+// True when `touched` overlaps nothing that a launch possibly still in flight on `st` writes, nor its written part anything
+// that such a launch reads; records this launch.  may_overlap false (the caller did not opt in): records it and answers false.
 // share: of the machine, if as many of its CTAs share an SM as fit; share_alone: if each has an SM to itself, which *alone
 // asks the caller to arrange (and which is recorded then).
-bool independent_of_in_flight(cudaStream_t st, unsigned long long capture, bool may_overlap, const Range* touched, int nt,
-                               const Range* written, double share, double share_alone, bool* alone) {
+bool independent_of_in_flight(cudaStream_t st, unsigned long long capture, bool may_overlap, const Range (&touched)[NTOUCHED],
+                              double share, double share_alone, bool* alone) {
   std::lock_guard<std::mutex> lock(g_hist_mutex);
   StreamHistory* h = history_of(st, capture, true);
   // Launches too few CTAs wide for the ones between two steps of a cache to fill the machine would have to wait.  Alone on
@@ -1052,7 +1053,7 @@ bool independent_of_in_flight(cudaStream_t st, unsigned long long capture, bool 
   // 48 x 2001, four caches, 13.3 and 9.3.
   int apart = h->count == HIST ? HIST : 0;       // launches since the last one on this cache
   for (int j = 0; j < h->count; ++j)
-    if (overlaps(touched[0], h->rec[(h->head - j + HIST) % HIST].w[0])) { apart = j; break; }
+    if (overlaps(touched[0], h->rec[(h->head - j + HIST) % HIST].r[0])) { apart = j; break; }
   *alone = may_overlap && apart * share < 1.0 && apart * share_alone >= 1.0;
   // The first recorded launch follows work this table knows nothing about (another kernel, the start of a
   // graph): it waits, and by the time it lets its successor start everything before it has completed.
@@ -1060,16 +1061,16 @@ bool independent_of_in_flight(cudaStream_t st, unsigned long long capture, bool 
   double between = 0.0;      // machine share of the launches between the candidate and this one
   for (int j = 0; indep && j < h->count && between < 1.0; ++j) {
     const LaunchRecord& r = h->rec[(h->head - j + HIST) % HIST];
-    for (int i = 0; i < nt && indep; ++i)
-      for (int k = 0; k < NRANGE; ++k)
-        if (overlaps(touched[i], r.w[k])) { indep = false; break; }
+    for (int i = 0; i < NTOUCHED && indep; ++i)
+      for (int k = 0; k < (i < NRANGE ? NTOUCHED : NRANGE); ++k)      // (two launches may read the same)
+        if (overlaps(touched[i], r.r[k])) { indep = false; break; }
     between += r.share;
     if (j == HIST - 1 && between < 1.0 && h->count == HIST) indep = false;   // history too short to tell
   }
   h->head = (h->head + 1) % HIST;
   if (h->count < HIST) ++h->count;
   LaunchRecord& r = h->rec[h->head];
-  for (int k = 0; k < NRANGE; ++k) r.w[k] = written[k];
+  for (int k = 0; k < NTOUCHED; ++k) r.r[k] = touched[k];
   r.share = *alone ? share_alone : share;
   return indep;
 }
@@ -1077,13 +1078,13 @@ bool independent_of_in_flight(cudaStream_t st, unsigned long long capture, bool 
 }  // namespace
 
 // Host-only probe of the overlap policy (no device work): feeds one pretend launch that touches and
-// writes the `n` byte ranges [begin[i], begin[i] + bytes[i]) on `stream` and occupies `share` of the
-// machine; returns whether it would have been allowed to run beside the launches before it.
+// writes the first NRANGE of the `n` byte ranges [begin[i], begin[i] + bytes[i]) and only reads the others, on `stream`, and
+// occupies `share` of the machine; returns whether it would have been allowed to run beside the launches before it.
 bool decode_overlap_policy_probe(void* stream, const uint64_t* begin, const uint64_t* bytes, int n, double share) {
-  Range r[NRANGE] = {};
-  for (int i = 0; i < n && i < NRANGE; ++i) r[i] = Range{reinterpret_cast<const char*>(begin[i]), (size_t)bytes[i]};
+  Range r[NTOUCHED] = {};
+  for (int i = 0; i < n && i < NTOUCHED; ++i) r[i] = Range{reinterpret_cast<const char*>(begin[i]), (size_t)bytes[i]};
   bool alone;
-  return independent_of_in_flight(static_cast<cudaStream_t>(stream), 0, true, r, NRANGE, r, share, share, &alone);
+  return independent_of_in_flight(static_cast<cudaStream_t>(stream), 0, true, r, share, share, &alone);
 }
 
 // Any other work this library enqueues on `st` (prefill, selection, compaction, the general decode kernel)
@@ -1170,7 +1171,7 @@ cudaError_t launch_hd(const Shape& s, int B, int F, int R, const vatp_cache& c, 
       !make_halves_map_bf16(&tm_v, c.v_cache, HD, (uint64_t)s.units * cap, GROUP))
     return cudaErrorInvalidValue;
   const size_t units = (size_t)s.units, slots = units * cap;
-  Range written[16] = {{(const char*)c.k_cache, slots * ROW_BYTES}, {(const char*)c.v_cache, slots * ROW_BYTES},
+  const Range touched[NTOUCHED] = {{(const char*)c.k_cache, slots * ROW_BYTES}, {(const char*)c.v_cache, slots * ROW_BYTES},
                        {(const char*)c.acc, slots * 4}, {(const char*)c.vnorm, slots * 4}, {(const char*)c.pos, slots * 4},
                        {(const char*)c.len, units * 4}, {(const char*)c.free_slot, units * 4},
                        {(const char*)c.next_pos, units * 4}, {(const char*)c.last_slot, units * 4},
@@ -1192,7 +1193,7 @@ cudaError_t launch_hd(const Shape& s, int B, int F, int R, const vatp_cache& c, 
   const bool half = dyn <= half_sm;
   const double share_alone = (double)grid / sms, share = half ? share_alone / 2 : share_alone;
   bool alone = false;
-  const int independent = independent_of_in_flight(st, capture_of(st), may_overlap, written, 16, written, share, share_alone, &alone) ? 1 : 0;
+  const int independent = independent_of_in_flight(st, capture_of(st), may_overlap, touched, share, share_alone, &alone) ? 1 : 0;
   dyn = half && !alone ? (dyn > third_sm ? dyn : third_sm) : whole_sm;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);

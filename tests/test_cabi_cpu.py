@@ -152,3 +152,31 @@ def test_decode_overlap_policy(V):
     assert [_probe(V, s, cache(i), 0.43) for i in range(4)] == [0, 1, 1, 1]
     assert _probe(V, s, cache(0), -1.0) == 0
     assert [_probe(V, s, cache(i), 0.43) for i in (7, 8, 7)] == [0, 1, 0]
+
+
+def test_decode_overlap_policy_keeps_what_a_launch_reads(V):
+    """A step may not write (its output, its state) what a launch that can still be running reads as its query, key or
+    value; that both read the same buffer is no reason to wait."""
+    MB = 1 << 20
+    X, Y, Z, W = (0xB0_0000_0000 + i * MB for i in range(4))
+
+    def step(stream, cache, q, out, kv=0xC0_0000_0000):
+        """13 ranges read and written (the cache, the output, the rest empty), then query, key, value."""
+        written = [(0x10_0000_0000 + cache * 64 * MB, 32 * MB), (out, 4096)] + [(0, 0)] * 11
+        return _probe(V, stream, written + [(q, 4096), (kv, 2048), (kv + 4096, 2048)], 0.6)
+
+    s = 0xA101
+    assert step(s, 0, X, Y) == 0                 # the first launch waits
+    assert step(s, 1, Z, W) == 1
+    # the output lands in the query of the launch before it (0.6 of the machine lies between this launch and the one before that)
+    assert step(s, 2, X, Z) == 0
+    assert step(s, 3, X, Y) == 1                 # the same query, key and value as the launch before it: read by both
+    assert step(s, 4, Y, W) == 0                 # reads the output of the launch before it
+    # a range written as part of the state (here: a key buffer of the launch before)
+    s = 0xA102
+    assert [step(s, i, X, Y + 8192 * i, kv=Z) for i in range(2)] == [0, 1]
+    assert step(s, 2, W, Z + 4096 + 1024) == 0   # the tail of its value buffer
+    # two launches of 0.6 in between: the reader has retired
+    s = 0xA103
+    assert [step(s, i, q, Y + 8192 * i) for i, q in enumerate((X, Z, W))] == [0, 1, 1]
+    assert step(s, 3, Z, X) == 1

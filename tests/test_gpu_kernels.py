@@ -236,3 +236,31 @@ def test_select_alignments_on_the_bounds_checking_build():
     r = subprocess.run([sys.executable, "-m", "pytest", "tests/test_gpu_kernels.py", "-x", "-q", "-m", "gpu", "-k", "every_length_and_alignment",
                         "-p", "no:cacheprovider"], cwd=root, env=env, capture_output=True, text=True)
     assert r.returncode == 0 and " passed" in r.stdout, (r.stdout + r.stderr)[-2000:]
+
+
+@pytest.mark.parametrize("units,B", [(320, 300), (16, 600)])     # several units per CTA, and one
+def test_overlapping_steps_whose_output_lands_in_an_earlier_steps_query(units, B):
+    """Steps of several caches over three query / output buffers in turn: a step's output replaces the query of the step
+    before it, which its launch may still be reading.  With and without leave to overlap: the same bits."""
+    V = P.vatp()
+    got = []
+    for overlap in (False, True):
+        g = torch.Generator(device="cuda").manual_seed(B)
+        rnd = lambda *s: torch.randn(*s, generator=g, device="cuda").bfloat16()  # noqa: E731
+        p = V.make_params(batch=1, heads=units, seq_len=2 * B, head_dim=128, dtype="bf16", budget=B, decode_overlap=overlap)
+        caches = [V.Cache(p) for _ in range(4)]
+        for c in caches:
+            c.k_cache[:, :, :B], c.v_cache[:, :, :B] = rnd(1, units, B, 128), rnd(1, units, B, 128)
+            c.pos[:, :, :B] = torch.arange(B, dtype=torch.int32, device="cuda")
+            c.vnorm[:, :, :B] = c.v_cache[:, :, :B].float().abs().sum(-1)
+            c.acc[:, :, :B] = torch.rand(1, units, B, generator=g, device="cuda")
+            c.len.fill_(B), c.free_slot.fill_(B), c.next_pos.fill_(2 * B)
+        buf, kv = [rnd(1, units, 128) for _ in range(3)], [(rnd(1, units, 128), rnd(1, units, 128)) for _ in range(24)]
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        for s in range(24):
+            V.vatp_decode_step(p, caches[s % 4], buf[s % 3], *kv[s], buf[(s + 2) % 3], dev_status=status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        got.append(buf + [t for c in caches for t in (c.k_cache, c.v_cache, c.acc, c.vnorm, c.pos, c.free_slot)])
+    assert all(torch.equal(a, b) for a, b in zip(*got))

@@ -1415,7 +1415,7 @@ window_ring_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
   auto emit = [&](const float (&p)[32], int c0, int cs, int n_cols) {
     const int j0 = T - w + c0 + cs;
     int rr = j0 >= 0 ? j0 % w : j0 + w;
-    uint32_t off = (uint32_t)rr * (uint32_t)cap;          // element offset of the ring row (w * cap < 2^31: checked on the host)
+    uint32_t off = (uint32_t)rr * (uint32_t)cap;          // element offset of the ring row (w * cap < 2^31: the caller's rule)
     const int live = min(32, n_cols - cs);
     const bool st_ok = slot < cap;
     if (live == 32 && rr + 32 <= w) {
@@ -1738,7 +1738,6 @@ cudaError_t launch_ring_hd(const Shape& s, int G, int B, const void* q, const fl
   sq.qsh = s.qsh / G;
   CUtensorMap tm_q, tm_kc;
   if (!make_map(&tm_q, q, sq, true) || !make_rows_map_bf16(&tm_kc, c.k_cache, HD, (uint64_t)s.units * cap, TILE)) return cudaErrorInvalidValue;
-  if ((int64_t)s.window * cap >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
   const size_t smem = sizeof(RingSmem<HD>) + 1024;
   auto kern = window_ring_tc_kernel<HD, GROUPED>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1756,7 +1755,7 @@ cudaError_t launch_prefill_tc(const Shape& s, const void* q, const void* k, cons
                    : launch_prefill_hd<128>(s, q, k, v, lse_ws, lse_out, attn_acc, vnorm, score, win_rows, dev_status, st, lse_in, attn_out);
 }
 
-// Window history from Q and the compacted keys on the tensor cores (bf16); see window_ring_tc_kernel.
+// Window history from Q and the compacted keys on the tensor cores (bf16, window * capacity < 2^31); see window_ring_tc_kernel.
 cudaError_t launch_window_ring_tc(const Shape& s, int G, int B, const void* q, const float* lse, const vatp_cache& c,
                                   int32_t* dev_status, cudaStream_t st) {
   if (G > 1)

@@ -8,7 +8,8 @@
 // a w x cap x d contraction per unit (tiny next to the T x T scoring passes), written straight into the ring's
 // layout.  With grouped queries the history holds the MEAN over the KV group's query heads of their probabilities (the
 // group-mean indicator's rows).  bf16 runs on the tensor cores (window_ring_tc_kernel, beside the scoring kernel whose
-// machinery it shares); this file holds the dispatch and the FMA kernel for fp32.  The sums are integers (2^52 fixed
+// machinery it shares); this file holds the dispatch and the FMA kernel for fp32 and for histories of 2^31 elements and more
+// per unit, which the tensor-core kernel's 32-bit ring offsets do not reach.  The sums are integers (2^52 fixed
 // point), so they do not depend on the order in which rows are added.
 #include <cooperative_groups.h>
 
@@ -147,7 +148,8 @@ cudaError_t launch_fma(const Shape& s, int G, int B, const void* q, const float*
 
 cudaError_t launch_window_ring(const Shape& s, int G, int dtype, int B, const void* q, const float* lse, const vatp_cache& c,
                                int32_t* dev_status, cudaStream_t st) {
-  if (dtype == VATP_BF16 && vatp_tc_available()) return launch_window_ring_tc(s, G, B, q, lse, c, dev_status, st);
+  if (dtype == VATP_BF16 && vatp_tc_available() && (int64_t)s.window * cache_capacity(B) < ((int64_t)1 << 31))
+    return launch_window_ring_tc(s, G, B, q, lse, c, dev_status, st);
   if (dtype == VATP_F32)
     return s.d == 64 ? launch_fma<float, 64>(s, G, B, q, lse, c, st) : launch_fma<float, 128>(s, G, B, q, lse, c, st);
   return s.d == 64 ? launch_fma<__nv_bfloat16, 64>(s, G, B, q, lse, c, st) : launch_fma<__nv_bfloat16, 128>(s, G, B, q, lse, c, st);

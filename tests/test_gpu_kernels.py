@@ -264,3 +264,37 @@ def test_overlapping_steps_whose_output_lands_in_an_earlier_steps_query(units, B
         assert int(status.item()) == 0
         got.append(buf + [t for c in caches for t in (c.k_cache, c.v_cache, c.acc, c.vnorm, c.pos, c.free_slot)])
     assert all(torch.equal(a, b) for a, b in zip(*got))
+
+
+def _probabilities(q, k, first, scale):
+    """float64 rows first .. T - 1 of the causal attention matrix of one unit ([T, d] each), and their normalisers."""
+    s = (q[first:].double() @ k.double().T) * scale
+    T = k.shape[0]
+    s.masked_fill_(torch.arange(T, device=q.device)[None] > torch.arange(first, T, device=q.device)[:, None], float("-inf"))
+    lse = torch.logsumexp(s, -1)
+    return torch.exp(s - lse[:, None]), lse
+
+
+@pytest.mark.parametrize("d,heads,kv", [(64, 1, 0), (128, 2, 1)])
+def test_history_of_more_elements_than_32_bits_index(d, heads, kv):
+    """A history window times a capacity beyond 2^31 elements (8.6 GB of rows per cache), head_dim 64 and grouped queries."""
+    V = P.vatp()
+    T, w, B = 300, 65536, 32768
+    p = V.make_params(batch=1, heads=heads, kv_heads=kv, seq_len=T, head_dim=d, dtype="bf16", budget=B, indicator="window", window=w)
+    g = torch.Generator(device="cuda").manual_seed(d)
+    q, k, v = (torch.randn(1, n, T, d, generator=g, device="cuda").bfloat16() for n in (heads, kv or heads, kv or heads))
+    rows = [_probabilities(q[0, h], k[0, 0], 0, d ** -0.5) for h in range(heads)]
+    want, lse = sum(r[0] for r in rows) / heads, torch.stack([r[1] for r in rows])[None].float().contiguous()
+    acc, vnorm = torch.zeros(1, 1, T, device="cuda"), v.float().abs().sum(-1)
+    kept = torch.full((1, 1, B), -1, dtype=torch.int32, device="cuda")
+    kept[..., :T] = torch.arange(T, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    c = V.Cache(p)
+    assert w * c.cap >= 1 << 31
+    V.vatp_compact_window(p, q, k, v, lse, acc, vnorm, kept, c, dev_status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    # 32-bit logits and normalisers of size up to 8: each rounding shows as 2^-21 of the probability at most, four of them
+    assert torch.all((c.ring[0, 0, :T, :T].double() - want).abs() <= 2.0 ** -19 * want)
+    assert torch.all(((c.acc[0, 0, :T].double() - want.sum(0)).abs() <= 2.0 ** -19 * want.sum(0)))
+    assert int(torch.count_nonzero(c.ring[0, 0, T:])) == 0 and int(torch.count_nonzero(c.ring[0, 0, :T, T:])) == 0

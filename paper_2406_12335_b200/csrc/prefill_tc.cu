@@ -1304,11 +1304,12 @@ __global__ void __launch_bounds__(VN_THREADS) vnorm_kernel(TcArgs a, const float
   // pass 2, a programmatic dependent, may set up while this kernel runs; it reads what is written here
   // only after its griddepcontrol.wait
   if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int u = blockIdx.x;
+  // (the grid is one-dimensional, all units of a group of tokens after one another: its other dimensions end at 65535)
+  const int block = blockIdx.x / a.kv_units, u = blockIdx.x - block * a.kv_units;
   if (lse_in) {
     // this CTA's tokens; the last CTA of the unit also fills the padding up to Tpad
-    const int last = blockIdx.y == gridDim.y - 1 ? a.Tpad : (blockIdx.y + 1) * VN_TOKENS;
-    for (int i = blockIdx.y * VN_TOKENS + threadIdx.x; i < last; i += VN_THREADS) {
+    const int last = blockIdx.x + a.kv_units >= gridDim.x ? a.Tpad : (block + 1) * VN_TOKENS;
+    for (int i = block * VN_TOKENS + threadIdx.x; i < last; i += VN_THREADS) {
       float x = -INFINITY;
       if (i < a.T) {
         const float l = __ldg(lse_in + (int64_t)u * a.T + i);
@@ -1322,7 +1323,7 @@ __global__ void __launch_bounds__(VN_THREADS) vnorm_kernel(TcArgs a, const float
   const __nv_bfloat16* vu = a.v + (int64_t)b * a.sb + (int64_t)h * a.sh;
   constexpr int LPR = HD / 8, RPP = VN_THREADS / LPR, NP = VN_TOKENS / RPP;     // lanes per row, rows per pass of the CTA, passes
   const int sub = threadIdx.x / LPR, part = threadIdx.x % LPR;
-  const int row0 = blockIdx.y * VN_TOKENS + sub;
+  const int row0 = block * VN_TOKENS + sub;
   uint4 raw[NP];
 #pragma unroll
   for (int j = 0; j < NP; ++j) {
@@ -1342,7 +1343,7 @@ __global__ void __launch_bounds__(VN_THREADS) vnorm_kernel(TcArgs a, const float
     const int tok = row0 + RPP * j;
     if (part == 0 && tok < a.T) a.vnorm[(int64_t)u * a.T + tok] = norm_finish(KIND, acc);
   }
-  if (!lse_in && blockIdx.x == 0 && blockIdx.y == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (!lse_in && blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 
@@ -1688,7 +1689,7 @@ cudaError_t launch_prefill_hd(const Shape& s, const void* q, const void* k, cons
   DependentLaunch dr(dim3(1), dim3(32), 0, st);
   if ((e = cudaLaunchKernelEx(&dr.cfg, reset_counters_kernel, a.counters)) != cudaSuccess) return e;
   auto value_norms = [&]() {
-    DependentLaunch dv(dim3(a.kv_units, (s.T + VN_TOKENS - 1) / VN_TOKENS), dim3(VN_THREADS), 0, st);
+    DependentLaunch dv(dim3((unsigned)a.kv_units * ((s.T + VN_TOKENS - 1) / VN_TOKENS)), dim3(VN_THREADS), 0, st);
     auto kern = a.norm == VATP_NORM_L1 ? vnorm_kernel<HD, VATP_NORM_L1> : a.norm == VATP_NORM_L2 ? vnorm_kernel<HD, VATP_NORM_L2> : vnorm_kernel<HD, VATP_NORM_LINF>;
     return cudaLaunchKernelEx(&dv.cfg, kern, a, lse_in);
   };

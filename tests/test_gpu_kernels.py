@@ -298,3 +298,30 @@ def test_history_of_more_elements_than_32_bits_index(d, heads, kv):
     assert torch.all((c.ring[0, 0, :T, :T].double() - want).abs() <= 2.0 ** -19 * want)
     assert torch.all(((c.acc[0, 0, :T].double() - want.sum(0)).abs() <= 2.0 ** -19 * want.sum(0)))
     assert int(torch.count_nonzero(c.ring[0, 0, T:])) == 0 and int(torch.count_nonzero(c.ring[0, 0, :T, T:])) == 0
+
+
+@pytest.mark.parametrize("call", ["scores", "lse"])
+def test_value_norms_of_a_very_long_prompt(call):
+    """One token more than 65535 groups of 64: the value norms beside a history window's scoring."""
+    V = P.vatp()
+    T, w, d = 65535 * 64 + 1, 16, 64
+    p = V.make_params(batch=1, heads=1, seq_len=T, head_dim=d, dtype="bf16", budget=64, indicator="window", window=w)
+    g = torch.Generator(device="cuda").manual_seed(7)
+    q, k, v = (torch.randn(1, 1, T, d, generator=g, device="cuda").bfloat16() for _ in range(3))
+    prob, lse = _probabilities(q[0, 0], k[0, 0], T - w, d ** -0.5)
+    acc, vnorm, score, given = (torch.zeros(1, 1, T, device="cuda") for _ in range(4))
+    given[0, 0, T - w:] = lse.float()
+    ws = torch.empty(V.vatp_workspace_bytes(p), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    to = dict(attn_acc=acc, vnorm=vnorm, score=score, workspace=ws, dev_status=status)
+    if call == "lse":
+        V.vatp_prefill_scores_from_lse(p, q, k, v, given, **to)
+    else:
+        V.vatp_prefill_scores(p, q, k, v, **to)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    norm = v[0, 0].float().abs().sum(-1)
+    assert torch.allclose(vnorm[0, 0], norm, rtol=1e-5, atol=0)
+    # logits and normalisers (size up to 22 in the log2 domain) rounded to 32 bits, exponentials good to 2^-20
+    assert torch.all((acc[0, 0].double() - prob.sum(0)).abs() <= 2.0 ** -17 * prob.sum(0))
+    assert torch.equal(score, acc * vnorm)

@@ -1489,7 +1489,7 @@ window_ring_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
 #pragma unroll
           for (int i4 = 0; i4 < 32; i4 += 4) {
             float4 nl;
-            asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(nl.x), "=f"(nl.y), "=f"(nl.z), "=f"(nl.w) : "r"(lp + 4 * i4));
+            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(nl.x), "=f"(nl.y), "=f"(nl.z), "=f"(nl.w) : "r"(lp + 4 * i4));
             const float nls[4] = {nl.x, nl.y, nl.z, nl.w};
 #pragma unroll
             for (int k = 0; k < 4; ++k) {

@@ -325,3 +325,30 @@ def test_value_norms_of_a_very_long_prompt(call):
     # logits and normalisers (size up to 22 in the log2 domain) rounded to 32 bits, exponentials good to 2^-20
     assert torch.all((acc[0, 0].double() - prob.sum(0)).abs() <= 2.0 ** -17 * prob.sum(0))
     assert torch.equal(score, acc * vnorm)
+
+
+@pytest.mark.parametrize("w,heads,kv", [(700, 2, 0), (300, 8, 2), (700, 12, 1)])
+def test_history_of_several_chunks_and_heads(w, heads, kv):
+    """Each chunk of 256 window rows and each head of a group meets its own normalisers: they differ widely from head to head
+    and from row to row (scaled queries)."""
+    V = P.vatp()
+    T, d, B, hk = 800, 128, 200, kv or heads
+    p = V.make_params(batch=1, heads=heads, kv_heads=kv, seq_len=T, head_dim=d, dtype="bf16", budget=B, indicator="window", window=w)
+    g = torch.Generator(device="cuda").manual_seed(w)
+    rnd = lambda n: torch.randn(1, n, T, d, generator=g, device="cuda")  # noqa: E731
+    size = (torch.arange(heads, device="cuda")[:, None] % 3 + 1) * (1 + torch.arange(T, device="cuda")[None] // 100 % 2)
+    q, k, v = (rnd(heads) * size[None, ..., None]).bfloat16(), rnd(hk).bfloat16(), rnd(hk).bfloat16()
+    G, f32 = heads // hk, dict(dtype=torch.float32, device="cuda")
+    rows = [_probabilities(q[0, h], k[0, h // G], 0, d ** -0.5) for h in range(heads)]
+    lse = torch.stack([r[1] for r in rows])[None].float().contiguous()
+    want = torch.stack([r[0] for r in rows]).view(hk, G, T, T).mean(1)[:, T - w:]
+    kept = torch.randperm(T, generator=torch.Generator().manual_seed(w))[:B].sort().values.cuda()
+    c, status = V.Cache(p), torch.zeros(1, dtype=torch.int32, device="cuda")
+    V.vatp_compact_window(p, q, k, v, lse, torch.zeros(1, hk, T, **f32), torch.ones(1, hk, T, **f32), kept.int().repeat(1, hk, 1).contiguous(),
+                          c, dev_status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    ring = c.ring[0][:, torch.arange(T - w, T, device="cuda") % w, :B].double()
+    want = want[..., kept]
+    # 32-bit logits and normalisers of size up to 64 in the log2 domain: a few roundings of 2^-19 each
+    assert torch.all((ring - want).abs() <= 2.0 ** -16 * want + 1e-30)

@@ -1362,6 +1362,7 @@ struct RingSmem {
   alignas(1024) unsigned char keys[tile_bytes<HD>];     // 128 cached keys: two K halves of [128 rows][128 bytes]
   alignas(1024) unsigned char qrows[chunk_bytes<HD>];   // 256 window queries: [K half][256 rows][128 bytes]
   float nlse[CHUNK];                                // their negated log2 normalisers (-inf: no such query)
+  float nres[CHUNK];                                // FINE: what the rounding of those lost
   long long part[3][TILE];                          // window sums of column groups 1-3
   alignas(8) uint64_t bar_ld, bar_mma;
   uint32_t tmem_base;
@@ -1371,16 +1372,23 @@ struct RingSmem {
 // GROUPED: the history of a KV group holds the MEAN over its G query heads; `heads` counts KV heads, q and lse have
 // heads * G.  The chunk's queries of one head after the other meet the same key tile, and the probabilities are summed in
 // registers (64 per thread: one CTA per SM), in ascending head order.  16 x 8 caches of 1025 slots, 32 query heads, w 256:
-// 2.5 ms on FMA units, the whole compaction with it now 0.19 ms.
+// 2.5 ms on FMA units, the whole compaction with it now 0.20 ms.
+// FINE (head_dim 64 and grouped queries, which FMA kernels with natural logarithms used to take): the exponent also gets what
+// the rounding of a normaliser to 32 bits in the log2 domain lost, and the logit's share of scale_lo: what the rounding of
+// the scale lost and what the tensor cores cut off the products, whose partial sums they truncate (DOT_LOSS, measured).
+// Error of the history against 64 bits given the normalisers (2-norm), FMA kernel, without FINE, with it: 16 heads x 64 channels,
+// 1531 tokens 2.46e-7, 2.92e-7, 1.97e-7; four heads to a group, 128 channels, 700 tokens 1.79e-7, 2.31e-7, 1.63e-7.
+// It takes 2 to 4.5 % of the compaction's time (16 x 8 caches of 1025 slots, 32 heads, w 256: 195 -> 203.5 us).
 template <int HD, bool GROUPED>
 __global__ void __launch_bounds__(RG_THREADS, GROUPED ? 1 : 2)
 window_ring_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kc, int heads, int G, int T,
-                      int w, int B, int cap, float scale_log2, const float* __restrict__ lse, vatp_cache c,
+                      int w, int B, int cap, float scale_log2, float scale_lo, const float* __restrict__ lse, vatp_cache c,
                       int32_t* dev_status) {
   extern __shared__ unsigned char smem_raw[];
   constexpr int TILE_BYTES = tile_bytes<HD>, CHUNK_BYTES = chunk_bytes<HD>;
   RingSmem<HD>& sm = *reinterpret_cast<RingSmem<HD>*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  constexpr bool FINE = GROUPED || HD == 64;
   const int u = blockIdx.y, slot0 = blockIdx.x * TILE;
   const int b = u / heads, h = u - b * heads;
   volatile int* abort_flag = &sm.abort_flag;
@@ -1450,7 +1458,10 @@ window_ring_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
       __syncthreads();
       for (int i = tid; i < CHUNK; i += RG_THREADS) {
         const int r = c0 + i, j = T - w + r;
-        sm.nlse[i] = (r < w && j >= 0) ? -__ldg(lse_h + j) * 1.4426950408889634f : -INFINITY;
+        const bool query = r < w && j >= 0;
+        const float l = query ? __ldg(lse_h + j) : 0.f, nl = -l * 1.4426950408889634f;
+        sm.nlse[i] = query ? nl : -INFINITY;
+        if constexpr (FINE) sm.nres[i] = fmaf(-l, 1.4426950408889634f, -nl) - l * 1.925963033e-8f;   // (log2 e - 1.4426950408889634f)
       }
       if (tid == 0) {
         mbar_expect_tx(&sm.bar_ld, CHUNK_BYTES + (it == 0 ? TILE_BYTES : 0));
@@ -1491,10 +1502,15 @@ window_ring_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             float4 nl;
             asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(nl.x), "=f"(nl.y), "=f"(nl.z), "=f"(nl.w) : "r"(lp + 4 * i4));
             const float nls[4] = {nl.x, nl.y, nl.z, nl.w};
+            float4 nr = make_float4(0.f, 0.f, 0.f, 0.f);
+            if constexpr (FINE)
+              asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(nr.x), "=f"(nr.y), "=f"(nr.z), "=f"(nr.w) : "r"(s32(&sm.nres[cs]) + 4 * i4));
+            const float res[4] = {nr.x, nr.y, nr.z, nr.w};
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
               const int i = i4 + k;
-              const float pr = i >= first ? ex2(fmaf(x[i], scale_log2, nls[k])) : 0.f;
+              const float arg = FINE ? fmaf(x[i], scale_log2, fmaf(x[i], scale_lo, res[k])) + nls[k] : fmaf(x[i], scale_log2, nls[k]);
+              const float pr = i >= first ? ex2(arg) : 0.f;
               if constexpr (GROUPED) sum[wave][i] = g == 0 ? pr : sum[wave][i] + pr;
               else x[i] = pr;
             }
@@ -1728,6 +1744,8 @@ cudaError_t launch_prefill_hd(const Shape& s, const void* q, const void* k, cons
                          : cudaLaunchKernelEx(&cfg, prefill_tc_kernel<HD, 2, false>, tm_q, tm_k, a);
 }
 
+// mean relative loss of magnitude of a product of HD channels in the tensor cores' truncating accumulation
+template <int HD> constexpr double DOT_LOSS = HD == 64 ? 6e-8 : 1e-7;
 template <int HD, bool GROUPED>
 cudaError_t launch_ring_hd(const Shape& s, int G, int B, const void* q, const float* lse, const vatp_cache& c, int32_t* dev_status,
                            cudaStream_t st) {
@@ -1744,7 +1762,9 @@ cudaError_t launch_ring_hd(const Shape& s, int G, int B, const void* q, const fl
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   DependentLaunch dl(dim3((cap + TILE - 1) / TILE, s.units), dim3(RG_THREADS), smem, st);
-  return cudaLaunchKernelEx(&dl.cfg, kern, tm_q, tm_kc, s.heads, G, s.T, s.window, B, cap, s.scale * 1.4426950408889634f, lse, c, dev_status);
+  const float scale_log2 = s.scale * 1.4426950408889634f;
+  const float scale_lo = (float)((double)s.scale * 1.4426950408889634 * (1.0 + DOT_LOSS<HD>) - (double)scale_log2);
+  return cudaLaunchKernelEx(&dl.cfg, kern, tm_q, tm_kc, s.heads, G, s.T, s.window, B, cap, scale_log2, scale_lo, lse, c, dev_status);
 }
 
 }  // namespace

@@ -352,3 +352,30 @@ def test_history_of_several_chunks_and_heads(w, heads, kv):
     want = want[..., kept]
     # 32-bit logits and normalisers of size up to 64 in the log2 domain: a few roundings of 2^-19 each
     assert torch.all((ring - want).abs() <= 2.0 ** -16 * want + 1e-30)
+
+
+@pytest.mark.parametrize("d,heads,kv,T,w", [(64, 16, 0, 1531, 256), (64, 8, 2, 700, 100), (128, 8, 2, 700, 100), (128, 32, 8, 900, 300)])
+def test_history_precision_of_head_dim_64_and_grouped_queries(d, heads, kv, T, w):
+    """The rebuilt history against float64 given the normalisers: no coarser than 32-bit arithmetic in natural logarithms."""
+    V = P.vatp()
+    B, hk = T // 2, kv or heads
+    G = heads // hk
+    p = V.make_params(batch=1, heads=heads, kv_heads=kv, seq_len=T, head_dim=d, dtype="bf16", budget=B, indicator="window", window=w)
+    g = torch.Generator(device="cuda").manual_seed(T + d)
+    q, k, v = (torch.randn(1, n, T, d, generator=g, device="cuda").bfloat16() for n in (heads, hk, hk))
+    lse = torch.stack([_probabilities(q[0, h], k[0, h // G], 0, d ** -0.5)[1] for h in range(heads)])[None].float().contiguous()
+    s = (q.double() @ k.double().repeat_interleave(G, 1).transpose(-1, -2)) * d ** -0.5
+    s.masked_fill_(torch.ones(T, T, dtype=torch.bool, device="cuda").triu(1), float("-inf"))
+    want = torch.exp(s - lse[..., None].double())[0].view(hk, G, T, T).mean(1)[:, T - w:]
+    kept = torch.randperm(T, generator=torch.Generator().manual_seed(w))[:B].sort().values.cuda()
+    c, status = V.Cache(p), torch.zeros(1, dtype=torch.int32, device="cuda")
+    ones = torch.ones(1, hk, T, device="cuda")
+    V.vatp_compact_window(p, q, k, v, lse, ones, ones, kept.int().repeat(1, hk, 1).contiguous(), c, dev_status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    ring, want = c.ring[0][:, torch.arange(T - w, T, device="cuda") % w, :B].double(), want[..., kept]
+    # exponents of magnitude 8 to 16 rounded once: 2^-20 / sqrt(12) * ln 2 = 1.9e-7 of a probability, 5e-8 for its exponential and
+    # the factor; a second rounding of that size (of the normaliser) would give 2.7e-7
+    e = float((ring - want).norm() / want.norm())
+    print(f"[history precision] d {d} heads {heads}/{hk}: {e:.3e}")
+    assert e <= 2.1e-7

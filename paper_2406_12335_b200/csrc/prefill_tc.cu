@@ -1375,10 +1375,13 @@ struct RingSmem {
 // 2.5 ms on FMA units, the whole compaction with it now 0.20 ms.
 // FINE (head_dim 64 and grouped queries, which FMA kernels with natural logarithms used to take): the exponent also gets what
 // the rounding of a normaliser to 32 bits in the log2 domain lost, and the logit's share of scale_lo: what the rounding of
-// the scale lost and what the tensor cores cut off the products, whose partial sums they truncate (DOT_LOSS, measured).
+// the scale lost and what the tensor cores cut off the products, whose partial sums they truncate (DOT_LOSS), and the mean
+// error of the special-function unit's exponential (EX2_LOSS, log2; both measured): the window sums add such means up.
 // Error of the history against 64 bits given the normalisers (2-norm), FMA kernel, without FINE, with it: 16 heads x 64 channels,
-// 1531 tokens 2.46e-7, 2.92e-7, 1.97e-7; four heads to a group, 128 channels, 700 tokens 1.79e-7, 2.31e-7, 1.63e-7.
+// 1531 tokens 2.46e-7, 2.92e-7, 1.92e-7; four heads to a group, 128 channels, 700 tokens 1.79e-7, 2.31e-7, 1.38e-7; of the window
+// sums 5.3e-8, 4.4e-8, 3.3e-8 and 3.6e-8, 6.1e-8, 3.4e-8.
 // It takes 2 to 4.5 % of the compaction's time (16 x 8 caches of 1025 slots, 32 heads, w 256: 195 -> 203.5 us).
+constexpr float EX2_LOSS = 7e-8f;
 template <int HD, bool GROUPED>
 __global__ void __launch_bounds__(RG_THREADS, GROUPED ? 1 : 2)
 window_ring_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kc, int heads, int G, int T,
@@ -1461,7 +1464,7 @@ window_ring_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         const bool query = r < w && j >= 0;
         const float l = query ? __ldg(lse_h + j) : 0.f, nl = -l * 1.4426950408889634f;
         sm.nlse[i] = query ? nl : -INFINITY;
-        if constexpr (FINE) sm.nres[i] = fmaf(-l, 1.4426950408889634f, -nl) - l * 1.925963033e-8f;   // (log2 e - 1.4426950408889634f)
+        if constexpr (FINE) sm.nres[i] = fmaf(-l, 1.4426950408889634f, -nl) - l * 1.925963033e-8f + EX2_LOSS;   // (log2 e - 1.4426950408889634f)
       }
       if (tid == 0) {
         mbar_expect_tx(&sm.bar_ld, CHUNK_BYTES + (it == 0 ? TILE_BYTES : 0));
@@ -1745,7 +1748,7 @@ cudaError_t launch_prefill_hd(const Shape& s, const void* q, const void* k, cons
 }
 
 // mean relative loss of magnitude of a product of HD channels in the tensor cores' truncating accumulation
-template <int HD> constexpr double DOT_LOSS = HD == 64 ? 6e-8 : 1e-7;
+template <int HD> constexpr double DOT_LOSS = HD == 64 ? 6e-8 : 1.2e-7;
 template <int HD, bool GROUPED>
 cudaError_t launch_ring_hd(const Shape& s, int G, int B, const void* q, const float* lse, const vatp_cache& c, int32_t* dev_status,
                            cudaStream_t st) {

@@ -374,6 +374,9 @@ def test_history_precision_of_head_dim_64_and_grouped_queries(d, heads, kv, T, w
     torch.cuda.synchronize()
     assert int(status.item()) == 0
     ring, want = c.ring[0][:, torch.arange(T - w, T, device="cuda") % w, :B].double(), want[..., kept]
+    sums = want.sum(1)
+    # their sums: rounded once to 32 bits (up to 3.4e-8), what is left of the means below 1.5e-8
+    assert float((c.acc[0, :, :B].double() - sums).norm() / sums.norm()) <= 3.8e-8
     # exponents of magnitude 8 to 16 rounded once: 2^-20 / sqrt(12) * ln 2 = 1.9e-7 of a probability, 5e-8 for its exponential and
     # the factor; a second rounding of that size (of the normaliser) would give 2.7e-7
     e = float((ring - want).norm() / want.norm())

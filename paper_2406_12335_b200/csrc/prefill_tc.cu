@@ -402,6 +402,7 @@ struct TcArgs {
   int norm;                 // vatp_norm_kind of the value norm
   int side_norm;            // pass 1 reduces the value norms in its side warp (else vnorm_kernel has, before it)
   unsigned* counters;       // [2] next work item of pass 1 / pass 2 (zeroed before pass 1 is launched)
+  float gain;               // head_dim 64: what pass 2's sums come out too large by (mean, relative)
   int wait_first;           // pass 1 was launched as a programmatic dependent (of the kernel that zeroes the counters):
                             // nothing in global memory is touched before griddepcontrol.wait
   float* win_rows;
@@ -419,6 +420,16 @@ struct TcArgs {
 //           lo = max(i, first tile of the window))
 // Softmax warpgroup g takes columns [128 g, 128 g + 128) of every accumulator, i.e. streamed tile
 // 2 c + g of chunk c; the two partial results of a row are combined once per item.
+
+// Mean errors, measured.  DOT_LOSS: a product of HD channels comes out of the tensor cores' truncating accumulation that much
+// smaller in magnitude (relative).  EX2_LOSS: the special-function unit's exponential is that much too small (log2).  SUM_LOSS:
+// so are pass 1's row sums (relative), whose rescaling factors are exponentials too, beyond the exponentials themselves,
+// whose error cancels against pass 2's.  head_dim 64, which an FMA kernel with natural logarithms used to take, makes up for
+// them where that costs nothing: in the scale, in given normalisers, in pass 2's totals, in lse_out, and in the history's
+// exponents.  Error against 64 bits (2-norm, 12 heads x 1531 tokens), FMA kernel, without, with: indicator 7.3e-8, 8.6e-8, 6.4e-8,
+// with a window of 256 7.0e-8, 9.8e-8, 5.8e-8; lse_out 2.9e-8, 4.6e-8, 2.8e-8; the same order from 130 to 3000 tokens.
+template <int HD> constexpr double DOT_LOSS = HD == 64 ? 6e-8 : 1.2e-7;
+constexpr float EX2_LOSS = 7e-8f, SUM_LOSS = 6e-8f;
 
 struct Item {
   int u, tile, c_first, c_count;
@@ -761,10 +772,16 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             a.lse2[(int64_t)u * a.Tpad + tok + TILE] = -INFINITY;
           // (head_dim 64 leaves the rows before a history window alone, head_dim 128 those before its first tile)
           if (a.lse_out && tok < a.T && (HD == 128 || tok >= a.first_row))
-            a.lse_out[(int64_t)(u / a.heads) * a.lse_sb + (int64_t)(u % a.heads) * a.lse_sh + tok] = lse2 * 0.69314718055994531f;
+            a.lse_out[(int64_t)(u / a.heads) * a.lse_sb + (int64_t)(u % a.heads) * a.lse_sh + tok] =
+                HD == 64 ? fmaf(m, 0.69314718055994531f, logf(l)) : lse2 * 0.69314718055994531f;
         } else {
-          const float tot = hsum2(add2(cs[0], cs[1])) + (sm.part_a[pi][0][row] + sm.part_a[pi][1][row]) + sm.part_a[pi][2][row];
+          const float first3 = hsum2(add2(cs[0], cs[1])) + (sm.part_a[pi][0][row] + sm.part_a[pi][1][row]), last = sm.part_a[pi][2][row];
+          float tot = first3 + last;
           mbar_arrive(&sm.comb_empty[pi]);
+          if (HD == 64) {      // a.gain of it less, rounded once
+            const float part = tot - first3;
+            tot += (first3 - (tot - part)) + (last - part) - a.gain * tot;
+          }
           if (tok < a.T && VATP_INB((int64_t)u * a.T + tok, (int64_t)a.units * a.T, a.dev_status)) {
             if (a.G == 1) {
               const int64_t o = (int64_t)u * a.T + tok;
@@ -1313,7 +1330,8 @@ __global__ void __launch_bounds__(VN_THREADS) vnorm_kernel(TcArgs a, const float
       float x = -INFINITY;
       if (i < a.T) {
         const float l = __ldg(lse_in + (int64_t)u * a.T + i);
-        if (i >= a.first_row) x = -l * 1.4426950408889634f;
+        // (log2 e - 1.4426950408889634f = 1.925963e-8)
+        if (i >= a.first_row) x = HD == 64 ? fmaf(-l, 1.4426950408889634f, fmaf(-l, 1.925963033e-8f, EX2_LOSS)) : -l * 1.4426950408889634f;
         if (a.lse_out && a.lse_out != lse_in) a.lse_out[(int64_t)u * a.T + i] = l;
       }
       a.lse2[(int64_t)u * a.Tpad + i] = x;
@@ -1376,12 +1394,11 @@ struct RingSmem {
 // FINE (head_dim 64 and grouped queries, which FMA kernels with natural logarithms used to take): the exponent also gets what
 // the rounding of a normaliser to 32 bits in the log2 domain lost, and the logit's share of scale_lo: what the rounding of
 // the scale lost and what the tensor cores cut off the products, whose partial sums they truncate (DOT_LOSS), and the mean
-// error of the special-function unit's exponential (EX2_LOSS, log2; both measured): the window sums add such means up.
+// error of the special-function unit's exponential (EX2_LOSS): the window sums add such means up.
 // Error of the history against 64 bits given the normalisers (2-norm), FMA kernel, without FINE, with it: 16 heads x 64 channels,
 // 1531 tokens 2.46e-7, 2.92e-7, 1.92e-7; four heads to a group, 128 channels, 700 tokens 1.79e-7, 2.31e-7, 1.38e-7; of the window
 // sums 5.3e-8, 4.4e-8, 3.3e-8 and 3.6e-8, 6.1e-8, 3.4e-8.
 // It takes 2 to 4.5 % of the compaction's time (16 x 8 caches of 1025 slots, 32 heads, w 256: 195 -> 203.5 us).
-constexpr float EX2_LOSS = 7e-8f;
 template <int HD, bool GROUPED>
 __global__ void __launch_bounds__(RG_THREADS, GROUPED ? 1 : 2)
 window_ring_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kc, int heads, int G, int T,
@@ -1668,7 +1685,7 @@ cudaError_t launch_prefill_hd(const Shape& s, const void* q, const void* k, cons
   a.nt = (s.T + TILE - 1) / TILE;
   a.nch = (a.nt + 1) / 2;
   a.Tpad = a.nch * CHUNK;
-  a.scale_log2 = s.scale * 1.4426950408889634f;
+  a.scale_log2 = HD == 64 ? (float)((double)s.scale * 1.4426950408889634 * (1.0 + DOT_LOSS<HD>)) : s.scale * 1.4426950408889634f;
   a.v = static_cast<const __nv_bfloat16*>(v);
   a.sb = s.sb; a.sh = s.sh; a.st = s.st;
   a.lse_sb = s.lse_sb; a.lse_sh = s.lse_sh;
@@ -1705,6 +1722,7 @@ cudaError_t launch_prefill_hd(const Shape& s, const void* q, const void* k, cons
   // The counters are zeroed first, by a one-warp kernel that waits for all earlier work; what follows is its programmatic
   // dependent (see reset_counters_kernel).
   a.wait_first = 1;
+  a.gain = lse_in || attn_out || a.nch == 1 ? 0.f : SUM_LOSS;      // (within one chunk there is hardly anything to rescale)
   DependentLaunch dr(dim3(1), dim3(32), 0, st);
   if ((e = cudaLaunchKernelEx(&dr.cfg, reset_counters_kernel, a.counters)) != cudaSuccess) return e;
   auto value_norms = [&]() {
@@ -1747,8 +1765,6 @@ cudaError_t launch_prefill_hd(const Shape& s, const void* q, const void* k, cons
                          : cudaLaunchKernelEx(&cfg, prefill_tc_kernel<HD, 2, false>, tm_q, tm_k, a);
 }
 
-// mean relative loss of magnitude of a product of HD channels in the tensor cores' truncating accumulation
-template <int HD> constexpr double DOT_LOSS = HD == 64 ? 6e-8 : 1.2e-7;
 template <int HD, bool GROUPED>
 cudaError_t launch_ring_hd(const Shape& s, int G, int B, const void* q, const float* lse, const vatp_cache& c, int32_t* dev_status,
                            cudaStream_t st) {

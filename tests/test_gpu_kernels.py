@@ -382,3 +382,36 @@ def test_history_precision_of_head_dim_64_and_grouped_queries(d, heads, kv, T, w
     e = float((ring - want).norm() / want.norm())
     print(f"[history precision] d {d} heads {heads}/{hk}: {e:.3e}")
     assert e <= 2.1e-7
+
+
+@pytest.mark.parametrize("kv", [0, 3])      # (groups of four: the factor of their mean is exact, a third would be 3e-8 off)
+@pytest.mark.parametrize("T,window", [(130, 0), (300, 100), (700, 0), (1531, 0), (1531, 256), (3000, 100), (3000, 256)])
+def test_head_dim_64_scoring_precision(T, window, kv):
+    """Normalisers and indicators against float64, and the mean error of the indicators: as good as 32-bit arithmetic in
+    natural logarithms gives them."""
+    V = P.vatp()
+    h, d, hk = 12, 64, kv or 12
+    p = V.make_params(batch=1, heads=h, kv_heads=kv, seq_len=T, head_dim=d, dtype="bf16", budget=T // 2, indicator="window" if window else "h2o",
+                      window=window)
+    e_lse, e, mean = [], [], []
+    for seed in range(3):
+        g = torch.Generator(device="cuda").manual_seed(T + seed)
+        q, k, v = (torch.randn(1, n, T, d, generator=g, device="cuda").bfloat16() for n in (h, hk, hk))
+        acc, vnorm, score = (torch.zeros(1, hk, T, device="cuda") for _ in range(3))
+        lse = torch.zeros(1, h, T, device="cuda")
+        status, ws = torch.zeros(1, dtype=torch.int32, device="cuda"), torch.empty(V.vatp_workspace_bytes(p), dtype=torch.uint8, device="cuda")
+        V.vatp_prefill_scores(p, q, k, v, lse_out=lse, attn_acc=acc, vnorm=vnorm, score=score, workspace=ws, dev_status=status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        first = max(T - window, 0) if window else 0
+        rows = [_probabilities(q[0, i], k[0, i * hk // h], first, d ** -0.5) for i in range(h)]
+        want_lse, want = torch.stack([r[1] for r in rows]), torch.stack([r[0].sum(0) for r in rows]).view(hk, h // hk, T).mean(1)
+        e_lse.append(float((lse[0, :, first:].double() - want_lse).norm() / want_lse.norm()))
+        e.append(float((acc[0].double() - want).norm() / want.norm()))
+        mean.append(float(((acc[0].double() - want) / want).mean()))
+    print(f"[scoring precision] T {T} window {window} heads {h}/{hk}: normalisers {sum(e_lse) / 3:.3e} indicators {sum(e) / 3:.3e} mean {sum(mean) / 3:.3e}")
+    # values of 3 to 8, the result's and the logarithm's rounding: up to 1.4e-7 of about 4.5 at the least, up to 2.7e-7 of 8 and more
+    assert sum(e_lse) / 3 <= 4.2e-8
+    # the terms' exponents, of magnitude 4 to 16, are rounded once each (2e-7 of a term, less the more rows are summed) and the sums
+    # in sixteen chains: 5e-8 to 8e-8, of which no more than 4e-8 may be common to all tokens
+    assert sum(e) / 3 <= 9e-8 and abs(sum(mean) / 3) <= 4e-8

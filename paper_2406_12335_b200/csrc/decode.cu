@@ -448,7 +448,8 @@ cudaError_t launch_t(const Shape& s, int B, int F, int R, const vatp_cache& c, c
   if (s.units * split > sms && split < MAX_SPLIT && dyn < 77 * 1024) dyn = 77 * 1024;
   if (dyn > most_dyn) return cudaErrorInvalidConfiguration;
   auto kern = decode_kernel<T, D, WINDOWED>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+  // (the kernel's limit is always the same: another thread's call may be about to launch with a larger size than this one's)
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most_dyn);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(s.units * split);

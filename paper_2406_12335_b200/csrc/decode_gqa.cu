@@ -35,6 +35,7 @@ __device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.c
 
 constexpr int GQ_THREADS = 512;
 constexpr int GQ_WARPS = GQ_THREADS / 32;
+constexpr size_t GQ_MAX_SMEM = 200 * 1024;     // dynamic shared memory of a CTA
 constexpr int GQ_FLY = 8;              // row steps a thread requests before it uses the first
 
 __device__ __forceinline__ float block_max(float x, float* red) {
@@ -400,7 +401,8 @@ template <typename T, int GT, int TPR>
 cudaError_t launch_gqa_t(int units, int G, int d, int split, int seg, size_t smem, int B, int cap, int F, int R, int window, int norm,
                          float scale, const vatp_cache& c, const void* q, const void* k, const void* v, void* out, int32_t* evicted,
                          int32_t* dev_status, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(decode_gqa_kernel<T, GT, TPR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // (always the same limit: another thread's call may be about to launch with a larger size than this one's)
+  cudaError_t e = cudaFuncSetAttribute(decode_gqa_kernel<T, GT, TPR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GQ_MAX_SMEM);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(units * split);
@@ -451,7 +453,7 @@ cudaError_t launch_decode_gqa(int units, int G, int d, int dtype, int B, int F, 
   const int split = units * 4 <= sms ? 4 : (units * 2 <= sms ? 2 : 1);
   const int seg = ((cap + split - 1) / split + 7) / 8 * 8;
   const size_t smem = sizeof(float) * ((size_t)G * seg + (size_t)G * d + (size_t)GQ_WARPS * G * d + (size_t)split * G * d);
-  if (smem > 200 * 1024) return cudaErrorNotSupported;
+  if (smem > GQ_MAX_SMEM) return cudaErrorNotSupported;
   if (dtype == VATP_F32) {
     if (G <= 4) return launch_gqa<float, 4>(units, G, d, split, seg, smem, B, cap, F, R, window, norm, scale, c, q, k, v, out, evicted, dev_status, st);
     if (G <= 8) return launch_gqa<float, 8>(units, G, d, split, seg, smem, B, cap, F, R, window, norm, scale, c, q, k, v, out, evicted, dev_status, st);

@@ -25,6 +25,7 @@ namespace {
 
 constexpr int SEL_THREADS = 1024;
 constexpr int SEL_WARPS = SEL_THREADS / 32;
+constexpr size_t SEL_MAX = 168 * 1024, SEL_CLUSTER_MAX = 185 * 1024;      // dynamic shared memory of a CTA (beside 1 and 42 KB)
 
 // order-preserving map float -> uint32 (larger float = larger key), valid for any sign
 __device__ __forceinline__ uint32_t order_key(float x) {
@@ -463,10 +464,11 @@ cudaError_t launch_select(int units, int T, int B, int F, int R, const float* sc
   // long prompts, few units: the middle range of a unit goes to a cluster of four or two CTAs
   const int sms = device_sm_count();
   const int split = n >= 8192 && B - F - R > 0 ? (units * 4 <= sms ? 4 : (units * 2 <= sms ? 2 : 1)) : 1;
-  if (split > 1) {
-    const int per = ((n + split - 1) / split + 31) / 32 * 32;
-    const size_t cbytes = (size_t)per * sizeof(uint32_t);
-    cudaError_t e = cudaFuncSetAttribute(select_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cbytes);
+  const int per = ((n + split - 1) / split + 31) / 32 * 32;
+  const size_t cbytes = (size_t)per * sizeof(uint32_t);
+  // (a kernel's limit is always the same: another thread's call may be about to launch with a larger size than this one's)
+  if (split > 1 && cbytes <= SEL_CLUSTER_MAX) {
+    cudaError_t e = cudaFuncSetAttribute(select_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_CLUSTER_MAX);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(units * split);
@@ -487,13 +489,13 @@ cudaError_t launch_select(int units, int T, int B, int F, int R, const float* sc
   const int copies = n <= 2048 ? 1 : (n <= 16384 ? 4 : 8);
   const size_t hist_bytes = (size_t)copies * 256 * sizeof(uint32_t);
   const size_t bytes = hist_bytes + (size_t)staged_words(n) * sizeof(uint32_t);
-  const bool staged = bytes <= 168 * 1024;
+  const bool staged = bytes <= SEL_MAX;
   // more units than SMs: CTAs of 512 threads, several to an SM
   const bool half = units > sms;
   auto kern = staged ? (half ? select_kernel<true, 512> : select_kernel<true, 1024>)
                      : (half ? select_kernel<false, 512> : select_kernel<false, 1024>);
   const size_t dyn = staged ? bytes : hist_bytes;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_MAX);
   if (e != cudaSuccess) return e;
   DependentLaunch dl(dim3(units), dim3(half ? 512 : 1024), dyn, st);
   return cudaLaunchKernelEx(&dl.cfg, kern, copies, T, B, F, R, score, kept, dev_status);

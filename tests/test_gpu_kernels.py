@@ -415,3 +415,59 @@ def test_head_dim_64_scoring_precision(T, window, kv):
     # the terms' exponents, of magnitude 4 to 16, are rounded once each (2e-7 of a term, less the more rows are summed) and the sums
     # in sixteen chains: 5e-8 to 8e-8, of which no more than 4e-8 may be common to all tokens
     assert sum(e) / 3 <= 9e-8 and abs(sum(mean) / 3) <= 4e-8
+
+
+@pytest.mark.parametrize("what", ["select", "select_clusters", "fp32_step", "grouped_step"])
+def test_host_threads_with_calls_of_different_sizes(what):
+    """Two threads launch the same kernel with different amounts of shared memory, each on a stream of its own."""
+    import threading
+    V = P.vatp()
+    failed, go = [], threading.Barrier(2)
+
+    def calls(size, stream):
+        with torch.cuda.stream(stream):
+            status = torch.zeros(1, dtype=torch.int32, device="cuda")
+            if what.startswith("select"):
+                T, B = size
+                p = V.make_params(batch=1, heads=2, seq_len=T, head_dim=64, dtype="f32", budget=B)
+                score, kept = torch.rand(1, 2, T, device="cuda"), torch.empty(1, 2, B, dtype=torch.int32, device="cuda")
+                run = lambda: V.vatp_select(p, score, kept, dev_status=status)  # noqa: E731
+            else:
+                kv = 2 if what == "grouped_step" else 0
+                p = V.make_params(batch=1, heads=32, kv_heads=kv, seq_len=2 * size, head_dim=64, dtype="f32", budget=size)
+                c, q = V.Cache(p), torch.zeros(1, 32, 64, device="cuda")
+                c.len.zero_(), c.free_slot.zero_()
+                k, out = torch.zeros(1, kv or 32, 64, device="cuda"), torch.empty(1, 32, 64, device="cuda")
+                run = lambda: V.vatp_decode_step(p, c, q, k, k, out, dev_status=status)  # noqa: E731
+            stream.synchronize()
+            go.wait()
+            try:
+                for _ in range(3000):
+                    run()
+            except V.VatpError as e:
+                failed.append(str(e))
+            stream.synchronize()
+            assert int(status.item()) == 0
+
+    sizes = {"select": ((1500, 100), (8000, 1000)), "select_clusters": ((9000, 1000), (100000, 20000)), "fp32_step": (100, 9000),
+             "grouped_step": (64, 1500)}[what]
+    threads = [threading.Thread(target=calls, args=(s, torch.cuda.Stream())) for s in sizes]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed
+
+
+@pytest.mark.parametrize("T", [189000, 192000])      # a cluster's shared memory holds the first in four parts, not the second
+def test_select_from_a_very_long_prompt(T):
+    from oracle import vatp_oracle as O
+    V = P.vatp()
+    score = torch.rand(1, 2, T, generator=torch.Generator().manual_seed(T))
+    p = V.make_params(batch=1, heads=2, seq_len=T, head_dim=64, dtype="f32", budget=T // 5, n_sink=3, n_recent=100)
+    kept, status = torch.empty(1, 2, T // 5, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    V.vatp_select(p, score.cuda(), kept, dev_status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    for u in range(2):
+        assert kept[0, u].cpu().numpy().tolist() == O.select_keep(score[0, u].numpy(), T // 5, 3, 100).tolist()

@@ -1140,7 +1140,10 @@ cudaError_t launch_hd(const Shape& s, int B, int F, int R, const vatp_cache& c, 
   // many units in flight per warp as fit there, at least two; the per-slot state beside them (1), in the rings' memory
   // after the streaming (2) or in global memory (0).  Only when not even that fits, a whole SM.
   const bool win = s.window > 0;
-  const size_t third_sm = 77 * 1024, half_sm = 111 * 1024, whole_sm = 222 * 1024;   // dynamic bytes, 1 KB of it alignment slack
+  // Dynamic bytes, 1 KB of it alignment slack.  (Two CTAs share 228 KB with 1 KB each for the system and their static arrays: 1376
+  // bytes at most, 2592 with grouped queries, which leaves 113,120 there.  512 caches of 1337 slots, two heads each, w 40, whose
+  // plan came to 113,408: 97.3 us per step with one CTA per SM, 70.2 so.)
+  const size_t third_sm = 77 * 1024, half_sm = (grouped ? 110 : 111) * 1024, whole_sm = 222 * 1024;
   const int groups_per_warp = ((chunk / GROUP) + MW - 1) / MW;
   const bool part_in_ring = grouped && one_unit;                // a warp's partial outputs land in its ring
   const size_t fixed = 1024 + (part_in_ring ? 0 : (size_t)MW * G * HD * 4) + (size_t)G * HD * 4 + (size_t)G * ld * 4;

@@ -109,6 +109,16 @@ def test_host_side_validation(V):
     assert V.lib.vatp_decode_step(C.byref(odd), null, 16, 16, 16, 16, null, null, null) == 1
 
 
+def test_current_stream_without_the_raw_handle(V, monkeypatch):
+    """A torch that does not give out the current stream's raw handle: the public way."""
+    class Stream:
+        cuda_stream = 1234
+    monkeypatch.setattr(V, "_raw_stream", None)
+    monkeypatch.setattr(V.torch.cuda, "current_stream", Stream)
+    assert V._stream() == 1234
+    assert V._stream(Stream()) == 1234
+
+
 def _probe(V, stream, caches, share):
     """One pretend decode launch touching the given (begin, bytes) ranges."""
     n = len(caches)

@@ -64,8 +64,7 @@ attention_fwd_general_kernel(int heads, int T_len, int d, float scale, const T* 
   for (int c = 0; c < FG_MAXC; ++c) {
     const int ch = lane + 32 * c;
     if (ch < d) {
-      if constexpr (sizeof(T) == 2) orow[ch] = __float2bfloat16(acc[c] * inv);
-      else orow[ch] = acc[c] * inv;
+      orow[ch] = acc[c] * inv;
     }
   }
   if (lane == 0) lse[(int64_t)b * lse_sb + (int64_t)h * lse_sh + j] = m + logf(l);
@@ -76,17 +75,11 @@ attention_fwd_general_kernel(int heads, int T_len, int d, float scale, const T* 
 // out: the inputs' dtype, unit (b, h)'s rows at b * osb + h * osh; lse: natural log, unit (b, h) at b * lse_sb + h * lse_sh.
 cudaError_t launch_attention_fwd_general(const Shape& s, int dtype, const void* q, const void* k, const void* v, void* out,
                                          float* lse, cudaStream_t st) {
-  if (s.d > 32 * FG_MAXC) return cudaErrorNotSupported;
+  if (dtype != VATP_F32 || s.d > 32 * FG_MAXC) return cudaErrorNotSupported;      // (bf16: attention_fwd_tc_kernel)
   const dim3 grid((s.T + FG_WARPS - 1) / FG_WARPS, s.units);
-  if (dtype == VATP_F32)
-    attention_fwd_general_kernel<float><<<grid, FG_WARPS * 32, 0, st>>>(
-        s.heads, s.T, s.d, s.scale, static_cast<const float*>(q), static_cast<const float*>(k), static_cast<const float*>(v),
-        s.sb, s.sh, s.st, s.qsb, s.qsh, static_cast<float*>(out), s.osb, s.osh, lse, s.lse_sb, s.lse_sh);
-  else
-    attention_fwd_general_kernel<__nv_bfloat16><<<grid, FG_WARPS * 32, 0, st>>>(
-        s.heads, s.T, s.d, s.scale, static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k),
-        static_cast<const __nv_bfloat16*>(v), s.sb, s.sh, s.st, s.qsb, s.qsh, static_cast<__nv_bfloat16*>(out), s.osb, s.osh, lse,
-        s.lse_sb, s.lse_sh);
+  attention_fwd_general_kernel<float><<<grid, FG_WARPS * 32, 0, st>>>(
+      s.heads, s.T, s.d, s.scale, static_cast<const float*>(q), static_cast<const float*>(k), static_cast<const float*>(v),
+      s.sb, s.sh, s.st, s.qsb, s.qsh, static_cast<float*>(out), s.osb, s.osh, lse, s.lse_sb, s.lse_sh);
   return cudaGetLastError();
 }
 

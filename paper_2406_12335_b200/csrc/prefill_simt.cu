@@ -3,7 +3,7 @@
 // Pass 1 gives every query row its log-sum-exp (the normaliser of Eq. 1); pass 2 recomputes the
 // logits tile by tile and adds exp(s - lse) into per-key sums (Eq. 2, or Eq. 3 when only the last
 // w query rows count), fused with the value norm and the Eq. 4 product.  This is the path for
-// fp32 inputs (tensor cores would round the operands) and for devices without the tensor-core kernels.
+// fp32 inputs (tensor cores would round the operands).
 // No float atomics: the CTAs of a cluster own a tile of rows (pass 1) or of keys (pass 2).
 //
 // Bound by the FMA pipes when there are many tiles, by latency when there are few.  So
@@ -314,11 +314,8 @@ cudaError_t launch_d(const Shape& s, const T* q, const T* k, const T* v, float* 
 cudaError_t launch_prefill_simt(const Shape& s, int dtype, const void* q, const void* k, const void* v, float* lse,
                                 float* attn_acc, float* vnorm, float* score, float* win_rows, cudaStream_t st,
                                 bool lse_given) {
-  if (dtype == VATP_F32)
-    return launch_d<float>(s, (const float*)q, (const float*)k, (const float*)v, lse, attn_acc, vnorm, score, win_rows, st,
-                           lse_given);
-  return launch_d<__nv_bfloat16>(s, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, lse,
-                                 attn_acc, vnorm, score, win_rows, st, lse_given);
+  if (dtype != VATP_F32) return cudaErrorNotSupported;      // (bf16: launch_prefill_tc)
+  return launch_d<float>(s, (const float*)q, (const float*)k, (const float*)v, lse, attn_acc, vnorm, score, win_rows, st, lse_given);
 }
 
 }  // namespace vatp

@@ -400,11 +400,9 @@ struct TcArgs {
   int first_row, ft, wrow0, window;
   int gu;                   // units per scheduling group (their K and Q fit in L2 together)
   int norm;                 // vatp_norm_kind of the value norm
-  int side_norm;            // pass 1 reduces the value norms in its side warp (else vnorm_kernel has, before it)
+  int side_norm;            // pass 1 (or the forward) reduces the value norms in its side warp (else vnorm_kernel does, beside it)
   unsigned* counters;       // [2] next work item of pass 1 / pass 2 (zeroed before pass 1 is launched)
   float gain;               // head_dim 64: what pass 2's sums come out too large by (mean, relative)
-  int wait_first;           // pass 1 was launched as a programmatic dependent (of the kernel that zeroes the counters):
-                            // nothing in global memory is touched before griddepcontrol.wait
   float* win_rows;
 };
 
@@ -530,7 +528,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
-  if (PASS == 1 && a.wait_first) asm volatile("griddepcontrol.wait;" ::: "memory");
+  // pass 1, a programmatic dependent of the kernel that zeroes the counters, touches nothing in global memory before
+  if (PASS == 1) asm volatile("griddepcontrol.wait;" ::: "memory");
 
   // Consumer side of the item FIFO: the itl-th item of this CTA (u < 0 ends the pass, also when the CTA
   // is aborting).  The producer has worked out what the item covers, once for the whole CTA (the index
@@ -971,7 +970,7 @@ attention_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
-  if (a.wait_first) asm volatile("griddepcontrol.wait;" ::: "memory");     // see reset_counters_kernel
+  asm volatile("griddepcontrol.wait;" ::: "memory");     // see reset_counters_kernel
   // pass 2, a programmatic dependent, may set up while this kernel runs
   if (tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
@@ -1721,7 +1720,6 @@ cudaError_t launch_prefill_hd(const Shape& s, const void* q, const void* k, cons
   a.side_norm = (a.ft == 0 || attn_out) && a.norm == VATP_NORM_L1 && !lse_in;
   // The counters are zeroed first, by a one-warp kernel that waits for all earlier work; what follows is its programmatic
   // dependent (see reset_counters_kernel).
-  a.wait_first = 1;
   a.gain = lse_in || attn_out || a.nch == 1 ? 0.f : SUM_LOSS;      // (within one chunk there is hardly anything to rescale)
   DependentLaunch dr(dim3(1), dim3(32), 0, st);
   if ((e = cudaLaunchKernelEx(&dr.cfg, reset_counters_kernel, a.counters)) != cudaSuccess) return e;

@@ -1,4 +1,4 @@
-// Register-tiled fp32 products of two sets of rows (fp32 inputs, and bf16 ones without tensor cores): shared by the scoring
+// Register-tiled fp32 products of two sets of rows (fp32 inputs, and bf16 ones of very large histories): shared by the scoring
 // passes and the history rebuild.  256 threads as 16 x 16, M x M results each; both operands transposed in shared memory.
 #pragma once
 #include "vatp_internal.cuh"

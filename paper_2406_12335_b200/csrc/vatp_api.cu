@@ -131,28 +131,23 @@ vatp_status prefill_impl(const vatp_params* p, const void* q, const void* k, con
       sq.osb = (int64_t)p->heads * sh.T * sh.d;
       e = launch_prefill_tc(sq, q, k, v, ws, lse_out, part, vnorm, score, nullptr, dev_status, st, nullptr, attn_out);
     }
-    for (int g = 0; g < G && e == cudaSuccess && !tc; ++g) {
+    for (int g = 0; g < G && e == cudaSuccess && !tc; ++g) {     // (fp32)
       const char* qg = static_cast<const char*>(q) + (size_t)g * sh.sh * eb;
       float* lse_g = lse_out ? lse_out + (size_t)g * sh.T : nullptr;
       // the fused call: this round's query heads' rows of the attention output (head kvh * G + g of every KV group)
       void* out_g = attn_out ? static_cast<char*>(attn_out) + (size_t)g * sh.T * sh.d * eb : nullptr;
-      if (tc) {
-        e = launch_prefill_tc(sh, qg, k, v, ws, lse_g, part + g * n, vnorm, score, nullptr, dev_status, st, nullptr, out_g);
+      Shape sg = sh;
+      float* lse_buf = lse_g;
+      if (!lse_buf) { lse_buf = ws; sg.lse_sb = (int64_t)sh.heads * sh.T; sg.lse_sh = sh.T; }   // plain [units][T] scratch
+      if (out_g) {
+        e = launch_attention_fwd_general(sg, p->dtype, qg, k, v, out_g, lse_buf, st);
+        if (e == cudaSuccess) e = launch_prefill_simt(sg, p->dtype, qg, k, v, lse_buf, part + g * n, vnorm, score, nullptr, st, true);
       } else {
-        Shape sg = sh;
-        float* lse_buf = lse_g;
-        if (!lse_buf) { lse_buf = ws; sg.lse_sb = (int64_t)sh.heads * sh.T; sg.lse_sh = sh.T; }   // plain [units][T] scratch
-        if (out_g) {
-          e = launch_attention_fwd_general(sg, p->dtype, qg, k, v, out_g, lse_buf, st);
-          if (e == cudaErrorNotSupported) return VATP_ERR_UNSUPPORTED;
-          if (e == cudaSuccess) e = launch_prefill_simt(sg, p->dtype, qg, k, v, lse_buf, part + g * n, vnorm, score, nullptr, st, true);
-        } else {
-          e = launch_prefill_simt(sg, p->dtype, qg, k, v, lse_buf, part + g * n, vnorm, score, nullptr, st);
-        }
+        e = launch_prefill_simt(sg, p->dtype, qg, k, v, lse_buf, part + g * n, vnorm, score, nullptr, st);
       }
     }
     if (e == cudaSuccess) e = launch_group_mean(G, (int64_t)n, part, vnorm, attn_acc, score, st);
-    return e == cudaSuccess ? VATP_OK : VATP_ERR_CUDA;
+    return e == cudaSuccess ? VATP_OK : (e == cudaErrorNotSupported ? VATP_ERR_UNSUPPORTED : VATP_ERR_CUDA);
   }
   if (p->dtype == VATP_BF16 && vatp_tc_available()) {
     e = launch_prefill_tc(sh, q, k, v, ws, lse_out, attn_acc, vnorm, score, win_rows, dev_status, st, lse_in, attn_out);
@@ -161,7 +156,6 @@ vatp_status prefill_impl(const vatp_params* p, const void* q, const void* k, con
     // the workspace in the same layout)
     float* lse_buf = lse_out ? lse_out : ws;
     e = launch_attention_fwd_general(sh, p->dtype, q, k, v, attn_out, lse_buf, st);
-    if (e == cudaErrorNotSupported) return VATP_ERR_UNSUPPORTED;
     if (e == cudaSuccess) e = launch_prefill_simt(sh, p->dtype, q, k, v, lse_buf, attn_acc, vnorm, score, win_rows, st, true);
   } else if (lse_in) {
     // pass 2 of the general kernel reads natural-log normalisers [units][T] directly
@@ -171,7 +165,7 @@ vatp_status prefill_impl(const vatp_params* p, const void* q, const void* k, con
   } else {
     e = launch_prefill_simt(sh, p->dtype, q, k, v, lse_out ? lse_out : ws, attn_acc, vnorm, score, win_rows, st);
   }
-  return e == cudaSuccess ? VATP_OK : VATP_ERR_CUDA;
+  return e == cudaSuccess ? VATP_OK : (e == cudaErrorNotSupported ? VATP_ERR_UNSUPPORTED : VATP_ERR_CUDA);
 }
 
 }  // namespace
@@ -284,7 +278,7 @@ vatp_status vatp_decode_step(const vatp_params* p, const vatp_cache* cache, cons
   if (group_of(p) > 1) {
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     if (p->dtype == VATP_BF16 && group_of(p) <= 8) {
-      // tensor-core step: the group's heads ride in the rows of the MMA tiles, every K and V row is read once
+      // tensor-core step: the group's heads ride in the columns of the MMA tiles, every K and V row is read once
       Shape sh;
       std::memset(&sh, 0, sizeof(sh));
       sh.units = p->batch * kv_heads_of(p);

@@ -56,15 +56,14 @@ def test_head_dim_64_window_leaves_earlier_normalisers_alone():
     (1, 2, 0, 128, 9000, 0),     # state beyond shared memory
     (1, 300, 0, 128, 2048, 30),  # several units per CTA, their state read from global memory in the tail
 ])
-@pytest.mark.parametrize("grow", [0, 5, 190])
+@pytest.mark.parametrize("grow", [0, 5, 190])       # (less where the budget is smaller)
 def test_decode_step_against_float64(b, h, kv, d, B, window, grow):
     """One-step arithmetic of every unit against float64 torch: output rows, indicators, evicted token; grow: the cache
     starts that many tokens short of its budget, so rows requested before the live range is known are dropped."""
     V = P.vatp()
     hk, T = kv or h, 2 * B
     G = h // hk
-    if grow >= B:
-        return
+    grow = min(grow, B - 1)
     p = V.make_params(batch=b, heads=h, kv_heads=kv, seq_len=T, head_dim=d, dtype="bf16", budget=B,
                       indicator="window" if window else "h2o", window=window)
     c, n = V.Cache(p), B - grow
@@ -471,3 +470,45 @@ def test_select_from_a_very_long_prompt(T):
     assert int(status.item()) == 0
     for u in range(2):
         assert kept[0, u].cpu().numpy().tolist() == O.select_keep(score[0, u].numpy(), T // 5, 3, 100).tolist()
+
+
+@pytest.mark.parametrize("d,units,T,window,call,norm,tile", [
+    (64, 49, 700, 0, "scores", "l1", 64),       # 294 rows of 128-row tiles: just below twice 148 SMs
+    (64, 50, 700, 0, "scores", "l1", 128),      # 300: the large tiles, the last of a unit ragged
+    (128, 49, 769, 0, "scores", "l2", 128),     # one row in the last tile
+    (128, 50, 700, 0, "lse", "linf", 128),
+    (64, 150, 500, 200, "scores", "l1", 128),   # history window, which starts inside a tile of keys
+    (128, 99, 530, 257, "lse", "l1", 128),
+    (128, 150, 300, 400, "scores", "l1", 128),  # window longer than the prompt
+])
+def test_fp32_scoring_tiles_against_float64(d, units, T, window, call, norm, tile):
+    """The fp32 passes either side of the line between 64- and 128-row tiles."""
+    V = P.vatp()
+    rows = window if 0 < window < T else T
+    assert (tile == 128) == (units * ((rows + 127) // 128) >= 2 * 148)
+    p = V.make_params(batch=1, heads=units, seq_len=T, head_dim=d, dtype="f32", budget=T // 2, indicator="window" if window else "h2o",
+                      window=window, norm=norm)
+    g = torch.Generator(device="cuda").manual_seed(T + d)
+    q, k, v = (torch.randn(1, units, T, d, generator=g, device="cuda") for _ in range(3))
+    first = max(T - window, 0) if window else 0
+    ref = [_probabilities(q[0, i], k[0, i], first, d ** -0.5) for i in range(units)]
+    want, want_lse = torch.stack([r[0].sum(0) for r in ref]), torch.stack([r[1] for r in ref])
+    acc, vnorm, score, lse = (torch.zeros(1, units, T, device="cuda") for _ in range(4))
+    status, ws = torch.zeros(1, dtype=torch.int32, device="cuda"), torch.empty(V.vatp_workspace_bytes(p), dtype=torch.uint8, device="cuda")
+    to = dict(attn_acc=acc, vnorm=vnorm, score=score, workspace=ws, dev_status=status)
+    if call == "lse":
+        given = torch.zeros_like(lse)
+        given[0, :, first:] = want_lse.float()
+        V.vatp_prefill_scores_from_lse(p, q, k, v, given, lse_out=lse, **to)
+        assert torch.equal(lse, given)
+    else:
+        V.vatp_prefill_scores(p, q, k, v, lse_out=lse, **to)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    tol = P.TOL["f32"]
+    assert torch.all((lse[0, :, first:].double() - want_lse).abs() <= 10 * tol)
+    assert torch.all(lse[0, :, :first] == 0)
+    assert torch.all((acc[0].double() - want).abs() <= tol * want)
+    n = v[0].double().norm(p={"l1": 1, "l2": 2, "linf": float("inf")}[norm], dim=-1)
+    assert torch.all((vnorm[0].double() - n).abs() <= tol * n)
+    assert torch.equal(score, acc * vnorm)

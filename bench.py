@@ -220,7 +220,7 @@ class LayerState:
 def prune_launches(wl, args):
     """Kernels of this library that one layer's scoring + selection + compaction launches (memsets not counted)."""
     windowed = wl.indicator == "window"
-    tensor_core = wl.dtype == "bf16" and wl.head_dim == 128
+    tensor_core = wl.dtype == "bf16"
     if tensor_core:
         # counter reset, pass 1 unless the normalisers are given, the norm kernel (Eq. 2 with the l1 norm: the side warp of
         # pass 1 instead), pass 2

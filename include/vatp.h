@@ -128,7 +128,8 @@ size_t vatp_workspace_bytes(const vatp_params* params);
  *           j >= max(T - w, k) (Eq. 3, last w queries); QK^T is recomputed, never stored
  *   vnorm[k] = sum_c |v[k][c]|,  score[k] = attn_acc[k] * vnorm[k]     (Eq. 4)
  * q, k, v: inputs as described above (read only).
- * lse_out:  [batch, heads, T] fp32 output (natural log), nullable.
+ * lse_out:  [batch, heads, T] fp32 output (natural log), nullable.  With VATP_IND_WINDOW its rows j >= T - w are the
+ *           output; earlier rows are left alone or receive their normalisers (which of them depends on the kernel).
  * attn_acc, vnorm, score: [batch, heads, T] fp32 outputs.
  * win_rows: VATP_IND_WINDOW only, nullable: [batch, heads, w, T] fp32 output, row r = probabilities
  *           of query T - w + r (zero where masked or where T - w + r < 0), for vatp_compact.  NULL

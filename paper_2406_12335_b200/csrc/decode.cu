@@ -479,7 +479,7 @@ cudaError_t launch_decode(const Shape& s, int dtype, int B, int F, int R, const 
     const cudaError_t e = launch_decode_mma(s, B, F, R, c, q, k, v, out, evicted, dev_status, st, may_overlap);
     if (e != cudaErrorNotSupported) return e;
   }
-  decode_history_forget(st);     // the general kernel is an ordinary launch: the record of overlapping launches ends here
+  decode_history_forget(st);     // the general kernel waits for all earlier work: the record of overlapping launches ends here
 #define VATP_DISPATCH(T, D)                                                                         \
   return win ? launch_t<T, D, true>(s, B, F, R, c, q, k, v, out, evicted, dev_status, st)           \
              : launch_t<T, D, false>(s, B, F, R, c, q, k, v, out, evicted, dev_status, st)

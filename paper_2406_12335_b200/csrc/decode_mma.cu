@@ -29,8 +29,8 @@
 //     of its own slots and sends its eviction candidate to rank 0, which picks.  No global scratch, one launch;
 //   * consecutive steps overlap (programmatic dependent launch).  By default a step requests
 //     K/V tiles early and reads everything else only after all earlier work in the stream has
-//     completed; it releases the next launch once that wait is over, so at most one
-//     unfinished predecessor exists while a step sets up, and the one cache row that predecessor
+//     completed; it releases the next launch after that wait (at once with a producer warp, else when its K rows are
+//     in), so at most one unfinished predecessor exists while a step sets up, and the one cache row that predecessor
 //     may have written - the row of its incoming token, recorded in last_slot - is re-read after
 //     the wait and patched in.  A caller that steps several independent caches on one stream may
 //     opt in (VATP_FLAG_DECODE_OVERLAP) to more: the host keeps, per stream, the buffers of the
@@ -43,7 +43,7 @@
 //     a group-wise score, read here as the MEAN of the heads' probabilities): up to eight heads of a group ride
 //     in the columns of the products (template parameter GT), so a K or V row is still read once per step.
 // Measured (us per step, first and latest version): 32 units x 2049 slots, every launch waiting 12.5 -> 9.15; 256 units x
-// 1639, launches overlapping 38 -> 33.4 (215 MB: 6.4 TB/s of the 6.56 a copy reaches); 512 units x 1025 with a history window
+// 1639, launches overlapping 37 -> 32.5 (221 MB: 6.8 TB/s; a copy reaches 6.5); 512 units x 1025 with a history window
 // 73 -> 55; 8 units x 2049, four heads each 11.0 -> 8.9.
 #include <cooperative_groups.h>
 

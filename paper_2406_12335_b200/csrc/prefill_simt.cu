@@ -12,8 +12,13 @@
 //     where one element per load made it 8 per 16.  The next tile's rows are on their way to registers under the products (M = 4);
 //   * few tiles are shared out over a cluster of up to eight CTAs along the other dimension, which combine their row
 //     statistics or column sums through distributed shared memory;
-//   * both passes are programmatic dependents: they are resident when the launch before them ends.
-// 2 heads x 512 tokens x 64 channels, scoring + selection + compaction: 93 -> 34 us.
+//   * both passes are programmatic dependents: they are resident when the launch before them ends, and pass 2 has its first
+//     tiles and the value norms by then, which depend on nothing that pass 1 writes;
+//   * the CTAs of a cluster push their partial results to rank 0 and meet once: with rank 0 reading them from its partners
+//     there were two meetings and a round trip between them.  Both operands of the first product travel together, and the 16
+//     threads of a row agree on its maximum before they exponentiate.
+// The scoring call, 2 heads x 512 tokens x 64 channels: 20.1 us before the last two points, 15.9 now; 12 heads of 128, 512 tokens,
+// a window of 256: 58.5 -> 51.7; 8 heads x 700 x 64: 67.5 -> 64.3.  128 x 128 tiles (32 heads x 2048 x 128) do not care: 974 us.
 #include <cooperative_groups.h>
 
 #include "simt_tile.cuh"
@@ -25,6 +30,11 @@ namespace {
 
 constexpr int MAX_CLUSTER = 8;
 
+// The CTAs of a cluster send what they have to rank 0's shared memory, which must have been claimed by then: every CTA
+// announces itself at once and waits for the others only when it sends, long after.
+__device__ __forceinline__ void cluster_announce() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_all_there() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
+
 // Pass 1: one cluster per (query tile, unit), its CTAs take every cs-th key tile.  lse[j] over keys i <= j.
 template <typename T, int M, int D>
 __global__ void __launch_bounds__(NTHREADS, M == 8 ? 2 : 1) rowstats_kernel(Shape sh, const T* __restrict__ q, const T* __restrict__ k,
@@ -33,7 +43,8 @@ __global__ void __launch_bounds__(NTHREADS, M == 8 ? 2 : 1) rowstats_kernel(Shap
   extern __shared__ __align__(16) float smem[];
   float* Qs = smem;
   float* Ks = smem + D * LD;
-  __shared__ float2 part[ROWS];
+  __shared__ float2 part[M == 4 ? MAX_CLUSTER : 1][ROWS];      // (M = 8 has tiles enough without clusters)
+  if (cs > 1) cluster_announce();
   // nothing is read before all earlier work has completed; pass 2 may set up from then on
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -51,14 +62,14 @@ __global__ void __launch_bounds__(NTHREADS, M == 8 ? 2 : 1) rowstats_kernel(Shap
   float m[M], l[M];
 #pragma unroll
   for (int i = 0; i < M; ++i) { m[i] = -INFINITY; l[i] = 0.f; }
+  [[maybe_unused]] float4 next[M == 4 ? NV : 1];
   {
     float4 r[NV];
     Tile<M, D>::fetch(r, qu, sh.st, q0, min(ROWS, sh.T - q0));
+    if constexpr (M == 4)      // (on its way together with the queries)
+      if (rank * ROWS < last_key) Tile<M, D>::fetch(next, ku, sh.st, rank * ROWS, min(ROWS, sh.T - rank * ROWS));
     Tile<M, D>::store(Qs, r);
   }
-  [[maybe_unused]] float4 next[M == 4 ? NV : 1];
-  if constexpr (M == 4)
-    if (rank * ROWS < last_key) Tile<M, D>::fetch(next, ku, sh.st, rank * ROWS, min(ROWS, sh.T - rank * ROWS));
   for (int k0 = rank * ROWS; k0 < last_key; k0 += cs * ROWS) {
     float s[M][M];
     if constexpr (M == 4) {
@@ -90,33 +101,30 @@ __global__ void __launch_bounds__(NTHREADS, M == 8 ? 2 : 1) rowstats_kernel(Shap
       }
     }
   }
-  // merge the 16 threads (same ty, consecutive lanes) that share each row
+  // merge the 16 threads (same ty, consecutive lanes) that share each row: the maximum first, then one factor a thread
+  if (cs > 1) cluster_all_there();
 #pragma unroll
   for (int i = 0; i < M; ++i) {
+    float mx = m[i];
 #pragma unroll
-    for (int off = 8; off >= 1; off >>= 1) {
-      const float m2 = __shfl_xor_sync(0xffffffffu, m[i], off);
-      const float l2 = __shfl_xor_sync(0xffffffffu, l[i], off);
-      const float mn = fmaxf(m[i], m2);
-      if (mn > -INFINITY) {
-        l[i] = l[i] * expf(m[i] - mn) + l2 * expf(m2 - mn);
-        m[i] = mn;
-      }
-    }
+    for (int off = 8; off >= 1; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+    float sum = m[i] > -INFINITY ? l[i] * expf(m[i] - mx) : 0.f;
+#pragma unroll
+    for (int off = 8; off >= 1; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
     const int at = micro_at<M>(ty, i);
     if (tx == 0) {
-      if (cs > 1) part[at] = make_float2(m[i], l[i]);
-      else if (q0 + at < sh.T) lse[unit_offset_lse(sh, u) + q0 + at] = m[i] + logf(l[i]);
+      if (cs > 1) cluster.map_shared_rank(&part[0][0], 0)[(M == 4 ? rank : 0) * ROWS + at] = make_float2(mx, sum);
+      else if (q0 + at < sh.T) lse[unit_offset_lse(sh, u) + q0 + at] = mx + logf(sum);
     }
   }
   if (cs > 1) {
-    cluster.sync();
+    cluster.sync();       // (nobody reads another CTA's shared memory after it)
     if (rank == 0 && (int)threadIdx.x < ROWS && q0 + (int)threadIdx.x < sh.T) {
       float2 p[MAX_CLUSTER];
       float mx = -INFINITY, sum = 0.f;
 #pragma unroll
       for (int r = 0; r < MAX_CLUSTER; ++r) {
-        p[r] = r < cs ? cluster.map_shared_rank(part, r)[threadIdx.x] : make_float2(-INFINITY, 0.f);
+        p[r] = r < cs ? part[M == 4 ? r : 0][threadIdx.x] : make_float2(-INFINITY, 0.f);
         mx = fmaxf(mx, p[r].x);
       }
 #pragma unroll
@@ -124,7 +132,6 @@ __global__ void __launch_bounds__(NTHREADS, M == 8 ? 2 : 1) rowstats_kernel(Shap
         if (p[r].x > -INFINITY) sum += p[r].y * expf(p[r].x - mx);
       lse[unit_offset_lse(sh, u) + q0 + threadIdx.x] = mx + logf(sum);
     }
-    cluster.sync();       // nobody leaves while rank 0 reads
   }
 }
 
@@ -134,7 +141,7 @@ template <typename T, int M, int D>
 __global__ void __launch_bounds__(NTHREADS, M == 8 ? 2 : 1)
 colsum_kernel(Shape sh, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
               const float* __restrict__ lse, float* __restrict__ attn_acc, float* __restrict__ vnorm,
-              float* __restrict__ score, float* __restrict__ win_rows, int first_row, int cs) {
+              float* __restrict__ score, float* __restrict__ win_rows, int first_row, int cs, bool after_pass1) {
   constexpr int ROWS = Tile<M, D>::ROWS, LD = Tile<M, D>::LD, NV = Tile<M, D>::NV;
   extern __shared__ __align__(16) float smem[];
   constexpr int DS = M == 4 ? D : 64;   // channels of the streamed tile in shared memory at a time
@@ -142,7 +149,8 @@ colsum_kernel(Shape sh, const T* __restrict__ q, const T* __restrict__ k, const 
   float* Qs = smem + D * LD;
   float* lse_s = Qs + DS * LD;          // [ROWS]
   float* red = Qs;                      // [16][ROWS], once the products are done (DS >= 16)
-  __shared__ float vn_s[ROWS], part[ROWS];
+  __shared__ float vn_s[ROWS], part[M == 4 ? MAX_CLUSTER : 1][ROWS];
+  if (cs > 1) cluster_announce();
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = cs > 1 ? (int)cluster.block_rank() : 0;
   const int item = blockIdx.x / cs, u = item % sh.units;      // the longest columns of all units first
@@ -153,22 +161,47 @@ colsum_kernel(Shape sh, const T* __restrict__ q, const T* __restrict__ k, const 
   const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
   const int keys_valid = min(ROWS, sh.T - k0);
   if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  // Everything this pass reads but the normalisers was complete before pass 1 released it; without a pass 1 before it
-  // (normalisers given) it waits first.
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-
-  {
-    float4 r[NV];
-    Tile<M, D>::fetch(r, ku, sh.st, k0, keys_valid);
-    Tile<M, D>::store(Ks, r);
-  }
-  float cs_sum[M];
-#pragma unroll
-  for (int j = 0; j < M; ++j) cs_sum[j] = 0.f;
+  // Everything this pass reads but the normalisers was complete before pass 1 released it: the first tiles and the value
+  // norms do not wait for pass 1.  Without a pass 1 before it (normalisers given) it waits first.
+  if (!after_pass1) asm volatile("griddepcontrol.wait;" ::: "memory");
 
   // query tiles are aligned to first_row so that window rows map to whole tiles
   int qstart = first_row;
   if (k0 > first_row) qstart = first_row + ((k0 - first_row) / ROWS) * ROWS;
+  const int qfirst = qstart + rank * ROWS;
+  [[maybe_unused]] float4 next[M == 4 ? NV : 1];
+  {
+    float4 r[NV];
+    Tile<M, D>::fetch(r, ku, sh.st, k0, keys_valid);
+    if constexpr (M == 4)
+      if (qfirst < sh.T) Tile<M, D>::fetch(next, qu, sh.st, qfirst, min(ROWS, sh.T - qfirst));
+    Tile<M, D>::store(Ks, r);
+  }
+  // value norms (Eq. 4): four threads per row, by the last CTA of the cluster, which has the fewest query tiles
+  auto value_norms = [&]() {
+    if (rank != cs - 1) return;
+    for (int r = threadIdx.x / 4; r < ROWS; r += NTHREADS / 4) {
+      const int part4 = threadIdx.x % 4;
+      float acc = 0.f;
+      if (r < keys_valid) {
+        const T* p = vu + (int64_t)(k0 + r) * sh.st;
+#pragma unroll 4
+        for (int c = part4 * 4; c < D; c += 16) {
+          const float4 x = load4(p + c);
+          acc = norm_fold(sh.norm, norm_fold(sh.norm, norm_fold(sh.norm, norm_fold(sh.norm, acc, x.x), x.y), x.z), x.w);
+        }
+      }
+      acc = norm_merge(sh.norm, acc, __shfl_xor_sync(0xffffffffu, acc, 1));
+      acc = norm_merge(sh.norm, acc, __shfl_xor_sync(0xffffffffu, acc, 2));
+      if (part4 == 0) vn_s[r] = norm_finish(sh.norm, acc);
+    }
+  };
+  if constexpr (M == 4) value_norms();      // (M = 8, whose launches fill the machine anyway: behind the products)
+  float cs_sum[M];
+#pragma unroll
+  for (int j = 0; j < M; ++j) cs_sum[j] = 0.f;
+  if (after_pass1) asm volatile("griddepcontrol.wait;" ::: "memory");
+
   const int wrow0 = sh.T - sh.window;   // query position of win_rows row 0 (may be negative)
   float* wr = win_rows ? win_rows + (int64_t)u * sh.window * sh.T : nullptr;
 
@@ -181,10 +214,6 @@ colsum_kernel(Shape sh, const T* __restrict__ q, const T* __restrict__ k, const 
       for (int c = threadIdx.x; c < keys_valid; c += NTHREADS) wr[(int64_t)r * sh.T + k0 + c] = 0.f;
   }
 
-  [[maybe_unused]] float4 next[M == 4 ? NV : 1];
-  const int qfirst = qstart + rank * ROWS;
-  if constexpr (M == 4)
-    if (qfirst < sh.T) Tile<M, D>::fetch(next, qu, sh.st, qfirst, min(ROWS, sh.T - qfirst));
   for (int q0 = qfirst; q0 < sh.T; q0 += cs * ROWS) {
     const int rows_valid = min(ROWS, sh.T - q0);
     // (s[i][j]: key k0 + micro_at(ty, i), query q0 + micro_at(tx, j))
@@ -216,24 +245,7 @@ colsum_kernel(Shape sh, const T* __restrict__ q, const T* __restrict__ k, const 
       }
     }
   }
-  // value norms (Eq. 4): four threads per row, by the last CTA of the cluster, which has the fewest query tiles
-  if (rank == cs - 1) {
-    for (int r = threadIdx.x / 4; r < ROWS; r += NTHREADS / 4) {
-      const int part4 = threadIdx.x % 4;
-      float acc = 0.f;
-      if (r < keys_valid) {
-        const T* p = vu + (int64_t)(k0 + r) * sh.st;
-#pragma unroll 4
-        for (int c = part4 * 4; c < D; c += 16) {
-          const float4 x = load4(p + c);
-          acc = norm_fold(sh.norm, norm_fold(sh.norm, norm_fold(sh.norm, norm_fold(sh.norm, acc, x.x), x.y), x.z), x.w);
-        }
-      }
-      acc = norm_merge(sh.norm, acc, __shfl_xor_sync(0xffffffffu, acc, 1));
-      acc = norm_merge(sh.norm, acc, __shfl_xor_sync(0xffffffffu, acc, 2));
-      if (part4 == 0) vn_s[r] = norm_finish(sh.norm, acc);
-    }
-  }
+  if constexpr (M == 8) value_norms();
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < M; ++i) red[tx * ROWS + micro_at<M>(ty, i)] = cs_sum[i];
@@ -242,26 +254,28 @@ colsum_kernel(Shape sh, const T* __restrict__ q, const T* __restrict__ k, const 
   if ((int)threadIdx.x < ROWS) {
 #pragma unroll
     for (int t = 0; t < 16; ++t) tot += red[t * ROWS + threadIdx.x];
-    part[threadIdx.x] = tot;
   }
-  if (cs > 1) cluster.sync(); else __syncthreads();
+  if (cs > 1) {
+    cluster_all_there();
+    if ((int)threadIdx.x < ROWS) {
+      cluster.map_shared_rank(&part[0][0], 0)[(M == 4 ? rank : 0) * ROWS + threadIdx.x] = tot;
+      if (rank == cs - 1) cluster.map_shared_rank(vn_s, 0)[threadIdx.x] = vn_s[threadIdx.x];
+    }
+    cluster.sync();       // (nobody reads another CTA's shared memory after it)
+  }
   if (rank == 0 && (int)threadIdx.x < keys_valid) {
-    float n1 = 0.f;
     if (cs > 1) {
       tot = 0.f;
 #pragma unroll
       for (int r = 0; r < MAX_CLUSTER; ++r)
-        if (r < cs) tot += cluster.map_shared_rank(part, r)[threadIdx.x];
-      n1 = cluster.map_shared_rank(vn_s, cs - 1)[threadIdx.x];
-    } else {
-      n1 = vn_s[threadIdx.x];
+        if (r < cs) tot += part[M == 4 ? r : 0][threadIdx.x];
     }
+    const float n1 = vn_s[threadIdx.x];
     const int64_t o = (int64_t)u * sh.T + k0 + threadIdx.x;
     attn_acc[o] = tot;
     vnorm[o] = n1;
     score[o] = tot * n1;
   }
-  if (cs > 1) cluster.sync();       // nobody leaves while rank 0 reads
 }
 
 template <typename T, int M, int D>
@@ -288,7 +302,7 @@ cudaError_t launch_m(const Shape& s, const T* q, const T* k, const T* v, float* 
   const int cs = cluster_for(ktiles, qtiles);
   ClusterLaunch c2(dim3((unsigned)(ktiles * s.units * cs)), smem2, st, cs);
   return cudaLaunchKernelEx(&c2.cfg, colsum_kernel<T, M, D>, s, q, k, v, (const float*)lse, attn_acc, vnorm, score,
-                            s.window > 0 ? win_rows : nullptr, first_row, cs);
+                            s.window > 0 ? win_rows : nullptr, first_row, cs, !lse_given);
 }
 
 template <typename T, int D>

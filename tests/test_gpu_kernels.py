@@ -512,3 +512,44 @@ def test_fp32_scoring_tiles_against_float64(d, units, T, window, call, norm, til
     n = v[0].double().norm(p={"l1": 1, "l2": 2, "linf": float("inf")}[norm], dim=-1)
     assert torch.all((vnorm[0].double() - n).abs() <= tol * n)
     assert torch.equal(score, acc * vnorm)
+
+
+@pytest.mark.parametrize("d,units,T,window", [
+    (64, 1, 1, 0),          # one token
+    (64, 1, 64, 0),         # one tile, no cluster
+    (64, 3, 65, 0),         # two tiles, one row in the second
+    (128, 2, 200, 0),       # clusters of four
+    (64, 2, 513, 0),        # clusters of eight, more CTAs than the first rows have key tiles
+    (128, 1, 700, 33),      # a window of less than a tile: pass 1 in one cluster a unit
+    (64, 9, 449, 0),        # clusters of two
+])
+def test_fp32_scoring_right_behind_the_inputs(d, units, T, window):
+    """The fp32 passes with clusters of every size, enqueued right behind the kernels that write their inputs, over and over:
+    pass 2 fetches its first tiles before pass 1 has finished, and the CTAs of a cluster send their parts to one of them."""
+    V = P.vatp()
+    p = V.make_params(batch=1, heads=units, seq_len=T, head_dim=d, dtype="f32", budget=T, indicator="window" if window else "h2o",
+                      window=window)
+    f32 = dict(dtype=torch.float32, device="cuda")
+    g = torch.Generator(device="cuda").manual_seed(17)
+    sets = [torch.randn(3, 1, units, T, d, generator=g, **f32) for _ in range(4)]
+    x = torch.empty_like(sets[0])
+    out = torch.zeros(4, 4, 1, units, T, **f32)
+    ws = torch.empty(max(V.vatp_workspace_bytes(p), 256), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for i in range(4):
+        x.copy_(sets[i])
+        V.vatp_prefill_scores(p, x[0], x[1], x[2], lse_out=out[i, 0], attn_acc=out[i, 1], vnorm=out[i, 2], score=out[i, 3], workspace=ws,
+                              dev_status=status)
+    torch.cuda.synchronize()
+    assert int(status) == 0
+    first = T - window if window else 0
+    for i in range(4):
+        q, k, v = sets[i].double()
+        s = (q @ k.transpose(-1, -2)) * p.scale
+        s.masked_fill_(torch.ones(T, T, dtype=torch.bool, device="cuda").triu(1), -torch.inf)
+        acc = torch.softmax(s, -1)[..., first:, :].sum(-2)
+        norm = v.abs().sum(-1)
+        tol = P.TOL["f32"]
+        assert (out[i, 0].double() - torch.logsumexp(s, -1))[..., first:].abs().max() <= 10 * tol
+        for got, want in ((out[i, 1], acc), (out[i, 2], norm), (out[i, 3], acc * norm)):
+            assert ((got.double() - want).abs() <= tol * want + 1e-30).all()

@@ -37,7 +37,7 @@ __device__ __forceinline__ void cluster_all_there() { asm volatile("barrier.clus
 
 // Pass 1: one cluster per (query tile, unit), its CTAs take every cs-th key tile.  lse[j] over keys i <= j.
 template <typename T, int M, int D>
-__global__ void __launch_bounds__(NTHREADS, M == 8 ? 2 : 1) rowstats_kernel(Shape sh, const T* __restrict__ q, const T* __restrict__ k,
+__global__ void __launch_bounds__(NTHREADS, M == 8 ? 2 : 1) rowstats_kernel(Shape sh, const T* q, const T* k,
                                                             float* __restrict__ lse, int first_row, int cs) {
   constexpr int ROWS = Tile<M, D>::ROWS, LD = Tile<M, D>::LD, NV = Tile<M, D>::NV;
   extern __shared__ __align__(16) float smem[];
@@ -139,8 +139,7 @@ __global__ void __launch_bounds__(NTHREADS, M == 8 ? 2 : 1) rowstats_kernel(Shap
 // j >= max(first_row, k).
 template <typename T, int M, int D>
 __global__ void __launch_bounds__(NTHREADS, M == 8 ? 2 : 1)
-colsum_kernel(Shape sh, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
-              const float* __restrict__ lse, float* __restrict__ attn_acc, float* __restrict__ vnorm,
+colsum_kernel(Shape sh, const T* q, const T* k, const T* v, const float* lse, float* __restrict__ attn_acc, float* __restrict__ vnorm,
               float* __restrict__ score, float* __restrict__ win_rows, int first_row, int cs, bool after_pass1) {
   constexpr int ROWS = Tile<M, D>::ROWS, LD = Tile<M, D>::LD, NV = Tile<M, D>::NV;
   extern __shared__ __align__(16) float smem[];
@@ -161,8 +160,9 @@ colsum_kernel(Shape sh, const T* __restrict__ q, const T* __restrict__ k, const 
   const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
   const int keys_valid = min(ROWS, sh.T - k0);
   if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  // Everything this pass reads but the normalisers was complete before pass 1 released it: the first tiles and the value
-  // norms do not wait for pass 1.  Without a pass 1 before it (normalisers given) it waits first.
+  // Everything this pass reads but the normalisers was complete before pass 1, which waits itself, released it: the first
+  // tiles do not wait for pass 1, nor with 64-row tiles the value norms.  Without a pass 1 before it (normalisers given) it
+  // waits first.  The normalisers are written while this kernel is resident: see DependentLaunch for how they may be loaded.
   if (!after_pass1) asm volatile("griddepcontrol.wait;" ::: "memory");
 
   // query tiles are aligned to first_row so that window rows map to whole tiles

@@ -86,7 +86,11 @@ bool make_row_gather_map(CUtensorMap* m, const void* base, uint32_t row_words, u
 
 // Launch configuration of a kernel that may be scheduled before the previous launch in the stream has
 // drained (programmatic dependent launch).  Such a kernel executes griddepcontrol.wait before it reads
-// anything an earlier launch wrote.
+// anything that an earlier launch may still be writing.  (Where the launch right before it executes its own wait before it
+// releases its dependents, everything older is complete by the time that this kernel starts, and needs no wait.)
+// What it reads it reads by ordinary loads: the read-only path - __ldg, or a `const ... __restrict__` parameter, for which the
+// compiler may take it - is for memory that nobody writes while the kernel is resident, and nothing holds such a load
+// behind the wait.
 struct DependentLaunch {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];

@@ -50,8 +50,7 @@ __device__ __forceinline__ bool cb_wait(uint64_t* bar, uint32_t parity) {
 // describe, and full batches are fetched with four-row gathers.
 __global__ void __launch_bounds__(CB_THREADS, 1)
 compact_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, int64_t gather_rs,
-               Shape sh, int elem_bytes, int B, int cap, const char* __restrict__ k, const char* __restrict__ v,
-               const float* __restrict__ attn_acc, const float* __restrict__ vnorm, const int32_t* __restrict__ kept,
+               Shape sh, int elem_bytes, int B, int cap, const char* k, const char* v, const float* attn_acc, const float* vnorm, const int32_t* kept,
                vatp_cache c, int rows_pb, int nbuf, int release, int32_t* dev_status) {
   extern __shared__ __align__(128) unsigned char cb_smem[];
   __shared__ __align__(8) uint64_t bars[CB_WARPS][CB_MAXBUF];
@@ -85,7 +84,7 @@ compact_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     const int s0 = (int)(bi - (int64_t)u * nb) * rows_pb;
     const int s = s0 + l16;                                       // this lane's destination slot
     int src = -1;
-    if (l16 < rows_pb && s < len) src = __ldg(kept + (int64_t)u * B + s);
+    if (l16 < rows_pb && s < len) src = kept[(int64_t)u * B + s];
     const int live = min(max(len - s0, 0), rows_pb);              // rows of the batch that hold a token
     uint64_t* bar = &bars[wid][slot];
     if (live > 0) {
@@ -123,9 +122,10 @@ compact_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     // per-slot decode state, and the unit's scalars with its first slot
     if (lane < rows_pb && s < cap && VATP_INB((int64_t)u * cap + s, (int64_t)sh.units * cap, dev_status)) {
       const int64_t o = (int64_t)u * cap + s;
+      const float a = src >= 0 ? attn_acc[(int64_t)u * sh.T + src] : 0.f, n = src >= 0 ? vnorm[(int64_t)u * sh.T + src] : 0.f;
       c.pos[o] = src;
-      c.acc[o] = src >= 0 ? __ldg(attn_acc + (int64_t)u * sh.T + src) : 0.f;
-      c.vnorm[o] = src >= 0 ? __ldg(vnorm + (int64_t)u * sh.T + src) : 0.f;
+      c.acc[o] = a;
+      c.vnorm[o] = n;
       if (s == 0) {
         c.len[u] = len;
         c.free_slot[u] = len;

@@ -383,18 +383,19 @@ decode_gqa_kernel(int G, int d, int B, int cap, int F, int R, int w, int norm, f
 }
 
 // attn_acc[u][t] = mean over the group's G partial indicators; score = that mean times the value norm (Eq. 4)
-__global__ void group_mean_kernel(int G, int64_t n, const float* __restrict__ part, const float* __restrict__ vnorm,
+__global__ void group_mean_kernel(int G, int64_t n, const float* part, const float* vnorm,
                                   float* __restrict__ attn_acc, float* __restrict__ score) {
   // a programmatic dependent of pass 2; the selection, its own dependent, may set up
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
+  const float norm = vnorm[i];
   float s = 0.f;
   for (int g = 0; g < G; ++g) s += part[(int64_t)g * n + i];       // fixed order
   s *= 1.f / (float)G;
   attn_acc[i] = s;
-  score[i] = s * vnorm[i];
+  score[i] = s * norm;
 }
 
 template <typename T, int GT, int TPR>

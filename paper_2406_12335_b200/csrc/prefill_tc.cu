@@ -27,6 +27,7 @@
 #include <cuda.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "vatp_internal.cuh"
 
@@ -478,7 +479,7 @@ __device__ __forceinline__ void side_value_norms(const TcArgs& a, int lane) {
       for (int j = 0; j < 16; ++j) {
         const int tok = it.tile * TILE + r0 + RPI * j + sub;
         raw[j] = make_uint4(0u, 0u, 0u, 0u);
-        if (tok < a.T) raw[j] = __ldg(reinterpret_cast<const uint4*>(vu + (int64_t)tok * a.st) + part);
+        if (tok < a.T) raw[j] = load_behind_wait(reinterpret_cast<const uint4*>(vu + (int64_t)tok * a.st) + part);
       }
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
@@ -671,7 +672,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
       const int tok = it.tile * TILE + row;       // query (pass 1) or key (pass 2) index of this thread
       // pass 2: this key's value norm, written by pass 1; fetched now, used in the item's epilogue
       float n1 = 0.f;
-      if (PASS == 2 && g == 0 && tok < a.T) n1 = __ldg(a.vnorm + (int64_t)kv_unit_of(a, u) * a.T + tok);
+      if (PASS == 2 && g == 0 && tok < a.T) n1 = load_behind_wait(a.vnorm + (int64_t)kv_unit_of(a, u) * a.T + tok);
       float m_run = -INFINITY, l_run = 0.f;       // pass 1
       f32x2 cs[2] = {pk2(0.f, 0.f), pk2(0.f, 0.f)};   // pass 2: four running sums, packed
       const uint32_t n0 = n;
@@ -1312,23 +1313,24 @@ __global__ void reset_counters_kernel(unsigned* counters) {
 // complete, and it runs beside that pass - small CTAs, for the registers a pass-1 CTA leaves on its SM - instead of before
 // it; only the first CTA stays until that pass has completed, so that whatever waits for this launch waits for both (32 heads
 // x 2048 tokens with a window of 256, scoring + selection + compaction + history: 70 -> 61 us with the counters' memset
-// gone).  With the caller's normalisers it stands in for pass 1 and waits first.
+// gone).  With the caller's normalisers (GIVEN) it stands in for pass 1 and waits first.
+// (Without them the values are complete, and read by __ldg: the windowed prompt above takes 0.3 us more with ordinary loads.)
 constexpr int VN_THREADS = 128, VN_TOKENS = 64;
-template <int HD, int KIND>
-__global__ void __launch_bounds__(VN_THREADS) vnorm_kernel(TcArgs a, const float* __restrict__ lse_in) {
-  if (lse_in) asm volatile("griddepcontrol.wait;" ::: "memory");
+template <int HD, int KIND, bool GIVEN>
+__global__ void __launch_bounds__(VN_THREADS) vnorm_kernel(TcArgs a, const float* lse_in) {
+  if (GIVEN) asm volatile("griddepcontrol.wait;" ::: "memory");
   // pass 2, a programmatic dependent, may set up while this kernel runs; it reads what is written here
   // only after its griddepcontrol.wait
   if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // (the grid is one-dimensional, all units of a group of tokens after one another: its other dimensions end at 65535)
   const int block = blockIdx.x / a.kv_units, u = blockIdx.x - block * a.kv_units;
-  if (lse_in) {
+  if (GIVEN) {
     // this CTA's tokens; the last CTA of the unit also fills the padding up to Tpad
     const int last = blockIdx.x + a.kv_units >= gridDim.x ? a.Tpad : (block + 1) * VN_TOKENS;
     for (int i = block * VN_TOKENS + threadIdx.x; i < last; i += VN_THREADS) {
       float x = -INFINITY;
       if (i < a.T) {
-        const float l = __ldg(lse_in + (int64_t)u * a.T + i);
+        const float l = load_behind_wait(lse_in + (int64_t)u * a.T + i);
         // (log2 e - 1.4426950408889634f = 1.925963e-8)
         if (i >= a.first_row) x = HD == 64 ? fmaf(-l, 1.4426950408889634f, fmaf(-l, 1.925963033e-8f, EX2_LOSS)) : -l * 1.4426950408889634f;
         if (a.lse_out && a.lse_out != lse_in) a.lse_out[(int64_t)u * a.T + i] = l;
@@ -1346,7 +1348,10 @@ __global__ void __launch_bounds__(VN_THREADS) vnorm_kernel(TcArgs a, const float
   for (int j = 0; j < NP; ++j) {
     const int tok = row0 + RPP * j;
     raw[j] = make_uint4(0u, 0u, 0u, 0u);
-    if (tok < a.T) raw[j] = __ldg(reinterpret_cast<const uint4*>(vu + (int64_t)tok * a.st) + part);
+    if (tok < a.T) {
+      const uint4* from = reinterpret_cast<const uint4*>(vu + (int64_t)tok * a.st) + part;
+      if (GIVEN) raw[j] = load_behind_wait(from); else raw[j] = __ldg(from);
+    }
   }
 #pragma unroll
   for (int j = 0; j < NP; ++j) {
@@ -1360,7 +1365,7 @@ __global__ void __launch_bounds__(VN_THREADS) vnorm_kernel(TcArgs a, const float
     const int tok = row0 + RPP * j;
     if (part == 0 && tok < a.T) a.vnorm[(int64_t)u * a.T + tok] = norm_finish(KIND, acc);
   }
-  if (!lse_in && blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (!GIVEN && blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 
@@ -1401,7 +1406,7 @@ struct RingSmem {
 template <int HD, bool GROUPED>
 __global__ void __launch_bounds__(RG_THREADS, GROUPED ? 1 : 2)
 window_ring_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kc, int heads, int G, int T,
-                      int w, int B, int cap, float scale_log2, float scale_lo, const float* __restrict__ lse, vatp_cache c,
+                      int w, int B, int cap, float scale_log2, float scale_lo, const float* lse, vatp_cache c,
                       int32_t* dev_status) {
   extern __shared__ unsigned char smem_raw[];
   constexpr int TILE_BYTES = tile_bytes<HD>, CHUNK_BYTES = chunk_bytes<HD>;
@@ -1478,7 +1483,7 @@ window_ring_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
       for (int i = tid; i < CHUNK; i += RG_THREADS) {
         const int r = c0 + i, j = T - w + r;
         const bool query = r < w && j >= 0;
-        const float l = query ? __ldg(lse_h + j) : 0.f, nl = -l * 1.4426950408889634f;
+        const float l = query ? load_behind_wait(lse_h + j) : 0.f, nl = -l * 1.4426950408889634f;
         sm.nlse[i] = query ? nl : -INFINITY;
         if constexpr (FINE) sm.nres[i] = fmaf(-l, 1.4426950408889634f, -nl) - l * 1.925963033e-8f + EX2_LOSS;   // (log2 e - 1.4426950408889634f)
       }
@@ -1725,8 +1730,11 @@ cudaError_t launch_prefill_hd(const Shape& s, const void* q, const void* k, cons
   if ((e = cudaLaunchKernelEx(&dr.cfg, reset_counters_kernel, a.counters)) != cudaSuccess) return e;
   auto value_norms = [&]() {
     DependentLaunch dv(dim3((unsigned)a.kv_units * ((s.T + VN_TOKENS - 1) / VN_TOKENS)), dim3(VN_THREADS), 0, st);
-    auto kern = a.norm == VATP_NORM_L1 ? vnorm_kernel<HD, VATP_NORM_L1> : a.norm == VATP_NORM_L2 ? vnorm_kernel<HD, VATP_NORM_L2> : vnorm_kernel<HD, VATP_NORM_LINF>;
-    return cudaLaunchKernelEx(&dv.cfg, kern, a, lse_in);
+    auto kernel_for = [&](auto given) {
+      constexpr bool G = decltype(given)::value;
+      return a.norm == VATP_NORM_L1 ? vnorm_kernel<HD, VATP_NORM_L1, G> : a.norm == VATP_NORM_L2 ? vnorm_kernel<HD, VATP_NORM_L2, G> : vnorm_kernel<HD, VATP_NORM_LINF, G>;
+    };
+    return cudaLaunchKernelEx(&dv.cfg, lse_in ? kernel_for(std::true_type{}) : kernel_for(std::false_type{}), a, lse_in);
   };
   if (attn_out) {
     // the forward sweep stands in for pass 1; it streams K and V, so a group's units share the L2 three ways

@@ -37,7 +37,7 @@ __device__ __forceinline__ uint32_t order_key(float x) {
 // of short phases; two or more CTAs per SM fill one another's).  copies: histograms the warps share out among them - one
 // for short ranges, where clearing and summing 32 of them took longer than the counting.
 template <bool STAGED, int THREADS>
-__global__ void __launch_bounds__(THREADS) select_kernel(int copies, int T, int B, int F, int R, const float* __restrict__ score,
+__global__ void __launch_bounds__(THREADS) select_kernel(int copies, int T, int B, int F, int R, const float* score,
                                                              int32_t* __restrict__ kept, int32_t* dev_status) {
   constexpr int WARPS = THREADS / 32;
   extern __shared__ __align__(16) uint32_t sel_smem[];
@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(THREADS) select_kernel(int copies, int T, int 
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int v = v0 + j * THREADS + tid;
-        if (v < nvec) x[j] = __ldg(src4 + v);
+        if (v < nvec) x[j] = load_behind_wait(src4 + v);
       }
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -306,7 +306,7 @@ __device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier
 __device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 __global__ void __launch_bounds__(SEL_THREADS) select_cluster_kernel(int T, int B, int F, int R, int split, int per,
-                                                                     const float* __restrict__ score, int32_t* __restrict__ kept,
+                                                                     const float* score, int32_t* __restrict__ kept,
                                                                      int32_t* dev_status) {
   extern __shared__ __align__(16) uint32_t keys_s[];  // keys of this CTA's part of the middle range
   __shared__ uint32_t hist[256];
@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(SEL_THREADS) select_cluster_kernel(int T, int 
     for (int i = tid; i < R; i += SEL_THREADS) out[B - R + i] = T - R + i;
   }
   const int lo_c = min(rank * per, n), hi_c = min(lo_c + per, n), n_c = hi_c - lo_c;    // this CTA's keys [lo_c, hi_c)
-  for (int i = tid; i < n_c; i += SEL_THREADS) keys_s[i] = order_key(__ldg(sc + F + lo_c + i));
+  for (int i = tid; i < n_c; i += SEL_THREADS) keys_s[i] = order_key(load_behind_wait(sc + F + lo_c + i));
   __syncthreads();
   cluster_wait_acquire();
 

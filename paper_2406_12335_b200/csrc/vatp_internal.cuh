@@ -64,6 +64,23 @@ __host__ __device__ inline int64_t unit_offset_lse(const Shape& s, int u) {
   return (int64_t)(u / s.heads) * s.lse_sb + (int64_t)(u % s.heads) * s.lse_sh;
 }
 
+// see DependentLaunch below (for memory that this kernel does not write itself)
+__device__ __forceinline__ float load_behind_wait(const float* p) {
+  float x;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(x) : "l"(p));
+  return x;
+}
+__device__ __forceinline__ float4 load_behind_wait(const float4* p) {
+  float4 x;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "l"(p));
+  return x;
+}
+__device__ __forceinline__ uint4 load_behind_wait(const uint4* p) {
+  uint4 x;
+  asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w) : "l"(p));
+  return x;
+}
+
 __device__ __forceinline__ float to_f32(float x) { return x; }
 __device__ __forceinline__ float to_f32(__nv_bfloat16 x) { return __bfloat162float(x); }
 
@@ -90,7 +107,8 @@ bool make_row_gather_map(CUtensorMap* m, const void* base, uint32_t row_words, u
 // releases its dependents, everything older is complete by the time that this kernel starts, and needs no wait.)
 // What it reads it reads by ordinary loads: the read-only path - __ldg, or a `const ... __restrict__` parameter, for which the
 // compiler may take it - is for memory that nobody writes while the kernel is resident, and nothing holds such a load
-// behind the wait.
+// behind the wait.  load_behind_wait() is an ordinary load that the compiler keeps in the order of the asm statements around
+// it, the waits, but not of the stores: a batch of them is in flight at once also where the results are stored in between.
 struct DependentLaunch {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];

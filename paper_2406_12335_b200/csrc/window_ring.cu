@@ -28,7 +28,7 @@ namespace {
 constexpr int RW_MAX_CLUSTER = 8;
 template <typename T, int D>
 __global__ void __launch_bounds__(NTHREADS)
-window_ring_fma_kernel(Shape sh, int G, int B, int cap, const T* __restrict__ q, int64_t q_head, const float* __restrict__ lse,
+window_ring_fma_kernel(Shape sh, int G, int B, int cap, const T* q, int64_t q_head, const float* lse,
                        vatp_cache c, int cs) {
   using Tl = Tile<4, D>;
   constexpr int ROWS = Tl::ROWS, LD = Tl::LD, NV = Tl::NV;

@@ -10,6 +10,9 @@ import re
 import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2406_12335_b200", "csrc")
+# What is complete before the kernel starts: the value norms' kernel follows a pass that has waited itself before it lets this
+# one start, unless the caller's normalisers stand in for that pass.
+COMPLETE = {"prefill_tc.cu": ["if (GIVEN) raw[j] = load_behind_wait(from); else raw[j] = __ldg(from);"]}
 
 
 def _code(name):
@@ -48,6 +51,11 @@ def _dependent_kernels(text):
 
 @pytest.mark.parametrize("name,kernels", [
     ("prefill_simt.cu", {"rowstats_kernel", "colsum_kernel"}),
+    ("prefill_tc.cu", {"prefill_tc_kernel", "attention_fwd_tc_kernel", "reset_counters_kernel", "vnorm_kernel", "window_ring_tc_kernel"}),
+    ("select.cu", {"select_kernel", "select_cluster_kernel"}),
+    ("compact.cu", {"compact_kernel"}),
+    ("window_ring.cu", {"window_ring_fma_kernel"}),
+    ("decode_gqa.cu", {"group_mean_kernel"}),
 ])
 def test_dependents_read_by_ordinary_loads(name, kernels):
     text = _code(name)
@@ -57,4 +65,8 @@ def test_dependents_read_by_ordinary_loads(name, kernels):
         read_only = re.findall(r"const\s+[\w:]+\s*\*\s*__restrict__\s+\w+", params)
         assert not read_only, (kernel, read_only)
     for f in (name, "simt_tile.cuh", "vatp_internal.cuh"):
-        assert "__ldg" not in _code(f) and "ld.global.nc" not in _code(f), f
+        code = _code(f)
+        for known in COMPLETE.get(f, ()):
+            assert code.count(known) == 1
+            code = code.replace(known, "")
+        assert "__ldg" not in code and "ld.global.nc" not in code, f

@@ -21,6 +21,8 @@
 // a window of 256: 58.5 -> 51.7; 8 heads x 700 x 64: 67.5 -> 64.3.  128 x 128 tiles (32 heads x 2048 x 128) do not care: 974 us.
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "simt_tile.cuh"
 
 namespace cg = cooperative_groups;
@@ -135,12 +137,16 @@ __global__ void __launch_bounds__(NTHREADS, M == 8 ? 2 : 1) rowstats_kernel(Shap
   }
 }
 
+// Queries, keys and values of pass 2.  128-row tiles read them by the read-only path (32 heads x 2048 x 128 971 us, 1004 with
+// ordinary loads): they are complete before the kernel starts, see launch_m.
+template <typename T, int M> using Input = std::conditional_t<M == 8, const T* __restrict__, const T*>;
+
 // Pass 2: one cluster per (key tile, unit), its CTAs take every cs-th query tile.  Column sums over query rows
 // j >= max(first_row, k).
 template <typename T, int M, int D>
 __global__ void __launch_bounds__(NTHREADS, M == 8 ? 2 : 1)
-colsum_kernel(Shape sh, const T* q, const T* k, const T* v, const float* lse, float* __restrict__ attn_acc, float* __restrict__ vnorm,
-              float* __restrict__ score, float* __restrict__ win_rows, int first_row, int cs, bool after_pass1) {
+colsum_kernel(Shape sh, Input<T, M> q, Input<T, M> k, Input<T, M> v, const float* lse, float* __restrict__ attn_acc,
+              float* __restrict__ vnorm, float* __restrict__ score, float* __restrict__ win_rows, int first_row, int cs, bool after_pass1) {
   constexpr int ROWS = Tile<M, D>::ROWS, LD = Tile<M, D>::LD, NV = Tile<M, D>::NV;
   extern __shared__ __align__(16) float smem[];
   constexpr int DS = M == 4 ? D : 64;   // channels of the streamed tile in shared memory at a time
@@ -301,6 +307,11 @@ cudaError_t launch_m(const Shape& s, const T* q, const T* k, const T* v, float* 
   }
   const int cs = cluster_for(ktiles, qtiles);
   ClusterLaunch c2(dim3((unsigned)(ktiles * s.units * cs)), smem2, st, cs);
+  // Large tiles with the normalisers given, i.e. no pass 1 that has waited for what came before: an ordinary launch, when
+  // everything is complete.  32 heads x 2048 x 128 506 -> 486 us, 50 x 700 x 64 106 -> 89 (as a dependent the next such call
+  // takes SMs from this one), 32 x 2048 x 64 284 -> 288.  Short calls would lose the launch's latency (2 x 512 x 64 9.4 -> 10.7)
+  // and stay dependents, with ordinary loads.
+  if (M == 8 && lse_given) c2.attr[0].val.programmaticStreamSerializationAllowed = 0;
   return cudaLaunchKernelEx(&c2.cfg, colsum_kernel<T, M, D>, s, q, k, v, (const float*)lse, attn_acc, vnorm, score,
                             s.window > 0 ? win_rows : nullptr, first_row, cs, !lse_given);
 }

@@ -10,9 +10,14 @@ import re
 import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2406_12335_b200", "csrc")
-# What is complete before the kernel starts: the value norms' kernel follows a pass that has waited itself before it lets this
-# one start, unless the caller's normalisers stand in for that pass.
-COMPLETE = {"prefill_tc.cu": ["if (GIVEN) raw[j] = load_behind_wait(from); else raw[j] = __ldg(from);"]}
+# What is complete before the kernel starts: the value norms' kernel and the fp32 pass 2 follow a pass that has waited itself
+# before it lets them start, unless the caller's normalisers stand in for that pass; the large tiles are no dependents then.
+COMPLETE = {"prefill_tc.cu": ["if (GIVEN) raw[j] = load_behind_wait(from); else raw[j] = __ldg(from);"],
+            "prefill_simt.cu": ["template <typename T, int M> using Input = std::conditional_t<M == 8, const T* __restrict__, const T*>;"]}
+
+
+def test_large_fp32_tiles_without_a_pass_before_them_are_launched_ordinarily():
+    assert "if (M == 8 && lse_given) c2.attr[0].val.programmaticStreamSerializationAllowed = 0;" in _code("prefill_simt.cu")
 
 
 def _code(name):
@@ -62,7 +67,7 @@ def test_dependents_read_by_ordinary_loads(name, kernels):
     found = _dependent_kernels(text)
     assert {k for k, _, _ in found} == kernels
     for kernel, params, _ in found:
-        read_only = re.findall(r"const\s+[\w:]+\s*\*\s*__restrict__\s+\w+", params)
+        read_only = re.findall(r"const\s+[\w:]+\s*\*\s*__restrict__", params)
         assert not read_only, (kernel, read_only)
     for f in (name, "simt_tile.cuh", "vatp_internal.cuh"):
         code = _code(f)
@@ -70,3 +75,4 @@ def test_dependents_read_by_ordinary_loads(name, kernels):
             assert code.count(known) == 1
             code = code.replace(known, "")
         assert "__ldg" not in code and "ld.global.nc" not in code, f
+        assert not re.search(r"(using|typedef).*__restrict__", code), f

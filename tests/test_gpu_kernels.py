@@ -514,42 +514,92 @@ def test_fp32_scoring_tiles_against_float64(d, units, T, window, call, norm, til
     assert torch.equal(score, acc * vnorm)
 
 
-@pytest.mark.parametrize("d,units,T,window", [
-    (64, 1, 1, 0),          # one token
-    (64, 1, 64, 0),         # one tile, no cluster
-    (64, 3, 65, 0),         # two tiles, one row in the second
-    (128, 2, 200, 0),       # clusters of four
-    (64, 2, 513, 0),        # clusters of eight, more CTAs than the first rows have key tiles
-    (128, 1, 700, 33),      # a window of less than a tile: pass 1 in one cluster a unit
-    (64, 9, 449, 0),        # clusters of two
+def _simt_clusters(units, T, window):
+    """Tile rows and the two passes' cluster sizes of an fp32 scoring call on 148 SMs."""
+    rows = window if 0 < window < T else T
+    size = 128 if units * ((rows + 127) // 128) >= 2 * 148 else 64
+    qtiles, ktiles = (rows + size - 1) // size, (T + size - 1) // size
+
+    def clusters(tiles, most):
+        cs = 1
+        while cs < 8 and tiles * units * cs * 2 <= 2 * 148 and cs < most:
+            cs *= 2
+        return cs
+    return size, clusters(qtiles, ktiles), clusters(ktiles, qtiles)
+
+
+@pytest.mark.parametrize("d,units,kv,T,window,call,plan", [
+    (64, 1, 0, 1, 0, "scores", (64, 1, 1)),         # one token
+    (64, 1, 0, 64, 0, "scores", (64, 1, 1)),        # one tile
+    (64, 3, 0, 66, 0, "scores", (64, 2, 2)),        # two tiles, two rows in the second
+    (128, 2, 0, 200, 0, "scores", (64, 4, 4)),
+    (64, 2, 0, 514, 0, "scores", (64, 8, 8)),       # more CTAs than the first rows have key tiles
+    (128, 1, 0, 700, 33, "scores", (64, 8, 1)),     # a window of less than a tile
+    (64, 9, 0, 450, 0, "scores", (64, 4, 4)),
+    (64, 8, 0, 700, 0, "scores", (64, 2, 2)),       # up to six tiles per CTA of a cluster
+    (64, 50, 0, 700, 0, "scores", (128, 1, 1)),     # the large tiles
+    (128, 50, 0, 700, 0, "scores", (128, 1, 1)),
+    (64, 8, 2, 514, 0, "scores", (64, 8, 8)),       # grouped queries: four rounds of both passes, on two units each
+    (64, 200, 100, 300, 0, "scores", (128, 1, 1)),
+    (64, 2, 0, 514, 0, "lse", (64, 8, 8)),          # normalisers given: pass 2 alone
+    (64, 50, 0, 700, 0, "lse", (128, 1, 1)),
+    (64, 3, 0, 514, 100, "lse", (64, 8, 2)),
 ])
-def test_fp32_scoring_right_behind_the_inputs(d, units, T, window):
-    """The fp32 passes with clusters of every size, enqueued right behind the kernels that write their inputs, over and over:
-    pass 2 fetches its first tiles before pass 1 has finished, and the CTAs of a cluster send their parts to one of them."""
+def test_fp32_scoring_right_behind_a_kernel_that_releases_it_early(d, units, kv, T, window, call, plan):
+    """The fp32 passes enqueued right behind the kernel that writes their queries, keys and values and that lets its dependents
+    start long before: another scoring call, whose indicators, norms and scores are the inputs.  With clusters of every size and
+    both tiles, over and over on the same buffers: an input read too early is the one of the round before."""
     V = P.vatp()
-    p = V.make_params(batch=1, heads=units, seq_len=T, head_dim=d, dtype="f32", budget=T, indicator="window" if window else "h2o",
-                      window=window)
+    hk = kv or units
+    assert _simt_clusters(hk, T, window) == plan
     f32 = dict(dtype=torch.float32, device="cuda")
-    g = torch.Generator(device="cuda").manual_seed(17)
-    sets = [torch.randn(3, 1, units, T, d, generator=g, **f32) for _ in range(4)]
-    x = torch.empty_like(sets[0])
-    out = torch.zeros(4, 4, 1, units, T, **f32)
-    ws = torch.empty(max(V.vatp_workspace_bytes(p), 256), dtype=torch.uint8, device="cuda")
-    status = torch.zeros(1, dtype=torch.int32, device="cuda")
-    for i in range(4):
-        x.copy_(sets[i])
-        V.vatp_prefill_scores(p, x[0], x[1], x[2], lse_out=out[i, 0], attn_acc=out[i, 1], vnorm=out[i, 2], score=out[i, 3], workspace=ws,
-                              dev_status=status)
+    g = torch.Generator(device="cuda").manual_seed(T + d)
+    n = units * T * d
+    T0 = 128 if n % 128 == 0 else 64                  # the writer: short prompts, as many as it takes
+    assert n % T0 == 0
+    p0 = V.make_params(batch=1, heads=n // T0, seq_len=T0, head_dim=64, dtype="f32", budget=T0)
+    p = V.make_params(batch=1, heads=units, kv_heads=kv, seq_len=T, head_dim=d, dtype="f32", budget=T, scale=0.001,
+                      indicator="window" if window else "h2o", window=window)
+    first = max(T - window, 0) if window else 0
+    sources = [torch.randn(1, n // T0, T0, 64, generator=g, **f32) for _ in range(3)]
+    made, ws0 = torch.zeros(3, 1, n // T0, T0, **f32), torch.empty(V.vatp_workspace_bytes(p0), dtype=torch.uint8, device="cuda")
+    ws, status = torch.empty(V.vatp_workspace_bytes(p), dtype=torch.uint8, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    rows = [made[0].view(1, units, T, d)] + [made[i].view(-1)[:hk * T * d].view(1, hk, T, d) for i in (1, 2)]
+
+    def write(src):
+        V.vatp_prefill_scores(p0, src, src, src, attn_acc=made[0], vnorm=made[1], score=made[2], workspace=ws0, dev_status=status)
+
+    def score(given):
+        lse = torch.zeros(1, units, T, **f32)
+        out = torch.zeros(3, 1, hk, T, **f32)
+        to = dict(attn_acc=out[0], vnorm=out[1], score=out[2], workspace=ws, dev_status=status)
+        if call == "lse":
+            return lambda: V.vatp_prefill_scores_from_lse(p, *rows, given, lse_out=lse, **to), lse, out
+        return lambda: V.vatp_prefill_scores(p, *rows, lse_out=lse, **to), lse, out
+
+    want = []
+    for src in sources:
+        write(src)
+        torch.cuda.synchronize()
+        q, k, v = (x.double() for x in rows)
+        s = (q @ k.repeat_interleave(units // hk, 1).transpose(-1, -2)) * p.scale
+        s.masked_fill_(torch.ones(T, T, dtype=torch.bool, device="cuda").triu(1), -torch.inf)
+        lse = torch.logsumexp(s, -1)
+        acc = torch.softmax(s, -1)[..., first:, :].sum(-2).view(1, hk, units // hk, T).mean(2)
+        norm = v.abs().sum(-1)
+        want.append((lse.float(), lse, acc, norm))
+        del s
+    calls = [score(want[i % 3][0]) for i in range(9)]
+    torch.cuda.synchronize()
+    for i, (run, _, _) in enumerate(calls):
+        write(sources[i % 3])
+        run()
     torch.cuda.synchronize()
     assert int(status) == 0
-    first = T - window if window else 0
-    for i in range(4):
-        q, k, v = sets[i].double()
-        s = (q @ k.transpose(-1, -2)) * p.scale
-        s.masked_fill_(torch.ones(T, T, dtype=torch.bool, device="cuda").triu(1), -torch.inf)
-        acc = torch.softmax(s, -1)[..., first:, :].sum(-2)
-        norm = v.abs().sum(-1)
-        tol = P.TOL["f32"]
-        assert (out[i, 0].double() - torch.logsumexp(s, -1))[..., first:].abs().max() <= 10 * tol
-        for got, want in ((out[i, 1], acc), (out[i, 2], norm), (out[i, 3], acc * norm)):
-            assert ((got.double() - want).abs() <= tol * want + 1e-30).all()
+    tol = P.TOL["f32"]
+    for i, (_, lse, out) in enumerate(calls):
+        _, want_lse, acc, norm = want[i % 3]
+        assert (lse.double() - want_lse)[..., first:].abs().max() <= 10 * tol
+        for got, ref in ((out[0], acc), (out[1], norm), (out[2], acc * norm)):
+            assert ((got.double() - ref).abs() <= 2 * tol * ref + 1e-30).all()      # (the score: two factors)
+        assert torch.equal(out, calls[i % 3][2])

@@ -98,7 +98,7 @@ __device__ __forceinline__ bool evicts_before(float Ia, int pa, float Ib, int pb
 template <typename T, int D, bool WINDOWED>
 __global__ void __launch_bounds__(DEC_THREADS)
 decode_kernel(int split, int chunk, int B, int cap, int F, int R, int w, int norm, float scale_log2, vatp_cache c,
-              const T* __restrict__ q_new, const T* __restrict__ k_new, const T* __restrict__ v_new,
+              const T* q_new, const T* k_new, const T* v_new,
               T* __restrict__ out, int32_t* __restrict__ evicted, int32_t* __restrict__ dev_status) {
   constexpr int EPV = Vec16<T>::N;       // elements per 16-byte vector
   constexpr int LPR = D / EPV;           // lanes per row

@@ -212,8 +212,8 @@ __global__ void __launch_bounds__(FEED ? DM_THREADS : WT, 2)
 decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, int independent, int G,
                   int units, int state_in_smem, int part_in_ring, int split, int chunk, int ld, int nslot, int B, int cap, int F, int R, int w, int norm,
                   float scale_log2, vatp_cache c,
-                  const __nv_bfloat16* __restrict__ q_new, const __nv_bfloat16* __restrict__ k_new,
-                  const __nv_bfloat16* __restrict__ v_new, __nv_bfloat16* __restrict__ out,
+                  const __nv_bfloat16* q_new, const __nv_bfloat16* k_new,
+                  const __nv_bfloat16* v_new, __nv_bfloat16* __restrict__ out,
                   int32_t* __restrict__ evicted, int32_t* __restrict__ dev_status) {
   constexpr int UNIT = unit_bytes<HD>, ROW_CHUNKS = HD / 8;   // 16-byte chunks of a row
   static_assert(WT >= HD, "one thread per output channel");
@@ -453,15 +453,15 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   const int t = c.next_pos[u];
   const int ls_m = c.last_slot[u];
   uint4 new_raw = make_uint4(0u, 0u, 0u, 0u), last_raw = make_uint4(0u, 0u, 0u, 0u);
-  if (!FEED && has_chunk) new_raw = __ldg(reinterpret_cast<const uint4*>((lane < 16 ? k_new : v_new) + (int64_t)u * HD) + (lane & 15));
+  if (!FEED && has_chunk) new_raw = load_behind_wait(reinterpret_cast<const uint4*>((lane < 16 ? k_new : v_new) + (int64_t)u * HD) + (lane & 15));
   // B operand of K q^T: q in every column (grouped queries: column g carries head g of the unit's group, columns beyond the
   // group repeat its last head)
   const __nv_bfloat16* qn = GT > 1 ? q_new + ((int64_t)u * G + min(lane >> 2, G - 1)) * HD : q_new + (int64_t)u * HD;
   uint32_t qb[HD / 16][2];
 #pragma unroll
   for (int ks = 0; ks < HD / 16; ++ks) {
-    qb[ks][0] = __ldg(reinterpret_cast<const uint32_t*>(qn + ks * 16 + 2 * j4));
-    qb[ks][1] = __ldg(reinterpret_cast<const uint32_t*>(qn + ks * 16 + 8 + 2 * j4));
+    qb[ks][0] = load_behind_wait(reinterpret_cast<const uint32_t*>(qn + ks * 16 + 2 * j4));
+    qb[ks][1] = load_behind_wait(reinterpret_cast<const uint32_t*>(qn + ks * 16 + 8 + 2 * j4));
   }
 #ifdef VATP_DEBUG_BOUNDS
   // the state words come from memory: out of range they are clamped and reported (every access below stays inside)
@@ -484,7 +484,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
   // the new row's norm is needed by the thread that updates its slot
   const int norm_warp = owns_new ? (fs_local % WT) / 32 : -1;
   if (FEED && has_chunk && (wid == new_warp || wid == norm_warp))
-    new_raw = __ldg(reinterpret_cast<const uint4*>((lane < 16 ? k_new : v_new) + (int64_t)u * HD) + (lane & 15));
+    new_raw = load_behind_wait(reinterpret_cast<const uint4*>((lane < 16 ? k_new : v_new) + (int64_t)u * HD) + (lane & 15));
   if (has_chunk && wid == last_warp)
     last_raw = *(reinterpret_cast<const uint4*>((const __nv_bfloat16*)(lane < 16 ? c.k_cache : c.v_cache) +
                                                 ((int64_t)u * cap + ls) * HD) + (lane & 15));

@@ -70,6 +70,11 @@ __device__ __forceinline__ float load_behind_wait(const float* p) {
   asm volatile("ld.global.f32 %0, [%1];" : "=f"(x) : "l"(p));
   return x;
 }
+__device__ __forceinline__ uint32_t load_behind_wait(const uint32_t* p) {
+  uint32_t x;
+  asm volatile("ld.global.u32 %0, [%1];" : "=r"(x) : "l"(p));
+  return x;
+}
 __device__ __forceinline__ float4 load_behind_wait(const float4* p) {
   float4 x;
   asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "l"(p));

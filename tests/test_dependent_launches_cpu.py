@@ -61,6 +61,8 @@ def _dependent_kernels(text):
     ("compact.cu", {"compact_kernel"}),
     ("window_ring.cu", {"window_ring_fma_kernel"}),
     ("decode_gqa.cu", {"group_mean_kernel"}),
+    ("decode.cu", {"decode_kernel"}),
+    ("decode_mma.cu", {"decode_mma_kernel"}),
 ])
 def test_dependents_read_by_ordinary_loads(name, kernels):
     text = _code(name)

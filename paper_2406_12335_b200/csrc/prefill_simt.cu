@@ -12,13 +12,15 @@
 //     where one element per load made it 8 per 16.  The next tile's rows are on their way to registers under the products (M = 4);
 //   * few tiles are shared out over a cluster of up to eight CTAs along the other dimension, which combine their row
 //     statistics or column sums through distributed shared memory;
-//   * both passes are programmatic dependents: they are resident when the launch before them ends, and pass 2 has its first
-//     tiles and the value norms by then, which depend on nothing that pass 1 writes;
+//   * both passes are programmatic dependents: they are resident when the launch before them ends, and by then pass 2 has its
+//     key tile and, with 64-row tiles, its first query tile and the value norms, which depend on nothing that pass 1 writes;
 //   * the CTAs of a cluster push their partial results to rank 0 and meet once: with rank 0 reading them from its partners
-//     there were two meetings and a round trip between them.  Both operands of the first product travel together, and the 16
-//     threads of a row agree on its maximum before they exponentiate.
-// The scoring call, 2 heads x 512 tokens x 64 channels: 20.1 us before the last two points, 15.9 now; 12 heads of 128, 512 tokens,
-// a window of 256: 58.5 -> 51.7; 8 heads x 700 x 64: 67.5 -> 64.3.  128 x 128 tiles (32 heads x 2048 x 128) do not care: 974 us.
+//     there were two meetings and a round trip between them.  The 16 threads of a row agree on its maximum before they
+//     exponentiate.
+// The scoring call, us: pass 2 starting late / two meetings a cluster / the rows merged pair by pair / all three / as it is:
+// 2 heads x 512 tokens x 64 channels 18.3 / 17.2 / 17.0 / 20.4 / 16.0; 12 heads of 128, 512 tokens, a window of 256
+// 53.2 / 54.2 / 52.4 / 58.5 / 50.8; 8 heads x 700 x 64 66.0 / 65.1 / 64.9 / 67.9 / 64.2.  128-row tiles (no clusters): 50 heads x
+// 700 x 64 203.1 / - / 203.9 / 204.4 / 202.1; the row merge is worth more there than the 36 bytes of registers that it spills.
 #include <cooperative_groups.h>
 
 #include <type_traits>
@@ -68,9 +70,9 @@ __global__ void __launch_bounds__(NTHREADS, M == 8 ? 2 : 1) rowstats_kernel(Shap
   {
     float4 r[NV];
     Tile<M, D>::fetch(r, qu, sh.st, q0, min(ROWS, sh.T - q0));
-    if constexpr (M == 4)      // (on its way together with the queries)
-      if (rank * ROWS < last_key) Tile<M, D>::fetch(next, ku, sh.st, rank * ROWS, min(ROWS, sh.T - rank * ROWS));
     Tile<M, D>::store(Qs, r);
+    if constexpr (M == 4)
+      if (rank * ROWS < last_key) Tile<M, D>::fetch(next, ku, sh.st, rank * ROWS, min(ROWS, sh.T - rank * ROWS));
   }
   for (int k0 = rank * ROWS; k0 < last_key; k0 += cs * ROWS) {
     float s[M][M];
@@ -179,9 +181,9 @@ colsum_kernel(Shape sh, Input<T, M> q, Input<T, M> k, Input<T, M> v, const float
   {
     float4 r[NV];
     Tile<M, D>::fetch(r, ku, sh.st, k0, keys_valid);
+    Tile<M, D>::store(Ks, r);
     if constexpr (M == 4)
       if (qfirst < sh.T) Tile<M, D>::fetch(next, qu, sh.st, qfirst, min(ROWS, sh.T - qfirst));
-    Tile<M, D>::store(Ks, r);
   }
   // value norms (Eq. 4): four threads per row, by the last CTA of the cluster, which has the fewest query tiles
   auto value_norms = [&]() {

@@ -30,9 +30,6 @@ namespace cg = cooperative_groups;
 namespace vatp {
 namespace {
 
-__device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-
 constexpr int GQ_THREADS = 512;
 constexpr int GQ_WARPS = GQ_THREADS / 32;
 constexpr size_t GQ_MAX_SMEM = 200 * 1024;     // dynamic shared memory of a CTA

@@ -15,8 +15,9 @@
 //   * both passes are programmatic dependents: they are resident when the launch before them ends, and by then pass 2 has its
 //     key tile and, with 64-row tiles, its first query tile and the value norms, which depend on nothing that pass 1 writes;
 //   * the CTAs of a cluster push their partial results to rank 0 and meet once: with rank 0 reading them from its partners
-//     there were two meetings and a round trip between them.  The 16 threads of a row agree on its maximum before they
-//     exponentiate.
+//     there were two meetings and a round trip between them.  (Rank 0's shared memory must have been claimed by then: every
+//     CTA announces itself at once and waits for the others only when it sends, long after.)  The 16 threads of a row agree on
+//     its maximum before they exponentiate.
 // The scoring call, us: pass 2 starting late / two meetings a cluster / the rows merged pair by pair / all three / as it is:
 // 2 heads x 512 tokens x 64 channels 18.3 / 17.2 / 17.0 / 20.4 / 16.0; 12 heads of 128, 512 tokens, a window of 256
 // 53.2 / 54.2 / 52.4 / 58.5 / 50.8; 8 heads x 700 x 64 66.0 / 65.1 / 64.9 / 67.9 / 64.2.  128-row tiles (no clusters): 50 heads x
@@ -34,11 +35,6 @@ namespace {
 
 constexpr int MAX_CLUSTER = 8;
 
-// The CTAs of a cluster send what they have to rank 0's shared memory, which must have been claimed by then: every CTA
-// announces itself at once and waits for the others only when it sends, long after.
-__device__ __forceinline__ void cluster_announce() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_all_there() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
-
 // Pass 1: one cluster per (query tile, unit), its CTAs take every cs-th key tile.  lse[j] over keys i <= j.
 template <typename T, int M, int D>
 __global__ void __launch_bounds__(NTHREADS, M == 8 ? 2 : 1) rowstats_kernel(Shape sh, const T* q, const T* k,
@@ -48,7 +44,7 @@ __global__ void __launch_bounds__(NTHREADS, M == 8 ? 2 : 1) rowstats_kernel(Shap
   float* Qs = smem;
   float* Ks = smem + D * LD;
   __shared__ float2 part[M == 4 ? MAX_CLUSTER : 1][ROWS];      // (M = 8 has tiles enough without clusters)
-  if (cs > 1) cluster_announce();
+  if (cs > 1) cluster_arrive_relaxed();
   // nothing is read before all earlier work has completed; pass 2 may set up from then on
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -106,7 +102,7 @@ __global__ void __launch_bounds__(NTHREADS, M == 8 ? 2 : 1) rowstats_kernel(Shap
     }
   }
   // merge the 16 threads (same ty, consecutive lanes) that share each row: the maximum first, then one factor a thread
-  if (cs > 1) cluster_all_there();
+  if (cs > 1) cluster_wait_acquire();
 #pragma unroll
   for (int i = 0; i < M; ++i) {
     float mx = m[i];
@@ -157,7 +153,7 @@ colsum_kernel(Shape sh, Input<T, M> q, Input<T, M> k, Input<T, M> v, const float
   float* lse_s = Qs + DS * LD;          // [ROWS]
   float* red = Qs;                      // [16][ROWS], once the products are done (DS >= 16)
   __shared__ float vn_s[ROWS], part[M == 4 ? MAX_CLUSTER : 1][ROWS];
-  if (cs > 1) cluster_announce();
+  if (cs > 1) cluster_arrive_relaxed();
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = cs > 1 ? (int)cluster.block_rank() : 0;
   const int item = blockIdx.x / cs, u = item % sh.units;      // the longest columns of all units first
@@ -264,7 +260,7 @@ colsum_kernel(Shape sh, Input<T, M> q, Input<T, M> k, Input<T, M> v, const float
     for (int t = 0; t < 16; ++t) tot += red[t * ROWS + threadIdx.x];
   }
   if (cs > 1) {
-    cluster_all_there();
+    cluster_wait_acquire();
     if ((int)threadIdx.x < ROWS) {
       cluster.map_shared_rank(&part[0][0], 0)[(M == 4 ? rank : 0) * ROWS + threadIdx.x] = tot;
       if (rank == cs - 1) cluster.map_shared_rank(vn_s, 0)[threadIdx.x] = vn_s[threadIdx.x];

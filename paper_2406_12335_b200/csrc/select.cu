@@ -302,8 +302,6 @@ struct SelExchange {
   uint32_t hist[2][SEL_MAXSPLIT][256];     // per pass parity and rank: that CTA's bin totals
   uint32_t n_gt[SEL_MAXSPLIT], n_eq[SEL_MAXSPLIT];
 };
-__device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 __global__ void __launch_bounds__(SEL_THREADS) select_cluster_kernel(int T, int B, int F, int R, int split, int per,
                                                                      const float* score, int32_t* __restrict__ kept,

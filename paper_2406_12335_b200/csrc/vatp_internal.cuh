@@ -64,6 +64,11 @@ __host__ __device__ inline int64_t unit_offset_lse(const Shape& s, int u) {
   return (int64_t)(u / s.heads) * s.lse_sb + (int64_t)(u % s.heads) * s.lse_sh;
 }
 
+// The halves of a cluster's barrier, for all threads of all its CTAs; relaxed: nothing that was written before is handed over.
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
 // see DependentLaunch below (for memory that this kernel does not write itself)
 __device__ __forceinline__ float load_behind_wait(const float* p) {
   float x;
